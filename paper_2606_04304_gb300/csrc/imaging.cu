@@ -14,8 +14,8 @@
 //      transform, which is exact because the mirror's footprint is the point
 //      reflection), with a separable 7 x 7 prolate-spheroidal kernel.  The uv
 //      position of a baseline moves by a fraction of a cell across a call's
-//      channels, so the host lists, once per call, the baselines that can
-//      touch each 4 x 8-cell tile of the grid; k_grid_tiles gives every tile
+//      channels, so the k_plan_* kernels list, once per call, the baselines that
+//      can touch each 4 x 4-cell tile of the grid; k_grid_tiles gives every tile
 //      to one warp whose 32 lanes are 32 adjacent channels: each lane takes
 //      the tile's records for its own channel (exact uv, keep test, weights)
 //      and accumulates the tile in registers, so no cell is written by two
@@ -74,36 +74,6 @@ struct ChanScale {
 
 __host__ __device__ __forceinline__ long long bl_index(int a, int b, int n) {
   return static_cast<long long>(a) * n - static_cast<long long>(a) * (a - 1) / 2 + (b - a);
-}
-
-__global__ void k_baselines(const double* __restrict__ ant, int n_ant, Baseline* __restrict__ out) {
-  const int a = blockIdx.y;
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= n_ant || b <= a) return;
-  const long long bl = bl_index(a, b, n_ant);
-  Baseline B;
-  B.dx = ant[3 * a] - ant[3 * b];
-  B.dy = ant[3 * a + 1] - ant[3 * b + 1];
-  B.dxh = static_cast<float>(B.dx);
-  B.dxl = static_cast<float>(B.dx - static_cast<double>(B.dxh));
-  B.dyh = static_cast<float>(B.dy);
-  B.dyl = static_cast<float>(B.dy - static_cast<double>(B.dyh));
-  B.bl = bl;
-  out[bl - a - 1] = B;            // cross baselines in (a, b), a < b, row-major order
-}
-
-__global__ void k_chan_scale(const double* __restrict__ freq, int n_chan, int n, double cell,
-                             ChanScale* __restrict__ out) {
-  const int f = blockIdx.x * blockDim.x + threadIdx.x;
-  if (f >= n_chan) return;
-  const double du = 1.0 / (static_cast<double>(n) * cell);
-  const double s = freq[f] / (kCLight * du);
-  ChanScale c;
-  c.s = s * static_cast<double>(kQ);          // exact: Q is a power of two
-  c.nu_c = freq[f] / kCLight;
-  c.sh = static_cast<float>(c.s);
-  c.sl = static_cast<float>(c.s - static_cast<double>(c.sh));
-  out[f] = c;
 }
 
 // rint(fl64(x * s)) decided in FP32: a float-float product, exact unless the
@@ -165,6 +135,9 @@ __global__ void k_uvw(const Baseline* __restrict__ base, int n_cross, const Chan
   pu[o] = static_cast<int32_t>(u > lim ? lim : (u < -lim ? -lim : u));
   pv[o] = static_cast<int32_t>(v > lim ? lim : (v < -lim ? -lim : v));
 }
+
+// device counters of one call's plan (ImgWs::counts)
+constexpr int kCountListed = 0, kCountRows = 1, kCountTiles = 2, kCounts = 3;
 
 struct GridEntry {
   int bl;            // baseline index in the visibility record
@@ -253,16 +226,17 @@ __host__ __device__ constexpr int tab_mirror(int g) { return 2 * (kTabD - g / 2)
 // visibilities are read (a warp reads consecutive baselines of one channel:
 // nearly sequential 32-byte records), and the records are turned around in
 // shared memory so each baseline's 32 channel records are stored as one
-// 512-byte run ([group][listed][lane]).  Kept visibilities are counted per
+// 512-byte run ([group][listed][lane], n_cross listed slots per group).  Kept visibilities are counted per
 // channel.
 constexpr int kPrepBl = 64;          // listed baselines per CTA of k_grid_prep
 constexpr int kPrepCh = kLanes / 8;  // channels per warp (8 warps)
 
 template <int LOG2G, bool CAL, bool BASES>
 __global__ void __launch_bounds__(256, CAL ? 1 : 4)
-k_grid_prep(const GridEntry* __restrict__ listed, int n_listed, const int32_t* __restrict__ vis, long long n_bl,
-            const Baseline* __restrict__ base, const ChanScale* __restrict__ cs, int ch0, int nb,
-            int* __restrict__ kept, PrepRec* __restrict__ prep, GridOpts opt) {
+k_grid_prep(const GridEntry* __restrict__ listed, const unsigned long long* __restrict__ counts, long long n_cross,
+            const int32_t* __restrict__ vis, long long n_bl, const Baseline* __restrict__ base,
+            const ChanScale* __restrict__ cs, int ch0, int nb, int* __restrict__ kept, PrepRec* __restrict__ prep,
+            GridOpts opt) {
   constexpr int G = 1 << LOG2G;
   // [baseline][channel] records, rows padded by one record so that the lanes'
   // 16-byte stores (lanes = baselines) fall in distinct banks
@@ -270,7 +244,8 @@ k_grid_prep(const GridEntry* __restrict__ listed, int n_listed, const int32_t* _
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int group = blockIdx.y;
   const int i0 = blockIdx.x * kPrepBl;
-  const int nbl = min(kPrepBl, n_listed - i0);
+  const int nbl = min(kPrepBl, static_cast<int>(counts[kCountListed]) - i0);
+  if (nbl <= 0) return;                                // the grid covers every cross baseline
   const int cmax = G / 2 - kHalfSup - 1;
   const int lim = (cmax + 1) * kQ;                     // < 2^21
   // this lane's two baselines (i0 + lane, i0 + lane + 32)
@@ -375,7 +350,7 @@ k_grid_prep(const GridEntry* __restrict__ listed, int n_listed, const int32_t* _
   }
   __syncthreads();
   // one baseline's 32 channel records per warp store: 512 contiguous bytes
-  int4* out = reinterpret_cast<int4*>(prep) + (static_cast<long long>(group) * n_listed + i0) * kLanes;
+  int4* out = reinterpret_cast<int4*>(prep) + (static_cast<long long>(group) * n_cross + i0) * kLanes;
   for (int bi = warp; bi < nbl; bi += 8) out[static_cast<long long>(bi) * kLanes + lane] = tile[bi][lane];
 }
 
@@ -405,8 +380,8 @@ constexpr size_t kTileSmem = static_cast<size_t>(kTabXLen) * sizeof(float);
 
 template <int LOG2G, bool BASES>
 __global__ void __launch_bounds__(kGridWarps * 32, 1)
-k_grid_tiles(const int* __restrict__ tile_idx, const int* __restrict__ tile_off, const int* __restrict__ tile_order,
-             const PrepRec* __restrict__ prep, int n_listed, const float* __restrict__ tabx_g, int nb,
+k_grid_tiles(const int* __restrict__ tile_idx, const int2* __restrict__ tile_rng, const int* __restrict__ tile_order,
+             const PrepRec* __restrict__ prep, long long n_cross, const float* __restrict__ tabx_g, int nb,
              float* __restrict__ grid) {
   constexpr int G = 1 << LOG2G;
   constexpr int NTU = n_tiles_u(G);
@@ -428,10 +403,11 @@ k_grid_tiles(const int* __restrict__ tile_idx, const int* __restrict__ tile_off,
     const int g = static_cast<int>(item / NT);
     const int tile = __ldg(tile_order + (item - static_cast<long long>(g) * NT));
     const int cb = g * kLanes + lane;                 // channel within the batch
-    const PrepRec* pg = prep + static_cast<long long>(g) * n_listed * kLanes + lane;
+    const PrepRec* pg = prep + static_cast<long long>(g) * n_cross * kLanes + lane;
     const int tv = tile / NTU, tu = tile - tv * NTU;
     const int r0 = G / 2 + tv * kTileV, c0 = tu * kTileU;
-    const int e0 = tile_off[tile], e1 = tile_off[tile + 1];
+    const int2 rng = __ldg(tile_rng + tile);
+    const int e0 = rng.x, e1 = rng.y;
     float acr[kTileV][kTileU], aci[kTileV][kTileU];
 #pragma unroll
     for (int i = 0; i < kTileV; ++i)
@@ -741,21 +717,372 @@ k_fft_cols(const void* __restrict__ h, const float* __restrict__ hs, int n_img, 
   }
 }
 
-__global__ void k_mask(int n, double cell, uint8_t* __restrict__ mask) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n * n) return;
-  const int r = i / n, c = i - r * n;
-  const double l = static_cast<double>(c - n / 2) * cell;
-  const double m = static_cast<double>(r - n / 2) * cell;
-  mask[i] = (l * l + m * m) < 1.0 ? 1 : 0;
+// ---------------------------------------------------------- per-call tables and lists
+// Everything one geometry and frequency axis needs is made on the device from
+// the antenna positions, the frequencies and the kernel table, in six
+// launches without a synchronisation.  Made by one host core (7169 N cosines
+// for the grid correction, a list push per tile and baseline) it took 13.5, 26
+// and 61 ms at 352 antennas and 256^2, 512^2 and 1024^2 images, five to twenty
+// times the gridding itself; whole calls now take 2.9 ms (1000 channels of
+// 256^2, 16.5 before), 3.1 ms (300 of 512^2, 29.7) and 3.4 ms (64 of 1024^2, 67).
+
+// Half of the even kernel table, C(m / Q) for m = 0 .. S Q / 2, passed by
+// value: the tables are built from it without a copy through memory.
+struct KernelHalf {
+  double c[kHalfTab + 1];
+};
+
+// The tables: the first n/2 + 1 CTAs form the reciprocal grid correction
+// 1 / C^(d), C^(d) = (1/Q) sum_m C(m/Q) cos(2 pi m d / (Q G)), one |d| each
+// (the table is even, and so is C^; the phase m d is reduced in integers, so
+// the cosine's argument is exact); the others fill the gap-indexed weights,
+// the twiddles, the horizon mask and the channel scales, one element a thread.
+// The cosines bound it: 3585 FP64 cospi per CTA.
+constexpr int kTabThreads = 256;
+__global__ void __launch_bounds__(kTabThreads)
+k_img_tables(const __grid_constant__ KernelHalf kh, int n, int g, double cell, const double* __restrict__ freq,
+             int n_chan, float* __restrict__ inv_corr, float* __restrict__ tabx, float2* __restrict__ tw,
+             uint8_t* __restrict__ mask, ChanScale* __restrict__ cs) {
+  const int n_corr = n / 2 + 1;
+  if (static_cast<int>(blockIdx.x) < n_corr) {
+    __shared__ double part[kTabThreads / 32];
+    const int d = blockIdx.x;
+    const int period = kQ * g;                         // a power of two, <= 2^21
+    double s = 0.0;
+    for (int m = threadIdx.x; m <= kHalfTab; m += kTabThreads) {
+      const int r = static_cast<int>((static_cast<long long>(m) * d) & (period - 1));
+      const double t = kh.c[m] * cospi(2.0 * static_cast<double>(r) / static_cast<double>(period));
+      s += m ? 2.0 * t : t;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < kTabThreads / 32; ++w) s += part[w];
+      const float v = static_cast<float>(1.0 / (s / kQ));
+      inv_corr[n / 2 - d] = v;                         // pixel offsets -d and d
+      if (d < n / 2) inv_corr[n / 2 + d] = v;
+    }
+    return;
+  }
+  long long i = static_cast<long long>(blockIdx.x - n_corr) * kTabThreads + threadIdx.x;
+  if (i < kTabXLen) {
+    const int d = static_cast<int>(i) / kTabStride - kTabD, off = kQ / 2 - static_cast<int>(i) % kTabStride;
+    tabx[i] = abs(d) <= kHalfSup ? static_cast<float>(kh.c[abs(d * kQ - off)]) : 0.0f;
+    return;
+  }
+  i -= kTabXLen;
+  if (i < g) {
+    double si, co;
+    sincospi(-2.0 * static_cast<double>(i) / static_cast<double>(g), &si, &co);
+    tw[i] = make_float2(static_cast<float>(co), static_cast<float>(si));
+    return;
+  }
+  i -= g;
+  if (i < static_cast<long long>(n) * n) {
+    const int r = static_cast<int>(i) / n, c = static_cast<int>(i) - r * n;
+    const double l = static_cast<double>(c - n / 2) * cell;
+    const double m = static_cast<double>(r - n / 2) * cell;
+    mask[i] = __dadd_rn(__dmul_rn(l, l), __dmul_rn(m, m)) < 1.0 ? 1 : 0;
+    return;
+  }
+  i -= static_cast<long long>(n) * n;
+  if (i < n_chan) {
+    const double du = 1.0 / (static_cast<double>(g) * cell);
+    const double sn = freq[i] / (kCLight * du);
+    ChanScale c;
+    c.s = sn * static_cast<double>(kQ);                // exact: Q is a power of two
+    c.nu_c = freq[i] / kCLight;
+    c.sh = static_cast<float>(c.s);
+    c.sl = static_cast<float>(c.s - static_cast<double>(c.sh));
+    cs[i] = c;
+  }
 }
 
-__global__ void k_twiddle_img(float2* tw, int n) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  double s, c;
-  sincospi(-2.0 * static_cast<double>(k) / static_cast<double>(n), &s, &c);
-  tw[k] = make_float2(static_cast<float>(c), static_cast<float>(s));
+// The frequency axis of a call as the lists need it: the extreme scales s_nu Q
+// and wavelengths per metre, and the uv range.
+struct PlanAxis {
+  double s_lo, s_hi;          // cells / Q per metre
+  double w_lo, w_hi;          // wavelengths per metre
+  double uv_min, uv_max;
+  int uv_cut;
+};
+
+// Centre cells of a cross baseline over the call's channels, and whether the
+// uv range must be decided per channel; u0 > u1: never gridded.
+struct PlanRange {
+  short u0, u1, v0, v1;
+  int check;
+};
+
+// Centre cell of a rounded position p (1/Q cells): p / Q rounded half away from zero.
+__device__ __forceinline__ long long centre_cell64(long long p) {
+  const long long c = (llabs(p) + kQ / 2) / kQ;
+  return p < 0 ? -c : c;
+}
+
+// Per cross baseline (a < b, row-major): its FP64 difference, length, and the
+// range of centre cells -- p = rint(dx s) is monotone in s, so every channel's
+// centre cells lie between those at the smallest and the largest scale.
+// blk[CTA] counts the CTA's baselines that can be gridded in some channel.
+constexpr int kPlanThreads = 256;
+__global__ void __launch_bounds__(kPlanThreads)
+k_plan_baselines(const double* __restrict__ ant, int n_ant, long long n_cross, int cmax, PlanAxis ax,
+                 Baseline* __restrict__ base, double* __restrict__ blen, PlanRange* __restrict__ rng,
+                 int* __restrict__ blk) {
+  const long long i = static_cast<long long>(blockIdx.x) * kPlanThreads + threadIdx.x;
+  bool live = false;
+  if (i < n_cross) {
+    // row a holds the pairs a (2n - a - 1) / 2 .. ; the root is exact to a row
+    const double q = 2.0 * n_ant - 1.0;
+    int a = static_cast<int>((q - sqrt(q * q - 8.0 * static_cast<double>(i))) * 0.5);
+    auto first = [&](long long r) { return r * (2LL * n_ant - r - 1) / 2; };
+    while (a > 0 && first(a) > i) --a;
+    while (first(a + 1) <= i) ++a;
+    const int b = static_cast<int>(i - first(a)) + a + 1;
+    Baseline B;
+    B.dx = __dsub_rn(ant[3 * a], ant[3 * b]);
+    B.dy = __dsub_rn(ant[3 * a + 1], ant[3 * b + 1]);
+    B.dxh = static_cast<float>(B.dx);
+    B.dxl = static_cast<float>(B.dx - static_cast<double>(B.dxh));
+    B.dyh = static_cast<float>(B.dy);
+    B.dyl = static_cast<float>(B.dy - static_cast<double>(B.dyh));
+    B.bl = bl_index(a, b, n_ant);
+    base[i] = B;
+    const double L = __dsqrt_rn(__dadd_rn(__dmul_rn(B.dx, B.dx), __dmul_rn(B.dy, B.dy)));
+    blen[i] = L;
+    auto cells = [&](double d, short& lo, short& hi) {
+      const long long x = centre_cell64(__double2ll_rn(__dmul_rn(d, ax.s_lo)));
+      const long long y = centre_cell64(__double2ll_rn(__dmul_rn(d, ax.s_hi)));
+      const long long l = max(min(x, y), static_cast<long long>(-cmax)), h = min(max(x, y), static_cast<long long>(cmax));
+      lo = static_cast<short>(l <= h ? l : 0);
+      hi = static_cast<short>(l <= h ? h : -1);
+      return l <= h;
+    };
+    PlanRange r;
+    live = cells(B.dx, r.u0, r.u1);
+    live = cells(B.dy, r.v0, r.v1) && live;
+    r.check = 0;
+    if (live && ax.uv_cut) {
+      // decided here when every channel of the call agrees (with a relative
+      // margin), per channel when the records are prepared otherwise
+      const double l0 = __dmul_rn(L, ax.w_lo), l1 = __dmul_rn(L, ax.w_hi), eps = 1e-9;
+      if (l1 < ax.uv_min * (1.0 - eps) || l0 >= ax.uv_max * (1.0 + eps)) live = false;
+      r.check = !(l0 >= ax.uv_min * (1.0 + eps) && l1 < ax.uv_max * (1.0 - eps));
+    }
+    if (!live) {
+      r.u0 = 0;
+      r.u1 = -1;
+    }
+    rng[i] = r;
+  }
+  const int c = __syncthreads_count(live);
+  if (threadIdx.x == 0) blk[blockIdx.x] = c;
+}
+
+// The listed baselines in cross order (a compaction: each CTA sums the counts
+// before its own), their ranges beside them, and how many there are.
+__global__ void __launch_bounds__(kPlanThreads)
+k_plan_list(int n_ant, long long n_cross, const Baseline* __restrict__ base, const PlanRange* __restrict__ rng,
+            const int* __restrict__ blk, GridEntry* __restrict__ listed, PlanRange* __restrict__ lrng,
+            unsigned long long* __restrict__ counts) {
+  __shared__ int wsum[kPlanThreads / 32];
+  __shared__ int wlive[kPlanThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int before = 0;
+  for (int j = threadIdx.x; j < static_cast<int>(blockIdx.x); j += kPlanThreads) before += blk[j];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+  const long long i = static_cast<long long>(blockIdx.x) * kPlanThreads + threadIdx.x;
+  PlanRange r;
+  r.u0 = 0;
+  r.u1 = -1;
+  if (i < n_cross) r = rng[i];
+  const bool live = r.u0 <= r.u1;
+  const unsigned m = __ballot_sync(0xffffffffu, live);
+  if (lane == 0) {
+    wsum[warp] = before;
+    wlive[warp] = __popc(m);
+  }
+  __syncthreads();
+  int pos = __popc(m & ((1u << lane) - 1u));
+  for (int w = 0; w < kPlanThreads / 32; ++w) pos += wsum[w] + (w < warp ? wlive[w] : 0);
+  if (live) {
+    const Baseline B = base[i];
+    GridEntry e;
+    e.bl = static_cast<int>(B.bl);
+    e.cross = static_cast<int>(i);
+    // the antennas: cross = bl - a - 1, b from a
+    const int a = static_cast<int>(B.bl - i) - 1;
+    e.a = a;
+    e.bf = static_cast<int>(B.bl - bl_index(a, a, n_ant)) + a;
+    if (r.check) e.bf |= kCheckUv;
+    e.dxh = B.dxh;
+    e.dxl = B.dxl;
+    e.dyh = B.dyh;
+    e.dyl = B.dyl;
+    listed[pos] = e;
+    lrng[pos] = r;
+  }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == kPlanThreads - 1)
+    counts[kCountListed] = static_cast<unsigned long long>(pos + (live ? 1 : 0));
+}
+
+// Tile rows a listed baseline's footprint (centre rows v0 .. v1 over the
+// call's channels, 3 cells to each side) touches among the gridded rows
+// G/2 .. G-1; the mirror's range is the negated one.
+__device__ __forceinline__ bool touches_row(int v0, int v1, int tv) {
+  return v1 + kHalfSup >= tv * kTileV && v0 - kHalfSup < (tv + 1) * kTileV;
+}
+
+// Per tile row, the records and mirrors that touch it, in listed order (a
+// record before its own mirror), each with its range of tile columns.  One CTA
+// per row: every warp counts its share of the list, the CTA reserves its range
+// of the buffer, every warp writes its share.  (A tile then scans its row's
+// few hundred entries, where it would scan tens of thousands of baselines.)
+constexpr int kRowWarps = 32;
+__global__ void __launch_bounds__(kRowWarps * 32)
+k_plan_rows(const PlanRange* __restrict__ lrng, int g, unsigned long long* __restrict__ counts,
+            int2* __restrict__ row_ent, long long cap, int2* __restrict__ row_rng) {
+  __shared__ int wcnt[kRowWarps];
+  __shared__ int start;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tv = blockIdx.x;
+  const unsigned lt = (1u << lane) - 1u;
+  const int n = static_cast<int>(counts[kCountListed]);
+  const int per = ((n + kRowWarps - 1) / kRowWarps + 31) & ~31;
+  const int i0 = min(n, warp * per), i1 = min(n, i0 + per);
+  auto hits = [&](int i, PlanRange& r, bool& rec, bool& mir) {
+    rec = mir = false;
+    if (i < i1) {
+      r = lrng[i];
+      rec = touches_row(r.v0, r.v1, tv);
+      mir = touches_row(-r.v1, -r.v0, tv);
+    }
+  };
+  int c = 0;
+#pragma unroll 4
+  for (int i = i0; i < i1; i += 32) {
+    PlanRange r;
+    bool rec, mir;
+    hits(i + lane, r, rec, mir);
+    c += (rec ? 1 : 0) + (mir ? 1 : 0);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+  if (lane == 0) wcnt[warp] = c;
+  __syncthreads();
+  int off = 0, total = 0;
+  for (int w = 0; w < kRowWarps; ++w) {
+    off += w < warp ? wcnt[w] : 0;
+    total += wcnt[w];
+  }
+  if (threadIdx.x == 0) {
+    // counts[kCountRows] may pass the capacity: the row stays empty then and
+    // the host reports the plan as too large
+    const unsigned long long s = atomicAdd(counts + kCountRows, static_cast<unsigned long long>(total));
+    start = s + total <= static_cast<unsigned long long>(cap) ? static_cast<int>(s) : -1;
+    row_rng[tv] = start < 0 ? make_int2(0, 0) : make_int2(start, start + total);
+  }
+  __syncthreads();
+  if (start < 0) return;
+  off += start;
+#pragma unroll 2
+  for (int i = i0; i < i1; i += 32) {
+    PlanRange r;
+    bool rec, mir;
+    hits(i + lane, r, rec, mir);
+    const unsigned mr = __ballot_sync(0xffffffffu, rec), mm = __ballot_sync(0xffffffffu, mir);
+    int pos = off + __popc(mr & lt) + __popc(mm & lt);
+    const int half = g / 2;
+    if (rec)
+      row_ent[pos++] = make_int2(i + lane, ((half + r.u0 - kHalfSup) / kTileU) | (((half + r.u1 + kHalfSup) / kTileU) << 16));
+    if (mir)
+      row_ent[pos] = make_int2((i + lane) | kMirror,
+                               ((half - r.u1 - kHalfSup) / kTileU) | (((half - r.u0 + kHalfSup) / kTileU) << 16));
+    off += __popc(mr) + __popc(mm);
+  }
+}
+
+// Per tile, its list in listed order: one warp per tile scans its row's entries
+// twice (count, then write to a range reserved by one atomic).
+constexpr int kTileListWarps = 8;
+__global__ void __launch_bounds__(kTileListWarps * 32)
+k_plan_tiles(const int2* __restrict__ row_ent, const int2* __restrict__ row_rng, int ntu, int nt,
+             unsigned long long* __restrict__ counts, int* __restrict__ tile_idx, long long cap,
+             int2* __restrict__ tile_rng) {
+  const int lane = threadIdx.x & 31;
+  const int tile = blockIdx.x * kTileListWarps + (threadIdx.x >> 5);
+  if (tile >= nt) return;
+  const int tv = tile / ntu, tu = tile - tv * ntu;
+  const int2 rr = row_rng[tv];
+  auto hit = [&](int i, int& ent) {
+    if (i >= rr.y) return false;
+    const int2 e = __ldg(row_ent + i);
+    ent = e.x;
+    return tu >= (e.y & 0xffff) && tu <= (e.y >> 16);
+  };
+  int c = 0;
+#pragma unroll 4
+  for (int i = rr.x; i < rr.y; i += 32) {
+    int ent;
+    c += hit(i + lane, ent) ? 1 : 0;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+  int start = 0;
+  if (lane == 0) {
+    const unsigned long long s = atomicAdd(counts + kCountTiles, static_cast<unsigned long long>(c));
+    start = s + c <= static_cast<unsigned long long>(cap) ? static_cast<int>(s) : -1;
+    tile_rng[tile] = start < 0 ? make_int2(0, 0) : make_int2(start, start + c);
+  }
+  start = __shfl_sync(0xffffffffu, start, 0);
+  if (start < 0) return;
+#pragma unroll 2
+  for (int i = rr.x; i < rr.y; i += 32) {
+    int ent = 0;
+    const bool h = hit(i + lane, ent);
+    const unsigned m = __ballot_sync(0xffffffffu, h);
+    if (h) tile_idx[start + __popc(m & ((1u << lane) - 1u))] = ent;
+    start += __popc(m);
+  }
+}
+
+// The tiles from the longest list to the shortest (lists of kOrderBins and
+// more together): a counting sort by one CTA.  The order only decides which
+// warp takes a tile when.
+constexpr int kOrderBins = 2048;
+__global__ void __launch_bounds__(1024)
+k_plan_order(const int2* __restrict__ tile_rng, int nt, int* __restrict__ order) {
+  __shared__ int bin[kOrderBins];
+  __shared__ int wtot[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int i = threadIdx.x; i < kOrderBins; i += 1024) bin[i] = 0;
+  __syncthreads();
+  auto cls = [&](int t) {
+    const int2 r = __ldg(tile_rng + t);
+    return kOrderBins - 1 - min(r.y - r.x, kOrderBins - 1);
+  };
+#pragma unroll 4
+  for (int t = threadIdx.x; t < nt; t += 1024) atomicAdd(&bin[cls(t)], 1);
+  __syncthreads();
+  // exclusive scan, kOrderBins / 1024 bins per thread
+  const int b0 = bin[2 * threadIdx.x], b1 = bin[2 * threadIdx.x + 1];
+  int v = b0 + b1;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += t;
+  }
+  if (lane == 31) wtot[warp] = v;
+  __syncthreads();
+  int run = v - b0 - b1;
+  for (int w = 0; w < warp; ++w) run += wtot[w];
+  bin[2 * threadIdx.x] = run;
+  bin[2 * threadIdx.x + 1] = run + b0;
+  __syncthreads();
+#pragma unroll 4
+  for (int t = threadIdx.x; t < nt; t += 1024) order[atomicAdd(&bin[cls(t)], 1)] = t;
 }
 
 __global__ void k_counts_out(const int* __restrict__ kept, int n_chan, int32_t* __restrict__ out) {
@@ -800,26 +1127,29 @@ ImgPlan make_plan(int n_ant, int n_chan, int n, int storage) {
 }
 
 struct ImgWs {
-  float* tab;
   float* tabx;       // [kTabXLen] weights by (tap offset, position offset)
   float* inv_corr;
   float2* tw;
   uint8_t* mask;
-  double* ant;
-  double* freq;
+  double* axis;      // antenna positions [n_ant][3], then frequencies [n_chan]
   Baseline* base;
   ChanScale* cs;
   int* kept;
+  PlanRange* rng;    // [n_cross] centre-cell ranges
+  int* blk;          // listed baselines per CTA of k_plan_baselines
   GridEntry* listed; // baselines that can be gridded in some channel of the call
-  int* tile_off;     // [n_tiles + 1]
+  PlanRange* lrng;   // their ranges
+  int2* row_ent;     // per tile row: (listed index | kMirror, first | last << 16 tile column)
+  int2* row_rng;     // [tile rows] their ranges in row_ent
+  int2* tile_rng;    // [n_tiles] ranges in tile_idx
   int* tile_order;   // [n_tiles] tiles by descending list length
-  int* tile_idx;     // per tile: indices into listed
+  int* tile_idx;     // per tile: indices into listed | kMirror
+  unsigned long long* counts;   // [kCounts]
   double* blen;      // [n_cross] baseline lengths (metres)
-  PrepRec* prep;     // [batch groups][n_cross][32] prepared records
+  PrepRec* prep;     // [batch groups][n_cross][32] prepared records (the listed ones first)
   float* grid;       // [batch][2][G][G] gridded planes (re, im)
   void* h;           // [batch][G][N] complex in the storage format
   float* hs;         // [batch][G] row scales (FP16 storage)
-  int n_listed = 0;
   bool bases = false;  // records carry weight-table offsets (footprints move < kTabMargin cells)
 };
 
@@ -835,20 +1165,24 @@ ImgWs carve_img(void* ws, size_t bytes, const ImgPlan& p, int n_ant, int n_chan,
   Carver c(ws, bytes);
   ImgWs w;
   const size_t nx = p.n_cross > 0 ? static_cast<size_t>(p.n_cross) : 1;
-  w.tab = c.take<float>(kTabLen);
   w.tabx = c.take<float>(kTabXLen);
   w.inv_corr = c.take<float>(p.n);
   w.tw = c.take<float2>(p.g);
   w.mask = c.take<uint8_t>(static_cast<size_t>(p.n) * p.n);
-  w.ant = c.take<double>(static_cast<size_t>(n_ant) * 3);
-  w.freq = c.take<double>(n_chan);
+  w.axis = c.take<double>(static_cast<size_t>(n_ant) * 3 + n_chan);
   w.base = c.take<Baseline>(nx);
   w.cs = c.take<ChanScale>(n_chan);
   w.kept = c.take<int>(n_chan);
+  w.rng = c.take<PlanRange>(nx);
+  w.blk = c.take<int>((nx + kPlanThreads - 1) / kPlanThreads);
   w.listed = c.take<GridEntry>(nx);
-  w.tile_off = c.take<int>(n_tiles(p.g) + 1);
+  w.lrng = c.take<PlanRange>(nx);
+  w.row_ent = c.take<int2>(entry_capacity(p));
+  w.row_rng = c.take<int2>(half_rows(p.g) / kTileV);
+  w.tile_rng = c.take<int2>(n_tiles(p.g));
   w.tile_order = c.take<int>(n_tiles(p.g));
   w.tile_idx = c.take<int>(entry_capacity(p));
+  w.counts = c.take<unsigned long long>(kCounts);
   w.blen = c.take<double>(nx);
   w.prep = c.take<PrepRec>(static_cast<size_t>((p.batch + kLanes - 1) / kLanes) * nx * kLanes);
   w.grid = c.take<float>(static_cast<size_t>(p.batch) * 2 * half_rows(p.g) * p.g);
@@ -856,103 +1190,6 @@ ImgWs carve_img(void* ws, size_t bytes, const ImgPlan& p, int n_ant, int n_chan,
   w.hs = c.take<float>(static_cast<size_t>(p.batch) * half_rows(p.g));
   *need = c.used;
   return w;
-}
-
-// Baseline length in metres, sqrt(dx^2 + dy^2) in FP64 (host code is built
-// without FMA contraction, so this rounds like the definition).
-double baseline_length(const double* ant, int a, int b) {
-  const double dx = ant[3 * a] - ant[3 * b], dy = ant[3 * a + 1] - ant[3 * b + 1];
-  const double x2 = dx * dx, y2 = dy * dy;
-  return std::sqrt(x2 + y2);
-}
-
-// Centre cell of a rounded position p (1/Q cells): p / Q rounded half away from zero.
-long long centre_cell_host(long long p) {
-  const long long c = (std::llabs(p) + kQ / 2) / kQ;
-  return p < 0 ? -c : c;
-}
-
-// Host: which baselines can touch which warp tile in some channel of the call.
-// The channel scales s_nu Q are computed exactly as the device computes them
-// (k_chan_scale), and p = rint(dx s) is monotone in s, so the centre cells of
-// every channel lie between those at the smallest and the largest scale.
-void build_entries(const ImgPlan& p, int n_ant, const double* ant, const double* freq, int n_chan,
-                   double cell, double uv_min, double uv_max, std::vector<GridEntry>& listed,
-                   std::vector<int>& idx, std::vector<int>& off, long long* spread) {
-  const double du = 1.0 / (static_cast<double>(p.g) * cell);
-  double s_lo = HUGE_VAL, s_hi = -HUGE_VAL, fmin = freq[0], fmax = freq[0];
-  for (int f = 0; f < n_chan; ++f) {
-    const double sq = (freq[f] / (kCLight * du)) * static_cast<double>(kQ);
-    s_lo = std::min(s_lo, sq);
-    s_hi = std::max(s_hi, sq);
-    fmin = std::min(fmin, freq[f]);
-    fmax = std::max(fmax, freq[f]);
-  }
-  const bool uv_cut = uv_min > 0.0 || std::isfinite(uv_max);
-  const double w_lo = fmin / kCLight, w_hi = fmax / kCLight;                  // wavelengths per metre
-  const long long cmax = p.g / 2 - kHalfSup - 1;
-  const int ntu = n_tiles_u(p.g), nt = n_tiles(p.g);
-  std::vector<std::vector<int>> tiles(nt);
-  // the centre cells over the call's channels; *spread: the most any listed
-  // footprint moves across them
-  *spread = 0;
-  long long move = 0;
-  auto cells = [&](double d, long long& lo, long long& hi) {
-    const long long a = centre_cell_host(std::llrint(d * s_lo)), b = centre_cell_host(std::llrint(d * s_hi));
-    lo = std::max(std::min(a, b), -cmax);
-    hi = std::min(std::max(a, b), cmax);
-    move = std::max(move, a > b ? a - b : b - a);
-    return lo <= hi;
-  };
-  listed.clear();
-  long long cross = 0;
-  for (int a = 0; a < n_ant; ++a)
-    for (int b = a + 1; b < n_ant; ++b, ++cross) {
-      const double dx = ant[3 * a] - ant[3 * b], dy = ant[3 * a + 1] - ant[3 * b + 1];
-      long long u0, u1, v0, v1;
-      move = 0;
-      if (!cells(dx, u0, u1) || !cells(dy, v0, v1)) continue;       // never on the grid
-      // uv range: decided here when every channel of the call agrees (with a
-      // relative margin), per channel on the device otherwise
-      bool check = false;
-      if (uv_cut) {
-        const double L = baseline_length(ant, a, b);
-        const double l0 = L * w_lo, l1 = L * w_hi, eps = 1e-9;
-        if (l1 < uv_min * (1.0 - eps) || l0 >= uv_max * (1.0 + eps)) continue;      // always outside
-        check = !(l0 >= uv_min * (1.0 + eps) && l1 < uv_max * (1.0 - eps));       // not always inside
-      }
-      GridEntry e;
-      e.bl = static_cast<int>(a * static_cast<long long>(n_ant) - static_cast<long long>(a) * (a - 1) / 2 + (b - a));
-      e.cross = static_cast<int>(cross);
-      e.a = a;
-      e.bf = b | (check ? kCheckUv : 0);
-      e.dxh = static_cast<float>(dx);
-      e.dxl = static_cast<float>(dx - static_cast<double>(e.dxh));
-      e.dyh = static_cast<float>(dy);
-      e.dyl = static_cast<float>(dy - static_cast<double>(e.dyh));
-      const int li = static_cast<int>(listed.size());
-      listed.push_back(e);
-      *spread = std::max(*spread, move);
-      // footprint rows / columns over the call (centre +- 3 cells), of the
-      // record and of its mirror, within the gridded rows G/2 .. G-1
-      auto add = [&](long long vl, long long vh, long long ul, long long uh, int flag) {
-        const int r_lo = static_cast<int>(std::max<long long>(p.g / 2, p.g / 2 + vl - kHalfSup));
-        const int r_hi = static_cast<int>(p.g / 2 + vh + kHalfSup);
-        if (r_hi < r_lo) return;
-        const int c_lo = static_cast<int>(p.g / 2 + ul - kHalfSup), c_hi = static_cast<int>(p.g / 2 + uh + kHalfSup);
-        for (int tv = (r_lo - p.g / 2) / kTileV; tv <= (r_hi - p.g / 2) / kTileV; ++tv)
-          for (int tu = c_lo / kTileU; tu <= c_hi / kTileU; ++tu) tiles[tv * ntu + tu].push_back(li | flag);
-      };
-      add(v0, v1, u0, u1, 0);
-      add(-v1, -v0, -u1, -u0, kMirror);
-    }
-  idx.clear();
-  off.assign(nt + 1, 0);
-  for (int t = 0; t < nt; ++t) {
-    off[t] = static_cast<int>(idx.size());
-    idx.insert(idx.end(), tiles[t].begin(), tiles[t].end());
-  }
-  off[nt] = static_cast<int>(idx.size());
 }
 
 template <int L, int S>
@@ -964,12 +1201,13 @@ int launch_batch(const ImgPlan& p, const ImgWs& w, const GridOpts& o, const int3
     // calibration corrections or a uv range select the variant that applies them
     const bool cal = o.gains != nullptr || o.uv_min > 0.0 || std::isfinite(o.uv_max);
     const int n_groups = (nb + kLanes - 1) / kLanes;
-    if (w.n_listed > 0) {
-      dim3 grid((w.n_listed + kPrepBl - 1) / kPrepBl, n_groups);
+    if (p.n_cross > 0) {
+      dim3 grid(static_cast<unsigned>((p.n_cross + kPrepBl - 1) / kPrepBl), n_groups);
       OVRO_PROF("k_grid_prep", st);
       auto prep = cal ? (w.bases ? k_grid_prep<L, true, true> : k_grid_prep<L, true, false>)
                       : (w.bases ? k_grid_prep<L, false, true> : k_grid_prep<L, false, false>);
-      prep<<<grid, 256, 0, st>>>(w.listed, w.n_listed, vis, n_bl, w.base, w.cs, ch0, nb, w.kept, w.prep, o);
+      prep<<<grid, 256, 0, st>>>(w.listed, w.counts, p.n_cross, vis, n_bl, w.base, w.cs, ch0, nb, w.kept, w.prep,
+                                o);
       OVRO_LAUNCH_CHECK();
     }
     auto tiles = w.bases ? k_grid_tiles<L, true> : k_grid_tiles<L, false>;
@@ -979,7 +1217,7 @@ int launch_batch(const ImgPlan& p, const ImgWs& w, const GridOpts& o, const int3
     const long long ctas = std::min<long long>(num_sms(), (items + kGridWarps - 1) / kGridWarps);
     OVRO_PROF("k_grid_tiles", st);
     tiles<<<static_cast<unsigned>(ctas), kGridWarps * 32, kTileSmem, st>>>(
-        w.tile_idx, w.tile_off, w.tile_order, w.prep, w.n_listed, w.tabx, nb, w.grid);
+        w.tile_idx, w.tile_rng, w.tile_order, w.prep, p.n_cross, w.tabx, nb, w.grid);
     OVRO_LAUNCH_CHECK();
   }
   {
@@ -1031,65 +1269,76 @@ int run_batch(const ImgPlan& p, const ImgWs& w, const GridOpts& o, const int32_t
   }
 }
 
+// The call's tables and lists, all made on the device.  bases: the prepared
+// records may hold weight-table offsets, because no listed footprint moves by
+// kTabMargin cells over the call's channels: a listed |d| s is below
+// (cmax + 1) Q at the smallest scale, so a centre moves by at most
+// (cmax + 1) (s_hi / s_lo - 1) + 1 cells; one more cell of slack for a
+// rounding of u Q that differs from the exact one.  A footprint that moves by
+// at most two cells touches 3 x 3 tiles, its mirror as many: 18 entries, within
+// the capacity of 24; a call over a wider band waits for its count and is
+// refused when it does not fit.
 int upload_common(const ImgPlan& p, ImgWs& w, int n_ant, const double* h_ant,
                   const double* h_freq, int n_chan, double cell, cudaStream_t st,
                   double uv_min = 0.0, double uv_max = HUGE_VAL) {
   const KernelTables& kt = kernel_tables();
-  std::vector<double> corr;
-  grid_correction(p.n, p.g, corr);
-  std::vector<float> inv(p.n);
-  for (int i = 0; i < p.n; ++i) inv[i] = static_cast<float>(1.0 / corr[i]);
-  std::vector<GridEntry> listed;
-  std::vector<int> idx, off;
-  long long spread = 0;
-  build_entries(p, n_ant, h_ant, h_freq, n_chan, cell, uv_min, uv_max, listed, idx, off, &spread);
-  if (static_cast<long long>(idx.size()) > entry_capacity(p)) return OVRO_ERR_CAPACITY;
-  w.n_listed = static_cast<int>(listed.size());
-  // one cell of slack for a host rounding of u Q that differs from the exact one
-  w.bases = spread + 1 <= kTabMargin;
-  std::vector<double> blen(p.n_cross > 0 ? p.n_cross : 1, 0.0);
-  {
-    long long x = 0;
-    for (int a = 0; a < n_ant; ++a)
-      for (int b = a + 1; b < n_ant; ++b) blen[x++] = baseline_length(h_ant, a, b);
+  KernelHalf kh;
+  std::copy(kt.table64.begin() + kHalfTab, kt.table64.end(), kh.c);
+  std::vector<double> axis(h_ant, h_ant + 3 * static_cast<size_t>(n_ant));
+  axis.insert(axis.end(), h_freq, h_freq + n_chan);
+  // the scales s_nu Q exactly as the device computes them
+  const double du = 1.0 / (static_cast<double>(p.g) * cell);
+  PlanAxis ax;
+  ax.s_lo = HUGE_VAL;
+  ax.s_hi = -HUGE_VAL;
+  double fmin = h_freq[0], fmax = h_freq[0];
+  for (int f = 0; f < n_chan; ++f) {
+    const double sq = (h_freq[f] / (kCLight * du)) * static_cast<double>(kQ);
+    ax.s_lo = std::min(ax.s_lo, sq);
+    ax.s_hi = std::max(ax.s_hi, sq);
+    fmin = std::min(fmin, h_freq[f]);
+    fmax = std::max(fmax, h_freq[f]);
   }
-  OVRO_CUDA_TRY(cudaMemcpyAsync(w.blen, blen.data(), blen.size() * sizeof(double), cudaMemcpyHostToDevice, st));
-  OVRO_CUDA_TRY(cudaMemcpyAsync(w.tab, kt.table32.data(), kTabLen * sizeof(float),
-                                cudaMemcpyHostToDevice, st));
-  std::vector<float> tabx(kTabXLen, 0.0f);
-  for (int d = -kHalfSup; d <= kHalfSup; ++d)
-    for (int off = -kQ / 2; off <= kQ / 2; ++off)
-      tabx[(d + kTabD) * kTabStride + kQ / 2 - off] = kt.table32[kHalfTab + d * kQ - off];
-  OVRO_CUDA_TRY(cudaMemcpyAsync(w.tabx, tabx.data(), kTabXLen * sizeof(float), cudaMemcpyHostToDevice, st));
-  OVRO_CUDA_TRY(cudaMemcpyAsync(w.inv_corr, inv.data(), p.n * sizeof(float), cudaMemcpyHostToDevice, st));
-  OVRO_CUDA_TRY(cudaMemcpyAsync(w.ant, h_ant, static_cast<size_t>(n_ant) * 3 * sizeof(double),
-                                cudaMemcpyHostToDevice, st));
-  OVRO_CUDA_TRY(cudaMemcpyAsync(w.freq, h_freq, static_cast<size_t>(n_chan) * sizeof(double),
-                                cudaMemcpyHostToDevice, st));
-  OVRO_CUDA_TRY(cudaMemcpyAsync(w.tile_off, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-  std::vector<int> order(off.size() - 1);
-  for (size_t t = 0; t < order.size(); ++t) order[t] = static_cast<int>(t);
-  std::stable_sort(order.begin(), order.end(),
-                   [&](int a, int b) { return off[a + 1] - off[a] > off[b + 1] - off[b]; });
-  OVRO_CUDA_TRY(cudaMemcpyAsync(w.tile_order, order.data(), order.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-  if (!listed.empty())
-    OVRO_CUDA_TRY(cudaMemcpyAsync(w.listed, listed.data(), listed.size() * sizeof(GridEntry),
-                                  cudaMemcpyHostToDevice, st));
-  if (!idx.empty())
-    OVRO_CUDA_TRY(cudaMemcpyAsync(w.tile_idx, idx.data(), idx.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-  // host->device copies from pageable memory are staged before cudaMemcpyAsync
-  // returns, so the temporaries above may go out of scope
-  k_twiddle_img<<<(p.g + 255) / 256, 256, 0, st>>>(w.tw, p.g);
+  ax.w_lo = fmin / kCLight;
+  ax.w_hi = fmax / kCLight;
+  ax.uv_min = uv_min;
+  ax.uv_max = uv_max;
+  ax.uv_cut = uv_min > 0.0 || std::isfinite(uv_max);
+  const int cmax = p.g / 2 - kHalfSup - 1;
+  const double move = ax.s_lo > 0.0 ? (cmax + 1) * (ax.s_hi / ax.s_lo - 1.0) + 1.0 : HUGE_VAL;
+  w.bases = move + 1.0 <= kTabMargin;
+  const double* d_ant = w.axis;
+  const double* d_freq = w.axis + 3 * static_cast<size_t>(n_ant);
+  // a copy from pageable memory is staged before cudaMemcpyAsync returns, so
+  // the vector may go out of scope
+  OVRO_CUDA_TRY(cudaMemcpyAsync(w.axis, axis.data(), axis.size() * sizeof(double), cudaMemcpyHostToDevice, st));
+  OVRO_CUDA_TRY(cudaMemsetAsync(w.counts, 0, kCounts * sizeof(unsigned long long), st));
+  const long long elems = kTabXLen + static_cast<long long>(p.g) + static_cast<long long>(p.n) * p.n + n_chan;
+  k_img_tables<<<static_cast<unsigned>(p.n / 2 + 1 + (elems + kTabThreads - 1) / kTabThreads), kTabThreads, 0, st>>>(
+      kh, p.n, p.g, cell, d_freq, n_chan, w.inv_corr, w.tabx, w.tw, w.mask, w.cs);
   OVRO_LAUNCH_CHECK();
-  k_mask<<<(p.n * p.n + 255) / 256, 256, 0, st>>>(p.n, cell, w.mask);
-  OVRO_LAUNCH_CHECK();
+  const int rows = half_rows(p.g) / kTileV, nt = n_tiles(p.g);
   if (p.n_cross > 0) {
-    dim3 g((n_ant + 127) / 128, n_ant);
-    k_baselines<<<g, 128, 0, st>>>(w.ant, n_ant, w.base);
+    const unsigned blocks = static_cast<unsigned>((p.n_cross + kPlanThreads - 1) / kPlanThreads);
+    k_plan_baselines<<<blocks, kPlanThreads, 0, st>>>(d_ant, n_ant, p.n_cross, cmax, ax, w.base, w.blen, w.rng, w.blk);
+    OVRO_LAUNCH_CHECK();
+    k_plan_list<<<blocks, kPlanThreads, 0, st>>>(n_ant, p.n_cross, w.base, w.rng, w.blk, w.listed, w.lrng, w.counts);
     OVRO_LAUNCH_CHECK();
   }
-  k_chan_scale<<<(n_chan + 255) / 256, 256, 0, st>>>(w.freq, n_chan, p.g, cell, w.cs);
+  k_plan_rows<<<rows, kRowWarps * 32, 0, st>>>(w.lrng, p.g, w.counts, w.row_ent, entry_capacity(p), w.row_rng);
   OVRO_LAUNCH_CHECK();
+  k_plan_tiles<<<(nt + kTileListWarps - 1) / kTileListWarps, kTileListWarps * 32, 0, st>>>(
+      w.row_ent, w.row_rng, n_tiles_u(p.g), nt, w.counts, w.tile_idx, entry_capacity(p), w.tile_rng);
+  OVRO_LAUNCH_CHECK();
+  k_plan_order<<<1, 1024, 0, st>>>(w.tile_rng, nt, w.tile_order);
+  OVRO_LAUNCH_CHECK();
+  if (!(move <= 2.0)) {
+    unsigned long long c[kCounts];
+    OVRO_CUDA_TRY(cudaMemcpyAsync(c, w.counts, sizeof(c), cudaMemcpyDeviceToHost, st));
+    OVRO_CUDA_TRY(cudaStreamSynchronize(st));
+    const unsigned long long cap = static_cast<unsigned long long>(entry_capacity(p));
+    if (c[kCountRows] > cap || c[kCountTiles] > cap) return OVRO_ERR_CAPACITY;
+  }
   return OVRO_OK;
 }
 

@@ -142,18 +142,4 @@ const KernelTables& kernel_tables() {
   return t;
 }
 
-void grid_correction(int n, int g, std::vector<double>& out) {
-  // C^(d) = (1/Q) sum_m C(m / Q) cos(2 pi m d / (Q G)), d = -N/2 .. N/2 - 1
-  const KernelTables& t = kernel_tables();
-  const int half = kSupport * kOversample / 2;
-  out.assign(n, 0.0);
-  for (int i = 0; i < n; ++i) {
-    const double d = i - n / 2;
-    double acc = 0.0;
-    for (int m = -half; m <= half; ++m)
-      acc += t.table64[m + half] * std::cos(2.0 * M_PI * m * d / (static_cast<double>(kOversample) * g));
-    out[i] = acc / kOversample;
-  }
-}
-
 }  // namespace ovro

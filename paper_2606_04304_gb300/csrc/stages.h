@@ -33,7 +33,7 @@ size_t grid_ctx_workspace(int n_ant, int n_chan, int image_size, int storage);
 int grid_ctx_init(GridCtx** out, int n_ant, int n_chan, int image_size, double cell, int storage, void* d_ws,
                   size_t ws_bytes, const void* d_gains = nullptr, double uv_min = 0.0,
                   double uv_max = HUGE_VAL);
-// Host lists and tables (pageable copies): once per geometry and frequency axis.
+// Tables and lists, made on the device (a pageable copy of the axis): once per geometry and frequency axis.
 int grid_ctx_upload(GridCtx* g, const double* h_ant_enu_m, const double* h_chan_freq_hz, cudaStream_t st);
 int grid_ctx_enqueue(GridCtx* g, const int32_t* d_vis, float* d_img, int32_t* d_counts_or_null, cudaStream_t st);
 // Cross visibilities gridded by the last enqueue (mirrors not counted; synchronises).
