@@ -7,13 +7,16 @@
 //                    FP64), giving FP64 statistics.
 //      k_ztrans      standardises (z = (x - med) / (1.4826 MAD)) and turns the
 //                    cube into per-pixel spectra [coarse][pixel][channel].
-//  a9  k_rank        per pixel spectrum: stable LSD radix sort (4 x 8-bit
-//                    digits, ballot multisplit for in-warp ranks) -> sorted values and
-//                    the rank of every channel.
-//      k_walk        one thread per pixel walks the channels keeping the
-//                    window's ranks in a bitset (shared memory, interleaved per
-//                    thread) and a cursor on the lower median, so every step of
-//                    the exact running median costs O(1) amortised.
+//  a9  k_rank_band   per pixel spectrum: the middle ranks by a histogram
+//                    selection and a counting sort over bins linear in the
+//                    value -> the band's sorted values and every channel's
+//                    rank, or its side of the band.
+//      k_walk        one thread per pixel and segment walks the channels
+//                    keeping the window's ranks in a bitset (shared memory,
+//                    interleaved per thread) and a pointer on the lower median,
+//                    so every step of the exact running median costs O(1).
+//      k_rank        full ranks (stable LSD radix sort) for the pixels whose
+//                    band or walk gave up; k_walk then takes them in full.
 //  a10 k_mf          per 8 consecutive channels a thread holds the 107-value
 //                    neighbourhood as register prefix sums and evaluates all 29
 //                    boxcars as prefix differences; keeps max SNR and width and
@@ -294,25 +297,21 @@ __host__ __device__ __forceinline__ int walk_stride(int nc, int h) {
   return (nc + ((h + 3) & ~3) + 3) & ~3;
 }
 
-// Stream codes: a rank word of 0xffff is no element; in a band stream
-// (band-relative ranks) 0xfffe is an element below the band and 0xfffd one
-// above it.
-constexpr uint32_t kRankNone = 0xffffu, kRankBelow = 0xfffeu, kRankAbove = 0xfffdu;
+// Stream codes, signed 16-bit like the ranks: in a band stream an element
+// below the band, and one above it, compare below and above every band rank.
+constexpr int kRankBelow = -32768, kRankAbove = 32767;
 
 // Stable LSD radix sort of m keys with 16-bit payloads in shared memory by the
 // whole CTA: four passes of 8 bits; each warp ranks a contiguous segment
 // (in-warp ranks by an 8-ballot multisplit, per-warp digit histograms at a
 // padded pitch, so an exclusive scan in digit-major order gives every
 // (digit, warp) its stable output offset).  The sorted keys end in ks / is.
-//   sw: the warps that rank segments (<= blockDim / 32).  All 32 for the band
-//   too: with 8 (a scan over a quarter of the digit counters) the idle warps
-//   waited at the barriers and the sort took longer.
 __device__ void lsd_sort(uint32_t* ks, uint16_t* is, uint32_t* kd, uint16_t* id, int m, uint32_t* hist,
-                         uint32_t* tot, int sw) {
-  const int W = sw;
+                         uint32_t* tot) {
+  const int W = blockDim.x >> 5;
   const int HP = W + 1;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int seg = warp < W ? ((m + W - 1) / W + 31) / 32 * 32 : 0;   // idle warps rank nothing
+  const int seg = ((m + W - 1) / W + 31) / 32 * 32;
   const unsigned lt_mask = (1u << lane) - 1u;
   for (int pass = 0; pass < 4; ++pass) {
     const int sh = 8 * pass;
@@ -355,18 +354,19 @@ __device__ void lsd_sort(uint32_t* ks, uint16_t* is, uint32_t* kd, uint16_t* id,
 // The step stream from per-channel ranks rk (shared memory): step k inserts
 // channel k + h and removes channel k - h - 1, stored at index k + H (H = h
 // rounded up to 4) as (insert rank, remove rank); indices below H hold the
-// insert-only steps that build the first window.  16-byte coalesced stores.
-__device__ void write_stream(const uint16_t* rk, int nc, int h, uint32_t* sp) {
+// insert-only steps that build the first window, and the half of a word
+// whose channel does not exist holds 0 (the walk knows which those are).
+// 16-byte coalesced stores.
+__device__ __forceinline__ void write_stream(const uint16_t* rk, int nc, int h, uint32_t* sp) {
   const int H = (h + 3) & ~3;
   const int S = walk_stride(nc, h);
   for (int q = threadIdx.x; q < S / 4; q += blockDim.x) {
     uint32_t wv[4];
+    const int ci = 4 * q - H + h, co = 4 * q - H - h - 1;
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int i = 4 * q + u;
-      const int cin = i - H + h, cout = i - H - h - 1;
-      const uint32_t rin = (cin >= 0 && cin < nc) ? rk[cin] : kRankNone;
-      const uint32_t rout = (cout >= 0 && i - H < nc) ? rk[cout] : kRankNone;
+      const uint32_t rin = static_cast<unsigned>(ci + u) < static_cast<unsigned>(nc) ? rk[ci + u] : 0u;
+      const uint32_t rout = static_cast<unsigned>(co + u) < static_cast<unsigned>(nc) ? rk[co + u] : 0u;
       wv[u] = rin | (rout << 16);
     }
     reinterpret_cast<uint4*>(sp)[q] = make_uint4(wv[0], wv[1], wv[2], wv[3]);
@@ -397,7 +397,7 @@ k_rank(const float* __restrict__ z, int n_valid, int nc, int h, float* __restric
       ia[k] = static_cast<uint16_t>(k);
     }
     __syncthreads();
-    lsd_sort(ka, ia, kb, ib, nc, hist, tot, W);
+    lsd_sort(ka, ia, kb, ib, nc, hist, tot);
     float* svp = sv + static_cast<long long>(p) * nc;
     for (int r = threadIdx.x; r < nc; r += blockDim.x) {
       svp[r] = key2f(ka[r]);
@@ -409,197 +409,264 @@ k_rank(const float* __restrict__ z, int n_valid, int nc, int h, float* __restric
   }
 }
 
-// Bin of the 256-bin histogram hg holding element `target` (0-based, in key
-// order) and the count below that bin; run by one warp.
-__device__ __forceinline__ void find_bin(const uint32_t* hg, int target, int* bin, int* below) {
-  const int lane = threadIdx.x & 31;
-  uint32_t c[8], s = 0;
-#pragma unroll
-  for (int u = 0; u < 8; ++u) {
-    c[u] = hg[lane * 8 + u];
-    s += c[u];
-  }
-  uint32_t incl = s;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += t;
-  }
-  uint32_t run = incl - s;
-  const uint32_t tg = static_cast<uint32_t>(target);
-#pragma unroll
-  for (int u = 0; u < 8; ++u) {
-    if (run <= tg && tg < run + c[u]) {
-      *bin = lane * 8 + u;
-      *below = static_cast<int>(run);
-    }
-    run += c[u];
-  }
+// Band ranks.  The walk of a long coarse channel needs exact ranks only inside
+// a band of middle ranks; below and above it a count suffices, and which band
+// it is does not matter as long as the window medians stay inside it.
+constexpr int kBins = 2048;             // histogram bins of the selection and of the ranking
+constexpr int kBandMax = 2048;          // ranks of a band at most
+
+// Ranks of the band (a multiple of 64): a window median's rank wanders about
+// nc / (2 sqrt(W)) from the middle for a stationary spectrum, by sqrt 2 more
+// for the half windows at the edges: 140 ranks at 8192 channels (W = 0.21 nc).
+// So the band grows as sqrt(nc); 22.6 sqrt(nc) is 7 deviations to each side
+// (half of that sent enough pixels of skewed noise images to the full walk to
+// cost more than the narrower band saved).  A short spectrum has them all.
+inline int band_ranks(int nc) {
+  const int b = std::min(nc, static_cast<int>(22.6 * std::sqrt(static_cast<double>(nc))));
+  return std::min(kBandMax, (b + 63) / 64 * 64);
 }
 
-constexpr int kRankMaxPerThread = 16;   // band ranking: nc <= 16 * 1024
+// Keys k_rank_band can rank: the band and its boundary bins, whose keys share
+// the sign, the exponent and two mantissa bits (2 to 6% of a spectrum each).
+inline int band_keys(int nc) { return std::min(nc, band_ranks(nc) + std::max(128, nc / 10)); }
 
-// Band ranks of one pixel spectrum per CTA iteration.  The walk of a long
-// coarse channel needs exact ranks only inside the band [r_lo, r_lo + B) of
-// the middle ranks; below and above it a count suffices.  Two radix-select
-// rounds over the 16 high key bits find the 16-bit buckets holding ranks r_lo
-// and r_lo + B - 1; the keys from the lower bucket's start to the upper
-// bucket's end (the band, its bucket mates and any ties) are compacted in
-// channel order and sorted stably, so the m-th of them has the stable rank
-// c_lo + m (c_lo = keys below the lower bucket), as in the full sort.  Output:
-// the band's sorted values (sv [pixel][0 .. B)) and the stream of band ranks
-// with the below / above codes.
-template <int KPT>   // keys per thread: nc <= KPT * 1024
-__global__ void __launch_bounds__(1024)
-k_rank_band(const float* __restrict__ z, int n_valid, int nc, int h, int r_lo, int B, float* __restrict__ sv,
-            uint32_t* __restrict__ steps) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int W = blockDim.x >> 5;
-  uint32_t* hist = reinterpret_cast<uint32_t*>(smem);           // 256 * (W + 1): sort; 3 * 256 + 512: select
-  uint32_t* tot = hist + 256 * (W + 1);                          // 32
-  uint32_t* ka = tot + 32;
-  uint32_t* kb = ka + nc;
-  uint16_t* ia = reinterpret_cast<uint16_t*>(kb + nc);
-  uint16_t* ib = ia + nc;
-  __shared__ int sel[8];                                         // d_lo, d_hi, c1_lo, c1_hi, e_lo, e_hi, c2_lo, m
+// Block-wide exclusive scan of the kBins counters of hist: this thread's bins
+// (kBins / T consecutive ones) are left in c and the count before them returned.
+template <int T>
+__device__ __forceinline__ uint32_t scan_bins(const uint32_t* hist, uint32_t* wtot, uint32_t (&c)[kBins / T]) {
+  constexpr int PER = kBins / T, NW = T / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned lt_mask = (1u << lane) - 1u;
-  const int r_hi = r_lo + B - 1;
+  if constexpr (PER == 2) {
+    const uint2 q = reinterpret_cast<const uint2*>(hist)[threadIdx.x];
+    c[0] = q.x;
+    c[1] = q.y;
+  } else {
+#pragma unroll
+    for (int u = 0; u < PER / 4; ++u) {
+      const uint4 q = reinterpret_cast<const uint4*>(hist)[threadIdx.x * (PER / 4) + u];
+      c[4 * u] = q.x;
+      c[4 * u + 1] = q.y;
+      c[4 * u + 2] = q.z;
+      c[4 * u + 3] = q.w;
+    }
+  }
+  uint32_t s = 0;
+#pragma unroll
+  for (int u = 0; u < PER; ++u) s += c[u];
+  uint32_t v = s;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += t;
+  }
+  if (lane == 31) wtot[warp] = v;
+  __syncthreads();
+  // every warp scans the warp totals for itself
+  uint32_t w = lane < NW ? wtot[lane] : 0u;
+#pragma unroll
+  for (int o = 1; o < NW; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, w, o);
+    if (lane >= o) w += t;
+  }
+  const uint32_t before = __shfl_sync(0xffffffffu, w, warp > 0 ? warp - 1 : 0);
+  return v - s + (warp > 0 ? before : 0u);
+}
+
+// One pixel spectrum per CTA iteration, its keys in registers.
+//  1. A histogram of the keys' top 11 bits (sign, exponent, two mantissa bits)
+//     gives the bins of the ranks r_lo and r_hi; the keys from the first bin's
+//     start to the second's end are the candidates.  When they are too many
+//     (a spectrum far from zero falls into a few of those bins), the interval
+//     is histogrammed again, finer.
+//  2. The candidates are counted into kBins bins linear in the value (the
+//     middle of a spectrum is close to uniform there: about one key a bin),
+//     and a scan of the counts gives every bin its range of ranks.
+//  3. The candidates are moved to their bins' ranges, and a key's rank is its
+//     bin's first rank plus the keys of its bin before it (by value, then by
+//     place: equal values may take their ranks in any order, the medians are
+//     values).  Threads take candidates here, not channels: a band is a
+//     quarter to a half of a spectrum.
+// Output: the sorted values of the band (sv [pixel][0 .. B)) and the stream
+// of band ranks; a spectrum whose candidates stay too many (ties) or are not
+// finite is listed in fail and marked in failed, to be ranked and walked in
+// full.
+// The kernel is issue bound (68% of issue slots, 190 instructions per 32 keys
+// where all are candidates).  Sorting the band by four 8-bit radix passes with
+// all 1024 threads of an SM on one pixel spent its time in the passes' counters
+// and barriers, as much for a short spectrum as for a long one.  51,468
+// pixels, radix passes -> now: 8192 channels 7.57 -> 2.02 ms, 4096 6.77 ->
+// 1.08 ms, 1024 (all ranks) 2.65 -> 0.62 ms.
+// T threads with KPT keys each: nc <= KPT T.
+template <int T, int KPT>
+__global__ void __launch_bounds__(T, 1024 / T)
+k_rank_band(const float* __restrict__ z, int n_valid, int nc, int h, int B, int cap, float* __restrict__ sv,
+            uint32_t* __restrict__ steps, int* __restrict__ fail, int* __restrict__ n_fail,
+            uint8_t* __restrict__ failed) {
+  constexpr int PER = kBins / T;
+  extern __shared__ __align__(16) unsigned char smem[];
+  uint32_t* hist = reinterpret_cast<uint32_t*>(smem);             // [kBins], then the number of candidates
+  uint32_t* ka = hist + kBins + 4;                                 // [cap] candidate keys by bin
+  float* sorted = reinterpret_cast<float*>(ka + cap);              // [cap]
+  uint16_t* rk = reinterpret_cast<uint16_t*>(sorted + cap);        // [nc] band rank or code
+  uint16_t* ic = rk + nc;                                          // [cap] candidate channels
+  const int r_lo = max(0, nc / 2 - B / 2), r_hi = min(nc - 1, r_lo + B - 1);
+  __shared__ uint32_t wtot[32];
+  __shared__ int sel[4];                 // bin of r_lo, keys before it, bin of r_hi, keys up to its end
+  const int t = threadIdx.x;
+  const bool vec = (nc & 3) == 0;
+  for (int i = t; i < kBins; i += T) hist[i] = 0u;
   for (int p = blockIdx.x; p < n_valid; p += gridDim.x) {
     const float* zp = z + static_cast<long long>(p) * nc;
-    // channel i * blockDim + t in register i: a warp's lanes hold 32 consecutive channels
+    // key 4 i + u is channel 4 (i T + t) + u
     uint32_t key[KPT];
 #pragma unroll
-    for (int i = 0; i < KPT; ++i) {
-      const int k = i * blockDim.x + threadIdx.x;
-      key[i] = k < nc ? f2key(__ldg(zp + k)) : 0u;
-    }
-    uint32_t* h1 = hist;
-    uint32_t* h2lo = hist + 256;
-    uint32_t* h2hi = hist + 512;
-    uint32_t* cnt = hist + 768;                                  // per-chunk candidate counts
-    for (int i = threadIdx.x; i < 768; i += blockDim.x) hist[i] = 0;
-    __syncthreads();
-    // round 1: the top byte (shared atomics; equal digits within a warp are
-    // serialised by the shared-memory pipe, not by issued instructions)
-#pragma unroll
-    for (int i = 0; i < KPT; ++i) {
-      if (i * static_cast<int>(blockDim.x) >= nc) break;
-      if (i * blockDim.x + threadIdx.x < nc) atomicAdd(&h1[key[i] >> 24], 1u);
-    }
-    __syncthreads();
-    if (warp == 0) {
-      find_bin(h1, r_lo, &sel[0], &sel[2]);
-      find_bin(h1, r_hi, &sel[1], &sel[3]);
-    }
-    __syncthreads();
-    const uint32_t d_lo = sel[0], d_hi = sel[1];
-    // round 2: the second byte among keys of the two boundary top bytes
-#pragma unroll
-    for (int i = 0; i < KPT; ++i) {
-      if (i * static_cast<int>(blockDim.x) >= nc) break;
-      const bool valid = i * blockDim.x + threadIdx.x < nc;
-      const uint32_t t = key[i] >> 24, d = (key[i] >> 16) & 255u;
-      if (valid && t == d_lo) atomicAdd(&h2lo[d], 1u);
-      else if (valid && t == d_hi) atomicAdd(&h2hi[d], 1u);
-    }
-    __syncthreads();
-    if (warp == 0) {
-      int dummy;
-      find_bin(h2lo, r_lo - sel[2], &sel[4], &sel[6]);
-      find_bin(d_hi == d_lo ? h2lo : h2hi, r_hi - sel[3], &sel[5], &dummy);
-    }
-    __syncthreads();
-    const uint32_t v_lo = (d_lo << 24) | (static_cast<uint32_t>(sel[4]) << 16);
-    const uint32_t v_hi = (d_hi << 24) | (static_cast<uint32_t>(sel[5]) << 16) | 0xffffu;
-    const int c_lo = sel[2] + sel[6];                            // keys below v_lo
-    // compaction of the candidates in channel order: chunk (i, warp) is
-    // channels [i * blockDim + 32 warp, + 32)
-    const int n_chunks = (nc + blockDim.x - 1) / blockDim.x * W;
-#pragma unroll
-    for (int i = 0; i < KPT; ++i) {
-      if (i * static_cast<int>(blockDim.x) >= nc) break;
-      const bool valid = i * blockDim.x + threadIdx.x < nc;
-      const bool cand = valid && key[i] >= v_lo && key[i] <= v_hi;
-      const unsigned bc = __ballot_sync(0xffffffffu, cand);
-      if (lane == 0) cnt[i * W + warp] = __popc(bc);
-    }
-    __syncthreads();
-    if (warp == 0) {
-      // exclusive scan of the n_chunks (<= 512) counts, 16 per lane
-      const int per = (n_chunks + 31) / 32;
-      uint32_t s = 0;
-      for (int u = 0; u < per; ++u) {
-        const int j = lane * per + u;
-        if (j < n_chunks) s += cnt[j];
+    for (int i = 0; i < KPT / 4; ++i) {
+      const int k = 4 * (i * T + t);
+      float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (vec) {
+        if (k < nc) q = __ldg(reinterpret_cast<const float4*>(zp + k));
+      } else {
+        if (k < nc) q.x = __ldg(zp + k);
+        if (k + 1 < nc) q.y = __ldg(zp + k + 1);
+        if (k + 2 < nc) q.z = __ldg(zp + k + 2);
+        if (k + 3 < nc) q.w = __ldg(zp + k + 3);
       }
-      uint32_t incl = s;
+      key[4 * i] = f2key(q.x);
+      key[4 * i + 1] = f2key(q.y);
+      key[4 * i + 2] = f2key(q.z);
+      key[4 * i + 3] = f2key(q.w);
+    }
+    auto exists = [&](int i) { return 4 * ((i >> 2) * T + t) + (i & 3) < nc; };
+    __syncthreads();                                               // hist is zero, the last pixel's arrays are free
+    // 1. the candidate interval [klo, khi], c_lo keys below it, m keys in it
+    uint32_t klo = 0u, khi = 0xffffffffu;
+    int sh = 21, c_lo = 0, m = nc;
+    for (;;) {
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-      }
-      uint32_t run = incl - s;
-      for (int u = 0; u < per; ++u) {
-        const int j = lane * per + u;
-        if (j < n_chunks) {
-          const uint32_t c = cnt[j];
-          cnt[j] = run;
-          run += c;
+      for (int i = 0; i < KPT; ++i)
+        if (exists(i) && key[i] >= klo && key[i] <= khi) atomicAdd(&hist[(key[i] - klo) >> sh], 1u);
+      __syncthreads();
+      uint32_t c[PER];
+      uint32_t run = static_cast<uint32_t>(c_lo) + scan_bins<T>(hist, wtot, c);
+#pragma unroll
+      for (int u = 0; u < PER; ++u) {
+        if (run <= static_cast<uint32_t>(r_lo) && static_cast<uint32_t>(r_lo) < run + c[u]) {
+          sel[0] = t * PER + u;
+          sel[1] = static_cast<int>(run);
         }
+        if (run <= static_cast<uint32_t>(r_hi) && static_cast<uint32_t>(r_hi) < run + c[u]) {
+          sel[2] = t * PER + u;
+          sel[3] = static_cast<int>(run + c[u]);
+        }
+        run += c[u];
+        hist[t * PER + u] = 0u;
       }
-      if (lane == 31) sel[7] = static_cast<int>(incl);
+      __syncthreads();
+      const uint32_t width = (static_cast<uint32_t>(sel[2] - sel[0]) << sh) + ((1u << sh) - 1u);
+      klo += static_cast<uint32_t>(sel[0]) << sh;
+      khi = min(khi, klo + width);
+      c_lo = sel[1];
+      m = sel[3] - sel[1];
+      if (m <= cap) break;
+      // finer bins, at most kBins of them over the interval (an interval across
+      // zero spans as many exponents as there are: it gets no finer)
+      const int next = max(0, 32 - __clz(static_cast<int>(khi - klo)) - 11);
+      if (next >= sh) break;
+      sh = next;
+      __syncthreads();                                             // sel is read
     }
-    __syncthreads();
-    const int m = sel[7];
-    uint16_t* rk = ib;                                           // channel -> band rank or code, after the sort
+    const float xlo = key2f(klo), xhi = key2f(khi);
+    const float span = xhi - xlo;
+    if (!(m <= cap && span >= 0.0f && span < INFINITY)) {          // the same for the whole CTA
+      if (t == 0) {
+        fail[atomicAdd(n_fail, 1)] = p;
+        failed[p] = 1;
+      }
+      continue;                                                    // hist is zero again
+    }
+    // 2. bins linear in the value: a monotone map, so bins order the keys
+    const float scale = span > 0.0f ? static_cast<float>(kBins) / span : 0.0f;
+    auto bin_of = [&](uint32_t k) { return min(static_cast<int>((key2f(k) - xlo) * scale), kBins - 1); };
+    uint32_t at[KPT];                                              // bin | place within the bin << 11
 #pragma unroll
     for (int i = 0; i < KPT; ++i) {
-      if (i * static_cast<int>(blockDim.x) >= nc) break;
-      const int k = i * blockDim.x + threadIdx.x;
-      const bool valid = k < nc;
-      const bool cand = valid && key[i] >= v_lo && key[i] <= v_hi;
-      const unsigned bc = __ballot_sync(0xffffffffu, cand);
-      if (cand) {
-        const uint32_t pos = cnt[i * W + warp] + __popc(bc & lt_mask);
-        ka[pos] = key[i];
-        ia[pos] = static_cast<uint16_t>(k);
+      at[i] = 0xffffffffu;
+      if (exists(i) && key[i] >= klo && key[i] <= khi) {
+        const int b = bin_of(key[i]);
+        at[i] = static_cast<uint32_t>(b) | (atomicAdd(&hist[b], 1u) << 11);
       }
     }
     __syncthreads();
-    lsd_sort(ka, ia, kb, ib, m, hist, tot, W);
-    // candidate j has stable rank c_lo + j, band rank j - (r_lo - c_lo)
-    const int off = r_lo - c_lo;
+    {
+      uint32_t c[PER];
+      uint32_t run = scan_bins<T>(hist, wtot, c);
+#pragma unroll
+      for (int u = 0; u < PER; ++u) {
+        hist[t * PER + u] = run;
+        run += c[u];
+      }
+      if (t == T - 1) hist[kBins] = run;
+    }
+    __syncthreads();
+    // 3. the candidates at their bins; codes for the other channels
+#pragma unroll
+    for (int i = 0; i < KPT; ++i)
+      if (at[i] != 0xffffffffu) {
+        const uint32_t j = hist[at[i] & (kBins - 1)] + (at[i] >> 11);
+        ka[j] = key[i];
+        ic[j] = static_cast<uint16_t>(4 * ((i >> 2) * T + t) + (i & 3));
+      }
+#pragma unroll
+    for (int i = 0; i < KPT; i += 4) {
+      uint32_t c[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) c[u] = static_cast<uint32_t>(key[i + u] < klo ? kRankBelow : kRankAbove) & 0xffffu;
+      const int k = 4 * ((i >> 2) * T + t);
+      if (k + 3 < nc) {
+        *reinterpret_cast<uint2*>(rk + k) = make_uint2(c[0] | (c[1] << 16), c[2] | (c[3] << 16));
+      } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (k + u < nc) rk[k + u] = static_cast<uint16_t>(c[u]);
+      }
+    }
+    __syncthreads();
+    for (int j = t; j < m; j += T) {
+      const uint32_t k = ka[j];
+      const int b = bin_of(k);
+      const int j0 = static_cast<int>(hist[b]), j1 = static_cast<int>(hist[b + 1]);
+      int r = j0;
+      for (int o = j0; o < j1; ++o) {
+        const uint32_t other = ka[o];
+        r += (other < k || (other == k && o < j)) ? 1 : 0;
+      }
+      sorted[r] = key2f(k);
+      r -= r_lo - c_lo;
+      rk[ic[j]] = static_cast<uint16_t>(r < 0 ? kRankBelow : (r >= B ? kRankAbove : r));
+    }
+    __syncthreads();
+    for (int i = t; i < kBins; i += T) hist[i] = 0u;
     float* svp = sv + static_cast<long long>(p) * nc;
-    for (int j = threadIdx.x; j < B; j += blockDim.x) svp[j] = key2f(ka[off + j]);
-    for (int j = threadIdx.x; j < m; j += blockDim.x) {
-      const int b = j - off;
-      rk[ia[j]] = static_cast<uint16_t>(b < 0 ? kRankBelow : (b >= B ? kRankAbove : static_cast<uint32_t>(b)));
-    }
-#pragma unroll
-    for (int i = 0; i < KPT; ++i) {
-      const int k = i * blockDim.x + threadIdx.x;
-      if (k < nc && (key[i] < v_lo || key[i] > v_hi))
-        rk[k] = static_cast<uint16_t>(key[i] < v_lo ? kRankBelow : kRankAbove);
-    }
-    __syncthreads();
+    for (int j = t; j <= r_hi - r_lo; j += T) svp[j] = sorted[r_lo - c_lo + j];
     write_stream(rk, nc, h, steps + static_cast<long long>(p) * walk_stride(nc, h));
-    __syncthreads();
   }
 }
 
 // --------------------------------------------------------- a9 running median
 // The walk keeps, per pixel spectrum, the set of ranks inside the current
-// window as a bitset over B ranks (the full walk: every rank, B >= nc; the
-// band walk: the middle 2048 ranks of the band stream, whose elements below
-// and above the band are only counted).  A cursor word W with lt = the number of
-// set bits in words below W finds any order statistic of the band in a few
-// word steps, since consecutive windows move it by at most one element; an
-// insert or remove below W moves lt by one, so no step needs a search for a
-// removed element.  A pixel's outputs may be split into S segments of
-// consecutive channels, each walked by its own thread from the window before
-// its first output (built from the inserts of the stream), so the chain of
-// dependent steps a thread runs is about nc / S + w instead of nc + w / 2.
+// window as a bitset (the full walk: every rank; the band walk: the ranks of
+// the band stream, whose elements below and above the band have no bit) and
+// the rank m of its lower median with the number of the window's elements below
+// m.  An inserted or removed element changes that number by one when it is
+// below m, so consecutive windows move m by a set bit or two, found in m's
+// word or the next; no order statistic is searched for.  A pixel's outputs
+// may be split into S segments of consecutive channels, each walked by its own
+// thread from the window before its first output (built from the inserts of
+// the stream), so the chain of dependent steps a thread runs is about
+// nc / S + w instead of nc + w / 2.  Bound by issue (61% of the slots at 95
+// instructions a step, 22 of 32 lanes active) and the latency of the chain;
+// with the median searched for from a cursor word in every step 51,468 pixels
+// of 8192 channels took 5.53 ms, now 3.44.
 
 // Position of the n-th (0-based) set bit of x, n < popc(x): binary search on
 // the population counts of the low halves.
@@ -616,92 +683,68 @@ __device__ __forceinline__ int select_bit(uint32_t x, int n) {
   return pos + (n >= static_cast<int>(x & 1u) ? 1 : 0);
 }
 
-struct WalkState {
-  int below, above, band;   // window elements below, above and inside the band
-  int W, lt;                // cursor word; set bits in the words below it
-};
-
-// Insert (sgn = +1) or remove (sgn = -1) band rank r (r < 0: below the band,
-// r >= B: above it).  Ranks are distinct, so both flip one bit.  Bit b of a
-// thread's set is word b / 32 at bits[(b / 32) * T] (the words of the
-// threads of a CTA interleave).
-template <bool BAND, int T>
-__device__ __forceinline__ void walk_update(uint32_t* bits, int r, int B, int sgn, WalkState& s) {
-  const bool inb = !BAND || static_cast<unsigned>(r) < static_cast<unsigned>(B);
-  if (BAND) {
-    s.below += r < 0 ? sgn : 0;
-    s.above += r >= B ? sgn : 0;
-  }
-  if (inb) bits[(r >> 5) * T] ^= 1u << (r & 31);
-  s.band += inb ? sgn : 0;
-  s.lt += (inb && (r >> 5) < s.W) ? sgn : 0;
+// Bit b of a thread's set is bit b % 32 of word bits[(b / 32) * T] (the words of
+// the threads of a CTA interleave, so every access is free of conflicts).
+// Words -1 and nwords are zero; word nwords + 1 takes the flips of elements
+// without a bit, so that a flip has no branch.
+template <int T>
+__device__ __forceinline__ void flip_bit(uint32_t* bits, int r, int nwords) {
+  uint32_t* w = bits + min(static_cast<uint32_t>(r) >> 5, static_cast<uint32_t>(nwords + 1)) * T;
+  *w ^= 1u << (r & 31);
 }
 
-// Band positions of the window's lower and upper median (equal for an odd
-// window); false if either lies outside the band.
-template <bool BAND, int T>
-__device__ __forceinline__ bool walk_median(const uint32_t* bits, WalkState& s, int& lo, int& hi) {
-  const int below = BAND ? s.below : 0;
-  const int size = below + s.band + (BAND ? s.above : 0);
-  const int tb = ((size - 1) >> 1) - below;
-  const bool even = (size & 1) == 0;
-  if (tb < 0 || tb + (even ? 1 : 0) >= s.band) return false;
-  // lt > tb >= 0 means a set bit below W; lt + popc(word W) <= tb < band means
-  // a set bit above it: the cursor stays inside the set's words
-  while (s.lt > tb) {
-    --s.W;
-    s.lt -= __popc(bits[s.W * T]);
+// The element at position `target` of the window, given m with `pos` of its
+// elements below m: the (target - pos)-th set bit at or above m, or, when pos
+// is larger, the (pos - target - 1)-th below it.  The search upwards and the
+// (bit-reversed) search downwards are one code path over m's word and its
+// neighbour, without a branch; only a longer way takes the loop (a band has a
+// set bit every five).  Returns false when the set has no such bit (m is then
+// left in place).
+template <int T>
+__device__ __forceinline__ bool seek_bit(const uint32_t* bits, int nwords, int target, int& m, int& pos) {
+  const int d = target - pos;
+  const int s = d >> 31;                               // 0 up, -1 down
+  const int skip = d ^ s;
+  const int dw = s | 1;
+  int w = m >> 5;
+  uint32_t x = bits[w * T], y = bits[(w + dw) * T];
+  x &= (0xffffffffu << (m & 31)) ^ static_cast<uint32_t>(s);
+  if (s) {
+    x = __brev(x);
+    y = __brev(y);
   }
-  uint32_t x = bits[s.W * T];
-  int pc = __popc(x);
-  while (s.lt + pc <= tb) {
-    s.lt += pc;
-    ++s.W;
-    x = bits[s.W * T];
-    pc = __popc(x);
-  }
-  const int b = select_bit(x, tb - s.lt);
-  lo = (s.W << 5) + b;
-  hi = lo;
-  if (even) {
-    // the next set bit: in this word above b, else in a following word
-    const uint32_t rest = b < 31 ? x & (0xfffffffeu << b) : 0u;
-    if (rest) {
-      hi = (s.W << 5) + __ffs(rest) - 1;
-    } else {
-      int w2 = s.W + 1;
-      uint32_t y = bits[w2 * T];
-      while (y == 0u) y = bits[++w2 * T];
-      hi = (w2 << 5) + __ffs(y) - 1;
+  // one set bit to skip: of this word, or of the neighbour when this one is empty
+  const uint32_t x1 = x & (x - 1u), y1 = y & (y - 1u);
+  const bool none = x == 0u;
+  if (skip) y = none ? y1 : y;
+  if (skip) x = x1;
+  if (none) x = 0u;
+  const bool cross = x == 0u;
+  x = cross ? y : x;
+  w += cross ? dw : 0;
+  if (x == 0u || skip > 1) {
+    w = m >> 5;
+    int left = skip;
+    x = bits[w * T] & ((0xffffffffu << (m & 31)) ^ static_cast<uint32_t>(s));
+    if (s) x = __brev(x);
+    for (;;) {
+      while (left > 0 && x) {
+        x &= x - 1u;
+        --left;
+      }
+      if (x) break;
+      w += dw;
+      if (static_cast<unsigned>(w) >= static_cast<unsigned>(nwords)) return false;
+      x = bits[w * T];
+      if (s) x = __brev(x);
     }
   }
-  return true;
-}
-
-// Applies f(index, word) to words [w0, w1) of a pixel's step stream, read in
-// 16-byte chunks two chunks ahead; stops when f returns false.
-template <class F>
-__device__ __forceinline__ bool for_steps(const uint4* __restrict__ st4, int w0, int w1, F&& f) {
-  const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
-  const int ce = (w1 + 3) >> 2;
-  int c = w0 >> 2;
-  uint4 a = c < ce ? st4[c] : zero4, b = c + 1 < ce ? st4[c + 1] : zero4;
-  for (; c < ce; ++c) {
-    const uint4 nx = c + 2 < ce ? st4[c + 2] : zero4;
-    const uint32_t sw[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int i = (c << 2) + q;
-      if (i >= w0 && i < w1 && !f(i, sw[q])) return false;
-    }
-    a = b;
-    b = nx;
-  }
+  m = (w << 5) + ((__ffs(x) - 1) ^ (s & 31));
+  pos = target;
   return true;
 }
 
 constexpr int kWalkThreads = 64;   // full walk: nc / 32 words per thread
-constexpr int kBandWordsMax = 64;  // band walk: up to 2048 ranks
 constexpr int kBandThreads = 128;
 
 // One thread per (pixel, segment) walks the segment's outputs over the step
@@ -710,71 +753,146 @@ constexpr int kBandThreads = 128;
 // stream), to med [pixel][nc]; k_median_sub then applies them with all
 // threads (the gathers of the sorted values would otherwise sit in the walk's
 // chain of dependent steps).
-//   BAND: the band stream (nwords * 32 band ranks); a segment whose median
+//   fail: the band stream (nwords * 32 band ranks); a segment whose median
 //     leaves the band gives up, and its pixel is listed once in fail (k_rank
-//     and the full walk redo it).
-//   !BAND: the full rank set (nwords = nc / 32 rounded up); with a pixel list
-//     (the band walk's failures) item i walks list[i], i < *n_list.
+//     and the full walk redo it), behind the pixels k_rank_band listed there.
+//   no fail: the full rank set (nwords = nc / 32 rounded up); with a pixel list
+//     (the band kernels' failures) item i walks list[i], i < *n_list.
 // seg_len is a multiple of 4, so every segment's steps start on a chunk.
-template <bool BAND, int T>
+//     The pixels marked in failed have no band stream and are left out.
+template <int T>
 __global__ void __launch_bounds__(T)
 k_walk(const uint32_t* __restrict__ steps, int n_valid, int nc, int h, int n_seg, int seg_len, int nwords,
        uint32_t* __restrict__ med, const int* __restrict__ list, const int* __restrict__ n_list,
-       int* __restrict__ fail, int* __restrict__ n_fail) {
+       int* __restrict__ fail, int* __restrict__ n_fail, const uint8_t* __restrict__ failed) {
   extern __shared__ uint32_t bits_all[];
   const int t = threadIdx.x;
   const int item = (blockIdx.x * T + t) / n_seg;
   const int sg = (blockIdx.x * T + t) - item * n_seg;
-  uint32_t* bits = bits_all + t;
+  uint32_t* bits = bits_all + T + t;                  // word -1 first
   int p = item;
   bool live = item < n_valid;
-  if (!BAND && list) {
+  if (list) {
     live = item < min(*n_list, n_valid);
     p = live ? list[item] : 0;
   }
-  bool gave_up = false;
+  if (failed) live = live && !failed[p];
+  bool ok = true;
   if (live) {
-    for (int w = 0; w < nwords; ++w) bits[w * T] = 0u;
-    const int B = nwords * 32;
+    for (int w = -1; w <= nwords; ++w) bits[w * T] = 0u;
     const int H = (h + 3) & ~3;
     const int k0 = sg * seg_len, k1 = min(nc, k0 + seg_len);
     const uint4* st4 = reinterpret_cast<const uint4*>(steps + static_cast<long long>(p) * walk_stride(nc, h));
-    uint32_t* mo = med + static_cast<long long>(p) * nc - H;
-    WalkState s{0, 0, 0, 0, 0};
-    auto rank_of = [&](uint32_t r) {
-      if (!BAND) return static_cast<int>(r);
-      return r == kRankBelow ? -1 : (r == kRankAbove ? B : static_cast<int>(r));
-    };
-    // the window before output k0: channels [k0 - 1 - h, k0 - 1 + h]; channel
-    // j is inserted by word j - h + H (the words below H build the first window)
-    const int wa = max(H - h, H + k0 - 1 - 2 * h), wb = H + k0;
-    bool ok = for_steps(st4, wa, wb, [&](int, uint32_t word) {
-      const uint32_t rin = word & 0xffffu;
-      if (rin != kRankNone) walk_update<BAND, T>(bits, rank_of(rin), B, 1, s);
-      return true;
-    });
-    ok = ok && for_steps(st4, H + k0, H + k1, [&](int i, uint32_t word) {
-      const uint32_t rin = word & 0xffffu, rout = word >> 16;
-      if (rin != kRankNone) walk_update<BAND, T>(bits, rank_of(rin), B, 1, s);
-      if (rout != kRankNone) walk_update<BAND, T>(bits, rank_of(rout), B, -1, s);
-      int lo, hi;
-      if (!walk_median<BAND, T>(bits, s, lo, hi)) return false;
-      mo[i] = static_cast<uint32_t>(lo) | (static_cast<uint32_t>(hi) << 16);
-      return true;
-    });
-    if (!ok) {
-      if (BAND) gave_up = true;
-      else atomicExch(&g_detect_status, 3);            // the full set always holds the median
+    uint4* mo = reinterpret_cast<uint4*>(med + static_cast<long long>(p) * nc);
+    const bool vec = (nc & 3) == 0;
+    auto rank_in = [](uint32_t w) { return static_cast<int>(static_cast<short>(w & 0xffffu)); };
+    auto rank_out = [](uint32_t w) { return static_cast<int>(w) >> 16; };
+    // the window before output k0, channels [k0 - 1 - h, k0 - 1 + h]: channel j
+    // is inserted by word j - h + H (the words below H build the first window)
+    int below = 0, size = 0;
+    {
+      const int wa = max(H - h, H + k0 - 1 - 2 * h), wb = min(H + k0, H + nc - h);
+      const int ce = (wb + 3) >> 2;
+      int c = wa >> 2;
+      const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
+      uint4 a = c < ce ? __ldg(st4 + c) : zero4, b = c + 1 < ce ? __ldg(st4 + c + 1) : zero4;
+      for (; c < ce; ++c) {
+        const uint4 nx = c + 2 < ce ? __ldg(st4 + c + 2) : zero4;
+        const uint32_t sw[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int i = (c << 2) + q;
+          if (i >= wa && i < wb) {
+            const int r = rank_in(sw[q]);
+            flip_bit<T>(bits, r, nwords);
+            below += r < 0 ? 1 : 0;
+            ++size;
+          }
+        }
+        a = b;
+        b = nx;
+      }
     }
+    // its lower median by the words' counts (an empty window: rank 0, with the
+    // elements below the set's first rank below it)
+    int m = 0, pos = below;
+    if (size > 0) {
+      int want = ((size - 1) >> 1) - below;
+      ok = want >= 0;
+      pos = below + want;
+      int w = 0;
+      for (; ok && w < nwords; ++w) {
+        const int c = __popc(bits[w * T]);
+        if (want < c) break;
+        want -= c;
+      }
+      ok = ok && w < nwords;
+      if (ok) m = (w << 5) + select_bit(bits[w * T], want);
+    }
+    const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
+    const int c0 = (H + k0) >> 2, ce = (H + k1 + 3) >> 2;
+    uint4 a = c0 < ce ? __ldg(st4 + c0) : zero4, b = c0 + 1 < ce ? __ldg(st4 + c0 + 1) : zero4;
+    for (int c = c0; c < ce && ok; ++c) {
+      const uint4 nx = c + 2 < ce ? __ldg(st4 + c + 2) : zero4;
+      const uint32_t sw[4] = {a.x, a.y, a.z, a.w};
+      uint32_t out[4] = {0u, 0u, 0u, 0u};
+      const int k = (c << 2) - H;
+      if (k > h && k + 3 + h < nc && k + 4 <= k1) {
+        // whole windows: one in, one out, an odd size
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int rin = rank_in(sw[q]), rout = rank_out(sw[q]);
+          flip_bit<T>(bits, rin, nwords);
+          flip_bit<T>(bits, rout, nwords);
+          pos += (rin < m ? 1 : 0) - (rout < m ? 1 : 0);
+          ok = seek_bit<T>(bits, nwords, h, m, pos) && ok;
+          out[q] = static_cast<uint32_t>(m) * 0x10001u;
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (ok && k + q < k1) {
+            if (k + q + h < nc) {
+              const int r = rank_in(sw[q]);
+              flip_bit<T>(bits, r, nwords);
+              pos += r < m ? 1 : 0;
+              ++size;
+            }
+            if (k + q - h - 1 >= 0) {
+              const int r = rank_out(sw[q]);
+              flip_bit<T>(bits, r, nwords);
+              pos -= r < m ? 1 : 0;
+              --size;
+            }
+            ok = seek_bit<T>(bits, nwords, (size - 1) >> 1, m, pos);
+            int hi = m;
+            if (ok && (size & 1) == 0) {
+              int above = pos;
+              ok = seek_bit<T>(bits, nwords, size >> 1, hi, above);
+            }
+            out[q] = static_cast<uint32_t>(m) | (static_cast<uint32_t>(hi) << 16);
+          }
+      }
+      if (vec) {
+        mo[k >> 2] = make_uint4(out[0], out[1], out[2], out[3]);
+      } else {
+        uint32_t* m1 = med + static_cast<long long>(p) * nc + k;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (k + q < k1) m1[q] = out[q];
+      }
+      a = b;
+      b = nx;
+    }
+    if (!ok && !fail) atomicExch(&g_detect_status, 3);   // the full set always holds the median
   }
-  if (BAND) {
+  if (fail) {
     // a pixel's segments are adjacent threads of one warp (n_seg divides 32)
-    const unsigned any = __ballot_sync(0xffffffffu, gave_up);
+    const unsigned any = __ballot_sync(0xffffffffu, live && !ok);
     const int lane = t & 31, first = lane - sg;
     const unsigned mine = ((n_seg >= 32) ? 0xffffffffu : ((1u << n_seg) - 1u)) << first;
     if (live && sg == 0 && (any & mine)) {
-      const int slot = atomicAdd(n_fail, 1);
-      if (slot < n_valid) fail[slot] = p;
+      fail[atomicAdd(n_fail, 1)] = p;                 // at most once per pixel
     }
   }
 }
@@ -1304,7 +1422,8 @@ struct DetectWs {
   float* sv;
   uint32_t* steps;
   uint32_t* med;         // [pixel][channel] median ranks of the current coarse block
-  int* fail;             // pixels whose band walk gave up
+  int* fail;             // pixels whose band ranking or band walk gave up
+  uint8_t* failed;       // [pixel] 1: the band ranking gave up
   float* snr;
   uint8_t* width;
   unsigned long long* hist;
@@ -1332,6 +1451,7 @@ DetectWs carve_detect(void* ws, size_t bytes, const DetectPlan& p, size_t* need)
   w.steps = c.take<uint32_t>(static_cast<size_t>(p.n_valid) * p.max_steps);
   w.med = c.take<uint32_t>(blk);
   w.fail = c.take<int>(p.n_valid > 0 ? p.n_valid : 1);
+  w.failed = c.take<uint8_t>(p.n_valid > 0 ? p.n_valid : 1);
   w.snr = c.take<float>(static_cast<size_t>(p.n_vox));
   w.width = c.take<uint8_t>(static_cast<size_t>(p.n_vox));
   w.hist = c.take<unsigned long long>(kMaxBins);
@@ -1395,75 +1515,67 @@ int run_filter_coarse(int c, const float* img_block, const DetectPlan& p, const 
     OVRO_LAUNCH_CHECK();
   }
   {
-    // Coarse channels longer than the band: band ranks and the band walk for
-    // every pixel, then full ranks and the full walk for the pixels whose
-    // median left the band.  Shorter ones: full ranks and the full walk.
-    // the band: the middle 2048 ranks (a window median's rank wanders about
-    // nc / (2 sqrt(W)) from the middle for a stationary spectrum: 99 ranks at
-    // 8192 channels, W = 1707; on the skewed noise images of the full workload
-    // a band of 1024 sent enough pixels to the full walk to cost more than the
-    // smaller sort saved: 13.7 against 12.6 ms per step for ranks and walk)
-    const int band_words = kBandWordsMax;
-    const int band = band_words * 32;
-    const bool use_band = nc > band && nc <= kRankMaxPerThread * 1024;
-    const int threads = 1024, W = threads / 32;      // one CTA per SM (shared memory): all 32 warps
+    // Band ranks and the band walk for every pixel, then full ranks and the full
+    // walk for the pixels either gave up (a median that left the band, ties).
+    const int band = band_ranks(nc), cap = band_keys(nc);
+    // 8 or 16 keys a thread: a short spectrum takes a small CTA, so that an SM
+    // has enough of them to cover one another's barriers
+    const int threads = nc <= 1024 ? 128 : nc <= 4096 ? 256 : nc <= 8192 ? 512 : 1024;
+    auto band_kernel = nc <= 1024 ? k_rank_band<128, 8> : nc <= 2048 ? k_rank_band<256, 8>
+                       : nc <= 4096 ? k_rank_band<256, 16> : nc <= 8192 ? k_rank_band<512, 16>
+                       : k_rank_band<1024, 16>;
+    const size_t sm_band = (kBins + 4 + 2 * static_cast<size_t>(cap)) * 4 + (static_cast<size_t>(nc) + cap) * 2;
+    OVRO_CUDA_TRY(cudaFuncSetAttribute(band_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(sm_band)));
+    const int W = 32;                                // k_rank: one CTA of 1024 threads per SM (shared memory)
     const size_t sm_rank = (256 * (W + 1) + 32) * 4 + static_cast<size_t>(nc) * 12;
     OVRO_CUDA_TRY(cudaFuncSetAttribute(k_rank, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(sm_rank)));
-    OVRO_CUDA_TRY(cudaFuncSetAttribute(k_rank_band<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(sm_rank)));
-    OVRO_CUDA_TRY(cudaFuncSetAttribute(k_rank_band<kRankMaxPerThread>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(sm_rank)));
     // CTAs per SM (each CTA loops over pixels; the outputs do not depend on it)
     auto rank = [&](int per_sm) -> int {
-      const int blocks = std::min(p.n_valid, per_sm * nsm);
+      OVRO_CUDA_TRY(cudaMemsetAsync(w.count + 3, 0, sizeof(int), st));
+      OVRO_CUDA_TRY(cudaMemsetAsync(w.failed, 0, p.n_valid, st));
       OVRO_PROF("k_rank", st);
-      if (use_band && nc <= 8 * 1024)
-        k_rank_band<8><<<blocks, threads, sm_rank, st>>>(w.zbuf, p.n_valid, nc, p.half[c], nc / 2 - band / 2, band,
-                                                         w.sv, w.steps);
-      else if (use_band)
-        k_rank_band<kRankMaxPerThread><<<blocks, threads, sm_rank, st>>>(w.zbuf, p.n_valid, nc, p.half[c],
-                                                                         nc / 2 - band / 2, band, w.sv, w.steps);
-      else
-        k_rank<<<blocks, threads, sm_rank, st>>>(w.zbuf, p.n_valid, nc, p.half[c], w.sv, w.steps, nullptr, nullptr);
+      band_kernel<<<std::min(p.n_valid, per_sm * nsm), threads, sm_band, st>>>(
+          w.zbuf, p.n_valid, nc, p.half[c], band, cap, w.sv, w.steps, w.fail, w.count + 3, w.failed);
       OVRO_LAUNCH_CHECK();
       return OVRO_OK;
     };
-    const std::string rkey = tune_key(use_band ? "k_rank_band" : "k_rank", {p.n_valid, nc});
+    const std::string rkey = tune_key("k_rank_band", {p.n_valid, nc});
     int per_sm = tuned(rkey, 16);
     if (tuning(st))
-      if (int e = tune_pick(rkey, {1, 2, 4, 16}, rank, st, &per_sm)) return e;
+      if (int e = tune_pick(rkey, {4, 8, 16, 32}, rank, st, &per_sm)) return e;
 
     // S segments per pixel (S divides 32), tuned per shape; a trial ranks
     // again, since the fallback rewrites the failed pixels' streams
     const int nwords = (nc + 31) / 32;
-    const size_t sm_full = static_cast<size_t>(nwords) * kWalkThreads * 4;
-    const size_t sm_band = static_cast<size_t>(band_words) * kBandThreads * 4;
-    OVRO_CUDA_TRY(cudaFuncSetAttribute(k_walk<false, kWalkThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const size_t sm_full = static_cast<size_t>(nwords + 3) * kWalkThreads * 4;
+    const size_t sm_walk = static_cast<size_t>(band / 32 + 3) * kBandThreads * 4;
+    OVRO_CUDA_TRY(cudaFuncSetAttribute(k_walk<kWalkThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(sm_full)));
+    OVRO_CUDA_TRY(cudaFuncSetAttribute(k_walk<kBandThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(sm_walk)));
     auto rank_walk = [&](int n_seg) -> int {
       if (int e = rank(per_sm)) return e;
       const int seg_len = ((nc + n_seg - 1) / n_seg + 3) & ~3;
       const long long thr = static_cast<long long>(p.n_valid) * n_seg;
-      if (use_band) {
-        OVRO_CUDA_TRY(cudaMemsetAsync(w.count + 3, 0, sizeof(int), st));
-        {
-          OVRO_PROF("k_walk", st);
-          k_walk<true, kBandThreads><<<static_cast<int>((thr + kBandThreads - 1) / kBandThreads), kBandThreads,
-                                       sm_band, st>>>(w.steps, p.n_valid, nc, p.half[c], n_seg, seg_len, band_words,
-                                                      w.med, nullptr, nullptr, w.fail, w.count + 3);
-          OVRO_LAUNCH_CHECK();
-        }
+      {
+        OVRO_PROF("k_walk", st);
+        k_walk<kBandThreads><<<static_cast<int>((thr + kBandThreads - 1) / kBandThreads), kBandThreads, sm_walk,
+                               st>>>(w.steps, p.n_valid, nc, p.half[c], n_seg, seg_len, band / 32, w.med, nullptr,
+                                     nullptr, w.fail, w.count + 3, w.failed);
+        OVRO_LAUNCH_CHECK();
+      }
+      {
         OVRO_PROF("k_rank", st);
-        k_rank<<<std::min(p.n_valid, nsm), threads, sm_rank, st>>>(w.zbuf, p.n_valid, nc, p.half[c], w.sv, w.steps,
-                                                                   w.fail, w.count + 3);
+        k_rank<<<std::min(p.n_valid, nsm), 1024, sm_rank, st>>>(w.zbuf, p.n_valid, nc, p.half[c], w.sv, w.steps,
+                                                                w.fail, w.count + 3);
         OVRO_LAUNCH_CHECK();
       }
       OVRO_PROF("k_walk", st);
-      k_walk<false, kWalkThreads><<<static_cast<int>((thr + kWalkThreads - 1) / kWalkThreads), kWalkThreads,
-                                    sm_full, st>>>(w.steps, p.n_valid, nc, p.half[c], n_seg, seg_len, nwords, w.med,
-                                                   use_band ? w.fail : nullptr, use_band ? w.count + 3 : nullptr,
-                                                   nullptr, nullptr);
+      k_walk<kWalkThreads><<<static_cast<int>((thr + kWalkThreads - 1) / kWalkThreads), kWalkThreads, sm_full,
+                             st>>>(w.steps, p.n_valid, nc, p.half[c], n_seg, seg_len, nwords, w.med, w.fail,
+                                   w.count + 3, nullptr, nullptr, nullptr);
       OVRO_LAUNCH_CHECK();
       return OVRO_OK;
     };
