@@ -194,7 +194,8 @@ def roofline_models(cfg, n_kept_vis, peaks):
         "k_rank": ("hbm", vox * 9, "B", cube),
         # walk: read the step stream, write the median ranks over it
         "k_walk": ("hbm", vox * 8, "B", cube),
-        # z' = z - median: read ranks and z, write z' (sorted-value gathers hit L1/L2)
+        # z' = z - median as a pass of its own (read ranks and z, write z'): k_mf
+        # does it while staging, so no launch carries this name
         "k_median_sub": ("hbm", vox * 12, "B", cube),
         # boxcars: read z', write SNR and width
         "k_mf": ("hbm", vox * 9, "B", cube),

@@ -17,10 +17,11 @@
 //                    so every step of the exact running median costs O(1).
 //      k_rank        full ranks (stable LSD radix sort) for the pixels whose
 //                    band or walk gave up; k_walk then takes them in full.
-//  a10 k_mf          per 8 consecutive channels a thread holds the 107-value
-//                    neighbourhood as register prefix sums and evaluates all 29
-//                    boxcars as prefix differences; keeps max SNR and width and
-//                    histograms the SNRs above the p = alpha floor.
+//  a10 k_mf          subtracts the medians and, per 8 consecutive channels, takes
+//                    the 107-value neighbourhood as register prefix sums and
+//                    evaluates all 29 boxcars as prefix differences; keeps max
+//                    SNR and width and histograms the SNRs above the p = alpha
+//                    floor.
 //  a11 host + k_gather_bins  Benjamini-Hochberg: counts above every
 //                    histogram bin edge are exact, so the step-up rule is
 //                    decided bin by bin in FP64; only the bins whose outcome
@@ -69,7 +70,7 @@ __host__ __device__ constexpr float rsqrt_width(int i) {
        : i == 27 ? 0.10540925533894598f : 0.10000000000000001f;
 }
 constexpr int kMaxLo = 49, kMaxHi = 50;
-constexpr int kVox = 8;                                  // voxels per thread in k_mf
+constexpr int kVox = 8;                                  // voxels per chunk in k_mf
 constexpr int kWin = kVox + kMaxLo + kMaxHi;             // 107
 
 // histogram of SNRs: bins of 2^-7 relative width from the floor up to 64, then overflow
@@ -750,7 +751,7 @@ constexpr int kBandThreads = 128;
 // One thread per (pixel, segment) walks the segment's outputs over the step
 // stream written by k_rank / k_rank_band and writes each window's median
 // ranks, lower | upper << 16 (equal for an odd window; band ranks for a band
-// stream), to med [pixel][nc]; k_median_sub then applies them with all
+// stream), to med [pixel][nc]; k_mf then applies them with all
 // threads (the gathers of the sorted values would otherwise sit in the walk's
 // chain of dependent steps).
 //   fail: the band stream (nwords * 32 band ranks); a segment whose median
@@ -897,51 +898,67 @@ k_walk(const uint32_t* __restrict__ steps, int n_valid, int nc, int h, int n_seg
   }
 }
 
-// z' = z - (v[lower] + v[upper]) / 2 for every voxel, v the pixel's sorted
-// values (the band's for a band stream) and med the median ranks the walk left.
-__global__ void k_median_sub(float* __restrict__ zbuf, const float* __restrict__ sv,
-                             const uint32_t* __restrict__ med, int n_valid, int nc) {
-  if ((nc & 3) == 0) {
-    // four channels per thread: 16-byte reads of z and of the rank words
-    const int nq = nc >> 2;
-    const long long n = static_cast<long long>(n_valid) * nq;
-    for (long long v = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; v < n;
-         v += static_cast<long long>(gridDim.x) * blockDim.x) {
-      const int p = static_cast<int>(v / nq);
-      const uint4 r = __ldg(reinterpret_cast<const uint4*>(med) + v);
-      const float* svp = sv + static_cast<long long>(p) * nc;
-      float4* zq = reinterpret_cast<float4*>(zbuf) + v;
-      float4 x = *zq;
-      x.x -= 0.5f * (__ldg(svp + (r.x & 0xffffu)) + __ldg(svp + (r.x >> 16)));
-      x.y -= 0.5f * (__ldg(svp + (r.y & 0xffffu)) + __ldg(svp + (r.y >> 16)));
-      x.z -= 0.5f * (__ldg(svp + (r.z & 0xffffu)) + __ldg(svp + (r.z >> 16)));
-      x.w -= 0.5f * (__ldg(svp + (r.w & 0xffffu)) + __ldg(svp + (r.w >> 16)));
-      *zq = x;
-    }
-    return;
-  }
-  const long long n = static_cast<long long>(n_valid) * nc;
-  for (long long v = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; v < n;
-       v += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const int p = static_cast<int>(v / nc);
-    const uint32_t r = __ldg(med + v);
-    const float* svp = sv + static_cast<long long>(p) * nc;
-    const float m = 0.5f * (__ldg(svp + (r & 0xffffu)) + __ldg(svp + (r >> 16)));
-    zbuf[v] -= m;
-  }
+// ----------------------------------- a9 median subtraction, a10 matched filter
+// k_mf takes tiles of whole pixel spectra through shared memory: the tile's z,
+// median ranks and sorted band values are copied in asynchronously (16 bytes at
+// a time where the rows allow it, a tile ahead where two fit), z' = z - median
+// is formed in place, then every thread takes chunks of kVox channels, sums the
+// 107 values around a chunk as register prefix sums and evaluates the 29
+// boxcars as prefix differences.
+//
+// Staged channel k of a pixel sits at index i = k + kMfPad of its row, slot
+// mf_slot(i): 4 words are left out after every 8, so a thread's window (28
+// 16-byte reads from index k0, k0 a multiple of 8, at constant offsets) falls
+// in distinct banks across a warp, and 16-byte copies stay aligned.  Rows are
+// padded with zeros to the left, whose sums are exactly 0, and with NaN to the
+// right: a boxcar that ends beyond the coarse channel is NaN and never larger.
+// Boxcars that would start before it are shut out the same way, by NaN prefix
+// sums (edge chunks only), so one code path serves edges and middle -- with
+// two unrolled ones a warp waited for instructions more than for anything else.
+constexpr int kMfPad = 52;                               // >= kMaxLo + 3, a multiple of 4
+constexpr int kMfThreads = 512;
+constexpr int kMfItems = 1024;                           // chunks a tile aims at
+__host__ __device__ constexpr int mf_slot(int i) { return i + ((i >> 3) << 2); }
+// words of a staged row: the last chunk's window ends at k0 + 112
+__host__ __device__ constexpr int mf_row(int nc) { return mf_slot((nc + kVox - 1) / kVox * kVox + 104); }
+
+// One tile's buffers: z rows, median ranks (pitch nc, rounded to 4) and the
+// band's values (pitch band) of px pixels, in 4-byte words.
+struct MfShape {
+  int nc, band, px, n_buf;
+  __host__ __device__ int med_pitch() const { return (nc + 3) & ~3; }
+  __host__ __device__ int buf_words() const { return px * (mf_row(nc) + med_pitch() + band); }
+};
+
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void* dst, const void* src) {
+  const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
+  if constexpr (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
 }
 
-// -------------------------------------------------------- a10 matched filter
-// Shared-memory slot of staged spectrum index i: one pad word after every 8,
-// so thread t's window (starting at index 8t, slot 9t) lies in its own banks
-// and every load of the window is the thread's base slot plus a constant.
-__host__ __device__ constexpr int mf_slot(int i) { return i + (i >> 3); }
-
-// Boxcars for kVox consecutive channels from the register prefix P; BOUNDS
-// keeps only widths that fit inside the coarse channel (edge chunks).
-template <bool BOUNDS>
-__device__ __forceinline__ void mf_chunk(const float (&P)[kWin + 1], int k0, int nc, float (&best)[kVox],
-                                         int (&bw)[kVox]) {
+// Boxcars of the kVox channels whose 112-value window starts at row (index k0;
+// value i of the window's 107 is channel k0 - 49 + i): a width is evaluated as
+// soon as the prefix reaches its right end, so sums to the right of the chunk
+// are dropped as they are used (96 registers; 156 with every sum held).
+__device__ __forceinline__ void mf_chunk(const float* row, int k0, float (&best)[kVox], int (&bw)[kVox]) {
+  constexpr int SH = kMfPad - kMaxLo;                    // the window's first value within its 16-byte reads
+  float P[kWin + 1];
+  float4 q;
+  auto value = [&](int i) {
+    const int o = i + SH;
+    if ((o & 3) == 0 || i == 0) q = *reinterpret_cast<const float4*>(row + mf_slot(o & ~3));
+    return (o & 3) == 0 ? q.x : (o & 3) == 1 ? q.y : (o & 3) == 2 ? q.z : q.w;
+  };
+  P[0] = 0.f;
+#pragma unroll
+  for (int i = 0; i < kMaxLo + kVox; ++i) P[i + 1] = P[i] + value(i);
+  if (k0 < kMaxLo) {
+    // prefix sums up to a channel before the first: no boxcar starts there
+#pragma unroll
+    for (int i = 0; i < kMaxLo; ++i)
+      if (k0 - kMaxLo + i < 0) P[i] = __int_as_float(0x7fc00000);
+  }
 #pragma unroll
   for (int j = 0; j < kVox; ++j) { best[j] = -INFINITY; bw[j] = 0; }
 #pragma unroll
@@ -949,64 +966,118 @@ __device__ __forceinline__ void mf_chunk(const float (&P)[kWin + 1], int k0, int
     const int w = width_of(wi);
     const int lo = (w - 1) / 2, hi = w - 1 - lo;
 #pragma unroll
+    for (int i = kMaxLo + kVox + (wi ? width_of(wi - 1) / 2 : 0); i < kMaxLo + kVox + hi; ++i)
+      P[i + 1] = P[i] + value(i);
+#pragma unroll
     for (int j = 0; j < kVox; ++j) {
-      if (!BOUNDS || (k0 + j - lo >= 0 && k0 + j + hi <= nc - 1)) {
-        const float S = P[j + kMaxLo + hi + 1] - P[j + kMaxLo - lo];
-        const float v = S * rsqrt_width(wi);
-        if (v > best[j]) { best[j] = v; bw[j] = w; }
-      }
+      const float S = P[j + kMaxLo + hi + 1] - P[j + kMaxLo - lo];
+      const float v = S * rsqrt_width(wi);
+      if (v > best[j]) { best[j] = v; bw[j] = w; }
     }
   }
 }
 
-__global__ void __launch_bounds__(128)
-k_mf(const float* __restrict__ zbuf, int n_valid, int nc, float* __restrict__ snr,
-     uint8_t* __restrict__ width, uint32_t hist_key0, int n_bins, unsigned long long* __restrict__ ghist) {
+// The CTA's warps start every round of chunks together, so the four warps of a
+// scheduler run the same instructions at the same time and share their
+// fetches (1500 instructions a chunk, 24 KB of code).  Bound by the compare and
+// the two selects per boxcar and channel (half-rate ALU, 61% active; 1.9 ms
+// per 51,468 pixels of 8192 channels at 100%).  51,468 pixels, with a separate
+// subtraction pass and two code paths at 12 warps per SM -> now: 8192 channels
+// 0.82 + 4.99 -> 3.57 ms, 4096 + 1024 channels 0.50 + 4.64 -> 2.41 ms.  z' goes
+// back to zbuf when the caller wants it.
+__global__ void __launch_bounds__(kMfThreads, 1)
+k_mf(float* __restrict__ zbuf, const float* __restrict__ sv, const uint32_t* __restrict__ med, int n_valid,
+     MfShape sh, int write_zp, float* __restrict__ snr, uint8_t* __restrict__ width, uint32_t hist_key0, int n_bins,
+     unsigned long long* __restrict__ ghist) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int n_s = kMaxLo + nc + kMaxHi + kVox;
-  float* s = reinterpret_cast<float*>(smem);                 // [mf_slot(n_s)]
-  uint32_t* hist = reinterpret_cast<uint32_t*>(s + mf_slot(n_s) + 1);
-  for (int i = threadIdx.x; i < n_bins; i += blockDim.x) hist[i] = 0;
+  uint32_t* hist = reinterpret_cast<uint32_t*>(smem);
+  float* buf0 = reinterpret_cast<float*>(hist + ((n_bins + 3) & ~3));
+  const int nc = sh.nc, px = sh.px, band = sh.band, row_w = mf_row(nc), med_w = sh.med_pitch();
+  const int tid = threadIdx.x;
+  const int chunks = (nc + kVox - 1) / kVox;
+  const int n_tiles = (n_valid + px - 1) / px;
+  const bool vec = (nc & 3) == 0;
   const float floor_snr = key2f(hist_key0 << kHistShift);
-  for (int p = blockIdx.x; p < n_valid; p += gridDim.x) {
-    const float* zp = zbuf + static_cast<long long>(p) * nc;
-    __syncthreads();
-    // stage the spectrum at slots kMaxLo .. kMaxLo + nc - 1, zeros around it;
-    // 16-byte loads, several in flight per thread
-    if ((nc & 3) == 0 && (reinterpret_cast<uintptr_t>(zp) & 15) == 0) {
-      const float4* z4 = reinterpret_cast<const float4*>(zp);
-      const int n4 = nc >> 2;
-#pragma unroll 4
-      for (int v = threadIdx.x; v < n4; v += blockDim.x) {
-        const float4 q = __ldg(z4 + v);
-        const int i = kMaxLo + 4 * v;
-        s[mf_slot(i)] = q.x;
-        s[mf_slot(i + 1)] = q.y;
-        s[mf_slot(i + 2)] = q.z;
-        s[mf_slot(i + 3)] = q.w;
-      }
-      for (int i = threadIdx.x; i < kMaxLo; i += blockDim.x) s[mf_slot(i)] = 0.f;
-      for (int i = kMaxLo + nc + threadIdx.x; i < n_s; i += blockDim.x) s[mf_slot(i)] = 0.f;
-    } else {
-#pragma unroll 4
-      for (int i = threadIdx.x; i < n_s; i += blockDim.x) {
-        const int k = i - kMaxLo;
-        s[mf_slot(i)] = (k >= 0 && k < nc) ? __ldg(zp + k) : 0.f;
+  for (int i = tid; i < n_bins; i += kMfThreads) hist[i] = 0u;
+  // the rows' padding, once: the copies never touch it
+  for (int r = 0; r < px * sh.n_buf; ++r) {
+    float* row = buf0 + (r / px) * sh.buf_words() + (r % px) * row_w;
+    for (int i = tid; i < kMfPad; i += kMfThreads) row[mf_slot(i)] = 0.f;
+    for (int i = kMfPad + nc + tid; i < chunks * kVox + 104; i += kMfThreads)
+      row[mf_slot(i)] = __int_as_float(0x7fc00000);
+  }
+  auto stage = [&](int tile, float* buf) {
+    const int p0 = tile * px, np = min(px, n_valid - p0);
+    uint32_t* mb = reinterpret_cast<uint32_t*>(buf + px * row_w);
+    float* sb = reinterpret_cast<float*>(mb + px * med_w);
+    const int nb = min(band, nc);
+    for (int r = 0; r < np; ++r) {
+      const long long o = static_cast<long long>(p0 + r) * nc;
+      if (vec) {
+        for (int v = tid; v < nc / 4; v += kMfThreads) {
+          copy_async<16>(buf + r * row_w + mf_slot(kMfPad + 4 * v), zbuf + o + 4 * v);
+          copy_async<16>(mb + r * med_w + 4 * v, med + o + 4 * v);
+        }
+        for (int v = tid; v < nb / 4; v += kMfThreads) copy_async<16>(sb + r * band + 4 * v, sv + o + 4 * v);
+        for (int v = (nb & ~3) + tid; v < nb; v += kMfThreads) copy_async<4>(sb + r * band + v, sv + o + v);
+      } else {
+        for (int v = tid; v < nc; v += kMfThreads) {
+          copy_async<4>(buf + r * row_w + mf_slot(kMfPad + v), zbuf + o + v);
+          copy_async<4>(mb + r * med_w + v, med + o + v);
+        }
+        for (int v = tid; v < nb; v += kMfThreads) copy_async<4>(sb + r * band + v, sv + o + v);
       }
     }
-    __syncthreads();
-    for (int k0 = threadIdx.x * kVox; k0 < nc; k0 += blockDim.x * kVox) {
-      const float* sw = s + mf_slot(k0);                     // k0 is a multiple of 8
-      float P[kWin + 1];
-      P[0] = 0.f;
-#pragma unroll
-      for (int i = 0; i < kWin; ++i) P[i + 1] = P[i] + sw[mf_slot(i)];   // channel k0 - 49 + i
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if (static_cast<int>(blockIdx.x) < n_tiles) stage(blockIdx.x, buf0);
+  int which = 0;
+  for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    float* buf = buf0 + which * sh.buf_words();
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();                                     // the tile is in; the last one is done with
+    if (sh.n_buf > 1) {
+      which ^= 1;
+      if (tile + gridDim.x < n_tiles) stage(tile + gridDim.x, buf0 + which * sh.buf_words());
+    }
+    const int p0 = tile * px, np = min(px, n_valid - p0);
+    {
+      const uint32_t* mb = reinterpret_cast<const uint32_t*>(buf + px * row_w);
+      const float* sb = reinterpret_cast<const float*>(mb + px * med_w);
+      for (int r = 0; r < np; ++r) {
+        const float* svp = sb + r * band;
+        const float* full = sv + static_cast<long long>(p0 + r) * nc;
+        // a pixel walked in full has ranks beyond the staged band
+        auto val = [&](uint32_t k) { return k < static_cast<uint32_t>(band) ? svp[k] : __ldg(full + k); };
+        for (int v = tid; v < nc / 4; v += kMfThreads) {
+          const uint4 m = *reinterpret_cast<const uint4*>(mb + r * med_w + 4 * v);
+          float4* zq = reinterpret_cast<float4*>(buf + r * row_w + mf_slot(kMfPad + 4 * v));
+          float4 x = *zq;
+          x.x -= 0.5f * (val(m.x & 0xffffu) + val(m.x >> 16));
+          x.y -= 0.5f * (val(m.y & 0xffffu) + val(m.y >> 16));
+          x.z -= 0.5f * (val(m.z & 0xffffu) + val(m.z >> 16));
+          x.w -= 0.5f * (val(m.w & 0xffffu) + val(m.w >> 16));
+          *zq = x;
+        }
+        for (int v = (nc & ~3) + tid; v < nc; v += kMfThreads) {
+          const uint32_t m = mb[r * med_w + v];
+          buf[r * row_w + mf_slot(kMfPad + v)] -= 0.5f * (val(m & 0xffffu) + val(m >> 16));
+        }
+      }
+    }
+    const int items = np * chunks;
+    for (int i0 = 0; i0 < items; i0 += kMfThreads) {
+      __syncthreads();                                   // z' is in place; the warps start together
+      const int it = i0 + tid;
+      if (it >= items) continue;
+      const int r = it / chunks, k0 = (it - r * chunks) * kVox;
+      const float* row = buf + r * row_w;
       float best[kVox];
       int bw[kVox];
-      if (k0 >= kMaxLo && k0 + kVox - 1 + kMaxHi <= nc - 1) mf_chunk<false>(P, k0, nc, best, bw);
-      else mf_chunk<true>(P, k0, nc, best, bw);
-      float* so = snr + static_cast<long long>(p) * nc + k0;
-      uint8_t* wo = width + static_cast<long long>(p) * nc + k0;
+      mf_chunk(row + mf_slot(k0), k0, best, bw);
+      const long long o = static_cast<long long>(p0 + r) * nc + k0;
+      float* so = snr + o;
+      uint8_t* wo = width + o;
       if (k0 + kVox <= nc && (reinterpret_cast<uintptr_t>(so) & 15) == 0 &&
           (reinterpret_cast<uintptr_t>(wo) & 7) == 0) {
         reinterpret_cast<float4*>(so)[0] = make_float4(best[0], best[1], best[2], best[3]);
@@ -1025,6 +1096,11 @@ k_mf(const float* __restrict__ zbuf, int n_valid, int nc, float* __restrict__ sn
             wo[j] = static_cast<uint8_t>(bw[j]);
           }
       }
+      if (write_zp) {
+#pragma unroll
+        for (int j = 0; j < kVox; ++j)
+          if (k0 + j < nc) zbuf[o + j] = row[mf_slot(k0 + kMfPad + j)];
+      }
 #pragma unroll
       for (int j = 0; j < kVox; ++j) {
         if (k0 + j < nc && best[j] >= floor_snr) {
@@ -1034,9 +1110,13 @@ k_mf(const float* __restrict__ zbuf, int n_valid, int nc, float* __restrict__ sn
         }
       }
     }
+    if (sh.n_buf == 1 && tile + gridDim.x < n_tiles) {
+      __syncthreads();                                   // the tile's reads are done
+      stage(tile + gridDim.x, buf0);
+    }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < n_bins; i += blockDim.x)
+  for (int i = tid; i < n_bins; i += kMfThreads)
     if (hist[i]) atomicAdd(ghist + i, static_cast<unsigned long long>(hist[i]));
 }
 
@@ -1584,35 +1664,44 @@ int run_filter_coarse(int c, const float* img_block, const DetectPlan& p, const 
     if (tuning(st))
       if (int e = tune_pick(key, {1, 2, 4}, rank_walk, st, &n_seg)) return e;
     if (int e = rank_walk(n_seg)) return e;
-    OVRO_PROF("k_median_sub", st);
-    k_median_sub<<<8 * nsm, 256, 0, st>>>(w.zbuf, w.sv, w.med, p.n_valid, nc);
-    OVRO_LAUNCH_CHECK();
-  }
-  if (d_zp_out) {
-    k_scatter<float><<<4 * nsm, 256, 0, st>>>(w.zbuf, w.pix, p.n_valid, nc, p.chan0[c], p.npix, d_zp_out);
-    OVRO_LAUNCH_CHECK();
   }
   {
-    const size_t sm = static_cast<size_t>(mf_slot(kMaxLo + nc + kMaxHi + kVox) + 1) * 4 +
-                      static_cast<size_t>(n_bins) * 4;
+    // a tile of kMfItems chunks or the pixels that half (or all, for the
+    // longest channels) of the shared memory holds
+    MfShape sh;
+    sh.nc = nc;
+    sh.band = band_ranks(nc);
+    sh.px = 1;
+    sh.n_buf = 2;
+    const size_t hist_b = (static_cast<size_t>(n_bins) + 3) / 4 * 16, room = 227 * 1024 - hist_b;
+    const int chunks = (nc + kVox - 1) / kVox;
+    const int one = sh.buf_words();
+    if (static_cast<size_t>(one) * 8 > room) sh.n_buf = 1;
+    else sh.px = std::max(1, std::min(static_cast<int>(room / 8 / one), (kMfItems + chunks - 1) / chunks));
+    const size_t sm = hist_b + static_cast<size_t>(sh.buf_words()) * 4 * sh.n_buf;
     OVRO_CUDA_TRY(cudaFuncSetAttribute(k_mf, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm)));
-    // CTAs per SM; trial launches histogram into scratch (the real histogram
-    // accumulates over coarse channels and must count every voxel once)
-    auto mf = [&](int per_sm, unsigned long long* hist) -> int {
-      const int blocks = std::min(p.n_valid, per_sm * nsm);
+    const int tiles = (p.n_valid + sh.px - 1) / sh.px;
+    // trial launches histogram into scratch (the real histogram accumulates
+    // over coarse channels and must count every voxel once) and keep z
+    auto mf = [&](int per_sm, unsigned long long* hist, int write_zp) -> int {
       OVRO_PROF("k_mf", st);
-      k_mf<<<blocks, 128, sm, st>>>(w.zbuf, p.n_valid, nc, w.snr + p.vox0[c], w.width + p.vox0[c], hist_key0,
-                                    n_bins, hist);
+      k_mf<<<std::min(tiles, per_sm * nsm), kMfThreads, sm, st>>>(w.zbuf, w.sv, w.med, p.n_valid, sh, write_zp,
+                                                                  w.snr + p.vox0[c], w.width + p.vox0[c], hist_key0,
+                                                                  n_bins, hist);
       OVRO_LAUNCH_CHECK();
       return OVRO_OK;
     };
     const std::string key = tune_key("k_mf", {p.n_valid, nc});
-    int per_sm = tuned(key, 24);
+    int per_sm = tuned(key, 1);
     if (tuning(st)) {
       unsigned long long* scratch = reinterpret_cast<unsigned long long*>(w.vals);
-      if (int e = tune_pick(key, {6, 12, 24, 48}, [&](int v) { return mf(v, scratch); }, st, &per_sm)) return e;
+      if (int e = tune_pick(key, {1, 2, 4}, [&](int v) { return mf(v, scratch, 0); }, st, &per_sm)) return e;
     }
-    if (int e = mf(per_sm, w.hist)) return e;
+    if (int e = mf(per_sm, w.hist, d_zp_out ? 1 : 0)) return e;
+  }
+  if (d_zp_out) {
+    k_scatter<float><<<4 * nsm, 256, 0, st>>>(w.zbuf, w.pix, p.n_valid, nc, p.chan0[c], p.npix, d_zp_out);
+    OVRO_LAUNCH_CHECK();
   }
   return OVRO_OK;
 }

@@ -1,4 +1,4 @@
-"""GPU parity of the running-median high-pass where the band ranking and the
+"""GPU parity of the running-median high-pass and the boxcars where the band ranking and the
 walk can go wrong: the shortest coarse channels, lengths just past a kernel's
 keys per thread, many equal values, dead channels, pixels far from zero (the
 finer selection) and pixels both kernels give up (the full walk)."""
@@ -36,7 +36,9 @@ def test_highpass_vs_oracle(lib, nfft, kind):
     mask = OI.horizon_mask(n, cell)
     d = torch.from_numpy(cube).cuda()
     st = lib.detect_stats(d, cell)
-    zp, _, _ = lib.detect_filter(d, st, cell, nfft, want_zp=True)
+    zp, snr, _ = lib.detect_filter(d, st, cell, nfft, want_zp=True)
+    plain = lib.detect_filter(d, st, cell, nfft)[1]
+    assert torch.equal(plain, snr)                   # with or without the high-passed cube
     s = st.cpu().numpy()
     z = np.zeros(cube.shape)
     for f in range(cube.shape[0]):
@@ -46,3 +48,8 @@ def test_highpass_vs_oracle(lib, nfft, kind):
     ref[:, ~mask] = 0
     # z is rounded to 24 bits before and after the subtraction
     assert np.abs(zp.cpu().numpy() - ref).max() <= 1e-5 * max(1.0, np.abs(z).max())
+    so, _ = OD.matched_filter(ref, OD.chan_bounds_of(nfft))
+    so[:, ~mask] = 0
+    # prefix sums of 107 values: at most 107 roundings of the largest sum
+    tol = 107 * 2.0 ** -24 * np.abs(ref).max() * 107 + 1e-5 * 10 * max(1.0, np.abs(z).max())
+    assert np.abs(snr.cpu().numpy() - so).max() <= tol
