@@ -54,7 +54,6 @@ namespace {
 constexpr double kCLight = 299792458.0;
 constexpr int kQ = kOversample;
 constexpr int kHalfTab = kSupport * kOversample / 2;
-constexpr int kTabLen = 2 * kHalfTab + 1;
 constexpr int kHalfSup = kSupport / 2;
 constexpr int kPad = 2;              // uv grid cells per image pixel, per axis
 // storage of the half-transformed grid between the row and column passes
@@ -137,7 +136,7 @@ __global__ void k_uvw(const Baseline* __restrict__ base, int n_cross, const Chan
 }
 
 // device counters of one call's plan (ImgWs::counts)
-constexpr int kCountListed = 0, kCountRows = 1, kCountTiles = 2, kCounts = 3;
+constexpr int kCountListed = 0, kCountRows = 1, kCountTiles = 2, kCountSlots = 3, kCounts = 4;
 
 struct GridEntry {
   int bl;            // baseline index in the visibility record
@@ -190,15 +189,17 @@ constexpr int kTabMargin = 4;
 constexpr int kTabD = kHalfSup + kTileU - 1 + kTabMargin;   // 10
 constexpr int kTabStride = kQ + 1;
 constexpr int kTabXLen = (2 * kTabD + 1) * kTabStride;
+constexpr int kTabBytes = 8;         // the tile kernel holds every weight twice, for packed arithmetic
 
 // Per-channel record of one listed baseline, prepared once per channel group
 // by k_grid_prep: its exact rounded position p = rint(u Q), rint(v Q) and its
 // value in the Hermitian part of the grid, conj(Stokes I) / 2, or V = 0 when
 // the visibility is not gridded in that channel.  Layout [group][listed][32].
 // With table bases (a call whose footprints move by less than kTabMargin
-// cells over its channels), pu and pv hold instead the weight-table offsets
-// of the position: column c's weight is tabx[pu + c (Q + 1)], row r's
-// tabx[pv + r (Q + 1)] (r, c grid indices), zero beyond the footprint.
+// cells over its channels), pu and pv hold instead the byte offsets of the
+// position in the tile kernel's table (8 bytes an entry): column c's weight is
+// entry pu / 8 + c (Q + 1), row r's pv / 8 + r (Q + 1) (r, c grid indices), zero
+// beyond the footprint.
 struct PrepRec {
   int pu, pv;
   float vr, vi;
@@ -310,8 +311,8 @@ k_grid_prep(const GridEntry* __restrict__ listed, const unsigned long long* __re
         int cu, cv, ou, ov;
         centre_cell32(pu, cu, ou);
         centre_cell32(pv, cv, ov);
-        r.pu = tab_base(G, cu, ou);
-        r.pv = tab_base(G, cv, ov);
+        r.pu = kTabBytes * tab_base(G, cu, ou);
+        r.pv = kTabBytes * tab_base(G, cv, ov);
       }
       if (keep) {
         float vr, vi;
@@ -358,183 +359,209 @@ k_grid_prep(const GridEntry* __restrict__ listed, const unsigned long long* __re
 // G/2 .. G-1 (v >= 0; a record whose footprint lies below is listed as its
 // mirror, one straddling row G/2 as both).  Work items are (group of 32
 // channels, warp tile) pairs, group-major, the tiles of a group taken from the
-// longest list to the shortest; every warp of the persistent grid (one CTA of
-// kGridWarps warps per SM) takes items kGridWarps * gridDim.x apart, so each
-// warp starts on a heavy tile and ends on light ones.  The gap-indexed weight
-// table sits in shared memory, loaded once per CTA.  For every list entry of
-// its tile, a lane reads its channel's prepared record (one 16-byte load, the
-// warp's 32 lanes contiguous), mirrors it if flagged, reads the tile's 4 row
-// and 4 column weights of the separable kernel and adds the products into its
-// accumulators; kRing records are in flight per warp and their list entries
-// are read 2 kRing ahead.
-//   BASES: the record holds the weight-table offsets of its position, so the
-//     weights are 8 loads at fixed strides from (offset + tile origin) and a
-//     lane off the footprint reads the table's zero rows;
+// longest list to the shortest; the warps of the persistent grid (one CTA of
+// kGridWarps warps per SM) draw items from a counter, the next one while they
+// work on the last.  The gap-indexed weight table sits in shared memory with
+// every weight twice, so that one 8-byte load gives both factors of a packed
+// multiply-add on a cell's (re, im): a record costs a lane one 16-byte load,
+// 8 table loads, 4 + 16 packed multiply(-add)s and its decoding, where scalar
+// arithmetic took 8 + 32.  kRing records are in flight per warp, a quad of
+// list entries ahead of them; whole quads run without a branch, so the loads
+// of one record overlap the arithmetic of the last.
+//   BASES: the record holds the table offsets of its position, so the weights
+//     are 8 loads at fixed strides from (offset + tile origin) and a lane off
+//     the footprint reads the table's zero rows;
 //   otherwise the lane takes the centre cells from the position and adds
 //     zeros when its footprint misses the tile.
-// The tile is written with the (-1)^(row + col) centring sign as two real
-// planes, grid [batch][2][G/2][G] (row j - G/2).
+// The tile is written with the (-1)^(row + col) centring sign to grid
+// [group][G/2][G][32] (row j - G/2; re, im of 32 channels), 256 contiguous bytes
+// a warp store: with a plane per channel every lane wrote half a sector of its
+// own, and that bounded sparse grids.  Before (scalar, plane per channel,
+// static items) -> now, 352 antennas: 1000 channels of 256^2 1.16 -> 0.72 ms,
+// 300 of 512^2 1.32 -> 0.49 ms, 64 of 1024^2 1.97 -> 0.33 ms.
 constexpr int kGridWarps = 20;
-constexpr int kRing = 4;           // records in flight per warp
-constexpr size_t kTileSmem = static_cast<size_t>(kTabXLen) * sizeof(float);
+constexpr int kRing = 4;           // records in flight per warp: one quad of list entries
+constexpr size_t kTileSmem = static_cast<size_t>(kTabXLen) * kTabBytes;
+
+// (a.x b.x, a.y b.y) and (a.x b.x + c.x, a.y b.y + c.y), each rounded once
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ unsigned long long pack2(int lo, int hi) {
+  unsigned long long d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
+  return d;
+}
 
 template <int LOG2G, bool BASES>
 __global__ void __launch_bounds__(kGridWarps * 32, 1)
-k_grid_tiles(const int* __restrict__ tile_idx, const int2* __restrict__ tile_rng, const int* __restrict__ tile_order,
+k_grid_tiles(const int4* __restrict__ tile_idx, const int2* __restrict__ tile_rng, const int* __restrict__ tile_order,
              const PrepRec* __restrict__ prep, long long n_cross, const float* __restrict__ tabx_g, int nb,
-             float* __restrict__ grid) {
+             unsigned* __restrict__ next_item, float2* __restrict__ grid) {
   constexpr int G = 1 << LOG2G;
   constexpr int NTU = n_tiles_u(G);
   constexpr int NT = n_tiles(G);
-  constexpr long long PLANE = static_cast<long long>(G / 2) * G;
+  constexpr int STEP = kTabStride * kTabBytes;        // bytes from one grid cell's weight to the next
   extern __shared__ __align__(16) unsigned char smem[];
-  float* tabx = reinterpret_cast<float*>(smem);
   const unsigned full = 0xffffffffu;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i = threadIdx.x; i < kTabXLen / 4; i += blockDim.x)
-    reinterpret_cast<float4*>(tabx)[i] = __ldg(reinterpret_cast<const float4*>(tabx_g) + i);
-  for (int i = (kTabXLen / 4) * 4 + threadIdx.x; i < kTabXLen; i += blockDim.x) tabx[i] = __ldg(tabx_g + i);
+  const int lane = threadIdx.x & 31;
+  for (int i = threadIdx.x; i < kTabXLen; i += blockDim.x) {
+    const float w = __ldg(tabx_g + i);
+    reinterpret_cast<float2*>(smem)[i] = make_float2(w, w);
+  }
   __syncthreads();
-  const int n_groups = (nb + kLanes - 1) / kLanes;
-  const long long n_items = static_cast<long long>(n_groups) * NT;
-  const int stride = gridDim.x * kGridWarps;
+  const unsigned n_items = static_cast<unsigned>((nb + kLanes - 1) / kLanes) * NT;
+  auto draw = [&]() {
+    unsigned i = 0;
+    if (lane == 0) i = atomicAdd(next_item, 1u);
+    return i;
+  };
+  unsigned item = __shfl_sync(full, draw(), 0);
 #pragma unroll 1
-  for (long long item = static_cast<long long>(blockIdx.x) * kGridWarps + warp; item < n_items; item += stride) {
+  while (item < n_items) {
+    const unsigned after = draw();                     // broadcast once this item is done
     const int g = static_cast<int>(item / NT);
-    const int tile = __ldg(tile_order + (item - static_cast<long long>(g) * NT));
-    const int cb = g * kLanes + lane;                 // channel within the batch
+    const int tile = __ldg(tile_order + (item - static_cast<unsigned>(g) * NT));
     const PrepRec* pg = prep + static_cast<long long>(g) * n_cross * kLanes + lane;
     const int tv = tile / NTU, tu = tile - tv * NTU;
     const int r0 = G / 2 + tv * kTileV, c0 = tu * kTileU;
     const int2 rng = __ldg(tile_rng + tile);
-    const int e0 = rng.x, e1 = rng.y;
-    float acr[kTileV][kTileU], aci[kTileV][kTileU];
+    unsigned long long acc[kTileV][kTileU];            // (re, im)
 #pragma unroll
     for (int i = 0; i < kTileV; ++i)
 #pragma unroll
-      for (int j = 0; j < kTileU; ++j) acr[i][j] = aci[i][j] = 0.0f;
-    auto index = [&](int e) { return e < e1 ? __ldg(tile_idx + e) : 0; };
+      for (int j = 0; j < kTileU; ++j) acc[i][j] = 0ull;
     auto load_rec = [&](int ent) {
       return __ldg(reinterpret_cast<const int4*>(pg + static_cast<long long>(ent & ~kMirror) * kLanes));
     };
-    auto accumulate = [&](const float* bu, const float* bv, float vr, float vi) {
-      float wv[kTileV], wu[kTileU];
+    // bu, bv: byte offsets of the tile's first column's and row's weights
+    auto accumulate = [&](int bu, int bv, unsigned long long v) {
+      unsigned long long wv[kTileV], wu[kTileU];
 #pragma unroll
-      for (int i = 0; i < kTileV; ++i) wv[i] = bv[i * kTabStride];
+      for (int i = 0; i < kTileV; ++i) wv[i] = *reinterpret_cast<const unsigned long long*>(smem + bv + i * STEP);
 #pragma unroll
-      for (int j = 0; j < kTileU; ++j) wu[j] = bu[j * kTabStride];
+      for (int j = 0; j < kTileU; ++j) wu[j] = *reinterpret_cast<const unsigned long long*>(smem + bu + j * STEP);
 #pragma unroll
       for (int i = 0; i < kTileV; ++i) {
-        const float br = wv[i] * vr, bi = wv[i] * vi;
+        const unsigned long long b = mul2(wv[i], v);
 #pragma unroll
-        for (int j = 0; j < kTileU; ++j) {
-          acr[i][j] = fmaf(br, wu[j], acr[i][j]);
-          aci[i][j] = fmaf(bi, wu[j], aci[i][j]);
-        }
+        for (int j = 0; j < kTileU; ++j) acc[i][j] = fma2(b, wu[j], acc[i][j]);
       }
     };
     // one list entry: the record (mirrored if flagged) decoded here, at its use
     auto grid_one = [&](int4 v, int ent) {
-      const bool m = ent & kMirror;
-      const float vr = __int_as_float(v.z), vi = m ? -__int_as_float(v.w) : __int_as_float(v.w);
+      const int s = ent >> 31;                         // -1: the mirror (-u, -v, conj V)
+      const unsigned long long val = pack2(v.z, v.w ^ (s & kMirror));
       if (BASES) {
-        // the table's zero rows stand for taps off the footprint
-        const int bu = m ? tab_mirror(G) - v.x : v.x, bv = m ? tab_mirror(G) - v.y : v.y;
-        accumulate(tabx + bu + c0 * kTabStride, tabx + bv + r0 * kTabStride, vr, vi);
+        // the mirror's offset is tab_mirror - offset = tab_mirror + 1 + ~offset
+        const int m = s & (kTabBytes * tab_mirror(G) + 1);
+        accumulate((v.x ^ s) + m + c0 * STEP, (v.y ^ s) + m + r0 * STEP, val);
         return;
       }
       int cu, offu, cv, offv;
-      centre_cell32(m ? -v.x : v.x, cu, offu);
-      centre_cell32(m ? -v.y : v.y, cv, offv);
+      centre_cell32(s ? -v.x : v.x, cu, offu);
+      centre_cell32(s ? -v.y : v.y, cv, offv);
       int dv0 = r0 - (G / 2 + cv), du0 = c0 - (G / 2 + cu);   // offsets of the tile's first row / column
       const bool touch = dv0 <= kHalfSup && dv0 >= -(kHalfSup + kTileV - 1) && du0 <= kHalfSup &&
                          du0 >= -(kHalfSup + kTileU - 1);
       if (__any_sync(full, touch)) {
-        float wr = vr, wi = vi;
-        if (!touch) {
-          // a lane whose footprint misses the tile adds zeros; its table
-          // reads stay inside the table
-          wr = wi = 0.0f;
-          dv0 = du0 = 0;
-          offu = offv = 0;
-        }
-        accumulate(tabx + (du0 + kTabD) * kTabStride + kQ / 2 - offu,
-                   tabx + (dv0 + kTabD) * kTabStride + kQ / 2 - offv, wr, wi);
+        // a lane whose footprint misses the tile adds zeros; its table reads
+        // stay inside the table
+        if (!touch) dv0 = du0 = offu = offv = 0;
+        accumulate(((du0 + kTabD) * kTabStride + kQ / 2 - offu) * kTabBytes,
+                   ((dv0 + kTabD) * kTabStride + kQ / 2 - offv) * kTabBytes, touch ? val : 0ull);
       }
     };
-    // a ring of kRing records in flight, each loaded kRing entries ahead of its
-    // use into its own slot (no register moves wait on a load), and their list
-    // entries, loaded 2 kRing ahead
-    int4 q[kRing];
-    int en[kRing], nx[kRing];
-#pragma unroll
-    for (int d = 0; d < kRing; ++d) en[d] = index(e0 + d);
-#pragma unroll
-    for (int d = 0; d < kRing; ++d) {
-      q[d] = load_rec(en[d]);
-      nx[d] = index(e0 + kRing + d);
-    }
+    if (rng.y > rng.x) {
+      // lists start on a quad and are padded to whole quads (entry 0)
+      const int last = (rng.y - 1) >> 2;
+      int q = rng.x >> 2;
+      int4 e = __ldg(tile_idx + q), en = __ldg(tile_idx + min(q + 1, last));
+      int4 rec[kRing] = {load_rec(e.x), load_rec(e.y), load_rec(e.z), load_rec(e.w)};
 #pragma unroll 1
-    for (int e = e0; e < e1; e += kRing) {
-#pragma unroll
-      for (int d = 0; d < kRing; ++d) {
-        if (e + d < e1) grid_one(q[d], en[d]);
-        en[d] = nx[d];
-        q[d] = load_rec(en[d]);
-        nx[d] = index(e + d + 2 * kRing);
+      for (const int whole = rng.y >> 2; q < whole; ++q) {
+        const int4 ahead = __ldg(tile_idx + min(q + 2, last));
+        grid_one(rec[0], e.x);
+        rec[0] = load_rec(en.x);
+        grid_one(rec[1], e.y);
+        rec[1] = load_rec(en.y);
+        grid_one(rec[2], e.z);
+        rec[2] = load_rec(en.z);
+        grid_one(rec[3], e.w);
+        rec[3] = load_rec(en.w);
+        e = en;
+        en = ahead;
       }
+      const int rest = rng.y & 3;
+      if (rest > 0) grid_one(rec[0], e.x);
+      if (rest > 1) grid_one(rec[1], e.y);
+      if (rest > 2) grid_one(rec[2], e.z);
     }
     // ---- the tile, with the centring sign (r0 and c0 are even)
-    if (cb < nb) {
-      float* gr = grid + static_cast<long long>(cb) * 2 * PLANE;
-      float* gi = gr + PLANE;
+    if (g * kLanes + lane < nb) {
+      float2* out = grid + ((static_cast<long long>(g) * (G / 2) + r0 - G / 2) * G + c0) * kLanes + lane;
 #pragma unroll
-      for (int i = 0; i < kTileV; ++i) {
-        float vr[kTileU], vi[kTileU];
+      for (int i = 0; i < kTileV; ++i)
 #pragma unroll
         for (int j = 0; j < kTileU; ++j) {
-          const bool neg = (i + j) & 1;
-          vr[j] = neg ? -acr[i][j] : acr[i][j];
-          vi[j] = neg ? -aci[i][j] : aci[i][j];
+          float2 z;
+          asm("mov.b64 {%0, %1}, %2;" : "=f"(z.x), "=f"(z.y) : "l"(acc[i][j]));
+          out[(i * G + j) * kLanes] = (i + j) & 1 ? make_float2(-z.x, -z.y) : z;
         }
-        const long long row = r0 + i - G / 2;
-        float4* pr = reinterpret_cast<float4*>(gr + row * G + c0);
-        float4* pi = reinterpret_cast<float4*>(gi + row * G + c0);
-#pragma unroll
-        for (int j = 0; j < kTileU / 4; ++j) {
-          pr[j] = make_float4(vr[4 * j], vr[4 * j + 1], vr[4 * j + 2], vr[4 * j + 3]);
-          pi[j] = make_float4(vi[4 * j], vi[4 * j + 1], vi[4 * j + 2], vi[4 * j + 3]);
-        }
-      }
     }
+    item = __shfl_sync(full, after, 0);
   }
 }
 
-// The central N columns of the row transforms of a band of rows in shared
-// memory, into the half-transformed grid h ([batch][G][N]) in its storage format.
+// Rows of the half-transformed grid kept per channel: the gridded plane is the
+// Hermitian part H of the grid on its rows j = G/2 .. G-1; the row transforms
+// of H satisfy R(G - j, k) = conj R(j, k), and row 0 is empty (no footprint
+// reaches it), so these G/2 rows carry everything the column pass needs.
+__host__ __device__ constexpr int half_rows(int g) { return g / 2; }
+
+// A row-pass CTA transforms row_lines(G) lines (8192 points; every row of the
+// smallest grids): row_chans(G) channels of as many rows each as fit.  The grid
+// holds a cell's channels together, so 8 channels make whole sectors (4 of
+// 2048 points still make 32 bytes).
+__host__ __device__ constexpr int row_lines(int g) { return 8192 / g < 4 * g ? 8192 / g : 4 * g; }
+__host__ __device__ constexpr int row_chans(int g) { return row_lines(g) < 8 ? row_lines(g) : 8; }
+__host__ __device__ constexpr int row_rows(int g) { return row_lines(g) / row_chans(g); }
+
+// The central N columns of the CTA's row transforms (line f = channel
+// f / row_rows, row f % row_rows), into the half-transformed grid h
+// ([batch][G/2][N]) in its storage format.
 template <int G, int LDP, int S>
-__device__ __forceinline__ void store_band(const float2* band, int band_h, int n_img, long long hrow0, void* h,
+__device__ __forceinline__ void store_band(const float2* band, int cb0, int row0, int nb, int n_img, void* h,
                                            float* hs) {
-  // band_h: the rows to store (the first rows of the band)
+  constexpr int R = row_rows(G);
   const int offc = G / 2 - n_img / 2;
+  const int lines = min(row_chans(G), nb - cb0) * R;    // the channels of the batch
+  auto hrow = [&](int f) { return static_cast<long long>(cb0 + f / R) * half_rows(G) + row0 + f % R; };
   if constexpr (S == kStoreF32) {
-    float2* hb = static_cast<float2*>(h) + hrow0 * n_img;
-    for (int i = threadIdx.x; i < band_h * n_img; i += blockDim.x) {
+    float2* hb = static_cast<float2*>(h);
+    for (int i = threadIdx.x; i < lines * n_img; i += blockDim.x) {
       const int r = i / n_img, c = i - r * n_img;
-      hb[static_cast<long long>(r) * n_img + c] = band[r * LDP + pad16(offc + c)];
+      hb[hrow(r) * n_img + c] = band[r * LDP + pad16(offc + c)];
     }
   } else if constexpr (S == kStoreBF16) {
-    __nv_bfloat162* hb = static_cast<__nv_bfloat162*>(h) + hrow0 * n_img;
-    for (int i = threadIdx.x; i < band_h * n_img; i += blockDim.x) {
+    __nv_bfloat162* hb = static_cast<__nv_bfloat162*>(h);
+    for (int i = threadIdx.x; i < lines * n_img; i += blockDim.x) {
       const int r = i / n_img, c = i - r * n_img;
-      hb[static_cast<long long>(r) * n_img + c] = __float22bfloat162_rn(band[r * LDP + pad16(offc + c)]);
+      hb[hrow(r) * n_img + c] = __float22bfloat162_rn(band[r * LDP + pad16(offc + c)]);
     }
   } else {
     // FP16 with a power-of-two scale per row: the row's largest component
     // lands in [2^13, 2^14), far from FP16 overflow; scaling is exact
-    __half2* hb = static_cast<__half2*>(h) + hrow0 * n_img;
+    __half2* hb = static_cast<__half2*>(h);
     const int lane = threadIdx.x & 31, n_w = blockDim.x >> 5;
-    for (int r = threadIdx.x >> 5; r < band_h; r += n_w) {
+    for (int r = threadIdx.x >> 5; r < lines; r += n_w) {
       float m = 0.f;
       for (int c = lane; c < n_img; c += 32) {
         const float2 v = band[r * LDP + pad16(offc + c)];
@@ -545,74 +572,56 @@ __device__ __forceinline__ void store_band(const float2* band, int band_h, int n
       int e = 0;
       if (m > 0.f) frexpf(m, &e);
       const float sc = m > 0.f ? ldexpf(1.0f, 14 - e) : 1.0f;
-      if (lane == 0) hs[hrow0 + r] = m > 0.f ? ldexpf(1.0f, e - 14) : 0.0f;
+      if (lane == 0) hs[hrow(r)] = m > 0.f ? ldexpf(1.0f, e - 14) : 0.0f;
       for (int c = lane; c < n_img; c += 32) {
         const float2 v = band[r * LDP + pad16(offc + c)];
-        hb[static_cast<long long>(r) * n_img + c] = __float22half2_rn(make_float2(v.x * sc, v.y * sc));
+        hb[hrow(r) * n_img + c] = __float22half2_rn(make_float2(v.x * sc, v.y * sc));
       }
     }
   }
 }
 
-// Row pitch (floats) of the two real planes of a band staged in shared
-// memory: G + 4, 16-byte rows (the planes overlap the FFT layout, which the
-// first Stockham pass only writes after all its reads).
-__host__ __device__ constexpr int planar_pitch(int g) { return g + 4; }
-
-// Rows of the half-transformed grid kept per channel: the gridded plane is the
-// Hermitian part H of the grid on its rows j = G/2 .. G-1; the row transforms
-// of H satisfy R(G - j, k) = conj R(j, k), and row 0 is empty (no footprint
-// reaches it), so these G/2 rows carry everything the column pass needs.
-__host__ __device__ constexpr int half_rows(int g) { return g / 2; }
-
-// Row transforms of one band of rows of the gridded half plane of one channel:
-// the two real planes are staged in shared memory with 16-byte loads (all in
-// flight at once), the first Stockham pass reads them, the rest run in place;
-// the central N columns go to h ([batch][G/2][N], row j - G/2).
+// Row transforms of the gridded half planes: a CTA stages its lines with
+// 16-byte loads (two channels of a cell each, all in flight at once), turned
+// into rows in shared memory, and transforms them in place; the central N
+// columns go to h ([batch][G/2][N], row j - G/2).
 template <int LOG2G, int S>
 __global__ void __launch_bounds__(1024)
-k_fft_rows(const float* __restrict__ grid, const float2* __restrict__ tw_g, int n_img, int band_h,
+k_fft_rows(const float2* __restrict__ grid, const float2* __restrict__ tw_g, int nb, int n_img,
            void* __restrict__ h, float* __restrict__ hs) {
   constexpr int G = 1 << LOG2G;
   constexpr int LDP = band_pitch(G);
-  constexpr int P = planar_pitch(G);
-  static_assert(2 * P <= 2 * LDP, "planar band fits in the FFT layout");
+  constexpr int CH = row_chans(G), R = row_rows(G), CP = CH / 2;
   extern __shared__ __align__(16) unsigned char smem[];
-  float2* band = reinterpret_cast<float2*>(smem);     // [band_h][LDP]
-  float* pre = reinterpret_cast<float*>(smem);        // [band_h][P] (staging)
-  float* pim = pre + band_h * P;
-  float2* tw = band + band_h * LDP;                   // [G]
-  const int b = blockIdx.x, cb = blockIdx.y;
-  const int row0 = b * band_h;
+  float2* band = reinterpret_cast<float2*>(smem);     // [row_lines][LDP]
+  float2* tw = band + row_lines(G) * LDP;             // [G]
+  const int cb0 = blockIdx.y * CH, row0 = blockIdx.x * R;
   for (int i = threadIdx.x; i < G; i += blockDim.x) tw[i] = tw_g[i];
-  const long long plane4 = static_cast<long long>(half_rows(G)) * G / 4;
-  const float4* src = reinterpret_cast<const float4*>(grid) + static_cast<long long>(cb) * 2 * plane4 +
-                      static_cast<long long>(row0) * (G / 4);
-  constexpr int RQ = G / 4;                           // float4 per row
-  // 2 band_h G / 4 float4 over band_h G / 16 threads: 8 per thread, all
+  // [group][row][col][32 channels] float2, read as channel pairs
+  const float4* src = reinterpret_cast<const float4*>(grid) +
+                      (static_cast<long long>(cb0 / kLanes) * half_rows(G) + row0) * G * (kLanes / 2) +
+                      (cb0 % kLanes) / 2;
+  // row_lines G / 2 float4 over row_lines G / 16 threads: 8 per thread, all
   // issued before the first is stored
   constexpr int PER = 8;
-  const int n1 = band_h * RQ;
   float4 q[PER];
 #pragma unroll
   for (int u = 0; u < PER; ++u) {
-    const int i = threadIdx.x + u * blockDim.x;
-    const int pl = i >= n1 ? 1 : 0, k = i - pl * n1;
-    q[u] = __ldg(src + pl * plane4 + k);
+    const int i = threadIdx.x + u * blockDim.x;       // (row, col, channel pair)
+    q[u] = __ldg(src + static_cast<long long>(i / CP) * (kLanes / 2) + i % CP);
   }
 #pragma unroll
   for (int u = 0; u < PER; ++u) {
     const int i = threadIdx.x + u * blockDim.x;
-    const int pl = i >= n1 ? 1 : 0, k = i - pl * n1;
-    const int r = k / RQ, c = k - r * RQ;
-    *reinterpret_cast<float4*>((pl ? pim : pre) + r * P + 4 * c) = q[u];
+    const int cp = i % CP, x = i / CP, r = x / G, c = x % G;
+    float2* d = band + (2 * cp * R + r) * LDP + pad16(c);
+    d[0] = make_float2(q[u].x, q[u].y);
+    d[R * LDP] = make_float2(q[u].z, q[u].w);
   }
   __syncthreads();
-  // the first pass reads the planar staging (which the band overlaps)
   fft_rows_inplace_f<LOG2G>(
-      band, LDP, [&](int f, int x) { return make_float2(pre[f * P + x], pim[f * P + x]); },
-      [&](int i) { return tw[i]; });
-  store_band<G, LDP, S>(band, band_h, n_img, static_cast<long long>(cb) * half_rows(G) + row0, h, hs);
+      band, LDP, [&](int f, int x) { return band[f * LDP + pad16(x)]; }, [&](int i) { return tw[i]; });
+  store_band<G, LDP, S>(band, cb0, row0, nb, n_img, h, hs);
 }
 
 // Two adjacent values (idx even) of the half-transformed grid in FP32.
@@ -1005,7 +1014,8 @@ k_plan_rows(const PlanRange* __restrict__ lrng, int g, unsigned long long* __res
 }
 
 // Per tile, its list in listed order: one warp per tile scans its row's entries
-// twice (count, then write to a range reserved by one atomic).
+// twice (count, then write to a range reserved by one atomic).  Ranges are
+// whole quads, the last one filled with entry 0.
 constexpr int kTileListWarps = 8;
 __global__ void __launch_bounds__(kTileListWarps * 32)
 k_plan_tiles(const int2* __restrict__ row_ent, const int2* __restrict__ row_rng, int ntu, int nt,
@@ -1032,8 +1042,10 @@ k_plan_tiles(const int2* __restrict__ row_ent, const int2* __restrict__ row_rng,
   for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
   int start = 0;
   if (lane == 0) {
-    const unsigned long long s = atomicAdd(counts + kCountTiles, static_cast<unsigned long long>(c));
-    start = s + c <= static_cast<unsigned long long>(cap) ? static_cast<int>(s) : -1;
+    const unsigned long long pad = static_cast<unsigned long long>((c + 3) & ~3);
+    if (c) atomicAdd(counts + kCountTiles, static_cast<unsigned long long>(c));
+    const unsigned long long s = c ? atomicAdd(counts + kCountSlots, pad) : 0ull;
+    start = s + pad <= static_cast<unsigned long long>(cap) ? static_cast<int>(s) : -1;
     tile_rng[tile] = start < 0 ? make_int2(0, 0) : make_int2(start, start + c);
   }
   start = __shfl_sync(0xffffffffu, start, 0);
@@ -1046,6 +1058,7 @@ k_plan_tiles(const int2* __restrict__ row_ent, const int2* __restrict__ row_rng,
     if (h) tile_idx[start + __popc(m & ((1u << lane) - 1u))] = ent;
     start += __popc(m);
   }
+  if (lane < (4 - (c & 3)) % 4) tile_idx[start + lane] = 0;
 }
 
 // The tiles from the longest list to the shortest (lists of kOrderBins and
@@ -1092,7 +1105,7 @@ __global__ void k_counts_out(const int* __restrict__ kept, int n_chan, int32_t* 
 
 // ---------------------------------------------------------------- planning
 struct ImgPlan {
-  int n, g, log2g, band_h, batch, cols_per_cta, storage;
+  int n, g, log2g, batch, cols_per_cta, storage;
   long long n_cross;
 };
 
@@ -1102,9 +1115,6 @@ ImgPlan make_plan(int n_ant, int n_chan, int n, int storage) {
   p.storage = storage;
   p.g = kPad * n;
   p.log2g = ilog2(p.g);
-  // row transforms: 8192 complex values per band, 512-thread CTAs (several
-  // per SM, so one band's loads overlap another's transforms)
-  p.band_h = 8192 / p.g < p.g / 2 ? 8192 / p.g : p.g / 2;
   p.n_cross = static_cast<long long>(n_ant) * (n_ant - 1) / 2;
   // channels per launch: whole groups of 32 (one per lane of a tile warp);
   // the gridded half planes, the prepared records and the half-transformed
@@ -1134,7 +1144,7 @@ struct ImgWs {
   double* axis;      // antenna positions [n_ant][3], then frequencies [n_chan]
   Baseline* base;
   ChanScale* cs;
-  int* kept;
+  int* kept;         // [n_chan] kept visibilities, then an item counter per batch (at most n_chan)
   PlanRange* rng;    // [n_cross] centre-cell ranges
   int* blk;          // listed baselines per CTA of k_plan_baselines
   GridEntry* listed; // baselines that can be gridded in some channel of the call
@@ -1147,7 +1157,7 @@ struct ImgWs {
   unsigned long long* counts;   // [kCounts]
   double* blen;      // [n_cross] baseline lengths (metres)
   PrepRec* prep;     // [batch groups][n_cross][32] prepared records (the listed ones first)
-  float* grid;       // [batch][2][G][G] gridded planes (re, im)
+  float2* grid;      // [batch groups][G/2][G][32] gridded half planes
   void* h;           // [batch][G][N] complex in the storage format
   float* hs;         // [batch][G] row scales (FP16 storage)
   bool bases = false;  // records carry weight-table offsets (footprints move < kTabMargin cells)
@@ -1160,6 +1170,8 @@ struct ImgWs {
 // as many more through its mirror).
 constexpr int kEntriesPerBaseline = 24;
 long long entry_capacity(const ImgPlan& p) { return std::max<long long>(1, p.n_cross * kEntriesPerBaseline); }
+// list slots: the entries, and up to 3 per tile to fill its last quad
+long long slot_capacity(const ImgPlan& p) { return entry_capacity(p) + 3LL * n_tiles(p.g); }
 
 ImgWs carve_img(void* ws, size_t bytes, const ImgPlan& p, int n_ant, int n_chan, size_t* need) {
   Carver c(ws, bytes);
@@ -1172,7 +1184,7 @@ ImgWs carve_img(void* ws, size_t bytes, const ImgPlan& p, int n_ant, int n_chan,
   w.axis = c.take<double>(static_cast<size_t>(n_ant) * 3 + n_chan);
   w.base = c.take<Baseline>(nx);
   w.cs = c.take<ChanScale>(n_chan);
-  w.kept = c.take<int>(n_chan);
+  w.kept = c.take<int>(2 * static_cast<size_t>(n_chan));
   w.rng = c.take<PlanRange>(nx);
   w.blk = c.take<int>((nx + kPlanThreads - 1) / kPlanThreads);
   w.listed = c.take<GridEntry>(nx);
@@ -1181,11 +1193,11 @@ ImgWs carve_img(void* ws, size_t bytes, const ImgPlan& p, int n_ant, int n_chan,
   w.row_rng = c.take<int2>(half_rows(p.g) / kTileV);
   w.tile_rng = c.take<int2>(n_tiles(p.g));
   w.tile_order = c.take<int>(n_tiles(p.g));
-  w.tile_idx = c.take<int>(entry_capacity(p));
+  w.tile_idx = c.take<int>(slot_capacity(p));
   w.counts = c.take<unsigned long long>(kCounts);
   w.blen = c.take<double>(nx);
   w.prep = c.take<PrepRec>(static_cast<size_t>((p.batch + kLanes - 1) / kLanes) * nx * kLanes);
-  w.grid = c.take<float>(static_cast<size_t>(p.batch) * 2 * half_rows(p.g) * p.g);
+  w.grid = c.take<float2>(static_cast<size_t>((p.batch + kLanes - 1) / kLanes) * kLanes * half_rows(p.g) * p.g);
   w.h = c.take<float2>(static_cast<size_t>(p.batch) * half_rows(p.g) * p.n);
   w.hs = c.take<float>(static_cast<size_t>(p.batch) * half_rows(p.g));
   *need = c.used;
@@ -1194,7 +1206,7 @@ ImgWs carve_img(void* ws, size_t bytes, const ImgPlan& p, int n_ant, int n_chan,
 
 template <int L, int S>
 int launch_batch(const ImgPlan& p, const ImgWs& w, const GridOpts& o, const int32_t* vis, long long n_bl, int ch0,
-                 int nb, float* img, cudaStream_t st) {
+                 int nb, unsigned* next_item, float* img, cudaStream_t st) {
   constexpr int G = 1 << L;
   constexpr int LDP = band_pitch(G);
   {
@@ -1217,17 +1229,17 @@ int launch_batch(const ImgPlan& p, const ImgWs& w, const GridOpts& o, const int3
     const long long ctas = std::min<long long>(num_sms(), (items + kGridWarps - 1) / kGridWarps);
     OVRO_PROF("k_grid_tiles", st);
     tiles<<<static_cast<unsigned>(ctas), kGridWarps * 32, kTileSmem, st>>>(
-        w.tile_idx, w.tile_rng, w.tile_order, w.prep, p.n_cross, w.tabx, nb, w.grid);
+        reinterpret_cast<const int4*>(w.tile_idx), w.tile_rng, w.tile_order, w.prep, p.n_cross, w.tabx, nb, next_item,
+        w.grid);
     OVRO_LAUNCH_CHECK();
   }
   {
-    const size_t sm = static_cast<size_t>(p.band_h) * LDP * sizeof(float2) + G * sizeof(float2);
+    const size_t sm = static_cast<size_t>(row_lines(G)) * LDP * sizeof(float2) + G * sizeof(float2);
     OVRO_CUDA_TRY(cudaFuncSetAttribute(k_fft_rows<L, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(sm)));
-    const int threads = p.band_h * G / 16;
-    dim3 grid(half_rows(G) / p.band_h, nb);
+    dim3 grid(half_rows(G) / row_rows(G), (nb + row_chans(G) - 1) / row_chans(G));
     OVRO_PROF("k_fft_rows", st);
-    k_fft_rows<L, S><<<grid, threads, sm, st>>>(w.grid, w.tw, p.n, p.band_h, w.h, w.hs);
+    k_fft_rows<L, S><<<grid, row_lines(G) * G / 16, sm, st>>>(w.grid, w.tw, nb, p.n, w.h, w.hs);
     OVRO_LAUNCH_CHECK();
   }
   {
@@ -1246,25 +1258,25 @@ int launch_batch(const ImgPlan& p, const ImgWs& w, const GridOpts& o, const int3
 
 template <int L>
 int launch_storage(const ImgPlan& p, const ImgWs& w, const GridOpts& o, const int32_t* vis, long long n_bl, int ch0,
-                   int nb, float* img, cudaStream_t st) {
+                   int nb, unsigned* next_item, float* img, cudaStream_t st) {
   switch (p.storage) {
-    case kStoreF32: return launch_batch<L, kStoreF32>(p, w, o, vis, n_bl, ch0, nb, img, st);
-    case kStoreBF16: return launch_batch<L, kStoreBF16>(p, w, o, vis, n_bl, ch0, nb, img, st);
-    case kStoreF16: return launch_batch<L, kStoreF16>(p, w, o, vis, n_bl, ch0, nb, img, st);
+    case kStoreF32: return launch_batch<L, kStoreF32>(p, w, o, vis, n_bl, ch0, nb, next_item, img, st);
+    case kStoreBF16: return launch_batch<L, kStoreBF16>(p, w, o, vis, n_bl, ch0, nb, next_item, img, st);
+    case kStoreF16: return launch_batch<L, kStoreF16>(p, w, o, vis, n_bl, ch0, nb, next_item, img, st);
     default: return OVRO_ERR_INVALID_ARG;
   }
 }
 
 int run_batch(const ImgPlan& p, const ImgWs& w, const GridOpts& o, const int32_t* vis, long long n_bl, int ch0,
-              int nb, float* img, cudaStream_t st) {
+              int nb, unsigned* next_item, float* img, cudaStream_t st) {
   switch (p.log2g) {
-    case 5: return launch_storage<5>(p, w, o, vis, n_bl, ch0, nb, img, st);
-    case 6: return launch_storage<6>(p, w, o, vis, n_bl, ch0, nb, img, st);
-    case 7: return launch_storage<7>(p, w, o, vis, n_bl, ch0, nb, img, st);
-    case 8: return launch_storage<8>(p, w, o, vis, n_bl, ch0, nb, img, st);
-    case 9: return launch_storage<9>(p, w, o, vis, n_bl, ch0, nb, img, st);
-    case 10: return launch_storage<10>(p, w, o, vis, n_bl, ch0, nb, img, st);
-    case 11: return launch_storage<11>(p, w, o, vis, n_bl, ch0, nb, img, st);
+    case 5: return launch_storage<5>(p, w, o, vis, n_bl, ch0, nb, next_item, img, st);
+    case 6: return launch_storage<6>(p, w, o, vis, n_bl, ch0, nb, next_item, img, st);
+    case 7: return launch_storage<7>(p, w, o, vis, n_bl, ch0, nb, next_item, img, st);
+    case 8: return launch_storage<8>(p, w, o, vis, n_bl, ch0, nb, next_item, img, st);
+    case 9: return launch_storage<9>(p, w, o, vis, n_bl, ch0, nb, next_item, img, st);
+    case 10: return launch_storage<10>(p, w, o, vis, n_bl, ch0, nb, next_item, img, st);
+    case 11: return launch_storage<11>(p, w, o, vis, n_bl, ch0, nb, next_item, img, st);
     default: return OVRO_ERR_UNSUPPORTED;
   }
 }
@@ -1328,7 +1340,7 @@ int upload_common(const ImgPlan& p, ImgWs& w, int n_ant, const double* h_ant,
   k_plan_rows<<<rows, kRowWarps * 32, 0, st>>>(w.lrng, p.g, w.counts, w.row_ent, entry_capacity(p), w.row_rng);
   OVRO_LAUNCH_CHECK();
   k_plan_tiles<<<(nt + kTileListWarps - 1) / kTileListWarps, kTileListWarps * 32, 0, st>>>(
-      w.row_ent, w.row_rng, n_tiles_u(p.g), nt, w.counts, w.tile_idx, entry_capacity(p), w.tile_rng);
+      w.row_ent, w.row_rng, n_tiles_u(p.g), nt, w.counts, w.tile_idx, slot_capacity(p), w.tile_rng);
   OVRO_LAUNCH_CHECK();
   k_plan_order<<<1, 1024, 0, st>>>(w.tile_rng, nt, w.tile_order);
   OVRO_LAUNCH_CHECK();
@@ -1417,10 +1429,11 @@ int grid_ctx_enqueue(GridCtx* g, const int32_t* d_vis, float* d_img, int32_t* d_
   // channels per launch pair (at most the workspace's batch): every choice
   // gives the same images and counts
   auto all = [&](int batch) -> int {
-    OVRO_CUDA_TRY(cudaMemsetAsync(g->w.kept, 0, g->n_chan * sizeof(int), st));
+    OVRO_CUDA_TRY(cudaMemsetAsync(g->w.kept, 0, 2 * static_cast<size_t>(g->n_chan) * sizeof(int), st));
+    unsigned* next_item = reinterpret_cast<unsigned*>(g->w.kept + g->n_chan);
     for (int ch0 = 0; ch0 < g->n_chan; ch0 += batch) {
       const int nb = g->n_chan - ch0 < batch ? g->n_chan - ch0 : batch;
-      if (int e = run_batch(p, g->w, o, d_vis, n_bl, ch0, nb, d_img, st)) return e;
+      if (int e = run_batch(p, g->w, o, d_vis, n_bl, ch0, nb, next_item++, d_img, st)) return e;
     }
     return OVRO_OK;
   };
