@@ -355,6 +355,20 @@ k_grid_prep(const GridEntry* __restrict__ listed, const unsigned long long* __re
   for (int bi = warp; bi < nbl; bi += 8) out[static_cast<long long>(bi) * kLanes + lane] = tile[bi][lane];
 }
 
+// Rows of the half-transformed grid kept per channel: the gridded plane is the
+// Hermitian part H of the grid on its rows j = G/2 .. G-1; the row transforms
+// of H satisfy R(G - j, k) = conj R(j, k), and row 0 is empty (no footprint
+// reaches it), so these G/2 rows carry everything the column pass needs.
+__host__ __device__ constexpr int half_rows(int g) { return g / 2; }
+
+// A row-pass CTA transforms row_lines(G) lines (8192 points; every row of the
+// smallest grids): row_chans(G) channels of as many rows each as fit.  The grid
+// holds these channels' values of four cells together, so the tile kernel's
+// stores are whole sectors and a CTA's input is one contiguous piece.
+__host__ __device__ constexpr int row_lines(int g) { return 8192 / g < 4 * g ? 8192 / g : 4 * g; }
+__host__ __device__ constexpr int row_chans(int g) { return row_lines(g) < 8 ? row_lines(g) : 8; }
+__host__ __device__ constexpr int row_rows(int g) { return row_lines(g) / row_chans(g); }
+
 // Gridding of one channel batch into the Hermitian part of the grid, rows
 // G/2 .. G-1 (v >= 0; a record whose footprint lies below is listed as its
 // mirror, one straddling row G/2 as both).  Work items are (group of 32
@@ -374,9 +388,10 @@ k_grid_prep(const GridEntry* __restrict__ listed, const unsigned long long* __re
 //   otherwise the lane takes the centre cells from the position and adds
 //     zeros when its footprint misses the tile.
 // The tile is written with the (-1)^(row + col) centring sign to grid
-// [group][G/2][G][32] (row j - G/2; re, im of 32 channels), 256 contiguous bytes
-// a warp store: with a plane per channel every lane wrote half a sector of its
-// own, and that bounded sparse grids.  Before (scalar, plane per channel,
+// [channels / row_chans][G/2][G/4][row_chans][4 cells] (row j - G/2; the
+// channels one row-pass CTA takes), a row of the tile and channel as one
+// 32-byte store and whole lines a warp: with a plane per channel every lane
+// wrote halves of sectors of its own, and that bounded sparse grids.  Before (scalar, plane per channel,
 // static items) -> now, 352 antennas: 1000 channels of 256^2 1.16 -> 0.72 ms,
 // 300 of 512^2 1.32 -> 0.49 ms, 64 of 1024^2 1.97 -> 0.33 ms.
 constexpr int kGridWarps = 20;
@@ -506,65 +521,48 @@ k_grid_tiles(const int4* __restrict__ tile_idx, const int2* __restrict__ tile_rn
     }
     // ---- the tile, with the centring sign (r0 and c0 are even)
     if (g * kLanes + lane < nb) {
-      float2* out = grid + ((static_cast<long long>(g) * (G / 2) + r0 - G / 2) * G + c0) * kLanes + lane;
+      constexpr int CH = row_chans(G);
+      const int cb = g * kLanes + lane;
+      float2* out = grid + ((static_cast<long long>(cb / CH) * (G / 2) + r0 - G / 2) * G + c0) * CH +
+                    (cb % CH) * kTileU;
 #pragma unroll
       for (int i = 0; i < kTileV; ++i)
+      {
+        unsigned long long z[kTileU];
 #pragma unroll
-        for (int j = 0; j < kTileU; ++j) {
-          float2 z;
-          asm("mov.b64 {%0, %1}, %2;" : "=f"(z.x), "=f"(z.y) : "l"(acc[i][j]));
-          out[(i * G + j) * kLanes] = (i + j) & 1 ? make_float2(-z.x, -z.y) : z;
-        }
+        for (int j = 0; j < kTileU; ++j) z[j] = (i + j) & 1 ? acc[i][j] ^ 0x8000000080000000ull : acc[i][j];
+        asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(out + i * G * CH), "l"(z[0]), "l"(z[1]),
+                     "l"(z[2]), "l"(z[3])
+                     : "memory");
+      }
     }
     item = __shfl_sync(full, after, 0);
   }
 }
 
-// Rows of the half-transformed grid kept per channel: the gridded plane is the
-// Hermitian part H of the grid on its rows j = G/2 .. G-1; the row transforms
-// of H satisfy R(G - j, k) = conj R(j, k), and row 0 is empty (no footprint
-// reaches it), so these G/2 rows carry everything the column pass needs.
-__host__ __device__ constexpr int half_rows(int g) { return g / 2; }
-
-// A row-pass CTA transforms row_lines(G) lines (8192 points; every row of the
-// smallest grids): row_chans(G) channels of as many rows each as fit.  The grid
-// holds a cell's channels together, so 8 channels make whole sectors (4 of
-// 2048 points still make 32 bytes).
-__host__ __device__ constexpr int row_lines(int g) { return 8192 / g < 4 * g ? 8192 / g : 4 * g; }
-__host__ __device__ constexpr int row_chans(int g) { return row_lines(g) < 8 ? row_lines(g) : 8; }
-__host__ __device__ constexpr int row_rows(int g) { return row_lines(g) / row_chans(g); }
-
 // The central N columns of the CTA's row transforms (line f = channel
-// f / row_rows, row f % row_rows), into the half-transformed grid h
-// ([batch][G/2][N]) in its storage format.
+// f / row_rows, row f % row_rows) in 16-bit storage.
 template <int G, int LDP, int S>
 __device__ __forceinline__ void store_band(const float2* band, int cb0, int row0, int nb, int n_img, void* h,
                                            float* hs) {
   constexpr int R = row_rows(G);
   const int offc = G / 2 - n_img / 2;
   const int lines = min(row_chans(G), nb - cb0) * R;    // the channels of the batch
-  auto hrow = [&](int f) { return static_cast<long long>(cb0 + f / R) * half_rows(G) + row0 + f % R; };
-  if constexpr (S == kStoreF32) {
-    float2* hb = static_cast<float2*>(h);
+  auto row_of = [&](int f) { return static_cast<long long>(cb0 + f / R) * half_rows(G) + row0 + f % R; };
+  if constexpr (S == kStoreBF16) {
     for (int i = threadIdx.x; i < lines * n_img; i += blockDim.x) {
-      const int r = i / n_img, c = i - r * n_img;
-      hb[hrow(r) * n_img + c] = band[r * LDP + pad16(offc + c)];
-    }
-  } else if constexpr (S == kStoreBF16) {
-    __nv_bfloat162* hb = static_cast<__nv_bfloat162*>(h);
-    for (int i = threadIdx.x; i < lines * n_img; i += blockDim.x) {
-      const int r = i / n_img, c = i - r * n_img;
-      hb[hrow(r) * n_img + c] = __float22bfloat162_rn(band[r * LDP + pad16(offc + c)]);
+      const int f = i / n_img, c = i - f * n_img;
+      static_cast<__nv_bfloat162*>(h)[row_of(f) * n_img + c] = __float22bfloat162_rn(band[f * LDP + pad16(offc + c)]);
     }
   } else {
     // FP16 with a power-of-two scale per row: the row's largest component
     // lands in [2^13, 2^14), far from FP16 overflow; scaling is exact
-    __half2* hb = static_cast<__half2*>(h);
     const int lane = threadIdx.x & 31, n_w = blockDim.x >> 5;
-    for (int r = threadIdx.x >> 5; r < lines; r += n_w) {
+    for (int f = threadIdx.x >> 5; f < lines; f += n_w) {
+      const long long row = row_of(f);
       float m = 0.f;
       for (int c = lane; c < n_img; c += 32) {
-        const float2 v = band[r * LDP + pad16(offc + c)];
+        const float2 v = band[f * LDP + pad16(offc + c)];
         m = fmaxf(m, fmaxf(fabsf(v.x), fabsf(v.y)));
       }
 #pragma unroll
@@ -572,56 +570,231 @@ __device__ __forceinline__ void store_band(const float2* band, int cb0, int row0
       int e = 0;
       if (m > 0.f) frexpf(m, &e);
       const float sc = m > 0.f ? ldexpf(1.0f, 14 - e) : 1.0f;
-      if (lane == 0) hs[hrow(r)] = m > 0.f ? ldexpf(1.0f, e - 14) : 0.0f;
+      if (lane == 0) hs[row] = m > 0.f ? ldexpf(1.0f, e - 14) : 0.0f;
       for (int c = lane; c < n_img; c += 32) {
-        const float2 v = band[r * LDP + pad16(offc + c)];
-        hb[hrow(r) * n_img + c] = __float22half2_rn(make_float2(v.x * sc, v.y * sc));
+        const float2 v = band[f * LDP + pad16(offc + c)];
+        static_cast<__half2*>(h)[row * n_img + c] = __float22half2_rn(make_float2(v.x * sc, v.y * sc));
       }
     }
   }
 }
 
-// Row transforms of the gridded half planes: a CTA stages its lines with
-// 16-byte loads (two channels of a cell each, all in flight at once), turned
-// into rows in shared memory, and transforms them in place; the central N
-// columns go to h ([batch][G/2][N], row j - G/2).
+// ------------------------------------------------------------ line FFTs
+// Forward FFTs of G = 2^LOG2G points (32 .. 2048) along lines in shared memory:
+// a radix-16 pass, one of radix 2 .. 16 (16 points done) and, from 512 points
+// on, one of radix 2, 4 or 8 (256 done).  Every thread holds 16 values.  The
+// passes are issue bound, so the additions are packed (re, im), the twiddles
+// of a pass are read from a table of its own laid out [factor][k] (a warp's
+// reads are consecutive; from one table of powers they met in few banks, which
+// had to be traded against products of powers), the first pass reads wherever
+// the lines come from and the last one hands its values to a functor instead
+// of another trip through shared memory.  Against the shared passes of
+// fft.cuh with staged input and output, 352 antennas: 1000 channels of 256^2
+// rows 0.60 -> 0.44 ms, columns 0.42 -> 0.32 ms; 300 of 512^2 0.72 -> 0.49 and
+// 0.54 -> 0.40 ms.
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 p, q, r;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %5};\n\tadd.rn.f32x2 r, p, q;\n\t"
+      "mov.b64 {%0, %1}, r;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+// a + s b for a pair of signs or factors s
+__device__ __forceinline__ float2 axpy2(float2 a, float s, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 p, q, r;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %5};\n\tmov.b64 r, {%6, %6};\n\t"
+      "fma.rn.f32x2 r, q, r, p;\n\tmov.b64 {%0, %1}, r;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(s));
+  return d;
+}
+
+// (a, b) <- (a + w b, a - w b), w = exp(-2 pi i Q / 16)
+template <int Q>
+__device__ __forceinline__ void bfly(float2& a, float2& b) {
+  constexpr float r2 = 0.70710678118654752f;
+  if constexpr (Q == 0) {
+    const float2 x = b;
+    b = axpy2(a, -1.0f, x);
+    a = add2(a, x);
+  } else if constexpr (Q == 4) {
+    const float2 x = b, y = a;                          // -i x = (x.y, -x.x)
+    a = make_float2(y.x + x.y, y.y - x.x);
+    b = make_float2(y.x - x.y, y.y + x.x);
+  } else if constexpr (Q == 2 || Q == 6) {
+    // r2 (1 - i) x and r2 (-1 - i) x: the factor goes into the sums
+    const float2 u = Q == 2 ? make_float2(b.x + b.y, b.y - b.x) : make_float2(b.y - b.x, -b.x - b.y);
+    const float2 y = a;
+    a = axpy2(y, r2, u);
+    b = axpy2(y, -r2, u);
+  } else {
+    constexpr float cw = Q == 1 ? 0.92387953251128674f : Q == 3 ? 0.38268343236508977f
+                         : Q == 5 ? -0.38268343236508977f : -0.92387953251128674f;
+    constexpr float sw = Q == 1 || Q == 7 ? -0.38268343236508977f : -0.92387953251128674f;
+    const float2 x = cmul(b, make_float2(cw, sw));
+    b = axpy2(a, -1.0f, x);
+    a = add2(a, x);
+  }
+}
+
+// V[k] = sum_r v[r] exp(-2 pi i r k / R), in natural order; R = 2, 4, 8, 16.
+template <int R>
+__device__ __forceinline__ void dft_line(float2* v) {
+  float2 t[R];
+#pragma unroll
+  for (int i = 0; i < R; ++i) t[i] = v[BitRev<R>::of(i)];
+#pragma unroll
+  for (int i = 0; i < R; i += 2) bfly<0>(t[i], t[i + 1]);
+  if constexpr (R >= 4) {
+#pragma unroll
+    for (int i = 0; i < R; i += 4) {
+      bfly<0>(t[i], t[i + 2]);
+      bfly<4>(t[i + 1], t[i + 3]);
+    }
+  }
+  if constexpr (R >= 8) {
+#pragma unroll
+    for (int i = 0; i < R; i += 8) {
+      bfly<0>(t[i], t[i + 4]);
+      bfly<2>(t[i + 1], t[i + 5]);
+      bfly<4>(t[i + 2], t[i + 6]);
+      bfly<6>(t[i + 3], t[i + 7]);
+    }
+  }
+  if constexpr (R >= 16) {
+    bfly<0>(t[0], t[8]);
+    bfly<1>(t[1], t[9]);
+    bfly<2>(t[2], t[10]);
+    bfly<3>(t[3], t[11]);
+    bfly<4>(t[4], t[12]);
+    bfly<5>(t[5], t[13]);
+    bfly<6>(t[6], t[14]);
+    bfly<7>(t[7], t[15]);
+  }
+#pragma unroll
+  for (int i = 0; i < R; ++i) v[i] = t[i];
+}
+
+// Twiddle tables of the second and third pass: [R2][16] with R2 = min(G / 16, 16)
+// of exp(-2 pi i r k / (16 R2)), then, from 512 points on, [G / 256][256] of
+// exp(-2 pi i r k / G).  Behind them omega_G^k, k < G, for 16-bit storage.
+__host__ __device__ constexpr int tw_entries(int g) { return g <= 256 ? g : 256 + g; }
+__host__ __device__ constexpr int tw_all(int g) { return tw_entries(g) + g; }
+
+// One pass of radix R over `NS` done points: load(f, x) gives point x of line f
+// and store(f, x, v) takes point x of its result; split(i, f, j) the line and
+// index of butterfly i (all of the CTA's, in the order the threads take them).
+// in_place: the results overwrite the input.
+template <int R, int NS, int G, class Split, class Load, class Store>
+__device__ __forceinline__ void line_pass(const float2* tw, bool in_place, Split&& split, Load&& load, Store&& store) {
+  constexpr int NB = 16 / R;
+  float2 v[16];
+  int f[NB], j[NB];
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    split(static_cast<int>(threadIdx.x + b * blockDim.x), f[b], j[b]);
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[b * R + r] = load(f[b], j[b] + r * (G / R));
+  }
+  if (in_place) __syncthreads();                        // every read before the first write
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    const int k = j[b] & (NS - 1);
+    if constexpr (NS > 1) {
+#pragma unroll
+      for (int r = 1; r < R; ++r) v[b * R + r] = cmul(v[b * R + r], tw[r * NS + k]);
+    }
+    dft_line<R>(v + b * R);
+    const int o = (j[b] / NS) * NS * R + k;
+#pragma unroll
+    for (int r = 0; r < R; ++r) store(f[b], o + r * NS, v[b * R + r]);
+  }
+  if (in_place) __syncthreads();
+}
+
+// load0(f, x), split0: the first pass's input and item order; store(f, x, v),
+// split1: the last pass's output and item order.
+// Lines lie at a[f * ldp], element x at pad16(x), in between; blockDim.x * 16 ==
+// lines * G.
+template <int LOG2G, class Split0, class Load0, class Split1, class Store>
+__device__ __forceinline__ void fft_lines(float2* a, int ldp, const float2* tw, Split0&& split0, Load0&& load0,
+                                          Split1&& split1, Store&& store) {
+  constexpr int G = 1 << LOG2G;
+  constexpr int R2 = G / 16 < 16 ? G / 16 : 16;
+  static_assert(G >= 32 && G <= 2048, "two or three passes");
+  auto put = [&](int f, int x, float2 v) { a[f * ldp + pad16(x)] = v; };
+  auto get = [&](int f, int x) { return a[f * ldp + pad16(x)]; };
+  line_pass<16, 1, G>(tw, true, split0, load0, put);
+  if constexpr (G <= 256) {
+    line_pass<R2, 16, G>(tw, false, split1, get, store);
+  } else {
+    auto split = [&](int i, int& f, int& j) {
+      f = i / (G / 16);
+      j = i % (G / 16);
+    };
+    line_pass<16, 16, G>(tw, true, split, get, put);
+    line_pass<G / 256, 256, G>(tw + 256, false, split1, get, store);
+  }
+}
+
+// The row transforms' last butterflies have radix last_radix(G).
+__host__ __device__ constexpr int last_radix(int g) { return g <= 256 ? g / 16 : g / 256; }
+
+// Row transforms of the gridded half planes: a CTA copies its channels' rows in
+// (64 KB, contiguous) and transforms them; the central N columns go to h
+// ([batch][G/2][N], row j - G/2), straight from the last pass.  With 16-bit
+// storage the rows go through fft_rows_inplace_f instead: rounding to 16 bits
+// turns a last-bit difference of a row into one of 2^-9 or 2^-12, and images
+// keep the bits they had.
 template <int LOG2G, int S>
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(512, 2)
 k_fft_rows(const float2* __restrict__ grid, const float2* __restrict__ tw_g, int nb, int n_img,
            void* __restrict__ h, float* __restrict__ hs) {
   constexpr int G = 1 << LOG2G;
   constexpr int LDP = band_pitch(G);
-  constexpr int CH = row_chans(G), R = row_rows(G), CP = CH / 2;
+  constexpr int CH = row_chans(G), R = row_rows(G);
   extern __shared__ __align__(16) unsigned char smem[];
-  float2* band = reinterpret_cast<float2*>(smem);     // [row_lines][LDP]
-  float2* tw = band + row_lines(G) * LDP;             // [G]
+  float2* band = reinterpret_cast<float2*>(smem);     // [row_lines][LDP]; first the input [R][G/4][CH][4]
+  float2* tw = band + row_lines(G) * LDP;
   const int cb0 = blockIdx.y * CH, row0 = blockIdx.x * R;
-  for (int i = threadIdx.x; i < G; i += blockDim.x) tw[i] = tw_g[i];
-  // [group][row][col][32 channels] float2, read as channel pairs
-  const float4* src = reinterpret_cast<const float4*>(grid) +
-                      (static_cast<long long>(cb0 / kLanes) * half_rows(G) + row0) * G * (kLanes / 2) +
-                      (cb0 % kLanes) / 2;
-  // row_lines G / 2 float4 over row_lines G / 16 threads: 8 per thread, all
-  // issued before the first is stored
-  constexpr int PER = 8;
-  float4 q[PER];
+  const float4* src = reinterpret_cast<const float4*>(
+      grid + (static_cast<long long>(blockIdx.y) * half_rows(G) + row0) * G * CH);
+  float4 q[8];
 #pragma unroll
-  for (int u = 0; u < PER; ++u) {
-    const int i = threadIdx.x + u * blockDim.x;       // (row, col, channel pair)
-    q[u] = __ldg(src + static_cast<long long>(i / CP) * (kLanes / 2) + i % CP);
-  }
+  for (int u = 0; u < 8; ++u) q[u] = __ldg(src + threadIdx.x + u * blockDim.x);
+  constexpr int TW0 = S == kStoreF32 ? 0 : tw_entries(G), TWN = S == kStoreF32 ? tw_entries(G) : G;
+  for (int i = threadIdx.x; i < TWN; i += blockDim.x) tw[i] = __ldg(tw_g + TW0 + i);
 #pragma unroll
-  for (int u = 0; u < PER; ++u) {
-    const int i = threadIdx.x + u * blockDim.x;
-    const int cp = i % CP, x = i / CP, r = x / G, c = x % G;
-    float2* d = band + (2 * cp * R + r) * LDP + pad16(c);
-    d[0] = make_float2(q[u].x, q[u].y);
-    d[R * LDP] = make_float2(q[u].z, q[u].w);
-  }
+  for (int u = 0; u < 8; ++u) reinterpret_cast<float4*>(band)[threadIdx.x + u * blockDim.x] = q[u];
   __syncthreads();
-  fft_rows_inplace_f<LOG2G>(
-      band, LDP, [&](int f, int x) { return band[f * LDP + pad16(x)]; }, [&](int i) { return tw[i]; });
-  store_band<G, LDP, S>(band, cb0, row0, nb, n_img, h, hs);
+  // the first pass takes four cells and the channels in adjacent lanes, as
+  // they lie in shared memory
+  constexpr int J = G / 16 < 4 ? G / 16 : 4;
+  auto split0 = [&](int i, int& f, int& j) {
+    const int x = i / (J * CH);                       // (row, group of J butterflies)
+    f = (i / J % CH) * R + x / (G / 16 / J);
+    j = x % (G / 16 / J) * J + i % J;
+  };
+  auto load0 = [&](int f, int x) { return band[(((f % R) * (G / 4) + x / 4) * CH + f / R) * 4 + x % 4]; };
+  if constexpr (S == kStoreF32) {
+    constexpr int PER = G / last_radix(G);
+    const int offc = G / 2 - n_img / 2;
+    fft_lines<LOG2G>(
+        band, LDP, tw, split0, load0,
+        [&](int i, int& f, int& j) {
+          f = i / PER;
+          j = i % PER;
+        },
+        [&](int f, int x, float2 v) {
+          const int cb = cb0 + f / R, c = x - offc;
+          if (cb < nb && static_cast<unsigned>(c) < static_cast<unsigned>(n_img))
+            static_cast<float2*>(h)[(static_cast<long long>(cb) * half_rows(G) + row0 + f % R) * n_img + c] = v;
+        });
+  } else {
+    fft_rows_inplace_f<LOG2G>(band, LDP, load0, [&](int i) { return tw[i]; });
+    store_band<G, LDP, S>(band, cb0, row0, nb, n_img, h, hs);
+  }
 }
 
 // Two adjacent values (idx even) of the half-transformed grid in FP32.
@@ -676,7 +849,7 @@ k_fft_cols(const void* __restrict__ h, const float* __restrict__ hs, int n_img, 
   const int cb = blockIdx.y;
   const int c0 = blockIdx.x * C;
   const long long hrow0 = static_cast<long long>(cb) * half_rows(G);
-  for (int i = threadIdx.x; i < G; i += blockDim.x) tw[i] = tw_g[i];
+  for (int i = threadIdx.x; i < tw_entries(G); i += blockDim.x) tw[i] = __ldg(tw_g + i);
   // U items per thread in flight: the reads come from L2 and would otherwise
   // wait one round trip each
   constexpr int U = 8;
@@ -705,25 +878,43 @@ k_fft_cols(const void* __restrict__ h, const float* __restrict__ hs, int n_img, 
     }
   }
   __syncthreads();
-  fft_rows_inplace_f<LOG2G>(
-      A, LDP, [&](int f, int x) { return A[f * LDP + pad16(x)]; }, [&](int i) { return tw[i]; });
   const long long chan = ch0 + cb;
   const int k = kept[chan];
   const float norm = k > 0 ? 0.5f / static_cast<float>(k) : 0.0f;
   const int off = G / 2 - n_img / 2;
-  float* out = img + chan * n_img * n_img;
-#pragma unroll 4
-  for (int i = threadIdx.x; i < n_img * C; i += blockDim.x) {
-    const int r = i >> (cp_shift + 1), c = i & (C - 1);
-    const int col = c0 + c;
-    float v = 0.0f;
-    if (mask[r * n_img + col]) {
-      const float2 z = A[(c >> 1) * LDP + pad16(off + r)];
-      v = (c & 1 ? z.y : z.x) * norm * inv_corr[r] * inv_corr[col];
-      if ((r + col) & 1) v = -v;
-    }
-    out[static_cast<long long>(r) * n_img + col] = v;
-  }
+  float* out = img + chan * n_img * n_img + c0;
+  // the last pass takes the column pairs in adjacent lanes, so a warp writes
+  // whole pieces of image rows; a thread keeps its pair
+  const int pair = threadIdx.x & (CP - 1);
+  const float2 ic = __ldg(reinterpret_cast<const float2*>(inv_corr + c0) + pair);
+  fft_lines<LOG2G>(
+      A, LDP, tw, [&](int i, int& f, int& j) {
+        f = i / (G / 16);
+        j = i % (G / 16);
+      },
+      [&](int f, int x) { return A[f * LDP + pad16(x)]; },
+      [&](int i, int& f, int& j) {
+        f = i & (CP - 1);
+        j = i >> cp_shift;
+      },
+      [&](int, int x, float2 z) {
+        const int r = x - off;
+        if (static_cast<unsigned>(r) >= static_cast<unsigned>(n_img)) return;
+        const uchar2 m = *reinterpret_cast<const uchar2*>(mask + r * n_img + c0 + 2 * pair);
+        const float ir = __ldg(inv_corr + r);
+        float2 v = make_float2(z.x * norm * ir * ic.x, z.y * norm * ir * ic.y);
+        // centring sign: (r + col) odd, c0 and the pair's first column even
+        if (r & 1) v.x = -v.x;
+        else v.y = -v.y;
+        if (!m.x) v.x = 0.0f;
+        if (!m.y) v.y = 0.0f;
+        *reinterpret_cast<float2*>(out + static_cast<long long>(r) * n_img + 2 * pair) = v;
+      });
+}
+
+__global__ void k_counts_out(const int* __restrict__ kept, int n_chan, int32_t* __restrict__ out) {
+  const int f = blockIdx.x * blockDim.x + threadIdx.x;
+  if (f < n_chan) out[f] = 2 * kept[f];
 }
 
 // ---------------------------------------------------------- per-call tables and lists
@@ -782,13 +973,18 @@ k_img_tables(const __grid_constant__ KernelHalf kh, int n, int g, double cell, c
     return;
   }
   i -= kTabXLen;
-  if (i < g) {
+  if (i < tw_all(g)) {
+    // exp(-2 pi i r k / len): the second pass's table, the third's, omega_G^k
+    const bool powers = i >= tw_entries(g), third = i >= 256;
+    const int e = static_cast<int>(third ? i - 256 : i);
+    const int rk = powers ? static_cast<int>(i) - tw_entries(g) : third ? (e >> 8) * (e & 255) : (e >> 4) * (e & 15);
+    const int len = powers || third ? g : min(g, 256);
     double si, co;
-    sincospi(-2.0 * static_cast<double>(i) / static_cast<double>(g), &si, &co);
+    sincospi(-2.0 * static_cast<double>(rk) / static_cast<double>(len), &si, &co);
     tw[i] = make_float2(static_cast<float>(co), static_cast<float>(si));
     return;
   }
-  i -= g;
+  i -= tw_all(g);
   if (i < static_cast<long long>(n) * n) {
     const int r = static_cast<int>(i) / n, c = static_cast<int>(i) - r * n;
     const double l = static_cast<double>(c - n / 2) * cell;
@@ -1098,11 +1294,6 @@ k_plan_order(const int2* __restrict__ tile_rng, int nt, int* __restrict__ order)
   for (int t = threadIdx.x; t < nt; t += 1024) order[atomicAdd(&bin[cls(t)], 1)] = t;
 }
 
-__global__ void k_counts_out(const int* __restrict__ kept, int n_chan, int32_t* __restrict__ out) {
-  const int f = blockIdx.x * blockDim.x + threadIdx.x;
-  if (f < n_chan) out[f] = 2 * kept[f];
-}
-
 // ---------------------------------------------------------------- planning
 struct ImgPlan {
   int n, g, log2g, batch, cols_per_cta, storage;
@@ -1128,9 +1319,9 @@ ImgPlan make_plan(int n_ant, int n_chan, int n, int storage) {
   p.batch = static_cast<int>(b);
   // an even number of columns per CTA (the column pass pairs them)
   int c = 8192 / p.g;
-  // 16-bit storage: at least 8 columns per CTA, so each row segment the
-  // column pass reads is a whole 32-byte sector
-  if (storage != kStoreF32 && c < 8 && 8 * p.g / 32 <= 512) c = 8;
+  // at least 8 columns per CTA, so each row segment the column pass reads (4
+  // bytes a value in 16-bit storage) and writes is a whole 32-byte sector
+  if (c < 8) c = 8;
   if (c > n) c = n;
   p.cols_per_cta = c;
   return p;
@@ -1157,7 +1348,7 @@ struct ImgWs {
   unsigned long long* counts;   // [kCounts]
   double* blen;      // [n_cross] baseline lengths (metres)
   PrepRec* prep;     // [batch groups][n_cross][32] prepared records (the listed ones first)
-  float2* grid;      // [batch groups][G/2][G][32] gridded half planes
+  float2* grid;      // [batch / row_chans][G/2][G/4][row_chans][4] gridded half planes
   void* h;           // [batch][G][N] complex in the storage format
   float* hs;         // [batch][G] row scales (FP16 storage)
   bool bases = false;  // records carry weight-table offsets (footprints move < kTabMargin cells)
@@ -1179,7 +1370,7 @@ ImgWs carve_img(void* ws, size_t bytes, const ImgPlan& p, int n_ant, int n_chan,
   const size_t nx = p.n_cross > 0 ? static_cast<size_t>(p.n_cross) : 1;
   w.tabx = c.take<float>(kTabXLen);
   w.inv_corr = c.take<float>(p.n);
-  w.tw = c.take<float2>(p.g);
+  w.tw = c.take<float2>(tw_all(p.g));
   w.mask = c.take<uint8_t>(static_cast<size_t>(p.n) * p.n);
   w.axis = c.take<double>(static_cast<size_t>(n_ant) * 3 + n_chan);
   w.base = c.take<Baseline>(nx);
@@ -1234,7 +1425,7 @@ int launch_batch(const ImgPlan& p, const ImgWs& w, const GridOpts& o, const int3
     OVRO_LAUNCH_CHECK();
   }
   {
-    const size_t sm = static_cast<size_t>(row_lines(G)) * LDP * sizeof(float2) + G * sizeof(float2);
+    const size_t sm = (static_cast<size_t>(row_lines(G)) * LDP + tw_entries(G)) * sizeof(float2);
     OVRO_CUDA_TRY(cudaFuncSetAttribute(k_fft_rows<L, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(sm)));
     dim3 grid(half_rows(G) / row_rows(G), (nb + row_chans(G) - 1) / row_chans(G));
@@ -1243,7 +1434,7 @@ int launch_batch(const ImgPlan& p, const ImgWs& w, const GridOpts& o, const int3
     OVRO_LAUNCH_CHECK();
   }
   {
-    const size_t sm = static_cast<size_t>(p.cols_per_cta / 2) * LDP * sizeof(float2) + G * sizeof(float2);
+    const size_t sm = (static_cast<size_t>(p.cols_per_cta / 2) * LDP + tw_entries(G)) * sizeof(float2);
     OVRO_CUDA_TRY(cudaFuncSetAttribute(k_fft_cols<L, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(sm)));
     const int threads = p.cols_per_cta * G / 32;
@@ -1325,7 +1516,7 @@ int upload_common(const ImgPlan& p, ImgWs& w, int n_ant, const double* h_ant,
   // the vector may go out of scope
   OVRO_CUDA_TRY(cudaMemcpyAsync(w.axis, axis.data(), axis.size() * sizeof(double), cudaMemcpyHostToDevice, st));
   OVRO_CUDA_TRY(cudaMemsetAsync(w.counts, 0, kCounts * sizeof(unsigned long long), st));
-  const long long elems = kTabXLen + static_cast<long long>(p.g) + static_cast<long long>(p.n) * p.n + n_chan;
+  const long long elems = kTabXLen + static_cast<long long>(tw_all(p.g)) + static_cast<long long>(p.n) * p.n + n_chan;
   k_img_tables<<<static_cast<unsigned>(p.n / 2 + 1 + (elems + kTabThreads - 1) / kTabThreads), kTabThreads, 0, st>>>(
       kh, p.n, p.g, cell, d_freq, n_chan, w.inv_corr, w.tabx, w.tw, w.mask, w.cs);
   OVRO_LAUNCH_CHECK();
