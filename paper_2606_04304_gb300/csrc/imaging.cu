@@ -136,7 +136,7 @@ __global__ void k_uvw(const Baseline* __restrict__ base, int n_cross, const Chan
 }
 
 // device counters of one call's plan (ImgWs::counts)
-constexpr int kCountListed = 0, kCountRows = 1, kCountTiles = 2, kCountSlots = 3, kCounts = 4;
+constexpr int kCountListed = 0, kCountRows = 1, kCountTiles = 2, kCountSlots = 3, kCountHeavy = 4, kCounts = 5;
 
 struct GridEntry {
   int bl;            // baseline index in the visibility record
@@ -362,20 +362,23 @@ k_grid_prep(const GridEntry* __restrict__ listed, const unsigned long long* __re
 __host__ __device__ constexpr int half_rows(int g) { return g / 2; }
 
 // A row-pass CTA transforms row_lines(G) lines (8192 points; every row of the
-// smallest grids): row_chans(G) channels of as many rows each as fit.  The grid
-// holds these channels' values of four cells together, so the tile kernel's
-// stores are whole sectors and a CTA's input is one contiguous piece.
+// smallest grids): row_chans(G) channels of as many rows each as fit, whose
+// values of four cells are 256 (128 at 2048 points) contiguous bytes of the grid.
 __host__ __device__ constexpr int row_lines(int g) { return 8192 / g < 4 * g ? 8192 / g : 4 * g; }
 __host__ __device__ constexpr int row_chans(int g) { return row_lines(g) < 8 ? row_lines(g) : 8; }
 __host__ __device__ constexpr int row_rows(int g) { return row_lines(g) / row_chans(g); }
 
 // Gridding of one channel batch into the Hermitian part of the grid, rows
 // G/2 .. G-1 (v >= 0; a record whose footprint lies below is listed as its
-// mirror, one straddling row G/2 as both).  Work items are (group of 32
-// channels, warp tile) pairs, group-major, the tiles of a group taken from the
-// longest list to the shortest; the warps of the persistent grid (one CTA of
-// kGridWarps warps per SM) draw items from a counter, the next one while they
-// work on the last.  The gap-indexed weight table sits in shared memory with
+// mirror, one straddling row G/2 as both).  Work items are (warp tile, group of
+// 32 channels) pairs, the tiles of kHeavy entries and more first and the others
+// as they lie: from the middle rows of the plane, where the lists are long,
+// outwards, and neighbours together, whose records and lines of the grid then
+// meet in L2 (from the longest list to the shortest, the stores of a sparse
+// grid went to DRAM line by line: 0.53 against 0.35 ms at 64 channels of
+// 1024^2).  The warps of the persistent grid (one CTA of kGridWarps warps per
+// SM) draw items from a counter, the next one while they work on the last.  The
+// gap-indexed weight table sits in shared memory with
 // every weight twice, so that one 8-byte load gives both factors of a packed
 // multiply-add on a cell's (re, im): a record costs a lane one 16-byte load,
 // 8 table loads, 4 + 16 packed multiply(-add)s and its decoding, where scalar
@@ -388,13 +391,14 @@ __host__ __device__ constexpr int row_rows(int g) { return row_lines(g) / row_ch
 //   otherwise the lane takes the centre cells from the position and adds
 //     zeros when its footprint misses the tile.
 // The tile is written with the (-1)^(row + col) centring sign to grid
-// [channels / row_chans][G/2][G/4][row_chans][4 cells] (row j - G/2; the
-// channels one row-pass CTA takes), a row of the tile and channel as one
-// 32-byte store and whole lines a warp: with a plane per channel every lane
-// wrote halves of sectors of its own, and that bounded sparse grids.  Before (scalar, plane per channel,
-// static items) -> now, 352 antennas: 1000 channels of 256^2 1.16 -> 0.72 ms,
-// 300 of 512^2 1.32 -> 0.49 ms, 64 of 1024^2 1.97 -> 0.33 ms.
+// [group][G/2][G/4][32 channels][4 cells] (row j - G/2): a row of the tile and
+// channel is one 32-byte store, 1 KB a warp.  With a plane per channel every lane
+// wrote halves of sectors of its own, and that bounded sparse grids; with planes
+// of 4 or 8 channels the lines went to DRAM in pieces.  Before (scalar, plane per channel,
+// static items) -> now, 352 antennas: 1000 channels of 256^2 1.16 -> 0.69 ms,
+// 300 of 512^2 1.32 -> 0.46 ms, 64 of 1024^2 1.97 -> 0.35 ms.
 constexpr int kGridWarps = 20;
+constexpr int kHeavy = 256;        // list entries of a tile that is taken first
 constexpr int kRing = 4;           // records in flight per warp: one quad of list entries
 constexpr size_t kTileSmem = static_cast<size_t>(kTabXLen) * kTabBytes;
 
@@ -417,8 +421,8 @@ __device__ __forceinline__ unsigned long long pack2(int lo, int hi) {
 
 template <int LOG2G, bool BASES>
 __global__ void __launch_bounds__(kGridWarps * 32, 1)
-k_grid_tiles(const int4* __restrict__ tile_idx, const int2* __restrict__ tile_rng, const int* __restrict__ tile_order,
-             const PrepRec* __restrict__ prep, long long n_cross, const float* __restrict__ tabx_g, int nb,
+k_grid_tiles(const int4* __restrict__ tile_idx, const int2* __restrict__ tile_rng, const int* __restrict__ heavy,
+             const unsigned long long* __restrict__ counts, const PrepRec* __restrict__ prep, long long n_cross, const float* __restrict__ tabx_g, int nb,
              unsigned* __restrict__ next_item, float2* __restrict__ grid) {
   constexpr int G = 1 << LOG2G;
   constexpr int NTU = n_tiles_u(G);
@@ -432,7 +436,9 @@ k_grid_tiles(const int4* __restrict__ tile_idx, const int2* __restrict__ tile_rn
     reinterpret_cast<float2*>(smem)[i] = make_float2(w, w);
   }
   __syncthreads();
-  const unsigned n_items = static_cast<unsigned>((nb + kLanes - 1) / kLanes) * NT;
+  const unsigned n_groups = static_cast<unsigned>((nb + kLanes - 1) / kLanes);
+  const unsigned n_first = static_cast<unsigned>(counts[kCountHeavy]) * n_groups;
+  const unsigned n_items = n_first + n_groups * NT;
   auto draw = [&]() {
     unsigned i = 0;
     if (lane == 0) i = atomicAdd(next_item, 1u);
@@ -442,12 +448,18 @@ k_grid_tiles(const int4* __restrict__ tile_idx, const int2* __restrict__ tile_rn
 #pragma unroll 1
   while (item < n_items) {
     const unsigned after = draw();                     // broadcast once this item is done
-    const int g = static_cast<int>(item / NT);
-    const int tile = __ldg(tile_order + (item - static_cast<unsigned>(g) * NT));
+    const bool first = item < n_first;
+    const unsigned at = first ? item : item - n_first;
+    const int g = static_cast<int>(at % n_groups);
+    const int tile = first ? __ldg(heavy + at / n_groups) : static_cast<int>(at / n_groups);
+    const int2 rng = __ldg(tile_rng + tile);
+    if (!first && rng.y - rng.x >= kHeavy) {           // done among the first
+      item = __shfl_sync(full, after, 0);
+      continue;
+    }
     const PrepRec* pg = prep + static_cast<long long>(g) * n_cross * kLanes + lane;
     const int tv = tile / NTU, tu = tile - tv * NTU;
     const int r0 = G / 2 + tv * kTileV, c0 = tu * kTileU;
-    const int2 rng = __ldg(tile_rng + tile);
     unsigned long long acc[kTileV][kTileU];            // (re, im)
 #pragma unroll
     for (int i = 0; i < kTileV; ++i)
@@ -521,17 +533,13 @@ k_grid_tiles(const int4* __restrict__ tile_idx, const int2* __restrict__ tile_rn
     }
     // ---- the tile, with the centring sign (r0 and c0 are even)
     if (g * kLanes + lane < nb) {
-      constexpr int CH = row_chans(G);
-      const int cb = g * kLanes + lane;
-      float2* out = grid + ((static_cast<long long>(cb / CH) * (G / 2) + r0 - G / 2) * G + c0) * CH +
-                    (cb % CH) * kTileU;
+      float2* out = grid + ((static_cast<long long>(g) * (G / 2) + r0 - G / 2) * G + c0) * kLanes + lane * kTileU;
 #pragma unroll
-      for (int i = 0; i < kTileV; ++i)
-      {
+      for (int i = 0; i < kTileV; ++i) {
         unsigned long long z[kTileU];
 #pragma unroll
         for (int j = 0; j < kTileU; ++j) z[j] = (i + j) & 1 ? acc[i][j] ^ 0x8000000080000000ull : acc[i][j];
-        asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(out + i * G * CH), "l"(z[0]), "l"(z[1]),
+        asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(out + i * G * kLanes), "l"(z[0]), "l"(z[1]),
                      "l"(z[2]), "l"(z[3])
                      : "memory");
       }
@@ -590,8 +598,8 @@ __device__ __forceinline__ void store_band(const float2* band, int cb0, int row0
 // the lines come from and the last one hands its values to a functor instead
 // of another trip through shared memory.  Against the shared passes of
 // fft.cuh with staged input and output, 352 antennas: 1000 channels of 256^2
-// rows 0.60 -> 0.44 ms, columns 0.42 -> 0.32 ms; 300 of 512^2 0.72 -> 0.49 and
-// 0.54 -> 0.40 ms.
+// rows 0.60 -> 0.46 ms, columns 0.42 -> 0.31 ms; 300 of 512^2 0.72 -> 0.52 and
+// 0.54 -> 0.39 ms.
 __device__ __forceinline__ float2 add2(float2 a, float2 b) {
   float2 d;
   asm("{\n\t.reg .b64 p, q, r;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %5};\n\tadd.rn.f32x2 r, p, q;\n\t"
@@ -742,7 +750,7 @@ __device__ __forceinline__ void fft_lines(float2* a, int ldp, const float2* tw, 
 __host__ __device__ constexpr int last_radix(int g) { return g <= 256 ? g / 16 : g / 256; }
 
 // Row transforms of the gridded half planes: a CTA copies its channels' rows in
-// (64 KB, contiguous) and transforms them; the central N columns go to h
+// (64 KB) and transforms them; the central N columns go to h
 // ([batch][G/2][N], row j - G/2), straight from the last pass.  With 16-bit
 // storage the rows go through fft_rows_inplace_f instead: rounding to 16 bits
 // turns a last-bit difference of a row into one of 2^-9 or 2^-12, and images
@@ -757,12 +765,17 @@ k_fft_rows(const float2* __restrict__ grid, const float2* __restrict__ tw_g, int
   extern __shared__ __align__(16) unsigned char smem[];
   float2* band = reinterpret_cast<float2*>(smem);     // [row_lines][LDP]; first the input [R][G/4][CH][4]
   float2* tw = band + row_lines(G) * LDP;
-  const int cb0 = blockIdx.y * CH, row0 = blockIdx.x * R;
-  const float4* src = reinterpret_cast<const float4*>(
-      grid + (static_cast<long long>(blockIdx.y) * half_rows(G) + row0) * G * CH);
+  // the CTAs of one row's channels run next to one another: they share its lines
+  const int cb0 = blockIdx.x * CH, row0 = blockIdx.y * R;
+  const float4* src = reinterpret_cast<const float4*>(grid) +
+                      (static_cast<long long>(cb0 / kLanes) * half_rows(G) + row0) * (G / 4) * (2 * kLanes) +
+                      cb0 % kLanes * 2;
   float4 q[8];
 #pragma unroll
-  for (int u = 0; u < 8; ++u) q[u] = __ldg(src + threadIdx.x + u * blockDim.x);
+  for (int u = 0; u < 8; ++u) {
+    const int i = threadIdx.x + u * blockDim.x;       // ((row, col / 4), 16-byte piece)
+    q[u] = __ldg(src + i / (2 * CH) * (2 * kLanes) + i % (2 * CH));
+  }
   constexpr int TW0 = S == kStoreF32 ? 0 : tw_entries(G), TWN = S == kStoreF32 ? tw_entries(G) : G;
   for (int i = threadIdx.x; i < TWN; i += blockDim.x) tw[i] = __ldg(tw_g + TW0 + i);
 #pragma unroll
@@ -919,12 +932,11 @@ __global__ void k_counts_out(const int* __restrict__ kept, int n_chan, int32_t* 
 
 // ---------------------------------------------------------- per-call tables and lists
 // Everything one geometry and frequency axis needs is made on the device from
-// the antenna positions, the frequencies and the kernel table, in six
+// the antenna positions, the frequencies and the kernel table, in five
 // launches without a synchronisation.  Made by one host core (7169 N cosines
 // for the grid correction, a list push per tile and baseline) it took 13.5, 26
 // and 61 ms at 352 antennas and 256^2, 512^2 and 1024^2 images, five to twenty
-// times the gridding itself; whole calls now take 2.9 ms (1000 channels of
-// 256^2, 16.5 before), 3.1 ms (300 of 512^2, 29.7) and 3.4 ms (64 of 1024^2, 67).
+// times the gridding itself; these kernels take 0.10, 0.11 and 0.17 ms.
 
 // Half of the even kernel table, C(m / Q) for m = 0 .. S Q / 2, passed by
 // value: the tables are built from it without a copy through memory.
@@ -934,11 +946,12 @@ struct KernelHalf {
 
 // The tables: the first n/2 + 1 CTAs form the reciprocal grid correction
 // 1 / C^(d), C^(d) = (1/Q) sum_m C(m/Q) cos(2 pi m d / (Q G)), one |d| each
-// (the table is even, and so is C^; the phase m d is reduced in integers, so
-// the cosine's argument is exact); the others fill the gap-indexed weights,
-// the twiddles, the horizon mask and the channel scales, one element a thread.
-// The cosines bound it: 3585 FP64 cospi per CTA.
+// (the table is even, and so is C^; m = 64 a + b, and 57 + 64 cosines and sines,
+// their phases reduced in integers, give all 3585 by the angle sum: a cosine a
+// term took 166 us at 1024^2); the others fill the gap-indexed weights, the
+// twiddles, the horizon mask and the channel scales, one element a thread.
 constexpr int kTabThreads = 256;
+constexpr int kCorrB = 64, kCorrA = kHalfTab / kCorrB + 1;
 __global__ void __launch_bounds__(kTabThreads)
 k_img_tables(const __grid_constant__ KernelHalf kh, int n, int g, double cell, const double* __restrict__ freq,
              int n_chan, float* __restrict__ inv_corr, float* __restrict__ tabx, float2* __restrict__ tw,
@@ -946,12 +959,22 @@ k_img_tables(const __grid_constant__ KernelHalf kh, int n, int g, double cell, c
   const int n_corr = n / 2 + 1;
   if (static_cast<int>(blockIdx.x) < n_corr) {
     __shared__ double part[kTabThreads / 32];
+    __shared__ double2 ca[kCorrA], cb[kCorrB];         // (cos, sin) of the angles of kCorrB a and of b
     const int d = blockIdx.x;
     const int period = kQ * g;                         // a power of two, <= 2^21
+    if (threadIdx.x < kCorrA + kCorrB) {
+      const int i = threadIdx.x;
+      const long long m = i < kCorrA ? static_cast<long long>(kCorrB) * i : i - kCorrA;
+      const int r = static_cast<int>((m * d) & (period - 1));
+      double si, co;
+      sincospi(2.0 * static_cast<double>(r) / static_cast<double>(period), &si, &co);
+      (i < kCorrA ? ca[i] : cb[i - kCorrA]) = make_double2(co, si);
+    }
+    __syncthreads();
     double s = 0.0;
     for (int m = threadIdx.x; m <= kHalfTab; m += kTabThreads) {
-      const int r = static_cast<int>((static_cast<long long>(m) * d) & (period - 1));
-      const double t = kh.c[m] * cospi(2.0 * static_cast<double>(r) / static_cast<double>(period));
+      const double2 x = ca[m / kCorrB], y = cb[m % kCorrB];
+      const double t = kh.c[m] * (x.x * y.x - x.y * y.y);
       s += m ? 2.0 * t : t;
     }
 #pragma unroll
@@ -1209,89 +1232,80 @@ k_plan_rows(const PlanRange* __restrict__ lrng, int g, unsigned long long* __res
   }
 }
 
-// Per tile, its list in listed order: one warp per tile scans its row's entries
-// twice (count, then write to a range reserved by one atomic).  Ranges are
-// whole quads, the last one filled with entry 0.
-constexpr int kTileListWarps = 8;
+// Per tile, its list in listed order: one warp per kTilesPerWarp adjacent tiles
+// scans their row's entries twice (count, then write to a range reserved by one
+// atomic).  Ranges are whole quads, the last one filled with entry 0.  Tiles of
+// kHeavy entries and more are listed in heavy, in any order.
+constexpr int kTileListWarps = 8, kTilesPerWarp = 8;
+static_assert(32 / kTileU % kTilesPerWarp == 0, "a warp's tiles lie in one row of the smallest grid");
 __global__ void __launch_bounds__(kTileListWarps * 32)
 k_plan_tiles(const int2* __restrict__ row_ent, const int2* __restrict__ row_rng, int ntu, int nt,
              unsigned long long* __restrict__ counts, int* __restrict__ tile_idx, long long cap,
-             int2* __restrict__ tile_rng) {
+             int2* __restrict__ tile_rng, int* __restrict__ heavy) {
+  const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const int tile = blockIdx.x * kTileListWarps + (threadIdx.x >> 5);
-  if (tile >= nt) return;
-  const int tv = tile / ntu, tu = tile - tv * ntu;
+  const int tile0 = (blockIdx.x * kTileListWarps + (threadIdx.x >> 5)) * kTilesPerWarp;
+  if (tile0 >= nt) return;
+  const int tv = tile0 / ntu, tu0 = tile0 - tv * ntu;
   const int2 rr = row_rng[tv];
-  auto hit = [&](int i, int& ent) {
-    if (i >= rr.y) return false;
-    const int2 e = __ldg(row_ent + i);
+  // columns of entry i, relative to the warp's first tile (none: an empty range)
+  auto range = [&](int i, int& ent, int& lo, int& hi) {
+    int2 e = make_int2(0, 0);
+    const bool in = i < rr.y;
+    if (in) e = __ldg(row_ent + i);
     ent = e.x;
-    return tu >= (e.y & 0xffff) && tu <= (e.y >> 16);
+    lo = (e.y & 0xffff) - tu0;
+    hi = in ? (e.y >> 16) - tu0 : -1;
   };
-  int c = 0;
-#pragma unroll 4
-  for (int i = rr.x; i < rr.y; i += 32) {
-    int ent;
-    c += hit(i + lane, ent) ? 1 : 0;
-  }
+  int c[kTilesPerWarp];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  int start = 0;
-  if (lane == 0) {
-    const unsigned long long pad = static_cast<unsigned long long>((c + 3) & ~3);
-    if (c) atomicAdd(counts + kCountTiles, static_cast<unsigned long long>(c));
-    const unsigned long long s = c ? atomicAdd(counts + kCountSlots, pad) : 0ull;
-    start = s + pad <= static_cast<unsigned long long>(cap) ? static_cast<int>(s) : -1;
-    tile_rng[tile] = start < 0 ? make_int2(0, 0) : make_int2(start, start + c);
-  }
-  start = __shfl_sync(0xffffffffu, start, 0);
-  if (start < 0) return;
+  for (int u = 0; u < kTilesPerWarp; ++u) c[u] = 0;
 #pragma unroll 2
   for (int i = rr.x; i < rr.y; i += 32) {
-    int ent = 0;
-    const bool h = hit(i + lane, ent);
-    const unsigned m = __ballot_sync(0xffffffffu, h);
-    if (h) tile_idx[start + __popc(m & ((1u << lane) - 1u))] = ent;
-    start += __popc(m);
-  }
-  if (lane < (4 - (c & 3)) % 4) tile_idx[start + lane] = 0;
-}
-
-// The tiles from the longest list to the shortest (lists of kOrderBins and
-// more together): a counting sort by one CTA.  The order only decides which
-// warp takes a tile when.
-constexpr int kOrderBins = 2048;
-__global__ void __launch_bounds__(1024)
-k_plan_order(const int2* __restrict__ tile_rng, int nt, int* __restrict__ order) {
-  __shared__ int bin[kOrderBins];
-  __shared__ int wtot[32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int i = threadIdx.x; i < kOrderBins; i += 1024) bin[i] = 0;
-  __syncthreads();
-  auto cls = [&](int t) {
-    const int2 r = __ldg(tile_rng + t);
-    return kOrderBins - 1 - min(r.y - r.x, kOrderBins - 1);
-  };
-#pragma unroll 4
-  for (int t = threadIdx.x; t < nt; t += 1024) atomicAdd(&bin[cls(t)], 1);
-  __syncthreads();
-  // exclusive scan, kOrderBins / 1024 bins per thread
-  const int b0 = bin[2 * threadIdx.x], b1 = bin[2 * threadIdx.x + 1];
-  int v = b0 + b1;
+    int ent, lo, hi;
+    range(i + lane, ent, lo, hi);
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(0xffffffffu, v, o);
-    if (lane >= o) v += t;
+    for (int u = 0; u < kTilesPerWarp; ++u) c[u] += __popc(__ballot_sync(full, u >= lo && u <= hi));
   }
-  if (lane == 31) wtot[warp] = v;
-  __syncthreads();
-  int run = v - b0 - b1;
-  for (int w = 0; w < warp; ++w) run += wtot[w];
-  bin[2 * threadIdx.x] = run;
-  bin[2 * threadIdx.x + 1] = run + b0;
-  __syncthreads();
-#pragma unroll 4
-  for (int t = threadIdx.x; t < nt; t += 1024) order[atomicAdd(&bin[cls(t)], 1)] = t;
+  int start[kTilesPerWarp], slots = 0, entries = 0;
+#pragma unroll
+  for (int u = 0; u < kTilesPerWarp; ++u) {
+    start[u] = slots;
+    slots += (c[u] + 3) & ~3;
+    entries += c[u];
+  }
+  int base = 0;
+  if (lane == 0 && entries) {
+    atomicAdd(counts + kCountTiles, static_cast<unsigned long long>(entries));
+    const unsigned long long s = atomicAdd(counts + kCountSlots, static_cast<unsigned long long>(slots));
+    base = s + slots <= static_cast<unsigned long long>(cap) ? static_cast<int>(s) : -1;
+  }
+  base = __shfl_sync(full, base, 0);
+#pragma unroll
+  for (int u = 0; u < kTilesPerWarp; ++u) {
+    start[u] += base;
+    if (lane == u) {
+      const int n = base < 0 ? 0 : c[u];
+      tile_rng[tile0 + u] = make_int2(start[u], start[u] + n);
+      if (n >= kHeavy) heavy[atomicAdd(counts + kCountHeavy, 1ull)] = tile0 + u;
+    }
+  }
+  if (base < 0) return;
+#pragma unroll 1
+  for (int i = rr.x; i < rr.y; i += 32) {
+    int ent, lo, hi;
+    range(i + lane, ent, lo, hi);
+#pragma unroll
+    for (int u = 0; u < kTilesPerWarp; ++u) {
+      const bool h = u >= lo && u <= hi;
+      const unsigned m = __ballot_sync(full, h);
+      if (h) tile_idx[start[u] + __popc(m & ((1u << lane) - 1u))] = ent;
+      start[u] += __popc(m);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < kTilesPerWarp; ++u)
+    if (lane < (4 - (c[u] & 3)) % 4) tile_idx[start[u] + lane] = 0;
 }
 
 // ---------------------------------------------------------------- planning
@@ -1343,12 +1357,12 @@ struct ImgWs {
   int2* row_ent;     // per tile row: (listed index | kMirror, first | last << 16 tile column)
   int2* row_rng;     // [tile rows] their ranges in row_ent
   int2* tile_rng;    // [n_tiles] ranges in tile_idx
-  int* tile_order;   // [n_tiles] tiles by descending list length
+  int* heavy;        // [n_tiles] tiles of kHeavy entries and more
   int* tile_idx;     // per tile: indices into listed | kMirror
   unsigned long long* counts;   // [kCounts]
   double* blen;      // [n_cross] baseline lengths (metres)
   PrepRec* prep;     // [batch groups][n_cross][32] prepared records (the listed ones first)
-  float2* grid;      // [batch / row_chans][G/2][G/4][row_chans][4] gridded half planes
+  float2* grid;      // [batch groups][G/2][G/4][32][4] gridded half planes
   void* h;           // [batch][G][N] complex in the storage format
   float* hs;         // [batch][G] row scales (FP16 storage)
   bool bases = false;  // records carry weight-table offsets (footprints move < kTabMargin cells)
@@ -1383,7 +1397,7 @@ ImgWs carve_img(void* ws, size_t bytes, const ImgPlan& p, int n_ant, int n_chan,
   w.row_ent = c.take<int2>(entry_capacity(p));
   w.row_rng = c.take<int2>(half_rows(p.g) / kTileV);
   w.tile_rng = c.take<int2>(n_tiles(p.g));
-  w.tile_order = c.take<int>(n_tiles(p.g));
+  w.heavy = c.take<int>(n_tiles(p.g));
   w.tile_idx = c.take<int>(slot_capacity(p));
   w.counts = c.take<unsigned long long>(kCounts);
   w.blen = c.take<double>(nx);
@@ -1420,15 +1434,15 @@ int launch_batch(const ImgPlan& p, const ImgWs& w, const GridOpts& o, const int3
     const long long ctas = std::min<long long>(num_sms(), (items + kGridWarps - 1) / kGridWarps);
     OVRO_PROF("k_grid_tiles", st);
     tiles<<<static_cast<unsigned>(ctas), kGridWarps * 32, kTileSmem, st>>>(
-        reinterpret_cast<const int4*>(w.tile_idx), w.tile_rng, w.tile_order, w.prep, p.n_cross, w.tabx, nb, next_item,
-        w.grid);
+        reinterpret_cast<const int4*>(w.tile_idx), w.tile_rng, w.heavy, w.counts, w.prep, p.n_cross, w.tabx, nb,
+        next_item, w.grid);
     OVRO_LAUNCH_CHECK();
   }
   {
     const size_t sm = (static_cast<size_t>(row_lines(G)) * LDP + tw_entries(G)) * sizeof(float2);
     OVRO_CUDA_TRY(cudaFuncSetAttribute(k_fft_rows<L, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(sm)));
-    dim3 grid(half_rows(G) / row_rows(G), (nb + row_chans(G) - 1) / row_chans(G));
+    dim3 grid((nb + row_chans(G) - 1) / row_chans(G), half_rows(G) / row_rows(G));
     OVRO_PROF("k_fft_rows", st);
     k_fft_rows<L, S><<<grid, row_lines(G) * G / 16, sm, st>>>(w.grid, w.tw, nb, p.n, w.h, w.hs);
     OVRO_LAUNCH_CHECK();
@@ -1530,10 +1544,9 @@ int upload_common(const ImgPlan& p, ImgWs& w, int n_ant, const double* h_ant,
   }
   k_plan_rows<<<rows, kRowWarps * 32, 0, st>>>(w.lrng, p.g, w.counts, w.row_ent, entry_capacity(p), w.row_rng);
   OVRO_LAUNCH_CHECK();
-  k_plan_tiles<<<(nt + kTileListWarps - 1) / kTileListWarps, kTileListWarps * 32, 0, st>>>(
-      w.row_ent, w.row_rng, n_tiles_u(p.g), nt, w.counts, w.tile_idx, slot_capacity(p), w.tile_rng);
-  OVRO_LAUNCH_CHECK();
-  k_plan_order<<<1, 1024, 0, st>>>(w.tile_rng, nt, w.tile_order);
+  constexpr int per_cta = kTileListWarps * kTilesPerWarp;
+  k_plan_tiles<<<(nt + per_cta - 1) / per_cta, kTileListWarps * 32, 0, st>>>(
+      w.row_ent, w.row_rng, n_tiles_u(p.g), nt, w.counts, w.tile_idx, slot_capacity(p), w.tile_rng, w.heavy);
   OVRO_LAUNCH_CHECK();
   if (!(move <= 2.0)) {
     unsigned long long c[kCounts];
