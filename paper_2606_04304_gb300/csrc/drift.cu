@@ -8,13 +8,12 @@
 // SNR = sum / sqrt(T) and its drift, then thresholds and runs Stage I's
 // greedy non-maximum suppression with the drifting line's width |d| + 1.
 //
-//   k_drift      CTA = 32 in-horizon pixels x 32 start channels: stages
-//                z'_t over the channels the tile's paths touch (a halo of
-//                T - 1 on each side, zero outside the coarse channel) in
-//                shared memory with lanes on pixels, then sums every path
-//                directly (2T - 1 drifts x T rows per output)
-//   k_drift_nms  one warp per (pixel, coarse channel): ballot-gathers the
-//                channels at or above the threshold, greedy NMS by warp argmax
+//   k_drift      lanes on in-horizon pixels, a few start channels per thread:
+//                every path's sum in a register, rows added in order, paths
+//                that begin alike sharing their first rows
+//   k_drift_nms  one warp per (pixel, coarse channel) with a hit: ballot-gathers
+//                the channels at or above the threshold, greedy NMS by warp
+//                argmax
 //   k_slice      one sub-integration's block of int8 spectra, for the X-engine
 #include <algorithm>
 #include <cmath>
@@ -39,11 +38,18 @@ struct DriftCand {
   float snr, pad;
 };
 
-__global__ void k_fill_snr(float* __restrict__ snr, int8_t* __restrict__ dr, long long n) {
-  for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
-       i += static_cast<long long>(gridDim.x) * blockDim.x) {
-    snr[i] = -INFINITY;
-    dr[i] = 0;
+// The maps' values below the horizon (the same FP64 test as the pixel list's):
+// a thread takes one pixel of one channel row, lanes along the columns.
+__global__ void k_fill_below(int n, double cell, int n_chan, float* __restrict__ snr, int32_t* __restrict__ drift) {
+  const int px = blockIdx.x * blockDim.x + threadIdx.x;
+  if (px >= n * n) return;
+  const int r = px / n, c = px - r * n;
+  const double l = __dmul_rn(static_cast<double>(c - n / 2), cell), m = __dmul_rn(static_cast<double>(r - n / 2), cell);
+  if (__dadd_rn(__dmul_rn(l, l), __dmul_rn(m, m)) < 1.0) return;
+  for (int f = blockIdx.y; f < n_chan; f += gridDim.y) {
+    const long long i = static_cast<long long>(f) * n * n + px;
+    if (snr) snr[i] = -INFINITY;
+    if (drift) drift[i] = 0;
   }
 }
 
@@ -53,61 +59,123 @@ __global__ void k_fill_snr(float* __restrict__ snr, int8_t* __restrict__ dr, lon
 constexpr int kDriftHistShift = 16;
 constexpr int kDriftMaxBins = 2048;
 
-// shift table: st[d * T + t], d, t < T (Taylor paths).  With ghist, every
-// voxel's best SNR at or above the floor of bin 0 is counted in its bin
-// (values above the top bin in the top bin).
-__global__ void __launch_bounds__(32 * kDriftWarps)
-k_drift(const float* __restrict__ zp, int T, long long chan_stride, long long sub_stride,
-        const int* __restrict__ pix, int n_valid, const DriftChunk* __restrict__ chunks,
-        const int* __restrict__ shift_tab, float inv_sqrt_t, float* __restrict__ snr, int8_t* __restrict__ dr,
+// Channel offset at row t of the Taylor path of total drift d over N rows: every
+// halving of the rows adds the larger half of the drift to the second half.  (A
+// loop, so that it folds into the indices of unrolled code.)
+template <int N>
+__device__ __forceinline__ int taylor_shift(int d, int t) {
+  int s = 0;
+#pragma unroll
+  for (int h = N / 2; h >= 1; h /= 2) {
+    if (t >= h) {
+      s += d - d / 2;
+      t -= h;
+    }
+    d /= 2;
+  }
+  return s;
+}
+
+// Sums over the first N rows of the paths of signed drift -(N-1) .. N-1 (index
+// D + N - 1) for F start channels, from those over the first N / 2: a path of N
+// rows begins as the path of half its drift, and the rows are added one after
+// the other, so a sum is rounded as ((z_0 + z_1) + z_2) + ... whoever shares it.
+template <int N, int F, class Load>
+struct PathSums {
+  static __device__ __forceinline__ void run(const Load& load, float (&s)[2 * N - 1][F]) {
+    float half[N - 1][F];
+    PathSums<N / 2, F, Load>::run(load, half);
+#pragma unroll
+    for (int i = 0; i < 2 * N - 1; ++i) {
+      const int d = i - (N - 1), p = (d < 0 ? -(-d / 2) : d / 2) + N / 2 - 1;
+#pragma unroll
+      for (int f = 0; f < F; ++f) s[i][f] = half[p][f];
+    }
+#pragma unroll
+    for (int t = N / 2; t < N; ++t) {
+      // row t at the offsets -t .. F - 1 + t its paths can reach
+      float z[F + 2 * (N - 1)];
+#pragma unroll
+      for (int o = 0; o < F + 2 * t; ++o) z[o] = load(t, o - t);
+#pragma unroll
+      for (int i = 0; i < 2 * N - 1; ++i) {
+        const int d = i - (N - 1), o = d < 0 ? -taylor_shift<N>(-d, t) : taylor_shift<N>(d, t);
+#pragma unroll
+        for (int f = 0; f < F; ++f) s[i][f] += z[f + o + t];
+      }
+    }
+  }
+};
+template <int F, class Load>
+struct PathSums<1, F, Load> {
+  static __device__ __forceinline__ void run(const Load& load, float (&s)[1][F]) {
+#pragma unroll
+    for (int f = 0; f < F; ++f) s[0][f] = 0.0f + load(0, f);
+  }
+};
+
+// start channels a thread holds: (2T - 1) F sums in registers
+__host__ __device__ constexpr int drift_chans(int T) { return T == 16 ? 2 : 4; }
+
+// CTA = 32 in-horizon pixels (lanes) x kTileF start channels, a warp
+// drift_chans(T) of them at a time; neighbouring warps read the same rows, which
+// L1 holds.  Bound by the additions and the compares: 78 + 45 a voxel at T = 8,
+// with 22 loads.  (Every path summed from shared memory took a load per addition,
+// 120 a voxel: 2.76 ms for 1024 channels of 256^2 at T = 8, now 0.82 ms.)
+// snr, dr and, when given, drift are written for in-horizon pixels; flag marks
+// the (pixel, coarse) pairs with a value at or above cut.  With ghist, every
+// voxel's best SNR at or above the floor of bin 0 is counted in its bin (values
+// above the top bin in the top bin).
+template <int T>
+__global__ void __launch_bounds__(32 * kDriftWarps, 2)
+k_drift(const float* __restrict__ zp, long long chan_stride, long long sub_stride, const int* __restrict__ pix,
+        int n_valid, const DriftChunk* __restrict__ chunks, int n_coarse, float inv_sqrt_t, float cut,
+        float* __restrict__ snr, int8_t* __restrict__ dr, int32_t* __restrict__ drift, uint8_t* __restrict__ flag,
         uint32_t hist_key0, int n_bins, unsigned long long* __restrict__ ghist) {
-  extern __shared__ __align__(16) float tile[];      // [T][W][32]
-  __shared__ int st[kMaxSub * kMaxSub];
+  constexpr int F = drift_chans(T);
   __shared__ uint32_t shist[kDriftMaxBins];
-  if (ghist)
+  if (ghist) {
     for (int i = threadIdx.x; i < n_bins; i += blockDim.x) shist[i] = 0u;
+    __syncthreads();
+  }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const DriftChunk ck = chunks[blockIdx.y];
   const int p = blockIdx.x * 32 + lane;
-  const int W = kTileF + 2 * (T - 1);
-  const int base = ck.f0 - (T - 1);                  // channel of tile column 0
-  for (int i = threadIdx.x; i < T * T; i += blockDim.x) st[i] = shift_tab[i];
-  const long long px = p < n_valid ? pix[p] : 0;
-  for (int row = warp; row < T * W; row += kDriftWarps) {
-    const int t = row / W, j = row - t * W;
-    const int f = base + j;
-    float v = 0.0f;
-    if (p < n_valid && f >= ck.c_lo && f < ck.c_hi)
-      v = __ldg(zp + t * sub_stride + static_cast<long long>(f) * chan_stride + px);
-    tile[(t * W + j) * 32 + lane] = v;
-  }
-  __syncthreads();
-  for (int o = warp; o < kTileF && p < n_valid; o += kDriftWarps) {
-    const int f = ck.f0 + o;
-    if (f >= ck.c_hi) break;
-    const int j0 = o + (T - 1);
-    float best = -INFINITY;
-    int bd = 0;
-    for (int d = 0; d < T; ++d) {
-      for (int sgn = 1; sgn >= -1; sgn -= 2) {
-        if (d == 0 && sgn < 0) continue;
-        const int end = f + sgn * d;
-        if (end < ck.c_lo || end >= ck.c_hi) continue;
-        float s = 0.0f;
-        for (int t = 0; t < T; ++t) s += tile[(t * W + j0 + sgn * st[d * T + t]) * 32 + lane];
-        s *= inv_sqrt_t;
-        if (s > best) {
-          best = s;
-          bd = sgn * d;
+  const long long px = pix[min(p, n_valid - 1)];
+  for (int f0 = ck.f0 + warp * F; f0 < min(ck.f0 + kTileF, ck.c_hi); f0 += kDriftWarps * F) {
+    // a path that ends inside the coarse channel stays inside it; what the
+    // others read does not matter
+    auto load = [&](int t, int o) {
+      const int f = min(max(f0 + o, ck.c_lo), ck.c_hi - 1);
+      return __ldg(zp + t * sub_stride + static_cast<long long>(f) * chan_stride + px);
+    };
+    float s[2 * T - 1][F];
+    PathSums<T, F, decltype(load)>::run(load, s);
+#pragma unroll
+    for (int j = 0; j < F; ++j) {
+      const int f = f0 + j;
+      float best = -INFINITY;
+      int bd = 0;
+#pragma unroll
+      for (int i = 0; i < 2 * T - 1; ++i) {
+        const int d = i & 1 ? (i + 1) / 2 : -(i / 2);    // 0, +1, -1, +2, ...
+        const float v = s[d + T - 1][j] * inv_sqrt_t;
+        if (f + d >= ck.c_lo && f + d < ck.c_hi && v > best) {
+          best = v;
+          bd = d;
         }
       }
-    }
-    const long long idx = static_cast<long long>(f) * chan_stride + px;
-    snr[idx] = best;
-    dr[idx] = static_cast<int8_t>(bd);
-    if (ghist) {
-      const uint32_t kb = f2key(best) >> kDriftHistShift;
-      if (kb >= hist_key0) atomicAdd(&shist[min(kb - hist_key0, static_cast<uint32_t>(n_bins - 1))], 1u);
+      if (p < n_valid && f < ck.c_hi) {
+        const long long idx = static_cast<long long>(f) * chan_stride + px;
+        snr[idx] = best;
+        dr[idx] = static_cast<int8_t>(bd);
+        if (drift) drift[idx] = bd;
+        if (best >= cut) flag[static_cast<long long>(p) * n_coarse + ck.coarse] = 1;
+        if (ghist) {
+          const uint32_t kb = f2key(best) >> kDriftHistShift;
+          if (kb >= hist_key0) atomicAdd(&shist[min(kb - hist_key0, static_cast<uint32_t>(n_bins - 1))], 1u);
+        }
+      }
     }
   }
   if (ghist) {
@@ -115,6 +183,22 @@ k_drift(const float* __restrict__ zp, int T, long long chan_stride, long long su
     for (int i = threadIdx.x; i < n_bins; i += blockDim.x)
       if (shist[i]) atomicAdd(ghist + i, static_cast<unsigned long long>(shist[i]));
   }
+}
+
+// Marks the (pixel, coarse) pairs with a value at or above a cut that was not
+// known when the map was made.
+__global__ void k_drift_flag(const float* __restrict__ snr, long long chan_stride, const int* __restrict__ pix,
+                             int n_valid, const DriftChunk* __restrict__ chunks, int n_coarse, float cut,
+                             uint8_t* __restrict__ flag) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= n_valid) return;
+  const DriftChunk ck = chunks[blockIdx.y];
+  const long long px = pix[p];
+  const int f1 = min(ck.f0 + kTileF, ck.c_hi);
+  bool hit = false;
+#pragma unroll 8
+  for (int f = ck.f0; f < f1; ++f) hit |= snr[static_cast<long long>(f) * chan_stride + px] >= cut;
+  if (hit) flag[static_cast<long long>(p) * n_coarse + ck.coarse] = 1;
 }
 
 // Values of histogram bin b of the in-horizon map (the top bin takes every
@@ -135,17 +219,20 @@ __global__ void k_drift_gather(const float* __restrict__ snr, long long chan_str
   }
 }
 
-// One warp per (pixel, coarse) pair q = p * n_coarse + c.
+// One warp per (pixel, coarse) pair q = p * n_coarse + c with a hit (lanes along
+// the channels read a line each, so the pairs without one are left out: 0.20 ms
+// for every pair of 1024 channels of 256^2).
 __global__ void __launch_bounds__(32 * kDriftWarps)
 k_drift_nms(const float* __restrict__ snr, const int8_t* __restrict__ dr, long long chan_stride,
             const int* __restrict__ pix, int n_valid, const int* __restrict__ c_lo, const int* __restrict__ c_hi,
-            int n_coarse, float cut, DriftCand* __restrict__ out, int out_cap, int* __restrict__ counters) {
+            int n_coarse, float cut, const uint8_t* __restrict__ flag, DriftCand* __restrict__ out, int out_cap,
+            int* __restrict__ counters) {
   __shared__ int lf[kDriftWarps][kNmsCapD];
   __shared__ float lv[kDriftWarps][kNmsCapD];
   __shared__ uint8_t ls[kDriftWarps][kNmsCapD];     // 0 undecided, 1 accepted, 2 suppressed
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long q = static_cast<long long>(blockIdx.x) * kDriftWarps + warp;
-  if (q >= static_cast<long long>(n_valid) * n_coarse) return;
+  if (q >= static_cast<long long>(n_valid) * n_coarse || !flag[q]) return;
   const int p = static_cast<int>(q / n_coarse), c = static_cast<int>(q % n_coarse);
   const long long px = pix[p];
   int n = 0;
@@ -209,12 +296,6 @@ k_drift_nms(const float* __restrict__ snr, const int8_t* __restrict__ dr, long l
   }
 }
 
-__global__ void k_widen(const int8_t* __restrict__ a, long long n, int32_t* __restrict__ b) {
-  for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < n;
-       i += static_cast<long long>(gridDim.x) * blockDim.x)
-    b[i] = a[i];
-}
-
 __global__ void k_slice(const int8_t* __restrict__ q, long long n_chan, long long n_spec, long long row_bytes,
                         int s0, int count, int8_t* __restrict__ out, bool vec) {
   // out[c][s][:] = q[c][s0 + s][:], row_bytes per spectrum; vec: 16-byte rows and pointers
@@ -232,13 +313,6 @@ __global__ void k_slice(const int8_t* __restrict__ q, long long n_chan, long lon
   }
 }
 
-int taylor_shift(int d, int n, int t) {
-  if (n == 1) return 0;
-  const int h = n / 2;
-  if (t < h) return taylor_shift(d / 2, h, t);
-  return (d - d / 2) + taylor_shift(d / 2, h, t - h);
-}
-
 // log10 of the one-sided Gaussian tail Q(x), FP64 (erfc below 30, the
 // asymptotic series above, where erfc underflows toward denormals).
 double log10_q(double x) {
@@ -254,12 +328,12 @@ struct DriftWs {
   unsigned long long* hist;
   float* vals;
   int* pix;
-  int* shift;
   DriftChunk* chunks;
   int* c_lo;
   int* c_hi;
   float* snr;
   int8_t* dr;
+  uint8_t* flag;     // [pixel][coarse] 1: a value at or above the cut
   DriftCand* cands;
   int* counters;
 };
@@ -274,12 +348,12 @@ DriftWs carve_drift(void* ws, size_t bytes, int n_chan, int image_size, int n_co
   w.hist = c.take<unsigned long long>(kDriftMaxBins);
   w.vals = c.take<float>(kDriftGatherCap);
   w.pix = c.take<int>(npix);
-  w.shift = c.take<int>(kMaxSub * kMaxSub);
   w.chunks = c.take<DriftChunk>(std::max<long long>(n_chunks, 1));
   w.c_lo = c.take<int>(n_coarse);
   w.c_hi = c.take<int>(n_coarse);
   w.snr = c.take<float>(static_cast<size_t>(n_chan) * npix);
   w.dr = c.take<int8_t>(static_cast<size_t>(n_chan) * npix);
+  w.flag = c.take<uint8_t>(static_cast<size_t>(n_coarse) * npix);
   w.cands = c.take<DriftCand>(kDriftCandCap);
   w.counters = c.take<int>(4);
   *need = c.used;
@@ -343,9 +417,6 @@ int ovro_drift_search(const float* d_zp, int n_sub, int n_chan, int image_size, 
   std::vector<DriftChunk> chunks;
   for (int c = 0; c < n_coarse; ++c)
     for (int f0 = lo[c]; f0 < hi[c]; f0 += kTileF) chunks.push_back(DriftChunk{lo[c], hi[c], f0, c});
-  std::vector<int> tab(kMaxSub * kMaxSub, 0);
-  for (int d = 0; d < n_sub; ++d)
-    for (int t = 0; t < n_sub; ++t) tab[d * n_sub + t] = taylor_shift(d, n_sub, t);
   size_t need = 0;
   DriftWs w = carve_drift(d_ws, ws_bytes, n_chan, n, n_coarse, static_cast<long long>(chunks.size()), &need);
   if (int e = check_workspace(d_ws, ws_bytes, need)) return e;
@@ -354,24 +425,30 @@ int ovro_drift_search(const float* d_zp, int n_sub, int n_chan, int image_size, 
   const long long npix = static_cast<long long>(n) * n;
   const long long nvox = npix * n_chan;
   OVRO_CUDA_TRY(cudaMemcpyAsync(w.pix, pix.data(), pix.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-  OVRO_CUDA_TRY(cudaMemcpyAsync(w.shift, tab.data(), tab.size() * sizeof(int), cudaMemcpyHostToDevice, st));
   OVRO_CUDA_TRY(cudaMemcpyAsync(w.chunks, chunks.data(), chunks.size() * sizeof(DriftChunk),
                                 cudaMemcpyHostToDevice, st));
   OVRO_CUDA_TRY(cudaMemcpyAsync(w.c_lo, lo.data(), lo.size() * sizeof(int), cudaMemcpyHostToDevice, st));
   OVRO_CUDA_TRY(cudaMemcpyAsync(w.c_hi, hi.data(), hi.size() * sizeof(int), cudaMemcpyHostToDevice, st));
   OVRO_CUDA_TRY(cudaMemsetAsync(w.counters, 0, 4 * sizeof(int), st));
   if (bh) OVRO_CUDA_TRY(cudaMemsetAsync(w.hist, 0, kDriftMaxBins * sizeof(unsigned long long), st));
-  k_fill_snr<<<4 * num_sms(), 256, 0, st>>>(w.snr, w.dr, nvox);
-  OVRO_LAUNCH_CHECK();
+  // the caller's map, when there is one, is the map the search works on
+  float* snr = d_snr_or_null ? d_snr_or_null : w.snr;
+  if (d_snr_or_null || d_drift_or_null) {
+    k_fill_below<<<dim3(static_cast<unsigned>((npix + 255) / 256), static_cast<unsigned>(std::min(n_chan, 64))), 256, 0,
+                   st>>>(n, cell_dircos, n_chan, d_snr_or_null, d_drift_or_null);
+    OVRO_LAUNCH_CHECK();
+  }
   if (n_valid > 0) {
-    const size_t sm = static_cast<size_t>(n_sub) * (kTileF + 2 * (n_sub - 1)) * 32 * sizeof(float);
-    OVRO_CUDA_TRY(cudaFuncSetAttribute(k_drift, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm)));
+    OVRO_CUDA_TRY(cudaMemsetAsync(w.flag, 0, static_cast<size_t>(n_valid) * n_coarse, st));
     dim3 grid((n_valid + 31) / 32, static_cast<unsigned>(chunks.size()));
     {
       OVRO_PROF("k_drift", st);
-      k_drift<<<grid, 32 * kDriftWarps, sm, st>>>(d_zp, n_sub, npix, nvox, w.pix, n_valid, w.chunks, w.shift,
-                                                   static_cast<float>(1.0 / std::sqrt(static_cast<double>(n_sub))),
-                                                   w.snr, w.dr, key0, nb, bh ? w.hist : nullptr);
+      auto kernel = n_sub == 2 ? k_drift<2> : n_sub == 4 ? k_drift<4> : n_sub == 8 ? k_drift<8> : k_drift<16>;
+      kernel<<<grid, 32 * kDriftWarps, 0, st>>>(
+          d_zp, npix, nvox, w.pix, n_valid, w.chunks, n_coarse,
+          static_cast<float>(1.0 / std::sqrt(static_cast<double>(n_sub))),
+          bh ? INFINITY : static_cast<float>(params->nsigma), snr, w.dr, d_drift_or_null, w.flag, key0, nb,
+          bh ? w.hist : nullptr);
       OVRO_LAUNCH_CHECK();
     }
     // the cut: the fixed threshold, or Benjamini-Hochberg over every
@@ -396,7 +473,7 @@ int ovro_drift_search(const float* d_zp, int n_sub, int n_chan, int image_size, 
         }
         if (hist[b] > static_cast<unsigned long long>(kDriftGatherCap)) return OVRO_ERR_CAPACITY;
         OVRO_CUDA_TRY(cudaMemsetAsync(w.counters + 2, 0, sizeof(int), st));
-        k_drift_gather<<<4 * num_sms(), 256, 0, st>>>(w.snr, npix, w.pix, n_valid, n_chan, key0 + b, b == nb - 1,
+        k_drift_gather<<<4 * num_sms(), 256, 0, st>>>(snr, npix, w.pix, n_valid, n_chan, key0 + b, b == nb - 1,
                                                      w.vals, kDriftGatherCap, w.counters + 2);
         OVRO_LAUNCH_CHECK();
         int nv = 0;
@@ -411,19 +488,15 @@ int ovro_drift_search(const float* d_zp, int n_sub, int n_chan, int image_size, 
       }
       if (!found) cut = INFINITY;                     // nothing is rejected
       OVRO_CUDA_TRY(cudaMemsetAsync(w.counters + 2, 0, sizeof(int), st));
+      k_drift_flag<<<dim3((n_valid + 255) / 256, static_cast<unsigned>(chunks.size())), 256, 0, st>>>(
+          snr, npix, w.pix, n_valid, w.chunks, n_coarse, cut, w.flag);
+      OVRO_LAUNCH_CHECK();
     }
     const long long pairs = static_cast<long long>(n_valid) * n_coarse;
     const long long blocks = (pairs + kDriftWarps - 1) / kDriftWarps;
     if (blocks > 0x7fffffffLL) return OVRO_ERR_UNSUPPORTED;
     k_drift_nms<<<static_cast<unsigned>(blocks), 32 * kDriftWarps, 0, st>>>(
-        w.snr, w.dr, npix, w.pix, n_valid, w.c_lo, w.c_hi, n_coarse, cut, w.cands, kDriftCandCap, w.counters);
-    OVRO_LAUNCH_CHECK();
-  }
-  // optional maps for the caller
-  if (d_snr_or_null)
-    OVRO_CUDA_TRY(cudaMemcpyAsync(d_snr_or_null, w.snr, nvox * sizeof(float), cudaMemcpyDeviceToDevice, st));
-  if (d_drift_or_null) {
-    k_widen<<<4 * num_sms(), 256, 0, st>>>(w.dr, nvox, d_drift_or_null);
+        snr, w.dr, npix, w.pix, n_valid, w.c_lo, w.c_hi, n_coarse, cut, w.flag, w.cands, kDriftCandCap, w.counters);
     OVRO_LAUNCH_CHECK();
   }
   int cnt[2] = {0, 0};
