@@ -3,8 +3,13 @@
 // with GELU hidden units scores 64-channel x 5 x 5-pixel cutouts of the
 // high-passed standardised cube around a trigger.  Weights are served in BF16
 // and every product is accumulated in FP32; training keeps FP32 master weights
-// and Adam moments.  All kernels are plain SIMT: the contractions are small
-// (a few hundred MFLOP per step) and memory/latency-bound at these sizes.
+// and Adam moments.  The inputs are FP32, so the contractions stay on the FP32
+// pipe (packed multiply-adds).  They are small (a few hundred MFLOP per step)
+// and a step is bound by launches and latency: the forward pass is two kernels
+// and the gradient a third, with the long sums (1600 inputs, the batch) split
+// over CTAs and thread groups so that a batch of 256 fills the chip.  Before, in
+// 12 launches of 32 x 32 tiles -> now, gradient and Adam step of 256 samples:
+// 197 -> 36 us (layer 1 forward 101 -> 7 us, weight gradients 47 -> 8 us).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -59,151 +64,310 @@ __global__ void k_cutouts(const float* __restrict__ zp, int n_chan, int n, const
 }
 
 // ------------------------------------------------------------ dense layers
-constexpr int kT = 32;
+// acc + (w, w) . (a, b) packed
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ unsigned long long dup2(float x) {
+  unsigned long long d;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
+  return d;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  float2 z;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(z.x), "=f"(z.y) : "l"(v));
+  return z;
+}
 
-// y[b][o] = act(sum_i x[b][i] w[o][i] + bias[o]); z (optional) keeps the pre-activation
+// Layer 1's products: part[split][b][o] = sum over the split's inputs of
+// x[b][i] w[o][i], 64 samples x all 128 outputs per CTA, 32 inputs staged at a
+// time (the next ones already in registers), 4 samples x 8 outputs per thread.
+// A batch of few tiles is split along the inputs until the CTAs fill the chip
+// (fwd_splits): 256 samples take 100 CTAs of two 32-input steps, where 32 CTAs
+// walked all 50 steps before.  x16, w16: the buffers start on 16 bytes (their
+// rows are multiples of 16).
+constexpr int kFB = 64, kFK = 32;
 template <bool BF16>
 __global__ void __launch_bounds__(256)
-k_dense_fwd(const float* __restrict__ x, const void* __restrict__ w, int w_off, int b_off, int B, int in, int out,
-            bool act, float* __restrict__ z, float* __restrict__ y) {
-  __shared__ float xs[kT][kT + 1];
-  __shared__ float ws[kT][kT + 1];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;       // 32 x 8
-  const int b0 = blockIdx.y * kT, o0 = blockIdx.x * kT;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int k0 = 0; k0 < in; k0 += kT) {
-    for (int r = ty; r < kT; r += 8) {
-      const int b = b0 + r, k = k0 + tx;
-      xs[r][tx] = (b < B && k < in) ? x[static_cast<long long>(b) * in + k] : 0.f;
-      const int o = o0 + r;
-      ws[r][tx] = (o < out && k < in) ? ldw<BF16>(w, w_off + static_cast<long long>(o) * in + k) : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int k = 0; k < kT; ++k) {
-      const float wv = ws[tx][k];
+k_dense_fwd(const float* __restrict__ x, const void* __restrict__ w, int B, int steps, bool x16, bool w16,
+            float* __restrict__ part) {
+  __shared__ __align__(16) float xs[kFK][kFB];
+  __shared__ __align__(16) float ws[kFK][kH1];
+  const int t = threadIdx.x;
+  const int b0 = blockIdx.x * kFB;
+  const int k0 = blockIdx.y * steps * kFK, k1 = min(kIn, k0 + steps * kFK);
+  // loads: 8 inputs of a sample, 16 weights of an output per thread
+  const int lb = t & 63, lk = (t >> 6) * 8, lo = t & 127, lw = (t >> 7) * 16;
+  const float* xp = x + static_cast<long long>(min(b0 + lb, B - 1)) * kIn + lk;
+  float xq[8], wq[16];
+  auto fetch = [&](int k) {
+    const long long o = kW1 + static_cast<long long>(lo) * kIn + k + lw;
+    if (x16) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc[q] = fmaf(xs[ty + 8 * q][k], wv, acc[q]);
+      for (int u = 0; u < 2; ++u) {
+        const float4 v = __ldg(reinterpret_cast<const float4*>(xp + k) + u);
+        xq[4 * u] = v.x; xq[4 * u + 1] = v.y; xq[4 * u + 2] = v.z; xq[4 * u + 3] = v.w;
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) xq[u] = __ldg(xp + k + u);
     }
+    if (!w16) {
+#pragma unroll
+      for (int u = 0; u < 16; ++u) wq[u] = ldw<BF16>(w, o + u);
+    } else if constexpr (BF16) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(w) + o) + u);
+        const uint32_t r[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {                     // a bf16 is the upper half of its float
+          wq[8 * u + 2 * q] = __uint_as_float(r[q] << 16);
+          wq[8 * u + 2 * q + 1] = __uint_as_float(r[q] & 0xffff0000u);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float4 v = __ldg(reinterpret_cast<const float4*>(static_cast<const float*>(w) + o) + u);
+        wq[4 * u] = v.x; wq[4 * u + 1] = v.y; wq[4 * u + 2] = v.z; wq[4 * u + 3] = v.w;
+      }
+    }
+  };
+  const int tb = (t >> 4) * 4, to = (t & 15) * 4;           // outputs to .. to + 3 and to + 64 ..
+  unsigned long long acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+  fetch(k0);
+  for (int k = k0; k < k1; k += kFK) {
     __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 8; ++u) xs[lk + u][lb] = xq[u];
+#pragma unroll
+    for (int u = 0; u < 16; ++u) ws[lw + u][lo] = wq[u];
+    __syncthreads();
+    if (k + kFK < k1) fetch(k + kFK);
+#pragma unroll 8
+    for (int i = 0; i < kFK; ++i) {
+      const float4 xv = *reinterpret_cast<const float4*>(&xs[i][tb]);
+      const ulonglong2 wa = *reinterpret_cast<const ulonglong2*>(&ws[i][to]);
+      const ulonglong2 wb = *reinterpret_cast<const ulonglong2*>(&ws[i][to + 64]);
+      const float xr[4] = {xv.x, xv.y, xv.z, xv.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const unsigned long long d = dup2(xr[q]);
+        acc[q][0] = fma2(d, wa.x, acc[q][0]);
+        acc[q][1] = fma2(d, wa.y, acc[q][1]);
+        acc[q][2] = fma2(d, wb.x, acc[q][2]);
+        acc[q][3] = fma2(d, wb.y, acc[q][3]);
+      }
+    }
   }
-  const int o = o0 + tx;
-  if (o >= out) return;
-  const float bias = ldw<BF16>(w, b_off + o);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const int b = b0 + ty + 8 * q;
+    const int b = b0 + tb + q;
     if (b >= B) continue;
-    const float v = acc[q] + bias;
-    if (z) z[static_cast<long long>(b) * out + o] = v;
-    y[static_cast<long long>(b) * out + o] = act ? gelu(v) : v;
+    float* o = part + (static_cast<long long>(blockIdx.y) * B + b) * kH1;
+    const float2 z0 = unpack2(acc[q][0]), z1 = unpack2(acc[q][1]), z2 = unpack2(acc[q][2]), z3 = unpack2(acc[q][3]);
+    *reinterpret_cast<float4*>(o + to) = make_float4(z0.x, z0.y, z1.x, z1.y);
+    *reinterpret_cast<float4*>(o + to + 64) = make_float4(z2.x, z2.y, z3.x, z3.y);
   }
 }
 
-// dx[b][i] = (sum_o dz[b][o] w[o][i]) * gelu'(zprev[b][i])
+// The rest of the network for kMB samples per CTA: layer 1's sums, bias and
+// GELU, layers 2 and 3; with targets also the loss of each sample and the
+// gradients with respect to the logits (d3) and the pre-activations (d2, d1),
+// dL/dlogit = (sigma(z) - y) / B.
+constexpr int kMB = 4;
 template <bool BF16>
 __global__ void __launch_bounds__(256)
-k_dense_bwd_x(const float* __restrict__ dz, const void* __restrict__ w, int w_off, int B, int in, int out,
-              const float* __restrict__ zprev, float* __restrict__ dx) {
-  __shared__ float ds[kT][kT + 1];
-  __shared__ float ws[kT][kT + 1];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int b0 = blockIdx.y * kT, i0 = blockIdx.x * kT;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int o0 = 0; o0 < out; o0 += kT) {
-    for (int r = ty; r < kT; r += 8) {
-      const int b = b0 + r, o = o0 + tx;
-      ds[r][tx] = (b < B && o < out) ? dz[static_cast<long long>(b) * out + o] : 0.f;
-      const int oo = o0 + r, i = i0 + tx;
-      ws[r][tx] = (oo < out && i < in) ? ldw<BF16>(w, w_off + static_cast<long long>(oo) * in + i) : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int o = 0; o < kT; ++o) {
-      const float wv = ws[o][tx];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[q] = fmaf(ds[ty + 8 * q][o], wv, acc[q]);
-    }
-    __syncthreads();
+k_dense_mid(const float* __restrict__ part, int n_split, const void* __restrict__ w, const float* __restrict__ y,
+            int B, float* __restrict__ logit, float* __restrict__ h1, float* __restrict__ h2, float* __restrict__ d1,
+            float* __restrict__ d2, float* __restrict__ d3, float* __restrict__ loss) {
+  __shared__ float w2[kH2][kH1 + 1];
+  __shared__ float z1s[kMB][kH1], h1s[kMB][kH1], z2s[kMB][kH2], d2s[kMB][kH2];
+  __shared__ float w3[kH2];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int b0 = blockIdx.x * kMB;
+  for (int i = t; i < kH2 * kH1; i += 256) w2[i / kH1][i % kH1] = ldw<BF16>(w, kW2 + i);
+  if (t < kH2) w3[t] = ldw<BF16>(w, kW3 + t);
+  for (int e = t; e < kMB * kH1; e += 256) {
+    const int q = e / kH1, o = e % kH1, b = min(b0 + q, B - 1);
+    float s = 0.f;
+#pragma unroll 5
+    for (int p = 0; p < n_split; ++p) s += __ldg(part + (static_cast<long long>(p) * B + b) * kH1 + o);
+    const float z = s + ldw<BF16>(w, kB1 + o), h = gelu(z);
+    z1s[q][o] = z;
+    h1s[q][o] = h;
+    if (h1 && b0 + q < B) h1[static_cast<long long>(b) * kH1 + o] = h;
   }
-  const int i = i0 + tx;
-  if (i >= in) return;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int b = b0 + ty + 8 * q;
-    if (b >= B) continue;
-    const long long e = static_cast<long long>(b) * in + i;
-    dx[e] = acc[q] * gelu_grad(zprev[e]);
-  }
-}
-
-// dw[o][i] = sum_b dz[b][o] x[b][i]
-__global__ void __launch_bounds__(256)
-k_dense_bwd_w(const float* __restrict__ dz, const float* __restrict__ x, int B, int in, int out,
-              float* __restrict__ dw) {
-  __shared__ float ds[kT][kT + 1];
-  __shared__ float xs[kT][kT + 1];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int o0 = blockIdx.y * kT, i0 = blockIdx.x * kT;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int b0 = 0; b0 < B; b0 += kT) {
-    for (int r = ty; r < kT; r += 8) {
-      const int b = b0 + r;
-      ds[r][tx] = (b < B && o0 + tx < out) ? dz[static_cast<long long>(b) * out + o0 + tx] : 0.f;
-      xs[r][tx] = (b < B && i0 + tx < in) ? x[static_cast<long long>(b) * in + i0 + tx] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int b = 0; b < kT; ++b) {
-      const float xv = xs[b][tx];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[q] = fmaf(ds[b][ty + 8 * q], xv, acc[q]);
-    }
-    __syncthreads();
-  }
-  const int i = i0 + tx;
-  if (i >= in) return;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int o = o0 + ty + 8 * q;
-    if (o < out) dw[static_cast<long long>(o) * in + i] = acc[q];
-  }
-}
-
-// db[o] = sum_b dz[b][o]  (one warp per output)
-__global__ void k_bias_grad(const float* __restrict__ dz, int B, int out, float* __restrict__ db) {
-  const int o = blockIdx.x;
-  float s = 0.f;
-  for (int b = threadIdx.x; b < B; b += blockDim.x) s += dz[static_cast<long long>(b) * out + o];
-  for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(0xffffffffu, s, d);
-  __shared__ float part[32];
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    s = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0.f;
-    for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(0xffffffffu, s, d);
-    if (threadIdx.x == 0) db[o] = s;
+  {
+    // two threads a sum: 4 samples x 32 outputs
+    const int q = t >> 6, o = (t >> 1) & 31, half = t & 1;
+    float s = 0.f;
+#pragma unroll 8
+    for (int k = 0; k < kH1 / 2; ++k) s = fmaf(h1s[q][2 * k + half], w2[o][2 * k + half], s);
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    if (half == 0) z2s[q][o] = s + ldw<BF16>(w, kB2 + o);
+  }
+  __syncthreads();
+  if (warp < kMB) {
+    const int q = warp, b = b0 + q;
+    const float z2 = z2s[q][lane], h = gelu(z2);
+    float s = h * w3[lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    const float z = s + ldw<BF16>(w, kB3);
+    if (lane == 0 && b < B && logit) logit[b] = z;
+    if (y) {
+      const float tgt = y[min(b, B - 1)];
+      const float g = (1.0f / (1.0f + expf(-z)) - tgt) / static_cast<float>(B);
+      const float v = g * w3[lane] * gelu_grad(z2);
+      d2s[q][lane] = v;
+      if (b < B) {
+        h2[static_cast<long long>(b) * kH2 + lane] = h;
+        d2[static_cast<long long>(b) * kH2 + lane] = v;
+        if (lane == 0) {
+          d3[b] = g;
+          loss[b] = fmaxf(z, 0.f) - tgt * z + log1pf(expf(-fabsf(z)));
+        }
+      }
+    }
+  }
+  if (!y) return;
+  __syncthreads();
+  for (int e = t; e < kMB * kH1; e += 256) {
+    const int q = e / kH1, k = e % kH1, b = b0 + q;
+    float s = 0.f;
+#pragma unroll 8
+    for (int o = 0; o < kH2; ++o) s = fmaf(d2s[q][o], w2[o][k], s);
+    if (b < B) d1[static_cast<long long>(b) * kH1 + k] = s * gelu_grad(z1s[q][k]);
   }
 }
 
-// mean BCE loss and dL/dlogit = (sigma(z) - y) / B; one block
-__global__ void k_bce(const float* __restrict__ z, const float* __restrict__ y, int B, float* __restrict__ dz,
-                      float* __restrict__ loss) {
-  float s = 0.f;
-  for (int b = threadIdx.x; b < B; b += blockDim.x) {
-    const float v = z[b], t = y[b];
-    s += fmaxf(v, 0.f) - t * v + log1pf(expf(-fabsf(v)));
-    dz[b] = (1.0f / (1.0f + expf(-v)) - t) / static_cast<float>(B);
+// All parameter gradients in one launch.  CTAs 0 .. kW1Tiles - 1: tiles of
+// dW1[o][i] = sum_b d1[b][o] x[b][i], 64 outputs x 32 inputs; then the tiles of
+// dW2 (d2, h1); then the sums over the batch that are single numbers (dW3,
+// biases, the mean loss), a warp each.  A tile's CTA has four groups of 128
+// threads, each taking every fourth 16 samples into sums of its own, which are
+// added in group order at the end.
+constexpr int kGO = 64, kGI = 32, kGB = 16, kGGroups = 4;
+constexpr int kW1Tiles = (kH1 / kGO) * (kIn / kGI), kW2Tiles = kH1 / kGI;
+constexpr int kSums = kH2 + kH1 + kH2 + 1 + 1;            // dW3, db1, db2, db3, loss
+constexpr int kSumCtas = (kSums + 15) / 16;
+__global__ void __launch_bounds__(128 * kGGroups)
+k_grads(const float* __restrict__ x, const float* __restrict__ h1, const float* __restrict__ h2,
+        const float* __restrict__ d1, const float* __restrict__ d2, const float* __restrict__ d3,
+        const float* __restrict__ loss, int B, bool x16, float* __restrict__ grad, float* __restrict__ loss_out) {
+  __shared__ __align__(16) float ds[kGGroups][kGB][kGO];
+  __shared__ __align__(16) float xs[kGGroups][kGB][kGI];
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (static_cast<int>(blockIdx.x) >= kW1Tiles + kW2Tiles) {
+    int o = (blockIdx.x - kW1Tiles - kW2Tiles) * 16 + (tid >> 5);
+    if (o >= kSums) return;
+    // the o-th sum: sum_b a[b sa] c[b sc]
+    const float *a, *c = nullptr;
+    int sa, sc = 0;
+    float* out;
+    if (o < kH2) { a = h2 + o; sa = kH2; c = d3; sc = 1; out = grad + kW3 + o; }
+    else if ((o -= kH2) < kH1) { a = d1 + o; sa = kH1; out = grad + kB1 + o; }
+    else if ((o -= kH1) < kH2) { a = d2 + o; sa = kH2; out = grad + kB2 + o; }
+    else if ((o -= kH2) < 1) { a = d3; sa = 1; out = grad + kB3; }
+    else { a = loss; sa = 1; out = loss_out; }
+    float s = 0.f;
+    for (int b = lane; b < B; b += 32) {
+      const float v = a[static_cast<long long>(b) * sa];
+      s = c ? fmaf(c[static_cast<long long>(b) * sc], v, s) : s + v;
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+    if (lane == 0 && out) *out = a == loss ? s / static_cast<float>(B) : s;
+    return;
   }
-  for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(0xffffffffu, s, d);
-  __shared__ float part[32];
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+  const bool second = static_cast<int>(blockIdx.x) >= kW1Tiles;
+  const int tile = second ? blockIdx.x - kW1Tiles : blockIdx.x;
+  const int in = second ? kH1 : kIn, out = second ? kH2 : kH1;
+  const float* dz = second ? d2 : d1;
+  const float* xv = second ? h1 : x;
+  float* dw = grad + (second ? kW2 : kW1);
+  const int i0 = tile % (in / kGI) * kGI, o0 = tile / (in / kGI) * kGO;
+  const int grp = tid >> 7, t = tid & 127;
+  const int to = (t >> 3) * 4, ti = (t & 7) * 4;              // 4 outputs x 4 inputs per thread
+  unsigned long long acc[4][2];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) acc[q][0] = acc[q][1] = 0ull;
+  const int lo = t & 63, lb = t >> 6, xi = (t & 7) * 4, xb = t >> 3;   // loads
+  // every group runs the same number of steps: the barriers are the CTA's
+  for (int s0 = 0; s0 < B; s0 += kGB * kGGroups) {
+    const int s = s0 + grp * kGB;
+    float dq[8];
+    float4 xq = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int b = s + lb + 2 * u;
+      dq[u] = b < B && o0 + lo < out ? __ldg(dz + static_cast<long long>(b) * out + o0 + lo) : 0.f;
+    }
+    if (s + xb < B) {
+      const float* xp = xv + static_cast<long long>(s + xb) * in + i0 + xi;
+      if (x16 || second) xq = __ldg(reinterpret_cast<const float4*>(xp));
+      else xq = make_float4(__ldg(xp), __ldg(xp + 1), __ldg(xp + 2), __ldg(xp + 3));
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 8; ++u) ds[grp][lb + 2 * u][lo] = dq[u];
+    *reinterpret_cast<float4*>(&xs[grp][xb][xi]) = xq;
+    __syncthreads();
+#pragma unroll
+    for (int b = 0; b < kGB; ++b) {
+      const float4 d = *reinterpret_cast<const float4*>(&ds[grp][b][to]);
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&xs[grp][b][ti]);
+      const float dr[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const unsigned long long dd = dup2(dr[q]);
+        acc[q][0] = fma2(dd, v.x, acc[q][0]);
+        acc[q][1] = fma2(dd, v.y, acc[q][1]);
+      }
+    }
+  }
+  // the groups' sums, through ds (64 x 32 a group fills two of its 16 x 64)
   __syncthreads();
-  if (threadIdx.x < 32) {
-    s = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0.f;
-    for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(0xffffffffu, s, d);
-    if (threadIdx.x == 0 && loss) *loss = s / static_cast<float>(B);
+  float* red = &ds[0][0][0];
+  for (int g = 1; g < kGGroups; ++g) {
+    if (grp == g)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float2 a = unpack2(acc[q][0]), c = unpack2(acc[q][1]);
+        *reinterpret_cast<float4*>(red + (to + q) * kGI + ti) = make_float4(a.x, a.y, c.x, c.y);
+      }
+    __syncthreads();
+    if (grp == 0)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 v = *reinterpret_cast<const float4*>(red + (to + q) * kGI + ti);
+        const float2 a = unpack2(acc[q][0]), c = unpack2(acc[q][1]);
+        const float2 p = make_float2(a.x + v.x, a.y + v.y), r = make_float2(c.x + v.z, c.y + v.w);
+        asm("mov.b64 %0, {%1, %2};" : "=l"(acc[q][0]) : "f"(p.x), "f"(p.y));
+        asm("mov.b64 %0, {%1, %2};" : "=l"(acc[q][1]) : "f"(r.x), "f"(r.y));
+      }
+    __syncthreads();
   }
+  if (grp == 0)
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (o0 + to + q < out) {
+        const float2 a = unpack2(acc[q][0]), c = unpack2(acc[q][1]);
+        float* p = dw + static_cast<long long>(o0 + to + q) * in + i0 + ti;
+        p[0] = a.x;                                         // (the caller's gradient may start anywhere)
+        p[1] = a.y;
+        p[2] = c.x;
+        p[3] = c.y;
+      }
 }
 
 // 1 - b is passed on its own (1 - 0.999f in FP32 is 1.3e-5 off) and the bias
@@ -229,36 +393,51 @@ __global__ void k_to_bf16(const float* __restrict__ w, int n, __nv_bfloat16* __r
 }
 
 struct ScorerWs {
-  float *z1, *h1, *z2, *h2, *z3, *d3, *d2, *d1, *loss;
+  float *part, *h1, *h2, *d3, *d2, *d1, *loss;
   int* chan0;
 };
+
+// Splits of layer 1's sum: CTAs for about every SM when the batch has few tiles
+// (at least two 32-input steps each), none beyond.
+constexpr int kFwdSteps = kIn / kFK;                        // 50
+int fwd_steps(int B) {
+  const int tiles = (B + kFB - 1) / kFB;
+  const int splits = std::max(1, std::min(kFwdSteps / 2, 152 / std::max(1, tiles)));
+  return (kFwdSteps + splits - 1) / splits;
+}
+int fwd_splits(int B) { return (kFwdSteps + fwd_steps(B) - 1) / fwd_steps(B); }
+// partial sums of a batch of B, and of every smaller one (a workspace sized for
+// a batch serves them): splits * B <= min(25 B, max(152 tiles, B))
+size_t part_rows(int B) {
+  return std::min<size_t>(static_cast<size_t>(B) * (kFwdSteps / 2), std::max<size_t>(152 * kFB, static_cast<size_t>(B)));
+}
+bool on16(const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; }
 
 ScorerWs carve_scorer(void* ws, size_t bytes, int B, int n_coarse, size_t* need) {
   Carver c(ws, bytes);
   ScorerWs w;
-  w.z1 = c.take<float>(static_cast<size_t>(B) * kH1);
+  w.part = c.take<float>(part_rows(B) * kH1);
   w.h1 = c.take<float>(static_cast<size_t>(B) * kH1);
-  w.z2 = c.take<float>(static_cast<size_t>(B) * kH2);
   w.h2 = c.take<float>(static_cast<size_t>(B) * kH2);
-  w.z3 = c.take<float>(B);
   w.d3 = c.take<float>(B);
   w.d2 = c.take<float>(static_cast<size_t>(B) * kH2);
   w.d1 = c.take<float>(static_cast<size_t>(B) * kH1);
-  w.loss = c.take<float>(1);
+  w.loss = c.take<float>(B);
   w.chan0 = c.take<int>(n_coarse + 1);
   *need = c.used;
   return w;
 }
 
-dim3 tiles(int cols, int rows) { return dim3((cols + kT - 1) / kT, (rows + kT - 1) / kT); }
-
+// logits, and with targets y what k_grads needs
 template <bool BF16>
-int forward_impl(const void* w, const float* x, int B, const ScorerWs& s, float* logit, cudaStream_t st) {
-  k_dense_fwd<BF16><<<tiles(kH1, B), 256, 0, st>>>(x, w, kW1, kB1, B, kIn, kH1, true, s.z1, s.h1);
+int forward_impl(const void* w, const float* x, const float* y, int B, const ScorerWs& s, float* logit,
+                 cudaStream_t st) {
+  const int splits = fwd_splits(B);
+  k_dense_fwd<BF16><<<dim3((B + kFB - 1) / kFB, splits), 256, 0, st>>>(x, w, B, fwd_steps(B), on16(x),
+                                                                            on16(w), s.part);
   OVRO_LAUNCH_CHECK();
-  k_dense_fwd<BF16><<<tiles(kH2, B), 256, 0, st>>>(s.h1, w, kW2, kB2, B, kH1, kH2, true, s.z2, s.h2);
-  OVRO_LAUNCH_CHECK();
-  k_dense_fwd<BF16><<<tiles(1, B), 256, 0, st>>>(s.h2, w, kW3, kB3, B, kH2, 1, false, nullptr, logit);
+  k_dense_mid<BF16><<<(B + kMB - 1) / kMB, 256, 0, st>>>(s.part, splits, w, y, B, logit, y ? s.h1 : nullptr, s.h2,
+                                                          s.d1, s.d2, s.d3, s.loss);
   OVRO_LAUNCH_CHECK();
   return OVRO_OK;
 }
@@ -266,29 +445,10 @@ int forward_impl(const void* w, const float* x, int B, const ScorerWs& s, float*
 template <bool BF16>
 int grad_impl(const void* w, const float* x, const float* y, int B, const ScorerWs& s, float* grad,
               float* loss_out, cudaStream_t st) {
-  if (int e = forward_impl<BF16>(w, x, B, s, s.z3, st)) return e;
-  k_bce<<<1, 1024, 0, st>>>(s.z3, y, B, s.d3, s.loss);
+  if (int e = forward_impl<BF16>(w, x, y, B, s, nullptr, st)) return e;
+  k_grads<<<kW1Tiles + kW2Tiles + kSumCtas, 128 * kGGroups, 0, st>>>(x, s.h1, s.h2, s.d1, s.d2, s.d3, s.loss, B,
+                                                                     on16(x), grad, loss_out);
   OVRO_LAUNCH_CHECK();
-  // layer 3
-  k_dense_bwd_w<<<tiles(kH2, 1), 256, 0, st>>>(s.d3, s.h2, B, kH2, 1, grad + kW3);
-  OVRO_LAUNCH_CHECK();
-  k_bias_grad<<<1, 256, 0, st>>>(s.d3, B, 1, grad + kB3);
-  OVRO_LAUNCH_CHECK();
-  k_dense_bwd_x<BF16><<<tiles(kH2, B), 256, 0, st>>>(s.d3, w, kW3, B, kH2, 1, s.z2, s.d2);
-  OVRO_LAUNCH_CHECK();
-  // layer 2
-  k_dense_bwd_w<<<tiles(kH1, kH2), 256, 0, st>>>(s.d2, s.h1, B, kH1, kH2, grad + kW2);
-  OVRO_LAUNCH_CHECK();
-  k_bias_grad<<<kH2, 256, 0, st>>>(s.d2, B, kH2, grad + kB2);
-  OVRO_LAUNCH_CHECK();
-  k_dense_bwd_x<BF16><<<tiles(kH1, B), 256, 0, st>>>(s.d2, w, kW2, B, kH1, kH2, s.z1, s.d1);
-  OVRO_LAUNCH_CHECK();
-  // layer 1
-  k_dense_bwd_w<<<tiles(kIn, kH1), 256, 0, st>>>(s.d1, x, B, kIn, kH1, grad + kW1);
-  OVRO_LAUNCH_CHECK();
-  k_bias_grad<<<kH1, 256, 0, st>>>(s.d1, B, kH1, grad + kB1);
-  OVRO_LAUNCH_CHECK();
-  if (loss_out) OVRO_CUDA_TRY(cudaMemcpyAsync(loss_out, s.loss, sizeof(float), cudaMemcpyDeviceToDevice, st));
   return OVRO_OK;
 }
 
@@ -340,7 +500,7 @@ int ovro_scorer_forward(const void* d_w_bf16, const float* d_x, int batch, float
   ScorerWs s = carve_scorer(d_ws, ws_bytes, batch, 1, &need);
   if (int e = check_workspace(d_ws, ws_bytes, need)) return e;
   OVRO_PROF("k_scorer_fwd", as_stream(stream));
-  return forward_impl<true>(d_w_bf16, d_x, batch, s, d_logit, as_stream(stream));
+  return forward_impl<true>(d_w_bf16, d_x, nullptr, batch, s, d_logit, as_stream(stream));
 }
 
 int ovro_scorer_grad(const void* d_w, int w_is_bf16, const float* d_x, const float* d_y, int batch,
