@@ -214,7 +214,7 @@ k_upchan_p2(UpchanArgs a) {
   const long long row0 = static_cast<long long>(s) * N;
   {
     const uint8_t* src = a.volt + row0 * a.n_input + i0;
-    if (gv == G && (G % 4) == 0 && (a.n_input % 4) == 0) {
+    if (gv == G && (G % 4) == 0 && ((reinterpret_cast<uintptr_t>(a.volt) | a.n_input) & 3) == 0) {
       const int wpr = G / 4;
       for (int idx = tid; idx < N * wpr; idx += T) {
         const int n = idx / wpr, w = idx - n * wpr;
@@ -272,8 +272,9 @@ k_upchan_p2(UpchanArgs a) {
   {
     int8_t* dst0 = a.out_q + (static_cast<long long>(s) * a.n_input + i0) * 2;
     const long long row_stride = static_cast<long long>(a.n_spec) * a.n_input * 2;
-    if (gv == G && (G % 2) == 0) {
-      const int wpr = G / 2;           // 4-byte words per row
+    // 4-byte words per row: the rows of an even number of inputs start on one
+    if (gv == G && (G % 2) == 0 && (a.n_input % 2) == 0 && (reinterpret_cast<uintptr_t>(a.out_q) & 3) == 0) {
+      const int wpr = G / 2;
       for (int idx = tid; idx < N * wpr; idx += T) {
         const int kp = idx / wpr, w = idx - kp * wpr;
         *reinterpret_cast<uint32_t*>(dst0 + kp * row_stride + 4 * w) =
@@ -472,7 +473,9 @@ int ovro_upchan_ex(const uint8_t* d_volt, int n_input, int n_coarse, int64_t n_t
     const int n = e.n;
     const long long n_used = (n_time / n) * n;
     if (!h_scale_or_null) {
-      const int vw = (n_input % 16 == 0) ? 16 : ((n_input % 4 == 0) ? 4 : 1);
+      // bytes a thread reads at a time: what every row starts on
+      const uintptr_t al = reinterpret_cast<uintptr_t>(d_volt) | static_cast<uintptr_t>(n_input);
+      const int vw = al % 16 == 0 ? 16 : (al % 4 == 0 ? 4 : 1);
       const int nvec = (n_input + vw - 1) / vw;
       const int threads = nvec >= 256 ? 256 : ((nvec + 31) / 32) * 32;
       const long long rows = n_used < 8LL * num_sms() ? n_used : 8LL * num_sms();

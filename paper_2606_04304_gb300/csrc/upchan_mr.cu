@@ -171,14 +171,15 @@ __global__ void __launch_bounds__(kMrThreads, MINB) k_upchan_mr(UpchanArgs a, Mr
     // stage the P N packed rows of this spectrum (G bytes each)
     const uint8_t* src = a.volt + static_cast<long long>(s) * N * a.n_input + i0;
     const int rows = P * N;
-    if (gv == G && (G % 4) == 0 && (a.n_input % 4) == 0) {
+    const uintptr_t al = reinterpret_cast<uintptr_t>(a.volt) | static_cast<uintptr_t>(a.n_input);
+    if (gv == G && (G % 4) == 0 && (al & 3) == 0) {
       const int wpr = G / 4;
       for (int idx = tid; idx < rows * wpr; idx += T) {
         const int n = idx / wpr, w = idx - n * wpr;
         reinterpret_cast<uint32_t*>(raw)[idx] =
             __ldg(reinterpret_cast<const uint32_t*>(src + static_cast<long long>(n) * a.n_input + 4 * w));
       }
-    } else if (gv == G && G == 2 && (a.n_input % 2) == 0) {
+    } else if (gv == G && G == 2 && (al & 1) == 0) {
       for (int n = tid; n < rows; n += T)
         reinterpret_cast<uint16_t*>(raw)[n] =
             __ldg(reinterpret_cast<const unsigned short*>(src + static_cast<long long>(n) * a.n_input));
@@ -213,7 +214,7 @@ __global__ void __launch_bounds__(kMrThreads, MINB) k_upchan_mr(UpchanArgs a, Mr
     int8_t* dst0 = a.out_q + (static_cast<long long>(s) * a.n_input + i0) * 2;
     const long long row_stride = static_cast<long long>(a.n_spec) * a.n_input * 2;
     const int cnt = a.chan_cnt;
-    if (gv == G && (G % 2) == 0 && (a.n_input % 2) == 0) {
+    if (gv == G && (G % 2) == 0 && ((reinterpret_cast<uintptr_t>(a.out_q) & 3) | (a.n_input & 1)) == 0) {
       const int wpr = G / 2;
       for (int idx = tid; idx < cnt * wpr; idx += T) {
         const int kp = idx / wpr, w = idx - kp * wpr;

@@ -1,0 +1,31 @@
+"""The upchannelizer on rows that do not start on a word: an odd number of
+inputs with whole groups of them, and a voltage buffer that starts off 16 bytes.
+Every input is transformed on its own, so the values are those of the same
+inputs inside wider, aligned rows, bit for bit."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("nfft,n_input,shift", [([2048], 23, 0), ([8192], 5, 0), ([1024, 256], 33, 0), ([4096], 17, 3),
+                                                ([8192], 16, 1), ([1024], 48, 4), ([480], 9, 0), ([2400], 12, 2),
+                                                ([16, 64], 31, 1)])
+def test_rows_off_a_word(lib, nfft, n_input, shift):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n_input)
+    n_time, wide = 3 * max(nfft) + 7, (n_input + 63) // 32 * 32
+    v = torch.randint(0, 256, (len(nfft), n_time, wide), generator=g, device="cuda", dtype=torch.int16).to(torch.uint8)
+    flat = torch.zeros(len(nfft) * n_time * n_input + shift, dtype=torch.uint8, device="cuda")
+    narrow = flat[shift:].view(len(nfft), n_time, n_input)
+    narrow.copy_(v[:, :, :n_input])
+    qw, fw = lib.upchan(v, nfft, want_f32=True)
+    qn, fn = lib.upchan(narrow, nfft, want_f32=True)
+    off_w = off_n = 0
+    for n in nfft:
+        k = n_time // n
+        for a, b in ((qw, qn), (fw, fn)):
+            w = a[off_w:off_w + n * k * wide * 2].view(n, k, wide, 2)[:, :, :n_input]
+            assert torch.equal(w, b[off_n:off_n + n * k * n_input * 2].view(n, k, n_input, 2))
+        off_w += n * k * wide * 2
+        off_n += n * k * n_input * 2
