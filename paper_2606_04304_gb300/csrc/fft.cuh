@@ -148,28 +148,37 @@ namespace ovro {
 // stride 16 become conflict-free.
 __device__ __forceinline__ int pad16(int x) { return x + (x >> 4); }
 
-// One Stockham pass in place over rows of G points, the first NS-point
-// transforms already done (G, R and NS are compile-time, so every index split
-// is a shift).  load(f, x) gives element x of row f of the pass's input (the
-// rows themselves, or another source for a first pass; every read completes
-// before the first write, so the source may overlap `a`); tw(i) = omega_G^i.
-template <int R, int NS, int G, class Load, class Tw>
-__device__ __forceinline__ void stockham_pass(float2* a, int ldp, Load&& load, Tw&& tw) {
+// The threads of one transform group: thread `tid` of `n`, and their barrier.
+struct CtaGroup {
+  __device__ __forceinline__ int tid() const { return threadIdx.x; }
+  __device__ __forceinline__ int size() const { return blockDim.x; }
+  __device__ __forceinline__ void sync() const { __syncthreads(); }
+};
+
+// One Stockham pass over rows of G points, the first NS-point transforms
+// already done (G, R and NS are compile-time, so every index split is a shift).
+// load(f, x, slot) gives element x of row f of the pass's input, slot (0 .. 15,
+// compile-time) being which of the thread's 16 values it is; store(f, x, v) takes
+// element x of its output.  in_place: the output may overlap the input (every
+// read completes before the first write) and is complete for the group when the
+// pass returns.  tw(i) = omega_G^i.
+template <int R, int NS, int G, class Group, class Load, class Tw, class Store>
+__device__ __forceinline__ void stockham_pass(const Group& group, bool in_place, Load&& load, Tw&& tw, Store&& store) {
   // every thread holds exactly 16 values: 16 / R butterflies of radix R
   constexpr int NB = 16 / R;
   constexpr int per = G / R;
-  const int T = blockDim.x;
+  const int T = group.size();
   float2 v[16];
   int fj[NB];
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
-    const int gb = threadIdx.x + b * T;
+    const int gb = group.tid() + b * T;
     const int f = gb / per, j = gb - f * per;
     fj[b] = gb;
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[b * R + r] = load(f, j + r * per);
+    for (int r = 0; r < R; ++r) v[b * R + r] = load(f, j + r * per, b * R + r);
   }
-  __syncthreads();
+  if (in_place) group.sync();
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
     const int f = fj[b] / per, j = fj[b] - f * per;
@@ -198,29 +207,53 @@ __device__ __forceinline__ void stockham_pass(float2* a, int ldp, Load&& load, T
     dft_reg<R>(x);
     const int o = (j / NS) * NS * R + k;
 #pragma unroll
-    for (int r = 0; r < R; ++r) a[f * ldp + pad16(o + r * NS)] = x[r];
+    for (int r = 0; r < R; ++r) store(f, o + r * NS, x[r]);
   }
-  __syncthreads();
+  if (in_place) group.sync();
 }
 
-// In-place forward FFTs of the rows of `a` (row f at a[f * ldp], element x at
-// pad16(x)), G = 2^LOG2G with 16 <= G <= 16384, with blockDim.x * 16 == rows * G:
-// radix-16 passes, then one of radix 2, 4 or 8.  The first pass reads its
-// input through load0(f, x); tw(i) = omega_G^i.
-template <int LOG2G, class Load, class Tw>
-__device__ void fft_rows_inplace_f(float2* a, int ldp, Load&& load0, Tw&& tw) {
+// Forward FFTs of rows of G = 2^LOG2G points, 16 <= G <= 16384, by a group of
+// threads with size * 16 == rows * G: radix-16 passes, then one of radix 2, 4 or
+// 8, exchanging through `a` (row f at a[f * ldp], element x at pad16(x)).  The
+// first pass reads its input through load0(f, x, slot) and may overlap `a`; the
+// last one hands its results to store(f, x, v): in_place when they overlap `a`.
+// tw(i) = omega_G^i.
+template <int LOG2G, class Group, class Load, class Tw, class Store>
+__device__ __forceinline__ void fft_rows_io(const Group& group, float2* a, int ldp, bool in_place, Load&& load0,
+                                            Tw&& tw, Store&& store) {
   constexpr int G = 1 << LOG2G;
   constexpr int n16 = LOG2G / 4;
   constexpr int rem = LOG2G % 4;
   constexpr int NSR = 1 << (4 * n16);                 // transforms done before the last radix-2/4/8 pass
   static_assert(n16 >= 1 && n16 <= 3, "16 <= G <= 16384");
-  auto rows = [&](int f, int x) { return a[f * ldp + pad16(x)]; };
-  stockham_pass<16, 1, G>(a, ldp, load0, tw);
-  if constexpr (n16 >= 2) stockham_pass<16, 16, G>(a, ldp, rows, tw);
-  if constexpr (n16 >= 3) stockham_pass<16, 256, G>(a, ldp, rows, tw);
-  if constexpr (rem == 1) stockham_pass<2, NSR, G>(a, ldp, rows, tw);
-  if constexpr (rem == 2) stockham_pass<4, NSR, G>(a, ldp, rows, tw);
-  if constexpr (rem == 3) stockham_pass<8, NSR, G>(a, ldp, rows, tw);
+  auto get = [&](int f, int x, int) { return a[f * ldp + pad16(x)]; };
+  auto put = [&](int f, int x, float2 v) { a[f * ldp + pad16(x)] = v; };
+  if constexpr (n16 == 1 && rem == 0) {
+    stockham_pass<16, 1, G>(group, in_place, load0, tw, store);
+  } else {
+    stockham_pass<16, 1, G>(group, true, load0, tw, put);
+    if constexpr (n16 == 2 && rem == 0) {
+      stockham_pass<16, 16, G>(group, in_place, get, tw, store);
+    } else {
+      if constexpr (n16 >= 2) stockham_pass<16, 16, G>(group, true, get, tw, put);
+      if constexpr (n16 == 3 && rem == 0) {
+        stockham_pass<16, 256, G>(group, in_place, get, tw, store);
+      } else {
+        if constexpr (n16 >= 3) stockham_pass<16, 256, G>(group, true, get, tw, put);
+        if constexpr (rem == 1) stockham_pass<2, NSR, G>(group, in_place, get, tw, store);
+        if constexpr (rem == 2) stockham_pass<4, NSR, G>(group, in_place, get, tw, store);
+        if constexpr (rem == 3) stockham_pass<8, NSR, G>(group, in_place, get, tw, store);
+      }
+    }
+  }
+}
+
+// The same by the whole CTA, in place.
+template <int LOG2G, class Load, class Tw>
+__device__ void fft_rows_inplace_f(float2* a, int ldp, Load&& load0, Tw&& tw) {
+  fft_rows_io<LOG2G>(
+      CtaGroup{}, a, ldp, true, [&](int f, int x, int) { return load0(f, x); }, tw,
+      [&](int f, int x, float2 v) { a[f * ldp + pad16(x)] = v; });
 }
 
 }  // namespace ovro

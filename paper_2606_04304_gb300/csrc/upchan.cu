@@ -33,40 +33,56 @@ __device__ __forceinline__ uint32_t sample_power(uint32_t b) {
   return static_cast<uint32_t>(re * re + im * im);
 }
 
+// Thread = one VW-byte column of R rows at a time (blockDim.x = R columns of
+// rows), so a CTA reads consecutive bytes; the R partial sums of a column meet in
+// shared memory.  Bound by the read: 169 MB took 122 us with one row per
+// 64-thread CTA step, now 63.
 template <int VW>
-__global__ void k_power(const uint8_t* __restrict__ volt, int n_input, long long n_used,
-                        unsigned long long* __restrict__ power) {
-  // thread = one VW-byte column of the row; blocks stride over rows
-  const int nvec = (n_input + VW - 1) / VW;
-  const int v = blockIdx.y * blockDim.x + threadIdx.x;
-  if (v >= nvec) return;
-  uint32_t acc[VW];
+__global__ void __launch_bounds__(256)
+k_power(const uint8_t* __restrict__ volt, int n_input, long long n_used, int nvec, int col0,
+        unsigned long long* __restrict__ power) {
+  extern __shared__ uint32_t sum[];                     // [columns of this CTA][VW]
+  const int cols = min(nvec - static_cast<int>(blockIdx.y) * col0, col0);
+  const int rows = blockDim.x / col0;
+  const int cv = threadIdx.x % col0, r0 = threadIdx.x / col0;
+  const int v = blockIdx.y * col0 + cv;
+  for (int i = threadIdx.x; i < col0 * VW; i += blockDim.x) sum[i] = 0u;
+  __syncthreads();
+  if (cv < cols && r0 < rows) {
+    uint32_t acc[VW];
 #pragma unroll
-  for (int j = 0; j < VW; ++j) acc[j] = 0;
-  const bool full = (v + 1) * VW <= n_input;
-#pragma unroll 4
-  for (long long r = blockIdx.x; r < n_used; r += gridDim.x) {
-    const uint8_t* p = volt + r * n_input + static_cast<long long>(v) * VW;
-    if (VW == 16) {
-      const uint4 w = __ldg(reinterpret_cast<const uint4*>(p));
-      const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
+    for (int j = 0; j < VW; ++j) acc[j] = 0;
+    const bool full = (v + 1) * VW <= n_input;
+    const long long step = static_cast<long long>(gridDim.x) * rows;
+#pragma unroll 8
+    for (long long r = static_cast<long long>(blockIdx.x) * rows + r0; r < n_used; r += step) {
+      const uint8_t* p = volt + r * n_input + static_cast<long long>(v) * VW;
+      if (VW == 16) {
+        const uint4 w = __ldg(reinterpret_cast<const uint4*>(p));
+        const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
+        for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[q * 4 + b] += sample_power((ws[q] >> (8 * b)) & 0xffu);
-    } else if (VW == 4) {
-      const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(p));
+          for (int b = 0; b < 4; ++b) acc[q * 4 + b] += sample_power((ws[q] >> (8 * b)) & 0xffu);
+      } else if (VW == 4) {
+        const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(p));
 #pragma unroll
-      for (int b = 0; b < 4; ++b) acc[b] += sample_power((w >> (8 * b)) & 0xffu);
-    } else {
+        for (int b = 0; b < 4; ++b) acc[b] += sample_power((w >> (8 * b)) & 0xffu);
+      } else {
 #pragma unroll
-      for (int b = 0; b < VW; ++b)
-        if (full || v * VW + b < n_input) acc[b] += sample_power(p[b]);
+        for (int b = 0; b < VW; ++b)
+          if (full || v * VW + b < n_input) acc[b] += sample_power(p[b]);
+      }
     }
-  }
 #pragma unroll
-  for (int j = 0; j < VW; ++j)
-    if (v * VW + j < n_input && acc[j]) atomicAdd(power + v * VW + j, static_cast<unsigned long long>(acc[j]));
+    for (int j = 0; j < VW; ++j)
+      if (acc[j]) atomicAdd(&sum[cv * VW + j], acc[j]);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < cols * VW; i += blockDim.x) {
+    const int in = blockIdx.y * col0 * VW + i;
+    if (in < n_input && sum[i]) atomicAdd(power + in, static_cast<unsigned long long>(sum[i]));
+  }
 }
 
 // s = 8 sqrt(2) / sqrt(W P), P = power / n_used, in FP64; rounded to FP32.
@@ -184,8 +200,10 @@ k_upchan(UpchanArgs a) {
 // FFTs of the group in flight (F N = 8192 points, 16 per thread; one FFT of
 // 16384), exchange rows padded by one slot per 16 so the stride-16 writes of
 // a pass hit distinct banks, every index split a shift.  The first pass
-// unpacks the staged 4+4-bit samples; the bins come out in natural order and
-// are requantised, fftshifted, into the staging rows.
+// unpacks the staged 4+4-bit samples; the last one requantises its bins,
+// fftshifted, into the staging rows straight from registers (through the exchange
+// buffer they cost a trip and a barrier more: with 704 inputs and 10 s 4096
+// points took 1.22 ms and now 1.10, 8192 points 1.47 and 1.44).
 template <int LOG2N>
 struct P2Plan {
   static constexpr int N = 1 << LOG2N;
@@ -233,9 +251,9 @@ k_upchan_p2(UpchanArgs a) {
   const int tw_stride = a.tw_n / N;
   auto tw = [&](int i) { return __ldg(a.tw + static_cast<long long>(i) * tw_stride); };
   for (int f0 = 0; f0 < G; f0 += F) {
-    fft_rows_inplace_f<LOG2N>(
-        buf, LDP,
-        [&](int f, int x) {
+    fft_rows_io<LOG2N>(
+        CtaGroup{}, buf, LDP, false,
+        [&](int f, int x, int) {
           // high nibble real, low nibble imaginary (two's complement)
           float2 v = make_float2(0.f, 0.f);
           const int g = f0 + f;
@@ -246,27 +264,25 @@ k_upchan_p2(UpchanArgs a) {
           }
           return v;
         },
-        tw);
-    for (int idx = tid; idx < F * N; idx += T) {
-      const int f = idx >> LOG2N, k = idx & (N - 1);
-      const int g = f0 + f;
-      if (g >= gv) continue;
-      const float2 X = buf[f * LDP + pad16(k)];
-      const float s_g = sc[g];
-      const int kp = (k + N / 2) & (N - 1);
-      float qr = rintf(__fmul_rn(s_g, X.x));
-      float qi = rintf(__fmul_rn(s_g, X.y));
-      qr = fminf(fmaxf(qr, -127.f), 127.f);
-      qi = fminf(fmaxf(qi, -127.f), 127.f);
-      char2 q2;
-      q2.x = static_cast<signed char>(qr);
-      q2.y = static_cast<signed char>(qi);
-      reinterpret_cast<char2*>(stg)[kp * G + g] = q2;
-      if (a.out_f) {
-        const long long o = ((static_cast<long long>(kp) * a.n_spec + s) * a.n_input + i0 + g);
-        reinterpret_cast<float2*>(a.out_f)[o] = X;
-      }
-    }
+        tw,
+        [&](int f, int k, float2 X) {
+          const int g = f0 + f;
+          if (g >= gv) return;
+          const float s_g = sc[g];
+          const int kp = (k + N / 2) & (N - 1);
+          float qr = rintf(__fmul_rn(s_g, X.x));
+          float qi = rintf(__fmul_rn(s_g, X.y));
+          qr = fminf(fmaxf(qr, -127.f), 127.f);
+          qi = fminf(fmaxf(qi, -127.f), 127.f);
+          char2 q2;
+          q2.x = static_cast<signed char>(qr);
+          q2.y = static_cast<signed char>(qi);
+          reinterpret_cast<char2*>(stg)[kp * G + g] = q2;
+          if (a.out_f) {
+            const long long o = ((static_cast<long long>(kp) * a.n_spec + s) * a.n_input + i0 + g);
+            reinterpret_cast<float2*>(a.out_f)[o] = X;
+          }
+        });
     __syncthreads();   // buf reused by the next F inputs; stg complete
   }
   {
@@ -477,17 +493,16 @@ int ovro_upchan_ex(const uint8_t* d_volt, int n_input, int n_coarse, int64_t n_t
       const uintptr_t al = reinterpret_cast<uintptr_t>(d_volt) | static_cast<uintptr_t>(n_input);
       const int vw = al % 16 == 0 ? 16 : (al % 4 == 0 ? 4 : 1);
       const int nvec = (n_input + vw - 1) / vw;
-      const int threads = nvec >= 256 ? 256 : ((nvec + 31) / 32) * 32;
-      const long long rows = n_used < 8LL * num_sms() ? n_used : 8LL * num_sms();
-      dim3 grid(static_cast<unsigned>(rows), (nvec + threads - 1) / threads);
+      const int col0 = std::min(nvec, 256), rows = 256 / col0;
+      const long long blocks = std::min<long long>((n_used + rows - 1) / rows, 4LL * num_sms());
+      // a CTA's 32-bit sums: at most 128 a sample over its share of the rows
+      const long long share = (n_used + blocks - 1) / blocks;
+      dim3 grid(static_cast<unsigned>(share < (1LL << 24) ? blocks : (n_used + (1LL << 24) - 1) >> 24),
+                (nvec + col0 - 1) / col0);
       const uint8_t* vc = d_volt + static_cast<long long>(c) * n_time * n_input;
       unsigned long long* pc = w.power + static_cast<size_t>(c) * n_input;
-      if (vw == 16)
-        k_power<16><<<grid, threads, 0, st>>>(vc, n_input, n_used, pc);
-      else if (vw == 4)
-        k_power<4><<<grid, threads, 0, st>>>(vc, n_input, n_used, pc);
-      else
-        k_power<1><<<grid, threads, 0, st>>>(vc, n_input, n_used, pc);
+      auto kern = vw == 16 ? k_power<16> : vw == 4 ? k_power<4> : k_power<1>;
+      kern<<<grid, col0 * rows, static_cast<size_t>(col0) * vw * 4, st>>>(vc, n_input, n_used, nvec, col0, pc);
       OVRO_LAUNCH_CHECK();
       if (taps) {
         k_sumsq<<<1, 256, 0, st>>>(opt->h_taps[c], n_tap * n, w.h2 + c);
