@@ -12,6 +12,7 @@
 // the X-engine reads.
 #include <cmath>
 #include <mutex>
+#include <numeric>
 #include <vector>
 
 #include "common.cuh"
@@ -33,30 +34,35 @@ __device__ __forceinline__ uint32_t sample_power(uint32_t b) {
   return static_cast<uint32_t>(re * re + im * im);
 }
 
-// Thread = one VW-byte column of R rows at a time (blockDim.x = R columns of
-// rows), so a CTA reads consecutive bytes; the R partial sums of a column meet in
-// shared memory.  Bound by the read: 169 MB took 122 us with one row per
-// 64-thread CTA step, now 63.
+// `fold` rows of n_input bytes laid end to end are one row of nvec VW-byte columns:
+// with fold = VW / gcd(n_input, VW) every such row starts on a VW-byte word and has
+// a whole number of them, so any width is read in full words.  Thread = one column
+// of R such rows at a time (blockDim.x = R columns of rows), a CTA reads
+// consecutive bytes, and the sums of one input meet in shared memory.  Bound by the
+// read: 169 MB in rows of 704 took 122 us with one row per 64-thread CTA step, now
+// 62; the same in rows of 574, read a byte at a time, cost another 0.5 ms.
 template <int VW>
 __global__ void __launch_bounds__(256)
-k_power(const uint8_t* __restrict__ volt, int n_input, long long n_used, int nvec, int col0,
+k_power(const uint8_t* __restrict__ volt, int n_input, int fold, long long n_rows, int nvec, int col0,
         unsigned long long* __restrict__ power) {
-  extern __shared__ uint32_t sum[];                     // [columns of this CTA][VW]
-  const int cols = min(nvec - static_cast<int>(blockIdx.y) * col0, col0);
+  extern __shared__ uint32_t sum[];                     // [inputs of this CTA's columns]
+  const int first = blockIdx.y * col0;
+  const int cols = min(nvec - first, col0);
+  const int n_sum = min(n_input, cols * VW);
   const int rows = blockDim.x / col0;
   const int cv = threadIdx.x % col0, r0 = threadIdx.x / col0;
-  const int v = blockIdx.y * col0 + cv;
-  for (int i = threadIdx.x; i < col0 * VW; i += blockDim.x) sum[i] = 0u;
+  for (int i = threadIdx.x; i < n_sum; i += blockDim.x) sum[i] = 0u;
   __syncthreads();
   if (cv < cols && r0 < rows) {
     uint32_t acc[VW];
 #pragma unroll
     for (int j = 0; j < VW; ++j) acc[j] = 0;
-    const bool full = (v + 1) * VW <= n_input;
     const long long step = static_cast<long long>(gridDim.x) * rows;
+    const long long pitch = static_cast<long long>(n_input) * fold;
+    const uint8_t* at = volt + static_cast<long long>(first + cv) * VW;
 #pragma unroll 8
-    for (long long r = static_cast<long long>(blockIdx.x) * rows + r0; r < n_used; r += step) {
-      const uint8_t* p = volt + r * n_input + static_cast<long long>(v) * VW;
+    for (long long r = static_cast<long long>(blockIdx.x) * rows + r0; r < n_rows; r += step) {
+      const uint8_t* p = at + r * pitch;
       if (VW == 16) {
         const uint4 w = __ldg(reinterpret_cast<const uint4*>(p));
         const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
@@ -69,20 +75,21 @@ k_power(const uint8_t* __restrict__ volt, int n_input, long long n_used, int nve
 #pragma unroll
         for (int b = 0; b < 4; ++b) acc[b] += sample_power((w >> (8 * b)) & 0xffu);
       } else {
-#pragma unroll
-        for (int b = 0; b < VW; ++b)
-          if (full || v * VW + b < n_input) acc[b] += sample_power(p[b]);
+        acc[0] += sample_power(*p);
       }
     }
+    int in = cv * VW % n_input;
 #pragma unroll
-    for (int j = 0; j < VW; ++j)
-      if (acc[j]) atomicAdd(&sum[cv * VW + j], acc[j]);
+    for (int j = 0; j < VW; ++j) {
+      if (acc[j]) atomicAdd(&sum[in], acc[j]);
+      if (++in == n_input) in = 0;
+    }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < cols * VW; i += blockDim.x) {
-    const int in = blockIdx.y * col0 * VW + i;
-    if (in < n_input && sum[i]) atomicAdd(power + in, static_cast<unsigned long long>(sum[i]));
-  }
+  const int in0 = static_cast<int>(static_cast<long long>(first) * VW % n_input);
+  for (int i = threadIdx.x; i < n_sum; i += blockDim.x)
+    if (sum[i])
+      atomicAdd(power + (in0 + i < n_input ? in0 + i : in0 + i - n_input), static_cast<unsigned long long>(sum[i]));
 }
 
 // s = 8 sqrt(2) / sqrt(W P), P = power / n_used, in FP64; rounded to FP32.
@@ -203,7 +210,7 @@ k_upchan(UpchanArgs a) {
 // unpacks the staged 4+4-bit samples; the last one requantises its bins,
 // fftshifted, into the staging rows straight from registers (through the exchange
 // buffer they cost a trip and a barrier more: with 704 inputs and 10 s 4096
-// points took 1.22 ms and now 1.10, 8192 points 1.47 and 1.44).
+// points took 1.22 ms and now 1.10, 8192 points 1.47 and 1.40).
 template <int LOG2N>
 struct P2Plan {
   static constexpr int N = 1 << LOG2N;
@@ -212,7 +219,9 @@ struct P2Plan {
   static constexpr int LDP = N + N / 16;             // pad16(x) < LDP for x < N
 };
 
-template <int LOG2N>
+// F32: FP32 spectra are asked for as well; known when compiled, as the test in the
+// last pass cost the transforms without them 2 to 4%.
+template <int LOG2N, bool F32>
 __global__ void __launch_bounds__(P2Plan<LOG2N>::THREADS, 1024 / P2Plan<LOG2N>::THREADS)
 k_upchan_p2(UpchanArgs a) {
   using P = P2Plan<LOG2N>;
@@ -232,13 +241,20 @@ k_upchan_p2(UpchanArgs a) {
   const long long row0 = static_cast<long long>(s) * N;
   {
     const uint8_t* src = a.volt + row0 * a.n_input + i0;
-    if (gv == G && (G % 4) == 0 && ((reinterpret_cast<uintptr_t>(a.volt) | a.n_input) & 3) == 0) {
-      const int wpr = G / 4;
+    auto words = [&](auto word) {
+      using W = decltype(word);
+      const int wpr = G / sizeof(W);
       for (int idx = tid; idx < N * wpr; idx += T) {
         const int n = idx / wpr, w = idx - n * wpr;
-        reinterpret_cast<uint32_t*>(raw)[idx] =
-            *reinterpret_cast<const uint32_t*>(src + static_cast<long long>(n) * a.n_input + 4 * w);
+        reinterpret_cast<W*>(raw)[idx] =
+            *reinterpret_cast<const W*>(src + static_cast<long long>(n) * a.n_input + sizeof(W) * w);
       }
+    };
+    const uintptr_t al = reinterpret_cast<uintptr_t>(a.volt) | a.n_input | G;   // where rows and groups start
+    if (gv == G && (al & 3) == 0) {
+      words(uint32_t{});
+    } else if (gv == G && (al & 1) == 0) {
+      words(uint16_t{});
     } else {
       for (int idx = tid; idx < N * G; idx += T) {
         const int n = idx / G, g = idx - n * G;
@@ -278,7 +294,7 @@ k_upchan_p2(UpchanArgs a) {
           q2.x = static_cast<signed char>(qr);
           q2.y = static_cast<signed char>(qi);
           reinterpret_cast<char2*>(stg)[kp * G + g] = q2;
-          if (a.out_f) {
+          if constexpr (F32) {
             const long long o = ((static_cast<long long>(kp) * a.n_spec + s) * a.n_input + i0 + g);
             reinterpret_cast<float2*>(a.out_f)[o] = X;
           }
@@ -342,7 +358,7 @@ int launch_upchan_t(const UpchanArgs& a, cudaStream_t st) {
   const size_t sm = smem_for(L, a.group);
   dim3 grid((a.n_input + a.group - 1) / a.group, a.n_spec);
   if constexpr (L >= 4) {
-    auto kern = k_upchan_p2<L>;
+    auto kern = a.out_f ? k_upchan_p2<L, true> : k_upchan_p2<L, false>;
     OVRO_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm)));
     OVRO_PROF("k_upchan", st);
     kern<<<grid, P2Plan<L>::THREADS, sm, st>>>(a);
@@ -489,20 +505,26 @@ int ovro_upchan_ex(const uint8_t* d_volt, int n_input, int n_coarse, int64_t n_t
     const int n = e.n;
     const long long n_used = (n_time / n) * n;
     if (!h_scale_or_null) {
-      // bytes a thread reads at a time: what every row starts on
-      const uintptr_t al = reinterpret_cast<uintptr_t>(d_volt) | static_cast<uintptr_t>(n_input);
-      const int vw = al % 16 == 0 ? 16 : (al % 4 == 0 ? 4 : 1);
-      const int nvec = (n_input + vw - 1) / vw;
-      const int col0 = std::min(nvec, 256), rows = 256 / col0;
-      const long long blocks = std::min<long long>((n_used + rows - 1) / rows, 4LL * num_sms());
-      // a CTA's 32-bit sums: at most 128 a sample over its share of the rows
-      const long long share = (n_used + blocks - 1) / blocks;
-      dim3 grid(static_cast<unsigned>(share < (1LL << 24) ? blocks : (n_used + (1LL << 24) - 1) >> 24),
-                (nvec + col0 - 1) / col0);
       const uint8_t* vc = d_volt + static_cast<long long>(c) * n_time * n_input;
       unsigned long long* pc = w.power + static_cast<size_t>(c) * n_input;
+      // bytes a thread reads at a time: the widest word the samples start on that
+      // whole numbers of rows make up, if the rows come out even
+      int vw = 16, fold = 1;
+      for (; vw > 1; vw /= 4) {
+        fold = vw / std::gcd(n_input, vw);
+        if (reinterpret_cast<uintptr_t>(vc) % vw == 0 && n_used % fold == 0) break;
+      }
+      if (vw == 1) fold = 1;
+      const long long n_rows = n_used / fold;
+      const int nvec = static_cast<int>(static_cast<long long>(n_input) * fold / vw), ny = (nvec + 255) / 256;
+      const int col0 = (nvec + ny - 1) / ny, rows = 256 / col0;
+      const long long blocks = std::min<long long>((n_rows + rows - 1) / rows, (vw == 16 ? 4LL : 8LL) * num_sms());
+      // a CTA's 32-bit sums: at most 128 a sample over its share of the rows
+      const long long share = (n_rows + blocks - 1) / blocks * fold;
+      dim3 grid(static_cast<unsigned>(share < (1LL << 24) ? blocks : (n_used + (1LL << 24) - 1) >> 24), ny);
       auto kern = vw == 16 ? k_power<16> : vw == 4 ? k_power<4> : k_power<1>;
-      kern<<<grid, col0 * rows, static_cast<size_t>(col0) * vw * 4, st>>>(vc, n_input, n_used, nvec, col0, pc);
+      kern<<<grid, col0 * rows, static_cast<size_t>(std::min(n_input, col0 * vw)) * 4, st>>>(vc, n_input, fold, n_rows,
+                                                                                              nvec, col0, pc);
       OVRO_LAUNCH_CHECK();
       if (taps) {
         k_sumsq<<<1, 256, 0, st>>>(opt->h_taps[c], n_tap * n, w.h2 + c);

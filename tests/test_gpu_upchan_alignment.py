@@ -10,7 +10,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("nfft,n_input,shift", [([2048], 23, 0), ([8192], 5, 0), ([1024, 256], 33, 0), ([4096], 17, 3),
                                                 ([8192], 16, 1), ([1024], 48, 4), ([480], 9, 0), ([2400], 12, 2),
-                                                ([16, 64], 31, 1)])
+                                                ([16, 64], 31, 1), ([8192], 34, 0), ([1024], 574, 0),
+                                                ([256], 4099, 0)])
 def test_rows_off_a_word(lib, nfft, n_input, shift):
     g = torch.Generator(device="cuda")
     g.manual_seed(n_input)
