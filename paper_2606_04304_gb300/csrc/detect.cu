@@ -41,6 +41,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "horizon.cuh"
 #include "stages.h"
 #include "tune.h"
 
@@ -1446,7 +1447,7 @@ constexpr int kCandCap = 1 << 21;       // candidates written by the NMS kernels
 struct DetectPlan {
   int n, n_coarse, n_chan;
   long long npix;
-  std::vector<int> pix;        // in-horizon pixel indices
+  Horizon disc;                // the in-horizon pixels
   std::vector<int> nfft, chan0, half;
   std::vector<long long> vox0; // voxel offset of each coarse block in snr/width
   long long n_vox = 0;
@@ -1465,13 +1466,8 @@ DetectPlan make_plan(int n_chan, int n, double cell, int n_coarse, const int32_t
   p.n_coarse = n_coarse;
   p.n_chan = n_chan;
   p.npix = static_cast<long long>(n) * n;
-  for (int r = 0; r < n; ++r)
-    for (int c = 0; c < n; ++c) {
-      const double l = static_cast<double>(c - n / 2) * cell;
-      const double m = static_cast<double>(r - n / 2) * cell;
-      if (l * l + m * m < 1.0) p.pix.push_back(r * n + c);
-    }
-  p.n_valid = static_cast<int>(p.pix.size());
+  p.disc = Horizon(n, cell);
+  p.n_valid = p.disc.size();
   int c0 = 0;
   for (int c = 0; c < n_coarse; ++c) {
     p.nfft.push_back(nfft[c]);
@@ -1495,6 +1491,7 @@ DetectPlan make_plan(int n_chan, int n, double cell, int n_coarse, const int32_t
 constexpr int kMaxBins = 2048;
 
 struct DetectWs {
+  int* rows;             // the horizon's rows, for k_horizon
   int* pix;
   double* stats64;
   float* stats32;
@@ -1523,6 +1520,7 @@ DetectWs carve_detect(void* ws, size_t bytes, const DetectPlan& p, size_t* need)
   DetectWs w;
   const size_t blk = static_cast<size_t>(p.n_valid) * p.max_nc;
   const long long np = std::max(1LL, n_pairs_of(p));
+  w.rows = c.take<int>(2 * static_cast<size_t>(p.n) + 1);
   w.pix = c.take<int>(p.n_valid > 0 ? p.n_valid : 1);
   w.stats64 = c.take<double>(2 * static_cast<size_t>(p.n_chan));
   w.stats32 = c.take<float>(2 * static_cast<size_t>(p.n_chan));
@@ -1784,12 +1782,12 @@ int bh_bin_verdict(const unsigned long long* hist, int nb, uint32_t key0, double
 // ranks above_next + 1, above_next + 2, ...; returns 1 and *cut, or 0.
 int bh_resolve(const float* v_desc, long long n, unsigned long long above_next, double m, double alpha,
                float* cut) {
-  long long best = -1;
-  for (long long j = 0; j < n; ++j)
-    if (log_q(v_desc[j]) <= std::log(alpha * static_cast<double>(above_next + j + 1) / m)) best = j;
-  if (best < 0) return 0;
-  *cut = v_desc[best];
-  return 1;
+  for (long long j = n - 1; j >= 0; --j)
+    if (log_q(v_desc[j]) <= std::log(alpha * static_cast<double>(above_next + j + 1) / m)) {
+      *cut = v_desc[j];
+      return 1;
+    }
+  return 0;
 }
 
 // Values of bin b of this search (device gather; synchronises).
@@ -1923,7 +1921,7 @@ int ovro_detect_stats(const float* d_img, int n_chan, int image_size, double cel
   DetectWs w = carve_detect(d_ws, ws_bytes, p, &need);
   if (int e = check_workspace(d_ws, ws_bytes, need)) return e;
   cudaStream_t st = as_stream(stream);
-  OVRO_CUDA_TRY(cudaMemcpyAsync(w.pix, p.pix.data(), p.pix.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+  if (int e = upload_horizon(p.disc, w.rows, w.pix, st)) return e;
   if (int e = run_stats_block(d_img, n_chan, w.stats64, w.stats32, p, w, st)) return e;
   OVRO_CUDA_TRY(cudaMemcpyAsync(d_stats, w.stats64, 2 * sizeof(double) * n_chan, cudaMemcpyDeviceToDevice, st));
   return OVRO_OK;
@@ -1943,7 +1941,7 @@ int ovro_detect_filter(const float* d_img, const double* d_stats, int n_chan, in
   DetectWs w = carve_detect(d_ws, ws_bytes, p, &need);
   if (int e = check_workspace(d_ws, ws_bytes, need)) return e;
   cudaStream_t st = as_stream(stream);
-  OVRO_CUDA_TRY(cudaMemcpyAsync(w.pix, p.pix.data(), p.pix.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+  if (int e = upload_horizon(p.disc, w.rows, w.pix, st)) return e;
   k_stats32<<<(n_chan + 255) / 256, 256, 0, st>>>(d_stats, n_chan, w.stats32);
   OVRO_LAUNCH_CHECK();
   uint32_t key0;
@@ -2028,7 +2026,7 @@ int detect_ctx_upload(DetectCtx* d, cudaStream_t st) {
   if (!d) return OVRO_ERR_INVALID_ARG;
   const DetectPlan& p = d->p;
   if (p.n_valid == 0) return OVRO_OK;
-  OVRO_CUDA_TRY(cudaMemcpyAsync(d->w.pix, p.pix.data(), p.pix.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+  if (int e = upload_horizon(p.disc, d->w.rows, d->w.pix, st)) return e;
   OVRO_CUDA_TRY(cudaMemcpyAsync(d->w.vox0, p.vox0.data(), p.n_coarse * sizeof(long long), cudaMemcpyHostToDevice, st));
   OVRO_CUDA_TRY(cudaMemcpyAsync(d->w.nfft, p.nfft.data(), p.n_coarse * sizeof(int), cudaMemcpyHostToDevice, st));
   return OVRO_OK;
@@ -2143,20 +2141,30 @@ int detect_ctx_candidates(DetectCtx* d, float cut, const double* h_chan_freq_hz,
     if (recs.size() < static_cast<size_t>(nw)) recs.resize(nw);
     OVRO_CUDA_TRY(cudaMemcpyAsync(recs.data(), w.recs, nw * sizeof(CandRec), cudaMemcpyDeviceToHost, st));
     OVRO_CUDA_TRY(cudaStreamSynchronize(st));
-    // (pixel, coarse) pair order, stable: a counting sort on q = p n_coarse + c
+    // (pixel, coarse) pair order, stable, q = p n_coarse + c: by comparison when
+    // the candidates are few beside the pairs, else a counting sort
     const long long n_q = np;
-    std::vector<int>& start = d->q_start;
-    start.assign(static_cast<size_t>(n_q) + 1, 0);
-    for (int i = 0; i < nw; ++i) ++start[static_cast<size_t>(recs[i].p) * p.n_coarse + recs[i].coarse + 1];
-    for (long long q = 0; q < n_q; ++q) start[q + 1] += start[q];
+    auto pair_of = [&](int i) { return static_cast<long long>(recs[i].p) * p.n_coarse + recs[i].coarse; };
     std::vector<int>& order = d->order;
     if (order.size() < static_cast<size_t>(nw)) order.resize(nw);
-    for (int i = 0; i < nw; ++i) order[start[static_cast<size_t>(recs[i].p) * p.n_coarse + recs[i].coarse]++] = i;
+    if (nw < n_q / 16) {
+      for (int i = 0; i < nw; ++i) order[i] = i;
+      std::sort(order.begin(), order.begin() + nw, [&](int a, int b) {
+        const long long qa = pair_of(a), qb = pair_of(b);
+        return qa != qb ? qa < qb : a < b;
+      });
+    } else {
+      std::vector<int>& start = d->q_start;
+      start.assign(static_cast<size_t>(n_q) + 1, 0);
+      for (int i = 0; i < nw; ++i) ++start[pair_of(i) + 1];
+      for (long long q = 0; q < n_q; ++q) start[q + 1] += start[q];
+      for (int i = 0; i < nw; ++i) order[start[pair_of(i)]++] = i;
+    }
     const int nout = std::min(nw, max_out);
     for (int q = 0; q < nout; ++q) {
       const CandRec& r = recs[order[q]];
       ovro_candidate& o = h_out[q];
-      const int pixel = p.pix[r.p];
+      const int pixel = p.disc.pixel(r.p);
       o.coarse = r.coarse;
       o.fine = r.k;
       o.chan = p.chan0[r.coarse] + r.k;

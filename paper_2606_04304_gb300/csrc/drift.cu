@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "horizon.cuh"
 
 namespace ovro {
 namespace {
@@ -327,6 +328,7 @@ constexpr int kDriftGatherCap = 1 << 22;
 struct DriftWs {
   unsigned long long* hist;
   float* vals;
+  int* rows;         // the horizon's rows, for k_horizon
   int* pix;
   DriftChunk* chunks;
   int* c_lo;
@@ -347,6 +349,7 @@ DriftWs carve_drift(void* ws, size_t bytes, int n_chan, int image_size, int n_co
   DriftWs w;
   w.hist = c.take<unsigned long long>(kDriftMaxBins);
   w.vals = c.take<float>(kDriftGatherCap);
+  w.rows = c.take<int>(2 * static_cast<size_t>(image_size) + 1);
   w.pix = c.take<int>(npix);
   w.chunks = c.take<DriftChunk>(std::max<long long>(n_chunks, 1));
   w.c_lo = c.take<int>(n_coarse);
@@ -406,14 +409,8 @@ int ovro_drift_search(const float* d_zp, int n_sub, int n_chan, int image_size, 
   }
   if (c0 != n_chan) return OVRO_ERR_INVALID_ARG;
   const int n = image_size;
-  std::vector<int> pix;
-  for (int r = 0; r < n; ++r)
-    for (int c = 0; c < n; ++c) {
-      const double l = static_cast<double>(c - n / 2) * cell_dircos;
-      const double m = static_cast<double>(r - n / 2) * cell_dircos;
-      if (l * l + m * m < 1.0) pix.push_back(r * n + c);
-    }
-  const int n_valid = static_cast<int>(pix.size());
+  const Horizon disc(n, cell_dircos);
+  const int n_valid = disc.size();
   std::vector<DriftChunk> chunks;
   for (int c = 0; c < n_coarse; ++c)
     for (int f0 = lo[c]; f0 < hi[c]; f0 += kTileF) chunks.push_back(DriftChunk{lo[c], hi[c], f0, c});
@@ -424,7 +421,7 @@ int ovro_drift_search(const float* d_zp, int n_sub, int n_chan, int image_size, 
   cudaStream_t st = as_stream(stream);
   const long long npix = static_cast<long long>(n) * n;
   const long long nvox = npix * n_chan;
-  OVRO_CUDA_TRY(cudaMemcpyAsync(w.pix, pix.data(), pix.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+  if (int e = upload_horizon(disc, w.rows, w.pix, st)) return e;
   OVRO_CUDA_TRY(cudaMemcpyAsync(w.chunks, chunks.data(), chunks.size() * sizeof(DriftChunk),
                                 cudaMemcpyHostToDevice, st));
   OVRO_CUDA_TRY(cudaMemcpyAsync(w.c_lo, lo.data(), lo.size() * sizeof(int), cudaMemcpyHostToDevice, st));
@@ -527,8 +524,8 @@ int ovro_drift_search(const float* d_zp, int n_sub, int n_chan, int image_size, 
     o.coarse = d.coarse;
     o.fine = d.chan - lo[d.coarse];
     o.chan = d.chan;
-    o.row = pix[d.p] / n;
-    o.col = pix[d.p] % n;
+    o.row = disc.pixel(d.p) / n;
+    o.col = disc.pixel(d.p) % n;
     o.width = std::abs(d.drift) + 1;
     o.snr = d.snr;
     o.score = 0.0f;
