@@ -2,6 +2,8 @@
 // upchannelizer and the imaging kernels.
 #pragma once
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace ovro {
@@ -155,13 +157,40 @@ struct CtaGroup {
   __device__ __forceinline__ void sync() const { __syncthreads(); }
 };
 
+// One radix-R butterfly of the pass after NS points, in registers: x[r] omega_G^(k r
+// G / (NS R)), then the DFT.
+template <int R, int NS, int G, class Tw>
+__device__ __forceinline__ void stockham_butterfly(float2 (&x)[R], int k, Tw&& tw) {
+  if (NS > 1) {
+    // twiddles w^r, w = omega_G^base: w^(2^m) read, the others products of
+    // those (at most three roundings deep), so a pass reads log2 R of them
+    const int base = k * (G / (NS * R));
+    float2 t[R];
+    constexpr std::integral_constant<int, NS> ns{};
+    t[1] = tw(base, ns, 0, k);
+    if (R >= 4) t[2] = tw(2 * base, ns, 1, k);
+    if (R >= 8) t[4] = tw(4 * base, ns, 2, k);
+    if (R >= 16) t[8] = tw(8 * base, ns, 3, k);
+#pragma unroll
+    for (int r = 3; r < R; ++r) {
+      if ((r & (r - 1)) == 0) continue;
+      const int hb = 1 << (31 - __clz(r));            // highest power of two in r (compile-time)
+      t[r] = cmul(t[hb], t[r - hb]);
+    }
+#pragma unroll
+    for (int r = 1; r < R; ++r) x[r] = cmul(x[r], t[r]);
+  }
+  dft_reg<R>(x);
+}
+
 // One Stockham pass over rows of G points, the first NS-point transforms
 // already done (G, R and NS are compile-time, so every index split is a shift).
 // load(f, x, slot) gives element x of row f of the pass's input, slot (0 .. 15,
 // compile-time) being which of the thread's 16 values it is; store(f, x, v) takes
 // element x of its output.  in_place: the output may overlap the input (every
 // read completes before the first write) and is complete for the group when the
-// pass returns.  tw(i) = omega_G^i.
+// pass returns.  tw(i, ns, m, k) = omega_G^i, i = k (G / (NS R)) 2^m: where it lies in
+// a table by passes, for tables laid out so.
 template <int R, int NS, int G, class Group, class Load, class Tw, class Store>
 __device__ __forceinline__ void stockham_pass(const Group& group, bool in_place, Load&& load, Tw&& tw, Store&& store) {
   // every thread holds exactly 16 values: 16 / R butterflies of radix R
@@ -186,25 +215,7 @@ __device__ __forceinline__ void stockham_pass(const Group& group, bool in_place,
     float2 x[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) x[r] = v[b * R + r];
-    if (NS > 1) {
-      // twiddles w^r, w = omega_G^base: w^(2^m) read, the others products of
-      // those (at most three roundings deep), so a pass reads log2 R of them
-      const int base = k * (G / (NS * R));
-      float2 t[R];
-      t[1] = tw(base);
-      if (R >= 4) t[2] = tw(2 * base);
-      if (R >= 8) t[4] = tw(4 * base);
-      if (R >= 16) t[8] = tw(8 * base);
-#pragma unroll
-      for (int r = 3; r < R; ++r) {
-        if ((r & (r - 1)) == 0) continue;
-        const int hb = 1 << (31 - __clz(r));            // highest power of two in r (compile-time)
-        t[r] = cmul(t[hb], t[r - hb]);
-      }
-#pragma unroll
-      for (int r = 1; r < R; ++r) x[r] = cmul(x[r], t[r]);
-    }
-    dft_reg<R>(x);
+    stockham_butterfly<R, NS, G>(x, k, tw);
     const int o = (j / NS) * NS * R + k;
 #pragma unroll
     for (int r = 0; r < R; ++r) store(f, o + r * NS, x[r]);
@@ -212,13 +223,54 @@ __device__ __forceinline__ void stockham_pass(const Group& group, bool in_place,
   if (in_place) group.sync();
 }
 
+// The last two passes at once, of radix 16 after NS points and of radix R after
+// 16 NS = G / R: the R butterflies whose outputs meet in the last pass are given to
+// lanes 32 / R apart and swap them by shuffles, which saves a trip through the
+// exchange buffer and its barriers (of radix 8 the outputs of a warp lie so far apart
+// that they cost as much).  The same arithmetic as the two passes.
+template <int R, int NS, int G, class Group, class Load, class Tw, class Store>
+__device__ __forceinline__ void stockham_tail(const Group& group, Load&& load, Tw&& tw, Store&& store) {
+  constexpr int per = G / 16, KK = 32 / R;
+  static_assert(per == NS * R && NS % KK == 0, "whole warps per row");
+  const int f = group.tid() / per, jj = group.tid() % per;
+  const int g = (jj & 31) / KK, k = (jj >> 5) * KK + (jj & (KK - 1)), j = g * NS + k;
+  float2 v[16];
+#pragma unroll
+  for (int r = 0; r < 16; ++r) v[r] = load(f, j + r * per, r);
+  stockham_butterfly<16, NS, G>(v, k, tw);
+  // R x R transposes: of v[i R + c] lane g keeps c = g, from every lane
+#pragma unroll
+  for (int bit = 1; bit < R; bit <<= 1) {
+    const bool up = (g & bit) != 0;
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      if (r & bit) continue;
+      const float2 send = up ? v[r] : v[r + bit];
+      const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, send.x, bit * KK),
+                                     __shfl_xor_sync(0xffffffffu, send.y, bit * KK));
+      if (up) v[r] = got;
+      else v[r + bit] = got;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 16 / R; ++i) {
+    const int k2 = k + (i * R + g) * NS;
+    float2 x[R];
+#pragma unroll
+    for (int c = 0; c < R; ++c) x[c] = v[i * R + c];
+    stockham_butterfly<R, 16 * NS, G>(x, k2, tw);
+#pragma unroll
+    for (int c = 0; c < R; ++c) store(f, k2 + c * 16 * NS, x[c]);
+  }
+}
+
 // Forward FFTs of rows of G = 2^LOG2G points, 16 <= G <= 16384, by a group of
 // threads with size * 16 == rows * G: radix-16 passes, then one of radix 2, 4 or
 // 8, exchanging through `a` (row f at a[f * ldp], element x at pad16(x)).  The
 // first pass reads its input through load0(f, x, slot) and may overlap `a`; the
-// last one hands its results to store(f, x, v): in_place when they overlap `a`.
-// tw(i) = omega_G^i.
-template <int LOG2G, class Group, class Load, class Tw, class Store>
+// last one hands its results to store(f, x, v): in_place when they overlap `a`, which
+// TAIL (the last two passes at once, where there are two and a shorter one) rules out.
+template <int LOG2G, bool TAIL, class Group, class Load, class Tw, class Store>
 __device__ __forceinline__ void fft_rows_io(const Group& group, float2* a, int ldp, bool in_place, Load&& load0,
                                             Tw&& tw, Store&& store) {
   constexpr int G = 1 << LOG2G;
@@ -235,14 +287,14 @@ __device__ __forceinline__ void fft_rows_io(const Group& group, float2* a, int l
     if constexpr (n16 == 2 && rem == 0) {
       stockham_pass<16, 16, G>(group, in_place, get, tw, store);
     } else {
-      if constexpr (n16 >= 2) stockham_pass<16, 16, G>(group, true, get, tw, put);
+      if constexpr (n16 == 3) stockham_pass<16, 16, G>(group, true, get, tw, put);
       if constexpr (n16 == 3 && rem == 0) {
         stockham_pass<16, 256, G>(group, in_place, get, tw, store);
+      } else if constexpr (n16 >= 2 && rem <= 2 && TAIL) {
+        stockham_tail<1 << rem, NSR / 16, G>(group, get, tw, store);
       } else {
-        if constexpr (n16 >= 3) stockham_pass<16, 256, G>(group, true, get, tw, put);
-        if constexpr (rem == 1) stockham_pass<2, NSR, G>(group, in_place, get, tw, store);
-        if constexpr (rem == 2) stockham_pass<4, NSR, G>(group, in_place, get, tw, store);
-        if constexpr (rem == 3) stockham_pass<8, NSR, G>(group, in_place, get, tw, store);
+        if constexpr (n16 >= 2) stockham_pass<16, NSR / 16, G>(group, true, get, tw, put);
+        stockham_pass<1 << rem, NSR, G>(group, in_place, get, tw, store);
       }
     }
   }
@@ -251,8 +303,9 @@ __device__ __forceinline__ void fft_rows_io(const Group& group, float2* a, int l
 // The same by the whole CTA, in place.
 template <int LOG2G, class Load, class Tw>
 __device__ void fft_rows_inplace_f(float2* a, int ldp, Load&& load0, Tw&& tw) {
-  fft_rows_io<LOG2G>(
-      CtaGroup{}, a, ldp, true, [&](int f, int x, int) { return load0(f, x); }, tw,
+  fft_rows_io<LOG2G, false>(
+      CtaGroup{}, a, ldp, true, [&](int f, int x, int) { return load0(f, x); },
+      [&](int i, auto, int, int) { return tw(i); },
       [&](int f, int x, float2 v) { a[f * ldp + pad16(x)] = v; });
 }
 

@@ -203,140 +203,218 @@ k_upchan(UpchanArgs a) {
   }
 }
 
-// Radix-16 Stockham kernel for N = 2^LOG2N >= 16 (fft.cuh's row passes): F
-// FFTs of the group in flight (F N = 8192 points, 16 per thread; one FFT of
-// 16384), exchange rows padded by one slot per 16 so the stride-16 writes of
-// a pass hit distinct banks, every index split a shift.  The first pass
-// unpacks the staged 4+4-bit samples; the last one requantises its bins,
-// fftshifted, into the staging rows straight from registers (through the exchange
-// buffer they cost a trip and a barrier more: with 704 inputs and 10 s 4096
-// points took 1.22 ms and now 1.10, 8192 points 1.47 and 1.40).
+// Radix-16 Stockham kernel for N = 2^LOG2N >= 16 (fft.cuh's row passes): F FFTs of
+// the group in flight (F N = 8192 points, 16 per thread; one FFT of 16384), exchange
+// rows padded by one slot per 16 so the stride-16 writes of a pass hit distinct
+// banks, every index split a shift.  The first pass unpacks the staged 4+4-bit
+// samples; the last one requantises its bins straight from registers.
+//
+// What bounds it is the load pipe, shared memory first, so every access is made to
+// be one wavefront:
+//  - a tile row per input (2 N bytes: first its packed samples, then, once they have
+//    been read, its int8 bins, fftshifted), so the threads of a pass touch
+//    consecutive bytes.  Rows are transposed four samples of four inputs at a time
+//    on the way in and two bins of four inputs on the way out; the row pitch spreads
+//    both over the banks.  With the inputs of a sample side by side half of all
+//    wavefronts were conflicts.
+//  - the twiddles of the passes after 16 and 256 points in shared memory, [m][k] =
+//    omega_N^(k 2^m N / (NS R)), as a warp reads them; from the global table they
+//    were scattered 8-byte reads.
+// With the samples in the bins' room two CTAs of 64 registers a thread share an SM;
+// from 2048 points they would hold too few inputs each for the rows to coalesce
+// (and spill), so there it is one with 128.  704 inputs x 240000 samples: 8192
+// points 1.40 -> 1.09 ms, 4096 1.06 -> 0.76, 1024 1.05 -> 0.61, 16384 3.0 -> 1.8 (the
+// power pass left out).
 template <int LOG2N>
 struct P2Plan {
   static constexpr int N = 1 << LOG2N;
   static constexpr int F = N >= 8192 ? 1 : 8192 / N;
   static constexpr int THREADS = F * N / 16;
+  static constexpr int CTAS = LOG2N < 11 ? 2 : 1;    // per SM
   static constexpr int LDP = N + N / 16;             // pad16(x) < LDP for x < N
+  static constexpr int TW16 = LOG2N > 4 ? 16 * (LOG2N < 8 ? LOG2N - 4 : 4) : 0;
+  static constexpr int TW256 = LOG2N > 8 ? 256 * (LOG2N < 12 ? LOG2N - 8 : 4) : 0;
 };
+
+// Bytes from one input's row of the tile to the next: lanes of four (or two) inputs
+// side by side and consecutive words of their rows hit distinct banks.
+__host__ __device__ inline int tile_pitch(int n, int G) { return 2 * n + 4 * (G < 32 ? 32 / G : 1); }
+
+// Packed samples of the inputs of one CTA, sizeof(W) inputs and four rows of them at a
+// time, transposed into the tile.
+template <class W>
+__device__ __forceinline__ void stage_samples(const uint8_t* __restrict__ src, long long row, int n, int lg, int gv,
+                                              uint8_t* tile, int pitch) {
+  constexpr int I = sizeof(W), LI = I == 4 ? 2 : I == 2 ? 1 : 0, U = 2;
+  const int sh = lg - LI, items = n / 4 << sh, T = blockDim.x;
+  for (int i1 = threadIdx.x; i1 < items; i1 += U * T) {
+    uint32_t v[U][4];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int idx = i1 + u * T, q = idx >> sh, g = (idx & ((1 << sh) - 1)) << LI;
+      const uint8_t* p = src + 4 * q * row + g;
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        v[u][j] = idx < items && g < gv ? static_cast<uint32_t>(*reinterpret_cast<const W*>(p + j * row)) : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int idx = i1 + u * T, q = idx >> sh, g = (idx & ((1 << sh) - 1)) << LI;
+      if (idx >= items) continue;
+#pragma unroll
+      for (int i = 0; i < I; ++i) {
+        const uint32_t lo = __byte_perm(v[u][0], v[u][1], i | (4 + i) << 4);
+        const uint32_t hi = __byte_perm(v[u][2], v[u][3], i | (4 + i) << 4);
+        *reinterpret_cast<uint32_t*>(tile + (g + i) * pitch + 4 * q) = __byte_perm(lo, hi, 0x5410);
+      }
+    }
+  }
+}
+
+// The tile's bins to rows of 2 G bytes, I inputs of two bins at a time.
+template <int I>
+__device__ __forceinline__ void write_bins(const uint8_t* tile, int pitch, int n, int lg, int gv, int8_t* dst,
+                                           long long row) {
+  constexpr int LI = I == 4 ? 2 : I == 2 ? 1 : 0;
+  const int sh = lg - LI, items = n / 2 << sh, T = blockDim.x;
+#pragma unroll 4
+  for (int idx = threadIdx.x; idx < items; idx += T) {
+    const int p = idx >> sh, g = (idx & ((1 << sh) - 1)) << LI;
+    if (g >= gv) continue;
+    uint32_t b[I];
+#pragma unroll
+    for (int i = 0; i < I; ++i) b[i] = *reinterpret_cast<const uint32_t*>(tile + (g + i) * pitch + 4 * p);
+    int8_t* d = dst + 2 * p * row + 2 * g;
+    if constexpr (I == 1) {
+      *reinterpret_cast<uint16_t*>(d) = static_cast<uint16_t>(b[0]);
+      *reinterpret_cast<uint16_t*>(d + row) = static_cast<uint16_t>(b[0] >> 16);
+    } else if constexpr (I == 2) {
+      *reinterpret_cast<uint32_t*>(d) = __byte_perm(b[0], b[1], 0x5410);
+      *reinterpret_cast<uint32_t*>(d + row) = __byte_perm(b[0], b[1], 0x7632);
+    } else {
+      *reinterpret_cast<uint2*>(d) = make_uint2(__byte_perm(b[0], b[1], 0x5410), __byte_perm(b[2], b[3], 0x5410));
+      *reinterpret_cast<uint2*>(d + row) = make_uint2(__byte_perm(b[0], b[1], 0x7632), __byte_perm(b[2], b[3], 0x7632));
+    }
+  }
+}
 
 // F32: FP32 spectra are asked for as well; known when compiled, as the test in the
 // last pass cost the transforms without them 2 to 4%.
 template <int LOG2N, bool F32>
-__global__ void __launch_bounds__(P2Plan<LOG2N>::THREADS, 1024 / P2Plan<LOG2N>::THREADS)
+__global__ void __launch_bounds__(P2Plan<LOG2N>::THREADS, P2Plan<LOG2N>::CTAS)
 k_upchan_p2(UpchanArgs a) {
   using P = P2Plan<LOG2N>;
-  constexpr int N = P::N, F = P::F, LDP = P::LDP;
+  constexpr int N = P::N, F = P::F;
+  // FP32 rows leave by F inputs at a time, in full sectors from F = 4 (1024 points x
+  // 574 inputs x 303090 samples: 2.5 -> 1.02 ms); one slot more, so that those hit
+  // distinct banks
+  constexpr bool wide = F32 && F > 1;
+  constexpr int LDP = P::LDP + (wide ? 1 : 0);
   extern __shared__ __align__(16) unsigned char smem[];
-  const int G = a.group;
+  const int G = a.group, lg = 31 - __clz(G);    // G is a power of two
+  const int pitch = tile_pitch(N, G);
   float2* buf = reinterpret_cast<float2*>(smem);                                 // [F][LDP]
-  uint8_t* raw = smem + static_cast<size_t>(F) * LDP * sizeof(float2);           // [N][G]
-  int8_t* stg = reinterpret_cast<int8_t*>(raw + static_cast<size_t>(N) * G);     // [N][G][2]
-  float* sc = reinterpret_cast<float*>(
-      stg + ((static_cast<size_t>(N) * G * 2 + 15) & ~static_cast<size_t>(15)));  // [G]
+  float2* tws = buf + F * LDP;
+  float* sc = reinterpret_cast<float*>(tws + P::TW16 + P::TW256);                // [G]
+  uint8_t* tile = reinterpret_cast<uint8_t*>(sc + G);                            // [G][pitch]
   const int tid = threadIdx.x;
   const int T = blockDim.x;
   const int s = blockIdx.y;
   const int i0 = blockIdx.x * G;
   const int gv = min(G, a.n_input - i0);        // valid inputs in this group
-  const long long row0 = static_cast<long long>(s) * N;
+  const int tw_stride = a.tw_n / N;
+  for (int i = tid; i < P::TW16 + P::TW256; i += T) {
+    const int NS = i < P::TW16 ? 16 : 256, x = i < P::TW16 ? i : i - P::TW16;
+    const int left = N / NS;                    // points left: a pass of radix 16, or the last one
+    tws[i] = __ldg(a.tw + ((x & (NS - 1)) * (left >= 16 ? left / 16 : 1) << (x / NS)) * tw_stride);
+  }
+  for (int g = tid; g < G; g += T) sc[g] = g < gv ? a.scale[i0 + g] : 0.0f;
   {
-    const uint8_t* src = a.volt + row0 * a.n_input + i0;
-    auto words = [&](auto word) {
-      using W = decltype(word);
-      const int wpr = G / sizeof(W);
-      for (int idx = tid; idx < N * wpr; idx += T) {
-        const int n = idx / wpr, w = idx - n * wpr;
-        reinterpret_cast<W*>(raw)[idx] =
-            *reinterpret_cast<const W*>(src + static_cast<long long>(n) * a.n_input + sizeof(W) * w);
-      }
-    };
+    const uint8_t* src = a.volt + static_cast<long long>(s) * N * a.n_input + i0;
     const uintptr_t al = reinterpret_cast<uintptr_t>(a.volt) | a.n_input | G;   // where rows and groups start
-    if (gv == G && (al & 3) == 0) {
-      words(uint32_t{});
-    } else if (gv == G && (al & 1) == 0) {
-      words(uint16_t{});
-    } else {
-      for (int idx = tid; idx < N * G; idx += T) {
-        const int n = idx / G, g = idx - n * G;
-        raw[idx] = g < gv ? src[static_cast<long long>(n) * a.n_input + g] : 0;
-      }
-    }
-    for (int g = tid; g < G; g += T) sc[g] = g < gv ? a.scale[i0 + g] : 0.0f;
+    if ((al & 3) == 0)
+      stage_samples<uint32_t>(src, a.n_input, N, lg, gv, tile, pitch);
+    else if ((al & 1) == 0)
+      stage_samples<uint16_t>(src, a.n_input, N, lg, gv, tile, pitch);
+    else
+      stage_samples<uint8_t>(src, a.n_input, N, lg, gv, tile, pitch);
   }
   __syncthreads();
-  const int tw_stride = a.tw_n / N;
-  auto tw = [&](int i) { return __ldg(a.tw + static_cast<long long>(i) * tw_stride); };
-  for (int f0 = 0; f0 < G; f0 += F) {
-    fft_rows_io<LOG2N>(
-        CtaGroup{}, buf, LDP, false,
-        [&](int f, int x, int) {
-          // high nibble real, low nibble imaginary (two's complement)
-          float2 v = make_float2(0.f, 0.f);
-          const int g = f0 + f;
-          if (g < G) {
-            const uint32_t byte = raw[x * G + g];
-            v.x = static_cast<float>(static_cast<int>(static_cast<int8_t>(byte)) >> 4);
-            v.y = static_cast<float>(static_cast<int>(static_cast<int8_t>(byte << 4)) >> 4);
-          }
-          return v;
-        },
-        tw,
-        [&](int f, int k, float2 X) {
-          const int g = f0 + f;
-          if (g >= gv) return;
-          const float s_g = sc[g];
-          const int kp = (k + N / 2) & (N - 1);
-          float qr = rintf(__fmul_rn(s_g, X.x));
-          float qi = rintf(__fmul_rn(s_g, X.y));
-          qr = fminf(fmaxf(qr, -127.f), 127.f);
-          qi = fminf(fmaxf(qi, -127.f), 127.f);
-          char2 q2;
-          q2.x = static_cast<signed char>(qr);
-          q2.y = static_cast<signed char>(qi);
-          reinterpret_cast<char2*>(stg)[kp * G + g] = q2;
-          if constexpr (F32) {
-            const long long o = ((static_cast<long long>(kp) * a.n_spec + s) * a.n_input + i0 + g);
-            reinterpret_cast<float2*>(a.out_f)[o] = X;
-          }
-        });
-    __syncthreads();   // buf reused by the next F inputs; stg complete
-  }
-  {
-    int8_t* dst0 = a.out_q + (static_cast<long long>(s) * a.n_input + i0) * 2;
-    const long long row_stride = static_cast<long long>(a.n_spec) * a.n_input * 2;
-    // 4-byte words per row: the rows of an even number of inputs start on one
-    if (gv == G && (G % 2) == 0 && (a.n_input % 2) == 0 && (reinterpret_cast<uintptr_t>(a.out_q) & 3) == 0) {
-      const int wpr = G / 2;
-      for (int idx = tid; idx < N * wpr; idx += T) {
-        const int kp = idx / wpr, w = idx - kp * wpr;
-        *reinterpret_cast<uint32_t*>(dst0 + kp * row_stride + 4 * w) =
-            reinterpret_cast<const uint32_t*>(stg)[idx];
+  auto tw = [&](int i, auto ns, int m, int k) {
+    if constexpr (decltype(ns)::value == 16) return tws[m * 16 + k];
+    if constexpr (decltype(ns)::value == 256) return tws[P::TW16 + m * 256 + k];
+    return __ldg(a.tw + i * tw_stride);
+  };
+  for (int f0 = 0; f0 < gv; f0 += F) {
+    auto sample = [&](int f, int x, int) {
+      // high nibble real, low nibble imaginary (two's complement)
+      float2 v = make_float2(0.f, 0.f);
+      const int g = f0 + f;
+      if (g < G) {
+        const uint32_t byte = tile[g * pitch + x];
+        v.x = static_cast<float>(static_cast<int>(static_cast<int8_t>(byte)) >> 4);
+        v.y = static_cast<float>(static_cast<int>(static_cast<int8_t>(byte << 4)) >> 4);
+      }
+      return v;
+    };
+    auto bin = [&](int f, int k, float2 X) {
+      const int g = f0 + f;
+      if (g >= gv) return;
+      const float s_g = sc[g];
+      const int kp = (k + N / 2) & (N - 1);
+      float qr = rintf(__fmul_rn(s_g, X.x));
+      float qi = rintf(__fmul_rn(s_g, X.y));
+      qr = fminf(fmaxf(qr, -127.f), 127.f);
+      qi = fminf(fmaxf(qi, -127.f), 127.f);
+      char2 q2;
+      q2.x = static_cast<signed char>(qr);
+      q2.y = static_cast<signed char>(qi);
+      *reinterpret_cast<char2*>(tile + g * pitch + 2 * kp) = q2;
+      if constexpr (F32) {
+        const long long o = ((static_cast<long long>(kp) * a.n_spec + s) * a.n_input + i0 + g);
+        reinterpret_cast<float2*>(a.out_f)[o] = X;
+      }
+    };
+    if constexpr (wide) {
+      // through the exchange buffer: F neighbouring inputs make a row of 8 F bytes
+      fft_rows_io<LOG2N, false>(CtaGroup{}, buf, LDP, true, sample, tw,
+                                [&](int f, int k, float2 X) { buf[f * LDP + pad16(k)] = X; });
+#pragma unroll 8
+      for (int idx = tid; idx < F * N; idx += P::THREADS) {
+        const int f = idx % F, k = idx / F;
+        bin(f, k, buf[f * LDP + pad16(k)]);
       }
     } else {
-      for (int idx = tid; idx < N * gv; idx += T) {
-        const int kp = idx / gv, g = idx - kp * gv;
-        *reinterpret_cast<char2*>(dst0 + kp * row_stride + 2 * g) =
-            reinterpret_cast<const char2*>(stg)[kp * G + g];
-      }
+      // one pass alone: its bins overlap its samples
+      fft_rows_io<LOG2N, true>(CtaGroup{}, buf, LDP, LOG2N == 4, sample, tw, bin);
     }
+    __syncthreads();       // buf reused by the next F inputs, the bins complete
   }
+  int8_t* dst = a.out_q + (static_cast<long long>(s) * a.n_input + i0) * 2;
+  const long long row = static_cast<long long>(a.n_spec) * a.n_input * 2;
+  const uintptr_t al = reinterpret_cast<uintptr_t>(a.out_q) | 2 * a.n_input | 2 * G;
+  if ((al & 7) == 0)
+    write_bins<4>(tile, pitch, N, lg, gv, dst, row);
+  else if ((al & 3) == 0)
+    write_bins<2>(tile, pitch, N, lg, gv, dst, row);
+  else
+    write_bins<1>(tile, pitch, N, lg, gv, dst, row);
 }
 
 size_t smem_p2(int log2n, int G) {
   const int N = 1 << log2n;
   const int F = N >= 8192 ? 1 : 8192 / N;
-  return static_cast<size_t>(F) * (N + N / 16) * 8 + static_cast<size_t>(N) * G +
-         ((static_cast<size_t>(N) * G * 2 + 15) & ~static_cast<size_t>(15)) + 4 * G + 16;
+  return static_cast<size_t>(F) * (N + N / 16 + (F > 1 ? 1 : 0)) * 8 + (log2n > 8 ? 1088 : 64) * sizeof(float2) + 4 * G +
+         static_cast<size_t>(G) * tile_pitch(N, G);
 }
 
 size_t smem_for(int log2n, int G);
 
 int group_for(int log2n, int n_input) {
-  // G inputs per CTA: the most whose shared memory (raw G N + staging 2 G N +
-  // exchange) fits one CTA per SM, at least F (wider groups coalesce the
-  // G-byte row reads and 2G-byte row writes)
+  // G inputs per CTA: the most that leave room for the CTAs planned per SM, at least F (wider groups coalesce the G-byte
+  // row reads and 2G-byte row writes)
   const int F = log2n >= 13 ? 1 : (log2n < 4 ? 256 : (8192 >> log2n));
-  const size_t budget = 200 * 1024;
+  const size_t budget = (log2n >= 4 && log2n < 11 ? 112 : 224) * 1024;
   int G = 1;
   while (G < 64 && smem_for(log2n, 2 * G) <= budget) G *= 2;
   if (G < F) G = F;
@@ -412,6 +490,7 @@ int launch_upchan_tuned(int l, UpchanArgs a, cudaStream_t st) {
   int g = tuned(key, g0);
   if (tuning(st) && cands.size() > 1)
     if (int e = tune_pick(key, cands, run, st, &g)) return e;
+  if (l >= 4 && (g <= 0 || (g & (g - 1)) || smem_for(l, g) > (size_t(227) << 10))) g = g0;
   return run(g);
 }
 

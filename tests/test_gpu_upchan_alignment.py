@@ -30,3 +30,24 @@ def test_rows_off_a_word(lib, nfft, n_input, shift):
             assert torch.equal(w, b[off_n:off_n + n * k * n_input * 2].view(n, k, n_input, 2))
         off_w += n * k * wide * 2
         off_n += n * k * n_input * 2
+
+
+@pytest.mark.parametrize("n_input", [3, 20])
+@pytest.mark.parametrize("log2n", range(4, 15))
+def test_every_power_of_two_both_ways(lib, log2n, n_input):
+    """The int8 spectra are the same whether FP32 ones are asked for or not (the
+    last passes differ), and the FP32 ones those of an FP64 transform.  Four passes,
+    each at most 4 additions and 6 roundings of twiddles and their products deep:
+    ||error|| <= 4 * 10 * 2^-24 ||X||."""
+    n = 1 << log2n
+    g = torch.Generator(device="cuda")
+    g.manual_seed(log2n)
+    v = torch.randint(0, 256, (1, 2 * n + 1, n_input), generator=g, device="cuda", dtype=torch.int16).to(torch.uint8)
+    q, f = lib.upchan(v, [n], want_f32=True)
+    q1, _ = lib.upchan(v, [n])
+    assert torch.equal(q, q1)
+    b = v[0, :2 * n].to(torch.int64).view(2, n, n_input)
+    x = torch.complex(((b >> 4) ^ 8).double() - 8, ((b & 15) ^ 8).double() - 8)
+    want = torch.fft.fftshift(torch.fft.fft(x, dim=1), dim=1).permute(1, 0, 2)
+    got = torch.view_as_complex(f.double().view(n, 2, n_input, 2).contiguous())
+    assert float((got - want).norm()) <= 40 * 2.0 ** -24 * float(want.norm())
