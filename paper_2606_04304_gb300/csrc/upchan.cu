@@ -540,6 +540,7 @@ int ovro_upchan_ex(const uint8_t* d_volt, int n_input, int n_coarse, int64_t n_t
   struct Coarse {
     int n, cnt, k;
     bool mixed;
+    MrPlan plan;                     // mixed only
   };
   std::vector<Coarse> cs(n_coarse);
   int max_pow2 = 2;
@@ -556,10 +557,9 @@ int ovro_upchan_ex(const uint8_t* d_volt, int n_input, int n_coarse, int64_t n_t
     if (static_cast<long long>(lo) + e.cnt > e.n) return OVRO_ERR_INVALID_ARG;
     e.mixed = taps || lo != 0 || e.cnt != e.n || !is_pow2(e.n) || e.n > kMaxN || k > 65535;
     if (e.mixed) {
-      MrPlan plan;
       int group = 0;
       size_t smem = 0;
-      if (!mr_plan(e.n, n_input, taps ? n_tap : 1, e.cnt, &plan, &group, &smem)) return OVRO_ERR_UNSUPPORTED;
+      if (!mr_plan(e.n, n_input, taps ? n_tap : 1, e.cnt, &e.plan, &group, &smem)) return OVRO_ERR_UNSUPPORTED;
     } else {
       if (e.n < 2) return OVRO_ERR_UNSUPPORTED;
       max_pow2 = std::max(max_pow2, e.n);
@@ -577,7 +577,8 @@ int ovro_upchan_ex(const uint8_t* d_volt, int n_input, int n_coarse, int64_t n_t
   } else {
     OVRO_CUDA_TRY(cudaMemsetAsync(w.power, 0, nsc * sizeof(unsigned long long), st));
   }
-  int table_n = 0;   // omega_{table_n}^k currently in w.tw
+  int table_n = 0;   // length of the table in w.tw
+  bool table_mr = false;   // by passes, else omega_{table_n}^k
   long long q_off = 0;
   for (int c = 0; c < n_coarse; ++c) {
     const Coarse& e = cs[c];
@@ -616,14 +617,18 @@ int ovro_upchan_ex(const uint8_t* d_volt, int n_input, int n_coarse, int64_t n_t
         n_used, taps ? w.h2 + c : nullptr, w.scale + static_cast<size_t>(c) * n_input);
     OVRO_LAUNCH_CHECK();
 
-    // twiddles: exactly omega_N for the mixed-radix kernel; any power-of-two
-    // table at least N long for the radix-16 kernel
-    const int want = e.mixed ? n : max_pow2;
-    const bool ok = e.mixed ? table_n == n : (is_pow2(table_n) && table_n >= n);
+    // twiddles: those of the plan's passes for the mixed-radix kernel; any
+    // power-of-two table at least N long for the radix-16 kernel
+    const bool ok = table_mr == e.mixed && (e.mixed ? table_n == n : table_n >= n);
     if (!ok) {
-      k_twiddle<<<(want + 255) / 256, 256, 0, st>>>(w.tw, want);
-      OVRO_LAUNCH_CHECK();
-      table_n = want;
+      table_n = e.mixed ? n : max_pow2;
+      table_mr = e.mixed;
+      if (e.mixed) {
+        if (int err = launch_twiddle_mr(w.tw, e.plan, st)) return err;
+      } else {
+        k_twiddle<<<(table_n + 255) / 256, 256, 0, st>>>(w.tw, table_n);
+        OVRO_LAUNCH_CHECK();
+      }
     }
 
     UpchanArgs a;
