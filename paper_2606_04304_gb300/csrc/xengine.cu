@@ -504,10 +504,22 @@ k_xeng_tc3(const int8_t* __restrict__ q, int n_ant, int n_spec, int n_tiles, int
 // 0..127 and Im in 128..255 against A = X rows of tile I.  Two 256-column
 // accumulators alternate: the MMAs of tile pair t+1 run while the epilogue
 // drains pair t.  The next channel's spectra are prefetched into L2.
-constexpr int kV2Threads = 256;
+// 16 warps drain an accumulator, 32 rows by 32 column inputs each: bound by the writing
+// of the records, whose latency 8 warps left open (352 antennas, 2048 channels x 29
+// spectra, 4.1 GB: 917 us with 8, 891 with whole() for the conversion unit, 800 with 16).
+// Whole 32-byte records from each lane by a swap between neighbours were slower (1.13
+// ms), and so were stores without the streaming hint (1.06 ms).
+constexpr int kV2Threads = 512;
 constexpr int kV2MaxTiles = 6;
 constexpr int kV2TileBytes = 2 * kTcM * kTcKc * 2;        // 32 KB: X rows then Z rows
 constexpr uint32_t kV2TmemCols = 512;
+
+// An integer below 2^22 in magnitude (K <= 32: at most 2^20) held in FP32, as int32:
+// an addition and a subtraction, where the conversion unit takes a quarter of the lanes
+// a cycle.
+__device__ __forceinline__ int whole(uint32_t f) {
+  return __float_as_int(__uint_as_float(f) + 12582912.f) - 0x4B400000;
+}
 
 __global__ void __launch_bounds__(kV2Threads, 1)
 k_xeng_tc2(const int8_t* __restrict__ q, int n_ant, int n_spec, int n_tiles, int n_chan, int prefetch,
@@ -620,8 +632,7 @@ k_xeng_tc2(const int8_t* __restrict__ q, int n_ant, int n_spec, int n_tiles, int
         int4* out = reinterpret_cast<int4*>(vis + static_cast<long long>(ch) * n_bl * 8);
         const uint32_t cb = static_cast<uint32_t>((t & 1) * 256);
 #pragma unroll 1
-        for (int hh = 0; hh < 2; ++hh) {
-          const int cin0 = wg * 64 + hh * 32;     // column inputs cin0 .. cin0 + 31
+        for (int cin0 = wg * 32; cin0 < kTcInputsN; cin0 += kV2Threads / 4) {     // column inputs cin0 .. cin0 + 31
           uint32_t re[32], im[32];
           const uint32_t tl = tmem + (static_cast<uint32_t>(q4 * 32) << 16) + cb + cin0;
           asm volatile(
@@ -652,10 +663,10 @@ k_xeng_tc2(const int8_t* __restrict__ q, int n_ant, int n_spec, int n_tiles, int
               const int b = b0 + bb;
               if (b >= n_ant || b < a) continue;
               int4 v;
-              v.x = __float2int_rn(__uint_as_float(re[2 * bb]));
-              v.y = __float2int_rn(__uint_as_float(im[2 * bb]));
-              v.z = __float2int_rn(__uint_as_float(re[2 * bb + 1]));
-              v.w = __float2int_rn(__uint_as_float(im[2 * bb + 1]));
+              v.x = whole(re[2 * bb]);
+              v.y = whole(im[2 * bb]);
+              v.z = whole(re[2 * bb + 1]);
+              v.w = whole(im[2 * bb + 1]);
               __stcs(out + bl_index(a, b, n_ant) * 2 + pa, v);
             }
           }
