@@ -116,7 +116,7 @@ def write_traffic_table(case, csv_path, command):
     # the upchannelizer's radix-16 kernel and the band ranks are traced under
     # the stage's kernel name)
     alias = {"k_xeng_tc2": "k_xeng_tc", "k_xeng_tc3": "k_xeng_tc", "k_upchan_p2": "k_upchan",
-             "k_rank_band": "k_rank"}
+             "k_upchan_mr_wide": "k_upchan_mr", "k_rank_band": "k_rank"}
     rows = [(lid, alias.get(k, k), m, v) for lid, k, m, v in _ncu_rows(csv_path)]
     if not rows:
         raise SystemExit(f"no kernel metrics in {csv_path}")
