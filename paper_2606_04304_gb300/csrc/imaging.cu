@@ -136,7 +136,7 @@ __global__ void k_uvw(const Baseline* __restrict__ base, int n_cross, const Chan
 }
 
 // device counters of one call's plan (ImgWs::counts)
-constexpr int kCountListed = 0, kCountRows = 1, kCountTiles = 2, kCountSlots = 3, kCountHeavy = 4, kCounts = 5;
+constexpr int kCountListed = 0, kCountRows = 1, kCountSlots = 2, kCountHeavy = 3, kCounts = 4;
 
 struct GridEntry {
   int bl;            // baseline index in the visibility record
@@ -1044,6 +1044,15 @@ struct PlanAxis {
   double w_lo, w_hi;          // wavelengths per metre
   double uv_min, uv_max;
   int uv_cut;
+  // a baseline of l0 .. l1 wavelengths is outside the uv range in every channel,
+  // or inside in every one, with a relative margin
+  static constexpr double kEps = 1e-9;
+  __host__ __device__ bool uv_outside(double l0, double l1) const {
+    return l1 < uv_min * (1.0 - kEps) || l0 >= uv_max * (1.0 + kEps);
+  }
+  __host__ __device__ bool uv_inside(double l0, double l1) const {
+    return l0 >= uv_min * (1.0 + kEps) && l1 < uv_max * (1.0 - kEps);
+  }
 };
 
 // Centre cells of a cross baseline over the call's channels, and whether the
@@ -1104,9 +1113,9 @@ k_plan_baselines(const double* __restrict__ ant, int n_ant, long long n_cross, i
     if (live && ax.uv_cut) {
       // decided here when every channel of the call agrees (with a relative
       // margin), per channel when the records are prepared otherwise
-      const double l0 = __dmul_rn(L, ax.w_lo), l1 = __dmul_rn(L, ax.w_hi), eps = 1e-9;
-      if (l1 < ax.uv_min * (1.0 - eps) || l0 >= ax.uv_max * (1.0 + eps)) live = false;
-      r.check = !(l0 >= ax.uv_min * (1.0 + eps) && l1 < ax.uv_max * (1.0 - eps));
+      const double l0 = __dmul_rn(L, ax.w_lo), l1 = __dmul_rn(L, ax.w_hi);
+      if (ax.uv_outside(l0, l1)) live = false;
+      r.check = !ax.uv_inside(l0, l1);
     }
     if (!live) {
       r.u0 = 0;
@@ -1215,8 +1224,8 @@ k_plan_rows(const PlanRange* __restrict__ lrng, int g, unsigned long long* __res
     total += wcnt[w];
   }
   if (threadIdx.x == 0) {
-    // counts[kCountRows] may pass the capacity: the row stays empty then and
-    // the host reports the plan as too large
+    // (a plan that does not fit was refused on the host: the test only keeps
+    // every store inside the buffer)
     const unsigned long long s = atomicAdd(counts + kCountRows, static_cast<unsigned long long>(total));
     start = s + total <= static_cast<unsigned long long>(cap) ? static_cast<int>(s) : -1;
     row_rng[tv] = start < 0 ? make_int2(0, 0) : make_int2(start, start + total);
@@ -1276,16 +1285,14 @@ k_plan_tiles(const int2* __restrict__ row_ent, const int2* __restrict__ row_rng,
 #pragma unroll
     for (int u = 0; u < kTilesPerWarp; ++u) c[u] += __popc(__ballot_sync(full, u >= lo && u <= hi));
   }
-  int start[kTilesPerWarp], slots = 0, entries = 0;
+  int start[kTilesPerWarp], slots = 0;
 #pragma unroll
   for (int u = 0; u < kTilesPerWarp; ++u) {
     start[u] = slots;
     slots += (c[u] + 3) & ~3;
-    entries += c[u];
   }
   int base = 0;
-  if (lane == 0 && entries) {
-    atomicAdd(counts + kCountTiles, static_cast<unsigned long long>(entries));
+  if (lane == 0 && slots) {
     const unsigned long long s = atomicAdd(counts + kCountSlots, static_cast<unsigned long long>(slots));
     base = s + slots <= static_cast<unsigned long long>(cap) ? static_cast<int>(s) : -1;
   }
@@ -1494,15 +1501,70 @@ int run_batch(const ImgPlan& p, const ImgWs& w, const GridOpts& o, const int32_t
   }
 }
 
-// The call's tables and lists, all made on the device.  bases: the prepared
-// records may hold weight-table offsets, because no listed footprint moves by
-// kTabMargin cells over the call's channels: a listed |d| s is below
-// (cmax + 1) Q at the smallest scale, so a centre moves by at most
-// (cmax + 1) (s_hi / s_lo - 1) + 1 cells; one more cell of slack for a
-// rounding of u Q that differs from the exact one.  A footprint that moves by
-// at most two cells touches 3 x 3 tiles, its mirror as many: 18 entries, within
-// the capacity of 24; a call over a wider band waits for its count and is
-// refused when it does not fit.
+// What a call over a wide band needs to know before anything is launched: the
+// most cells a listed footprint moves over the channels, and the tile list
+// entries there will be.  FP64 as in k_plan_baselines, k_plan_rows and
+// k_plan_tiles (host code is built without FMA contraction), so the two agree.
+struct PlanExtent {
+  int move = 0;
+  long long entries = 0;
+};
+
+PlanExtent plan_extent(int g, int n_ant, const double* ant, const PlanAxis& ax) {
+  PlanExtent out;
+  const int half = g / 2, cmax = half - kHalfSup - 1;
+  // a baseline that reaches past the grid at the smallest scale is never listed
+  const double reach = ax.s_lo > 0.0 ? (cmax + 1.0) * kQ / ax.s_lo : HUGE_VAL;
+  // centre cell of a product d s: rint by the addition of 1.5 2^52 (products far off
+  // the grid are held at 2^40), then half away from zero
+  auto centre = [](double v) {
+    constexpr double kRint = 6755399441055744.0, kFar = 1099511627776.0;
+    const double p = (std::min(std::max(v, -kFar), kFar) + kRint) - kRint;
+    return static_cast<int>((p + std::copysign(kQ / 2.0, p)) * (1.0 / kQ));
+  };
+  // tiles of the rows kept that centre rows v0 .. v1 and columns u0 .. u1 touch
+  auto tiles = [&](int v0, int v1, int u0, int u1) -> long long {
+    if (v1 + kHalfSup < 0) return 0;
+    const unsigned r = static_cast<unsigned>(v1 + kHalfSup) / kTileV - static_cast<unsigned>(std::max(0, v0 - kHalfSup)) / kTileV + 1;
+    const unsigned c = static_cast<unsigned>(half + u1 + kHalfSup) / kTileU - static_cast<unsigned>(half + u0 - kHalfSup) / kTileU + 1;
+    return r * c;
+  };
+  std::vector<double> x(n_ant), y(n_ant);
+  for (int a = 0; a < n_ant; ++a) {
+    x[a] = ant[3 * a];
+    y[a] = ant[3 * a + 1];
+  }
+  for (int a = 0; a < n_ant; ++a)
+    for (int b = a + 1; b < n_ant; ++b) {
+      const double dx = x[a] - x[b], dy = y[a] - y[b];
+      if (!(std::fabs(dx) <= reach && std::fabs(dy) <= reach)) continue;
+      const int ua = centre(dx * ax.s_lo), ub = centre(dx * ax.s_hi), va = centre(dy * ax.s_lo), vb = centre(dy * ax.s_hi);
+      const int u0 = std::max(std::min(ua, ub), -cmax), u1 = std::min(std::max(ua, ub), cmax);
+      const int v0 = std::max(std::min(va, vb), -cmax), v1 = std::min(std::max(va, vb), cmax);
+      if (u0 > u1 || v0 > v1) continue;
+      if (ax.uv_cut) {
+        const double x2 = dx * dx, y2 = dy * dy, len = std::sqrt(x2 + y2);
+        if (ax.uv_outside(len * ax.w_lo, len * ax.w_hi)) continue;
+      }
+      out.move = std::max(out.move, std::max(std::abs(ub - ua), std::abs(vb - va)));
+      out.entries += tiles(v0, v1, u0, u1) + tiles(-v1, -v0, -u1, -u0);
+    }
+  return out;
+}
+
+// The call's tables and lists, made on the device without a synchronisation.
+// bases: the prepared records may hold weight-table offsets, because no listed
+// footprint moves by kTabMargin cells over the call's channels (one cell of
+// slack for a rounding of u Q that differs from the exact one).  A listed
+// |d| s is below (cmax + 1) Q at the smallest scale, so no centre moves by more
+// than (cmax + 1) (s_hi / s_lo - 1) + 1 cells; a footprint that moves by at most
+// two touches 3 x 3 tiles, its mirror as many: 18 entries, within the capacity
+// of 24, and there is nothing more to know.  Over a wider band (60 kHz at 1024^2
+// and 60 MHz) the array itself decides, on the host: waiting for the device's
+// counts took the call's asynchrony, and the bound alone kept compact arrays from
+// the faster records.  352 antennas, 512 channels over 512 kHz at 256^2: the call
+// returns after 0.5 ms and is done after 1.7 (with the wait 1.4); the same array
+// ten times smaller 6.6 ms (general records 8.4).
 int upload_common(const ImgPlan& p, ImgWs& w, int n_ant, const double* h_ant,
                   const double* h_freq, int n_chan, double cell, cudaStream_t st,
                   double uv_min = 0.0, double uv_max = HUGE_VAL) {
@@ -1530,7 +1592,12 @@ int upload_common(const ImgPlan& p, ImgWs& w, int n_ant, const double* h_ant,
   ax.uv_max = uv_max;
   ax.uv_cut = uv_min > 0.0 || std::isfinite(uv_max);
   const int cmax = p.g / 2 - kHalfSup - 1;
-  const double move = ax.s_lo > 0.0 ? (cmax + 1) * (ax.s_hi / ax.s_lo - 1.0) + 1.0 : HUGE_VAL;
+  double move = ax.s_lo > 0.0 ? (cmax + 1) * (ax.s_hi / ax.s_lo - 1.0) + 1.0 : HUGE_VAL;
+  if (!(move <= 2.0)) {
+    const PlanExtent e = plan_extent(p.g, n_ant, h_ant, ax);
+    if (e.entries > entry_capacity(p)) return OVRO_ERR_CAPACITY;
+    move = e.move;
+  }
   w.bases = move + 1.0 <= kTabMargin;
   const double* d_ant = w.axis;
   const double* d_freq = w.axis + 3 * static_cast<size_t>(n_ant);
@@ -1556,13 +1623,6 @@ int upload_common(const ImgPlan& p, ImgWs& w, int n_ant, const double* h_ant,
   k_plan_tiles<<<(nt + per_cta - 1) / per_cta, kTileListWarps * 32, 0, st>>>(
       w.row_ent, w.row_rng, n_tiles_u(p.g), nt, w.counts, w.tile_idx, slot_capacity(p), w.tile_rng, w.heavy);
   OVRO_LAUNCH_CHECK();
-  if (!(move <= 2.0)) {
-    unsigned long long c[kCounts];
-    OVRO_CUDA_TRY(cudaMemcpyAsync(c, w.counts, sizeof(c), cudaMemcpyDeviceToHost, st));
-    OVRO_CUDA_TRY(cudaStreamSynchronize(st));
-    const unsigned long long cap = static_cast<unsigned long long>(entry_capacity(p));
-    if (c[kCountRows] > cap || c[kCountTiles] > cap) return OVRO_ERR_CAPACITY;
-  }
   return OVRO_OK;
 }
 
