@@ -1519,7 +1519,7 @@ PlanExtent plan_extent(int g, int n_ant, const double* ant, const PlanAxis& ax) 
   // the grid are held at 2^40), then half away from zero
   auto centre = [](double v) {
     constexpr double kRint = 6755399441055744.0, kFar = 1099511627776.0;
-    const double p = (std::min(std::max(v, -kFar), kFar) + kRint) - kRint;
+    const double p = ((v < kFar ? std::max(v, -kFar) : kFar) + kRint) - kRint;
     return static_cast<int>((p + std::copysign(kQ / 2.0, p)) * (1.0 / kQ));
   };
   // tiles of the rows kept that centre rows v0 .. v1 and columns u0 .. u1 touch
@@ -1555,7 +1555,9 @@ PlanExtent plan_extent(int g, int n_ant, const double* ant, const PlanAxis& ax) 
 // The call's tables and lists, made on the device without a synchronisation.
 // bases: the prepared records may hold weight-table offsets, because no listed
 // footprint moves by kTabMargin cells over the call's channels (one cell of
-// slack for a rounding of u Q that differs from the exact one).  A listed
+// slack for a rounding of u Q that differs from the exact one) and every frequency
+// is a number: with NaN among them the range spans the other channels alone, and the
+// offsets of that channel would lie outside the table.  A listed
 // |d| s is below (cmax + 1) Q at the smallest scale, so no centre moves by more
 // than (cmax + 1) (s_hi / s_lo - 1) + 1 cells; a footprint that moves by at most
 // two touches 3 x 3 tiles, its mirror as many: 18 entries, within the capacity
@@ -1579,8 +1581,10 @@ int upload_common(const ImgPlan& p, ImgWs& w, int n_ant, const double* h_ant,
   ax.s_lo = HUGE_VAL;
   ax.s_hi = -HUGE_VAL;
   double fmin = h_freq[0], fmax = h_freq[0];
+  bool finite = true;                                  // a channel without a position has no table offset
   for (int f = 0; f < n_chan; ++f) {
     const double sq = (h_freq[f] / (kCLight * du)) * static_cast<double>(kQ);
+    finite = finite && std::isfinite(sq);
     ax.s_lo = std::min(ax.s_lo, sq);
     ax.s_hi = std::max(ax.s_hi, sq);
     fmin = std::min(fmin, h_freq[f]);
@@ -1598,7 +1602,7 @@ int upload_common(const ImgPlan& p, ImgWs& w, int n_ant, const double* h_ant,
     if (e.entries > entry_capacity(p)) return OVRO_ERR_CAPACITY;
     move = e.move;
   }
-  w.bases = move + 1.0 <= kTabMargin;
+  w.bases = finite && move + 1.0 <= kTabMargin;
   const double* d_ant = w.axis;
   const double* d_freq = w.axis + 3 * static_cast<size_t>(n_ant);
   // a copy from pageable memory is staged before cudaMemcpyAsync returns, so
