@@ -16,7 +16,7 @@
 //                    interleaved per thread) and a pointer on the lower median,
 //                    so every step of the exact running median costs O(1).
 //      k_rank        full ranks (stable LSD radix sort) for the pixels whose
-//                    band or walk gave up; k_walk then takes them in full.
+//                    walk left the band; k_walk then takes them in full.
 //  a10 k_mf          subtracts the medians and, per 8 consecutive channels, takes
 //                    the 107-value neighbourhood as register prefix sums and
 //                    evaluates all 29 boxcars as prefix differences; keeps max
@@ -429,8 +429,32 @@ inline int band_ranks(int nc) {
 }
 
 // Keys k_rank_band can rank: the band and its boundary bins, whose keys share
-// the sign, the exponent and two mantissa bits (2 to 6% of a spectrum each).
+// the sign, the exponent and two mantissa bits (2 to 6% of a spectrum each).  When
+// more share them, many of them equal, the boundary keys are found exactly and
+// the candidates are the band itself.
 inline int band_keys(int nc) { return std::min(nc, band_ranks(nc) + std::max(128, nc / 10)); }
+
+// Words of k_rank_band's counters: the bins and their end, with ties lsd_sort's
+// digits by warp.
+__host__ __device__ constexpr int band_hist(int threads, bool ties) {
+  const int digits = 256 * (threads / 32 + 1);
+  return ties && digits > kBins + 4 ? digits : kBins + 4;
+}
+
+// No candidate: above the band, or below it (smaller than any bin | place << 11
+// otherwise).
+constexpr uint32_t kNoSlot = 0xffffffffu, kNoSlotBelow = 0xfffffffeu;
+// Keys of one bin beyond which k_rank_band gives a spectrum up: comparing 400 equal
+// ones of 4096 (51,468 pixels: 2.0 ms) costs less than the sort and the time
+// lost before it (2.7), 820 of them more (6.4).
+constexpr int kCrowd = 512;
+
+// A permutation of 0 .. n - 1 (n <= 16384, less than the prime) without order: equal values
+// come in the order of their channels, and a window's would then lie at one end
+// of the ranks they share, off the band when those outgrow it.  With this prime the
+// median of every fifth of them stays within 5 sqrt(n) ranks of the middle, for 400
+// drawn n (a band reaches 11 sqrt(nc) to each side).
+__device__ __forceinline__ uint32_t spread(uint32_t t, uint32_t n) { return t * 40529u % n; }
 
 // Block-wide exclusive scan of the kBins counters of hist: this thread's bins
 // (kBins / T consecutive ones) are left in c and the count before them returned.
@@ -489,9 +513,14 @@ __device__ __forceinline__ uint32_t scan_bins(const uint32_t* hist, uint32_t* wt
 //     values).  Threads take candidates here, not channels: a band is a
 //     quarter to a half of a spectrum.
 // Output: the sorted values of the band (sv [pixel][0 .. B)) and the stream
-// of band ranks; a spectrum whose candidates stay too many (ties) or are not
-// finite is listed in fail and marked in failed, to be ranked and walked in
-// full.
+// of band ranks.  Equal values spoil this: the candidates may stay too many, or the
+// comparisons within a bin cost their number squared (the channels whose deviation
+// is 0 are 0 in every pixel).  Those spectra, and those whose interval is not
+// finite, go to the list, and TIES ranks them: the two boundary keys are found
+// exactly, of the keys equal to one as many are taken as the band holds, and the
+// candidates are sorted.  A kernel of its own, as the code cost the others 7%.
+// 51,468 pixels x 4096 channels, 40% of them flagged: detection 35.1 -> 10.0 ms
+// (7.0 with none; 15.8 when every band was sorted by radix passes).
 // The kernel is issue bound (68% of issue slots, 190 instructions per 32 keys
 // where all are candidates).  Sorting the band by four 8-bit radix passes with
 // all 1024 threads of an SM on one pixel spent its time in the passes' counters
@@ -499,25 +528,28 @@ __device__ __forceinline__ uint32_t scan_bins(const uint32_t* hist, uint32_t* wt
 // pixels, radix passes -> now: 8192 channels 7.57 -> 2.02 ms, 4096 6.77 ->
 // 1.08 ms, 1024 (all ranks) 2.65 -> 0.62 ms.
 // T threads with KPT keys each: nc <= KPT T.
-template <int T, int KPT>
+template <int T, int KPT, bool TIES>
 __global__ void __launch_bounds__(T, 1024 / T)
 k_rank_band(const float* __restrict__ z, int n_valid, int nc, int h, int B, int cap, float* __restrict__ sv,
-            uint32_t* __restrict__ steps, int* __restrict__ fail, int* __restrict__ n_fail,
-            uint8_t* __restrict__ failed) {
+            uint32_t* __restrict__ steps, int* __restrict__ list, int* __restrict__ n_list) {
   constexpr int PER = kBins / T;
   extern __shared__ __align__(16) unsigned char smem[];
-  uint32_t* hist = reinterpret_cast<uint32_t*>(smem);             // [kBins], then the number of candidates
-  uint32_t* ka = hist + kBins + 4;                                 // [cap] candidate keys by bin
+  uint32_t* hist = reinterpret_cast<uint32_t*>(smem);             // [kBins], then the number of candidates; lsd_sort's
+  uint32_t* ka = hist + band_hist(T, TIES);                        // [cap] candidate keys by bin
   float* sorted = reinterpret_cast<float*>(ka + cap);              // [cap]
   uint16_t* rk = reinterpret_cast<uint16_t*>(sorted + cap);        // [nc] band rank or code
-  uint16_t* ic = rk + nc;                                          // [cap] candidate channels
+  uint16_t* ic = rk + nc;                                          // [cap] candidate channels, [cap] for lsd_sort
   const int r_lo = max(0, nc / 2 - B / 2), r_hi = min(nc - 1, r_lo + B - 1);
   __shared__ uint32_t wtot[32];
-  __shared__ int sel[4];                 // bin of r_lo, keys before it, bin of r_hi, keys up to its end
+  __shared__ int sel[5];                 // bin of ra, keys before it, bin of rb, keys up to its end and before it
+  __shared__ int2 same[2];               // rank of the first key equal to a boundary, and how many
+  __shared__ int ticket[2];              // of the keys equal to a boundary
   const int t = threadIdx.x;
   const bool vec = (nc & 3) == 0;
   for (int i = t; i < kBins; i += T) hist[i] = 0u;
-  for (int p = blockIdx.x; p < n_valid; p += gridDim.x) {
+  const int n_items = TIES ? min(*n_list, n_valid) : n_valid;
+  for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
+    const int p = TIES ? list[it] : it;
     const float* zp = z + static_cast<long long>(p) * nc;
     // key 4 i + u is channel 4 (i T + t) + u
     uint32_t key[KPT];
@@ -539,31 +571,38 @@ k_rank_band(const float* __restrict__ z, int n_valid, int nc, int h, int B, int 
       key[4 * i + 3] = f2key(q.w);
     }
     auto exists = [&](int i) { return 4 * ((i >> 2) * T + t) + (i & 3) < nc; };
+    if (TIES && t < 2) ticket[t] = 0;
     __syncthreads();                                               // hist is zero, the last pixel's arrays are free
-    // 1. the candidate interval [klo, khi], c_lo keys below it, m keys in it
-    uint32_t klo = 0u, khi = 0xffffffffu;
-    int sh = 21, c_lo = 0, m = nc;
-    for (;;) {
+    // histograms the keys of [base, top], `before` of them lower, and finds the bins
+    // of ranks ra and rb
+    auto locate = [&](uint32_t base, uint32_t top, int sh, int before, int ra, int rb) {
 #pragma unroll
       for (int i = 0; i < KPT; ++i)
-        if (exists(i) && key[i] >= klo && key[i] <= khi) atomicAdd(&hist[(key[i] - klo) >> sh], 1u);
+        if (exists(i) && key[i] >= base && key[i] <= top) atomicAdd(&hist[(key[i] - base) >> sh], 1u);
       __syncthreads();
       uint32_t c[PER];
-      uint32_t run = static_cast<uint32_t>(c_lo) + scan_bins<T>(hist, wtot, c);
+      uint32_t run = static_cast<uint32_t>(before) + scan_bins<T>(hist, wtot, c);
 #pragma unroll
       for (int u = 0; u < PER; ++u) {
-        if (run <= static_cast<uint32_t>(r_lo) && static_cast<uint32_t>(r_lo) < run + c[u]) {
+        if (run <= static_cast<uint32_t>(ra) && static_cast<uint32_t>(ra) < run + c[u]) {
           sel[0] = t * PER + u;
           sel[1] = static_cast<int>(run);
         }
-        if (run <= static_cast<uint32_t>(r_hi) && static_cast<uint32_t>(r_hi) < run + c[u]) {
+        if (run <= static_cast<uint32_t>(rb) && static_cast<uint32_t>(rb) < run + c[u]) {
           sel[2] = t * PER + u;
           sel[3] = static_cast<int>(run + c[u]);
+          if (TIES) sel[4] = static_cast<int>(run);
         }
         run += c[u];
         hist[t * PER + u] = 0u;
       }
       __syncthreads();
+    };
+    // 1. the candidates: keys of [klo, khi], c_lo keys below them, m in all
+    uint32_t klo = 0u, khi = 0xffffffffu;
+    int sh = 21, c_lo = 0, m = nc;
+    for (;;) {
+      locate(klo, khi, sh, c_lo, r_lo, r_hi);
       const uint32_t width = (static_cast<uint32_t>(sel[2] - sel[0]) << sh) + ((1u << sh) - 1u);
       klo += static_cast<uint32_t>(sel[0]) << sh;
       khi = min(khi, klo + width);
@@ -577,23 +616,67 @@ k_rank_band(const float* __restrict__ z, int n_valid, int nc, int h, int B, int 
       sh = next;
       __syncthreads();                                             // sel is read
     }
-    const float xlo = key2f(klo), xhi = key2f(khi);
-    const float span = xhi - xlo;
-    if (!(m <= cap && span >= 0.0f && span < INFINITY)) {          // the same for the whole CTA
-      if (t == 0) {
-        fail[atomicAdd(n_fail, 1)] = p;
-        failed[p] = 1;
+    const bool exact = TIES && m > cap;                            // many keys share a boundary's bin
+    if (TIES && exact) {
+      // the two boundary keys themselves: their bins by themselves, to single keys
+      const uint32_t first[2] = {klo, khi - ((1u << sh) - 1u)};
+      const int lower[2] = {c_lo, sel[4]};
+      for (int e = 0; e < 2; ++e) {
+        uint32_t base = e ? first[1] : first[0];
+        int before = e ? lower[1] : lower[0], s = sh;
+        do {
+          __syncthreads();                                         // sel is read
+          const uint32_t top = base + ((1u << s) - 1u);
+          s = max(0, s - 11);
+          locate(base, top, s, before, e ? r_hi : r_lo, e ? r_hi : r_lo);
+          base += static_cast<uint32_t>(sel[0]) << s;
+          before = sel[1];
+        } while (s > 0);
+        if (t == 0) same[e] = make_int2(before, sel[3] - before);
+        (e ? khi : klo) = base;
       }
+    }
+    const float xlo = key2f(klo), span = key2f(khi) - xlo;
+    const bool finite = span >= 0.0f && span < INFINITY;
+    if (!TIES && !(m <= cap && finite)) {                          // the same for the whole CTA
+      if (t == 0) list[atomicAdd(n_list, 1)] = p;
       continue;                                                    // hist is zero again
     }
-    // 2. bins linear in the value: a monotone map, so bins order the keys
-    const float scale = span > 0.0f ? static_cast<float>(kBins) / span : 0.0f;
-    auto bin_of = [&](uint32_t k) { return min(static_cast<int>((key2f(k) - xlo) * scale), kBins - 1); };
     uint32_t at[KPT];                                              // bin | place within the bin << 11
+    if constexpr (TIES) {
+#pragma unroll
+      for (int i = 0; i < KPT; ++i) at[i] = exists(i) && key[i] >= klo && key[i] <= khi ? 0u : key[i] < klo ? kNoSlotBelow : kNoSlot;
+      if (exact) {
+        // of the keys equal to a boundary, those whose ranks lie in the band
+        c_lo = r_lo;
+        m = r_hi - r_lo + 1;
+        const int lane = t & 31;
+        __syncthreads();                                           // same is written
+#pragma unroll
+        for (int i = 0; i < KPT; ++i)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const bool mine = at[i] == 0u && key[i] == (e ? khi : klo) && (e == 0 || khi != klo);
+            const unsigned all = __ballot_sync(0xffffffffu, mine);
+            if (all == 0u) continue;
+            int turn = 0;
+            if (lane == __ffs(all) - 1) turn = atomicAdd(&ticket[e], __popc(all));
+            turn = __shfl_sync(0xffffffffu, turn, __ffs(all) - 1) + __popc(all & ((1u << lane) - 1u));
+            if (mine) {
+              const int r = same[e].x + static_cast<int>(spread(turn, same[e].y));
+              if (r < r_lo || r > r_hi) at[i] = r < r_lo ? kNoSlotBelow : kNoSlot;
+            }
+          }
+      }
+    }
+    // 2. bins linear in the value: a monotone map, so bins order the keys (one bin
+    // when the interval has no finite width)
+    const float scale = span > 0.0f && finite ? static_cast<float>(kBins) / span : 0.0f;
+    auto bin_of = [&](uint32_t k) { return min(static_cast<int>((key2f(k) - xlo) * scale), kBins - 1); };
 #pragma unroll
     for (int i = 0; i < KPT; ++i) {
-      at[i] = 0xffffffffu;
-      if (exists(i) && key[i] >= klo && key[i] <= khi) {
+      if (!TIES) at[i] = kNoSlot;
+      if (TIES ? at[i] == 0u : exists(i) && key[i] >= klo && key[i] <= khi) {
         const int b = bin_of(key[i]);
         at[i] = static_cast<uint32_t>(b) | (atomicAdd(&hist[b], 1u) << 11);
       }
@@ -613,8 +696,14 @@ k_rank_band(const float* __restrict__ z, int n_valid, int nc, int h, int B, int 
     // 3. the candidates at their bins; codes for the other channels
 #pragma unroll
     for (int i = 0; i < KPT; ++i)
-      if (at[i] != 0xffffffffu) {
-        const uint32_t j = hist[at[i] & (kBins - 1)] + (at[i] >> 11);
+      if (at[i] < kNoSlotBelow) {
+        const uint32_t b = at[i] & (kBins - 1);
+        uint32_t j = at[i] >> 11;
+        if constexpr (TIES) {
+          const uint32_t n = hist[b + 1] - hist[b];
+          if (n > 32u) j = spread(j, n);
+        }
+        j += hist[b];
         ka[j] = key[i];
         ic[j] = static_cast<uint16_t>(4 * ((i >> 2) * T + t) + (i & 3));
       }
@@ -622,7 +711,8 @@ k_rank_band(const float* __restrict__ z, int n_valid, int nc, int h, int B, int 
     for (int i = 0; i < KPT; i += 4) {
       uint32_t c[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) c[u] = static_cast<uint32_t>(key[i + u] < klo ? kRankBelow : kRankAbove) & 0xffffu;
+      for (int u = 0; u < 4; ++u)
+        c[u] = static_cast<uint32_t>((TIES ? at[i + u] == kNoSlotBelow : key[i + u] < klo) ? kRankBelow : kRankAbove) & 0xffffu;
       const int k = 4 * ((i >> 2) * T + t);
       if (k + 3 < nc) {
         *reinterpret_cast<uint2*>(rk + k) = make_uint2(c[0] | (c[1] << 16), c[2] | (c[3] << 16));
@@ -633,20 +723,42 @@ k_rank_band(const float* __restrict__ z, int n_valid, int nc, int h, int B, int 
       }
     }
     __syncthreads();
-    for (int j = t; j < m; j += T) {
-      const uint32_t k = ka[j];
-      const int b = bin_of(k);
-      const int j0 = static_cast<int>(hist[b]), j1 = static_cast<int>(hist[b + 1]);
-      int r = j0;
-      for (int o = j0; o < j1; ++o) {
-        const uint32_t other = ka[o];
-        r += (other < k || (other == k && o < j)) ? 1 : 0;
-      }
-      sorted[r] = key2f(k);
+    auto code = [&](int r) {
       r -= r_lo - c_lo;
-      rk[ic[j]] = static_cast<uint16_t>(r < 0 ? kRankBelow : (r >= B ? kRankAbove : r));
+      return static_cast<uint16_t>(r < 0 ? kRankBelow : (r >= B ? kRankAbove : r));
+    };
+    if constexpr (TIES) {
+      lsd_sort(ka, ic, reinterpret_cast<uint32_t*>(sorted), ic + cap, m, hist, wtot);
+      for (int j = t; j < m; j += T) {
+        sorted[j] = key2f(ka[j]);
+        rk[ic[j]] = code(j);
+      }
+      __syncthreads();
+    } else {
+      bool crowded = false;
+      for (int j = t; j < m; j += T) {
+        const uint32_t k = ka[j];
+        const int b = bin_of(k);
+        const int j0 = static_cast<int>(hist[b]), j1 = static_cast<int>(hist[b + 1]);
+        if (j1 - j0 > kCrowd) {
+          crowded = true;
+          break;
+        }
+        int r = j0;
+        for (int o = j0; o < j1; ++o) {
+          const uint32_t other = ka[o];
+          r += (other < k || (other == k && o < j)) ? 1 : 0;
+        }
+        sorted[r] = key2f(k);
+        rk[ic[j]] = code(r);
+      }
+      crowded = __syncthreads_or(crowded);
+      if (crowded) {
+        if (t == 0) list[atomicAdd(n_list, 1)] = p;
+        for (int i = t; i < kBins; i += T) hist[i] = 0u;
+        continue;
+      }
     }
-    __syncthreads();
     for (int i = t; i < kBins; i += T) hist[i] = 0u;
     float* svp = sv + static_cast<long long>(p) * nc;
     for (int j = t; j <= r_hi - r_lo; j += T) svp[j] = sorted[r_lo - c_lo + j];
@@ -757,16 +869,15 @@ constexpr int kBandThreads = 128;
 // chain of dependent steps).
 //   fail: the band stream (nwords * 32 band ranks); a segment whose median
 //     leaves the band gives up, and its pixel is listed once in fail (k_rank
-//     and the full walk redo it), behind the pixels k_rank_band listed there.
+//     and the full walk redo it).
 //   no fail: the full rank set (nwords = nc / 32 rounded up); with a pixel list
-//     (the band kernels' failures) item i walks list[i], i < *n_list.
+//     (the band walk's failures) item i walks list[i], i < *n_list.
 // seg_len is a multiple of 4, so every segment's steps start on a chunk.
-//     The pixels marked in failed have no band stream and are left out.
 template <int T>
 __global__ void __launch_bounds__(T)
 k_walk(const uint32_t* __restrict__ steps, int n_valid, int nc, int h, int n_seg, int seg_len, int nwords,
        uint32_t* __restrict__ med, const int* __restrict__ list, const int* __restrict__ n_list,
-       int* __restrict__ fail, int* __restrict__ n_fail, const uint8_t* __restrict__ failed) {
+       int* __restrict__ fail, int* __restrict__ n_fail) {
   extern __shared__ uint32_t bits_all[];
   const int t = threadIdx.x;
   const int item = (blockIdx.x * T + t) / n_seg;
@@ -778,7 +889,6 @@ k_walk(const uint32_t* __restrict__ steps, int n_valid, int nc, int h, int n_seg
     live = item < min(*n_list, n_valid);
     p = live ? list[item] : 0;
   }
-  if (failed) live = live && !failed[p];
   bool ok = true;
   if (live) {
     for (int w = -1; w <= nwords; ++w) bits[w * T] = 0u;
@@ -1499,8 +1609,7 @@ struct DetectWs {
   float* sv;
   uint32_t* steps;
   uint32_t* med;         // [pixel][channel] median ranks of the current coarse block
-  int* fail;             // pixels whose band ranking or band walk gave up
-  uint8_t* failed;       // [pixel] 1: the band ranking gave up
+  int* fail;             // pixels left to the ties kernel, then those whose band walk gave up
   float* snr;
   uint8_t* width;
   unsigned long long* hist;
@@ -1509,7 +1618,8 @@ struct DetectWs {
   int* nfft;
   int* ovf;
   CandRec* recs;
-  int* count;            // [0] gathered values, [1] overflow pairs, [2] candidates, [3] band-walk failures
+  int* count;            // [0] gathered values, [1] overflow pairs, [2] candidates, [3] band-walk failures,
+                         // [4] spectra left to the ties kernel
   uint8_t* want;         // [kMaxBins] bins gathered in one pass
 };
 
@@ -1529,7 +1639,6 @@ DetectWs carve_detect(void* ws, size_t bytes, const DetectPlan& p, size_t* need)
   w.steps = c.take<uint32_t>(static_cast<size_t>(p.n_valid) * p.max_steps);
   w.med = c.take<uint32_t>(blk);
   w.fail = c.take<int>(p.n_valid > 0 ? p.n_valid : 1);
-  w.failed = c.take<uint8_t>(p.n_valid > 0 ? p.n_valid : 1);
   w.snr = c.take<float>(static_cast<size_t>(p.n_vox));
   w.width = c.take<uint8_t>(static_cast<size_t>(p.n_vox));
   w.hist = c.take<unsigned long long>(kMaxBins);
@@ -1538,7 +1647,7 @@ DetectWs carve_detect(void* ws, size_t bytes, const DetectPlan& p, size_t* need)
   w.nfft = c.take<int>(p.n_coarse);
   w.ovf = c.take<int>(np);
   w.recs = c.take<CandRec>(p.cand_cap);
-  w.count = c.take<int>(4);
+  w.count = c.take<int>(5);
   w.want = c.take<uint8_t>(kMaxBins);
   *need = c.used;
   return w;
@@ -1594,28 +1703,39 @@ int run_filter_coarse(int c, const float* img_block, const DetectPlan& p, const 
   }
   {
     // Band ranks and the band walk for every pixel, then full ranks and the full
-    // walk for the pixels either gave up (a median that left the band, ties).
+    // walk for the pixels whose median left the band.
     const int band = band_ranks(nc), cap = band_keys(nc);
     // 8 or 16 keys a thread: a short spectrum takes a small CTA, so that an SM
     // has enough of them to cover one another's barriers
     const int threads = nc <= 1024 ? 128 : nc <= 4096 ? 256 : nc <= 8192 ? 512 : 1024;
-    auto band_kernel = nc <= 1024 ? k_rank_band<128, 8> : nc <= 2048 ? k_rank_band<256, 8>
-                       : nc <= 4096 ? k_rank_band<256, 16> : nc <= 8192 ? k_rank_band<512, 16>
-                       : k_rank_band<1024, 16>;
-    const size_t sm_band = (kBins + 4 + 2 * static_cast<size_t>(cap)) * 4 + (static_cast<size_t>(nc) + cap) * 2;
+    auto band_kernel = nc <= 1024 ? k_rank_band<128, 8, false> : nc <= 2048 ? k_rank_band<256, 8, false>
+                       : nc <= 4096 ? k_rank_band<256, 16, false> : nc <= 8192 ? k_rank_band<512, 16, false>
+                       : k_rank_band<1024, 16, false>;
+    auto ties_kernel = nc <= 1024 ? k_rank_band<128, 8, true> : nc <= 2048 ? k_rank_band<256, 8, true>
+                       : nc <= 4096 ? k_rank_band<256, 16, true> : nc <= 8192 ? k_rank_band<512, 16, true>
+                       : k_rank_band<1024, 16, true>;
+    auto sm_bytes = [&](bool ties) {
+      return (band_hist(threads, ties) + 2 * static_cast<size_t>(cap)) * 4 +
+             (static_cast<size_t>(nc) + (ties ? 2 : 1) * cap) * 2;
+    };
+    const size_t sm_band = sm_bytes(false), sm_ties = sm_bytes(true);
     OVRO_CUDA_TRY(cudaFuncSetAttribute(band_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(sm_band)));
+    OVRO_CUDA_TRY(cudaFuncSetAttribute(ties_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(sm_ties)));
     const int W = 32;                                // k_rank: one CTA of 1024 threads per SM (shared memory)
     const size_t sm_rank = (256 * (W + 1) + 32) * 4 + static_cast<size_t>(nc) * 12;
     OVRO_CUDA_TRY(cudaFuncSetAttribute(k_rank, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(sm_rank)));
     // CTAs per SM (each CTA loops over pixels; the outputs do not depend on it)
     auto rank = [&](int per_sm) -> int {
-      OVRO_CUDA_TRY(cudaMemsetAsync(w.count + 3, 0, sizeof(int), st));
-      OVRO_CUDA_TRY(cudaMemsetAsync(w.failed, 0, p.n_valid, st));
+      OVRO_CUDA_TRY(cudaMemsetAsync(w.count + 3, 0, 2 * sizeof(int), st));
       OVRO_PROF("k_rank", st);
       band_kernel<<<std::min(p.n_valid, per_sm * nsm), threads, sm_band, st>>>(
-          w.zbuf, p.n_valid, nc, p.half[c], band, cap, w.sv, w.steps, w.fail, w.count + 3, w.failed);
+          w.zbuf, p.n_valid, nc, p.half[c], band, cap, w.sv, w.steps, w.fail, w.count + 4);
+      OVRO_LAUNCH_CHECK();
+      ties_kernel<<<std::min(p.n_valid, 1024 / threads * nsm), threads, sm_ties, st>>>(
+          w.zbuf, p.n_valid, nc, p.half[c], band, cap, w.sv, w.steps, w.fail, w.count + 4);
       OVRO_LAUNCH_CHECK();
       return OVRO_OK;
     };
@@ -1641,7 +1761,7 @@ int run_filter_coarse(int c, const float* img_block, const DetectPlan& p, const 
         OVRO_PROF("k_walk", st);
         k_walk<kBandThreads><<<static_cast<int>((thr + kBandThreads - 1) / kBandThreads), kBandThreads, sm_walk,
                                st>>>(w.steps, p.n_valid, nc, p.half[c], n_seg, seg_len, band / 32, w.med, nullptr,
-                                     nullptr, w.fail, w.count + 3, w.failed);
+                                     nullptr, w.fail, w.count + 3);
         OVRO_LAUNCH_CHECK();
       }
       {
@@ -1653,7 +1773,7 @@ int run_filter_coarse(int c, const float* img_block, const DetectPlan& p, const 
       OVRO_PROF("k_walk", st);
       k_walk<kWalkThreads><<<static_cast<int>((thr + kWalkThreads - 1) / kWalkThreads), kWalkThreads, sm_full,
                              st>>>(w.steps, p.n_valid, nc, p.half[c], n_seg, seg_len, nwords, w.med, w.fail,
-                                   w.count + 3, nullptr, nullptr, nullptr);
+                                   w.count + 3, nullptr, nullptr);
       OVRO_LAUNCH_CHECK();
       return OVRO_OK;
     };
