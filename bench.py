@@ -268,14 +268,16 @@ def next_row_measurements(volt, cfg, n_kept_vis, kern, steps, dev, vis_sub, pos,
     T, nc, N = 8, 1024, cfg.image_size
     g = torch.Generator(device=dev).manual_seed(5)
     zsub = torch.randn((T, nc, N, N), generator=g, device=dev, dtype=torch.float32)
-    freqs = np.arange(nc, dtype=np.float64)
-    ms = _kernel_ms(lambda: ovro.drift_search(zsub, cfg.cell, [nc], freqs, 12.0), ["k_drift"])
+    drift_freqs = np.arange(nc, dtype=np.float64)
+    ms = _kernel_ms(lambda: ovro.drift_search(zsub, cfg.cell, [nc], drift_freqs, 12.0), ["k_drift"])
     d = (np.arange(N) - N // 2) * cfg.cell
     nvox = int(((d[None, :] ** 2 + d[:, None] ** 2) < 1.0).sum()) * nc
     out["drift_search"] = {"workload": "T = 8 sub-integrations x 1024 channels x 256^2 (in-horizon voxels)",
                            "k_drift_ms": ms, "voxels_per_s": nvox / (ms * 1e-3),
                            "path_sums_per_s": nvox * (2 * T - 1) / (ms * 1e-3),
-                           "smem_loads_per_voxel": (2 * T - 1) * T}
+                           # T + T (T - 1) / 4: four start channels a thread, row t at the 4 + 2 t
+                           # channels its paths reach, through L1
+                           "loads_per_voxel": T + T * (T - 1) / 4}
     del zsub
     # vetting: 2000 candidates on a 256-channel 128^2 cube
     nc, N = 256, 128
