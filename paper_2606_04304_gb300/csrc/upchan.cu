@@ -471,12 +471,17 @@ int launch_upchan(int log2n, const UpchanArgs& a, cudaStream_t st) {
 }
 
 // G inputs per CTA from the autotuner: every G with F <= G <= 64 whose shared
-// memory fits (results do not depend on G).
+// memory fits (results do not depend on G).  Untuned, the widest, halved while the
+// CTAs still fit the SMs one each: a call of few spectra of few inputs is a chain of
+// the G / F transforms of a CTA (9 spectra of 8192 points: 16 inputs 57 us with G = 8,
+// 24 with 1, and 104 and 28 with FP32 spectra; 40 inputs 57 with G = 8, 34 with 4).
 int launch_upchan_tuned(int l, UpchanArgs a, cudaStream_t st) {
   const int F = l >= 13 ? 1 : (l < 4 ? 256 : (8192 >> l));
   int np2 = 1;
   while (np2 < a.n_input) np2 *= 2;
-  const int g0 = group_for(l, a.n_input);
+  int g0 = group_for(l, a.n_input);
+  auto ctas = [&](int g) { return static_cast<long long>((a.n_input + g - 1) / g) * a.n_spec; };
+  while (l >= 4 && g0 / 2 >= F && ctas(g0 / 2) <= num_sms()) g0 /= 2;
   std::vector<int> cands;
   for (int g = F; g <= 64; g *= 2) {
     if (g > np2 && g > F) break;
