@@ -64,98 +64,9 @@ __device__ __forceinline__ void dft_reg(float2 (&v)[R]) {
   for (int i = 0; i < R; ++i) v[i] = t[i];
 }
 
-
-// Forward FFTs (exp(-2 pi i k n / N)) of `count` rows of length N = 2^LOG2N
-// stored in `a` with row stride `ld` >= N; `b` is a scratch buffer of the same
-// shape.  Stockham auto-sort: radix-16 passes, then one radix-2/4/8 pass.
-// All threads of the block take part; returns the buffer holding the result.
-// tw: omega_{N * tw_stride}^k table.
-template <int LOG2N>
-__device__ float2* fft_rows_pingpong(float2* a, float2* b, int count, int ld,
-                                     const float2* __restrict__ tw, int tw_stride) {
-  constexpr int N = 1 << LOG2N;
-  constexpr int n16 = LOG2N / 4;
-  constexpr int rem = LOG2N % 4;
-  constexpr int n_pass = n16 + (rem ? 1 : 0);
-  int Ns = 1;
-  float2* src = a;
-  float2* dst = b;
-#pragma unroll 1
-  for (int p = 0; p < n_pass; ++p) {
-    const int R = (p < n16) ? 16 : (1 << rem);
-    const int per = N / R;
-    const int total = count * per;
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-      const int f = t / per, j = t - f * per;
-      const int k = j & (Ns - 1);
-      const float2* s = src + f * ld;
-      float2* d = dst + f * ld;
-      const int o = (j / Ns) * Ns * R + k;
-      const int base = k * (N / (Ns * R));
-      if (R == 16) {
-        float2 v[16];
-#pragma unroll
-        for (int r = 0; r < 16; ++r) v[r] = s[j + r * per];
-        if (Ns > 1) {
-#pragma unroll
-          for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], __ldg(tw + (r * base) * tw_stride));
-        }
-        dft_reg<16>(v);
-#pragma unroll
-        for (int r = 0; r < 16; ++r) d[o + r * Ns] = v[r];
-      } else if (R == 8) {
-        float2 v[8];
-#pragma unroll
-        for (int r = 0; r < 8; ++r) v[r] = s[j + r * per];
-        if (Ns > 1) {
-#pragma unroll
-          for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], __ldg(tw + (r * base) * tw_stride));
-        }
-        dft_reg<8>(v);
-#pragma unroll
-        for (int r = 0; r < 8; ++r) d[o + r * Ns] = v[r];
-      } else if (R == 4) {
-        float2 v[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) v[r] = s[j + r * per];
-        if (Ns > 1) {
-#pragma unroll
-          for (int r = 1; r < 4; ++r) v[r] = cmul(v[r], __ldg(tw + (r * base) * tw_stride));
-        }
-        dft_reg<4>(v);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) d[o + r * Ns] = v[r];
-      } else {
-        float2 v[2];
-        v[0] = s[j];
-        v[1] = s[j + per];
-        if (Ns > 1) v[1] = cmul(v[1], __ldg(tw + base * tw_stride));
-        dft_reg<2>(v);
-        d[o] = v[0];
-        d[o + Ns] = v[1];
-      }
-    }
-    __syncthreads();
-    float2* t = src; src = dst; dst = t;
-    Ns *= R;
-  }
-  return src;
-}
-
-}  // namespace ovro
-
-namespace ovro {
-
 // Shared-memory index with one pad slot per 16 elements: Stockham writes at
 // stride 16 become conflict-free.
 __device__ __forceinline__ int pad16(int x) { return x + (x >> 4); }
-
-// The threads of one transform group: thread `tid` of `n`, and their barrier.
-struct CtaGroup {
-  __device__ __forceinline__ int tid() const { return threadIdx.x; }
-  __device__ __forceinline__ int size() const { return blockDim.x; }
-  __device__ __forceinline__ void sync() const { __syncthreads(); }
-};
 
 // One radix-R butterfly of the pass after NS points, in registers: x[r] omega_G^(k r
 // G / (NS R)), then the DFT.
@@ -188,26 +99,26 @@ __device__ __forceinline__ void stockham_butterfly(float2 (&x)[R], int k, Tw&& t
 // load(f, x, slot) gives element x of row f of the pass's input, slot (0 .. 15,
 // compile-time) being which of the thread's 16 values it is; store(f, x, v) takes
 // element x of its output.  in_place: the output may overlap the input (every
-// read completes before the first write) and is complete for the group when the
+// read completes before the first write) and is complete for the CTA when the
 // pass returns.  tw(i, ns, m, k) = omega_G^i, i = k (G / (NS R)) 2^m: where it lies in
 // a table by passes, for tables laid out so.
-template <int R, int NS, int G, class Group, class Load, class Tw, class Store>
-__device__ __forceinline__ void stockham_pass(const Group& group, bool in_place, Load&& load, Tw&& tw, Store&& store) {
+template <int R, int NS, int G, class Load, class Tw, class Store>
+__device__ __forceinline__ void stockham_pass(bool in_place, Load&& load, Tw&& tw, Store&& store) {
   // every thread holds exactly 16 values: 16 / R butterflies of radix R
   constexpr int NB = 16 / R;
   constexpr int per = G / R;
-  const int T = group.size();
+  const int T = blockDim.x;
   float2 v[16];
   int fj[NB];
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
-    const int gb = group.tid() + b * T;
+    const int gb = threadIdx.x + b * T;
     const int f = gb / per, j = gb - f * per;
     fj[b] = gb;
 #pragma unroll
     for (int r = 0; r < R; ++r) v[b * R + r] = load(f, j + r * per, b * R + r);
   }
-  if (in_place) group.sync();
+  if (in_place) __syncthreads();
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
     const int f = fj[b] / per, j = fj[b] - f * per;
@@ -220,7 +131,7 @@ __device__ __forceinline__ void stockham_pass(const Group& group, bool in_place,
 #pragma unroll
     for (int r = 0; r < R; ++r) store(f, o + r * NS, x[r]);
   }
-  if (in_place) group.sync();
+  if (in_place) __syncthreads();
 }
 
 // The last two passes at once, of radix 16 after NS points and of radix R after
@@ -228,11 +139,11 @@ __device__ __forceinline__ void stockham_pass(const Group& group, bool in_place,
 // lanes 32 / R apart and swap them by shuffles, which saves a trip through the
 // exchange buffer and its barriers (of radix 8 the outputs of a warp lie so far apart
 // that they cost as much).  The same arithmetic as the two passes.
-template <int R, int NS, int G, class Group, class Load, class Tw, class Store>
-__device__ __forceinline__ void stockham_tail(const Group& group, Load&& load, Tw&& tw, Store&& store) {
+template <int R, int NS, int G, class Load, class Tw, class Store>
+__device__ __forceinline__ void stockham_tail(Load&& load, Tw&& tw, Store&& store) {
   constexpr int per = G / 16, KK = 32 / R;
   static_assert(per == NS * R && NS % KK == 0, "whole warps per row");
-  const int f = group.tid() / per, jj = group.tid() % per;
+  const int f = threadIdx.x / per, jj = threadIdx.x % per;
   const int g = (jj & 31) / KK, k = (jj >> 5) * KK + (jj & (KK - 1)), j = g * NS + k;
   float2 v[16];
 #pragma unroll
@@ -264,15 +175,14 @@ __device__ __forceinline__ void stockham_tail(const Group& group, Load&& load, T
   }
 }
 
-// Forward FFTs of rows of G = 2^LOG2G points, 16 <= G <= 16384, by a group of
-// threads with size * 16 == rows * G: radix-16 passes, then one of radix 2, 4 or
+// Forward FFTs of rows of G = 2^LOG2G points, 16 <= G <= 16384, by the whole CTA
+// with blockDim.x * 16 == rows * G: radix-16 passes, then one of radix 2, 4 or
 // 8, exchanging through `a` (row f at a[f * ldp], element x at pad16(x)).  The
 // first pass reads its input through load0(f, x, slot) and may overlap `a`; the
 // last one hands its results to store(f, x, v): in_place when they overlap `a`, which
 // TAIL (the last two passes at once, where there are two and a shorter one) rules out.
-template <int LOG2G, bool TAIL, class Group, class Load, class Tw, class Store>
-__device__ __forceinline__ void fft_rows_io(const Group& group, float2* a, int ldp, bool in_place, Load&& load0,
-                                            Tw&& tw, Store&& store) {
+template <int LOG2G, bool TAIL, class Load, class Tw, class Store>
+__device__ __forceinline__ void fft_rows_io(float2* a, int ldp, bool in_place, Load&& load0, Tw&& tw, Store&& store) {
   constexpr int G = 1 << LOG2G;
   constexpr int n16 = LOG2G / 4;
   constexpr int rem = LOG2G % 4;
@@ -281,30 +191,30 @@ __device__ __forceinline__ void fft_rows_io(const Group& group, float2* a, int l
   auto get = [&](int f, int x, int) { return a[f * ldp + pad16(x)]; };
   auto put = [&](int f, int x, float2 v) { a[f * ldp + pad16(x)] = v; };
   if constexpr (n16 == 1 && rem == 0) {
-    stockham_pass<16, 1, G>(group, in_place, load0, tw, store);
+    stockham_pass<16, 1, G>(in_place, load0, tw, store);
   } else {
-    stockham_pass<16, 1, G>(group, true, load0, tw, put);
+    stockham_pass<16, 1, G>(true, load0, tw, put);
     if constexpr (n16 == 2 && rem == 0) {
-      stockham_pass<16, 16, G>(group, in_place, get, tw, store);
+      stockham_pass<16, 16, G>(in_place, get, tw, store);
     } else {
-      if constexpr (n16 == 3) stockham_pass<16, 16, G>(group, true, get, tw, put);
+      if constexpr (n16 == 3) stockham_pass<16, 16, G>(true, get, tw, put);
       if constexpr (n16 == 3 && rem == 0) {
-        stockham_pass<16, 256, G>(group, in_place, get, tw, store);
+        stockham_pass<16, 256, G>(in_place, get, tw, store);
       } else if constexpr (n16 >= 2 && rem <= 2 && TAIL) {
-        stockham_tail<1 << rem, NSR / 16, G>(group, get, tw, store);
+        stockham_tail<1 << rem, NSR / 16, G>(get, tw, store);
       } else {
-        if constexpr (n16 >= 2) stockham_pass<16, NSR / 16, G>(group, true, get, tw, put);
-        stockham_pass<1 << rem, NSR, G>(group, in_place, get, tw, store);
+        if constexpr (n16 >= 2) stockham_pass<16, NSR / 16, G>(true, get, tw, put);
+        stockham_pass<1 << rem, NSR, G>(in_place, get, tw, store);
       }
     }
   }
 }
 
-// The same by the whole CTA, in place.
+// The same in place.
 template <int LOG2G, class Load, class Tw>
 __device__ void fft_rows_inplace_f(float2* a, int ldp, Load&& load0, Tw&& tw) {
   fft_rows_io<LOG2G, false>(
-      CtaGroup{}, a, ldp, true, [&](int f, int x, int) { return load0(f, x); },
+      a, ldp, true, [&](int f, int x, int) { return load0(f, x); },
       [&](int i, auto, int, int) { return tw(i); },
       [&](int f, int x, float2 v) { a[f * ldp + pad16(x)] = v; });
 }

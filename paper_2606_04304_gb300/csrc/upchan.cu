@@ -3,13 +3,14 @@
 // Section 2.1 of the paper: each ~24 kHz coarse channel is upchannelized by an
 // FFT over its time samples, and the fine-channel voltages are correlated by an
 // 8-bit X-engine.  One CTA handles one spectrum (N consecutive samples) of a
-// group of G adjacent inputs: it stages the G-byte-wide rows of packed samples
-// in shared memory, runs F FFTs at a time (Stockham auto-sort, radix-16 passes
-// through a padded shared exchange buffer, 16 complex values per thread in
-// registers), requantises the bins into a staging tile and writes the int8
-// spectra for all G inputs with row-contiguous stores, so the output for fine
-// channel k' is one 2G-byte run in [k'][spectrum][input] order -- the layout
-// the X-engine reads.
+// group of G adjacent inputs: it transposes the G-byte-wide rows of packed samples
+// into a tile of one row per input in shared memory, runs F FFTs at a time
+// (Stockham auto-sort, radix-16 passes through a padded exchange buffer, 16 complex
+// values per thread in registers), requantises the bins from registers into the
+// room of the samples they came from, and writes the int8 spectra for all G inputs
+// with row-contiguous stores, so the output for fine channel k' is one 2G-byte run
+// in [k'][spectrum][input] order -- the layout the X-engine reads.  (N < 16: a
+// thread an FFT, samples and bins staged side by side.)
 #include <cmath>
 #include <mutex>
 #include <numeric>
@@ -377,7 +378,7 @@ k_upchan_p2(UpchanArgs a) {
     };
     if constexpr (wide) {
       // through the exchange buffer: F neighbouring inputs make a row of 8 F bytes
-      fft_rows_io<LOG2N, false>(CtaGroup{}, buf, LDP, true, sample, tw,
+      fft_rows_io<LOG2N, false>(buf, LDP, true, sample, tw,
                                 [&](int f, int k, float2 X) { buf[f * LDP + pad16(k)] = X; });
 #pragma unroll 8
       for (int idx = tid; idx < F * N; idx += P::THREADS) {
@@ -386,7 +387,7 @@ k_upchan_p2(UpchanArgs a) {
       }
     } else {
       // one pass alone: its bins overlap its samples
-      fft_rows_io<LOG2N, true>(CtaGroup{}, buf, LDP, LOG2N == 4, sample, tw, bin);
+      fft_rows_io<LOG2N, true>(buf, LDP, LOG2N == 4, sample, tw, bin);
     }
     __syncthreads();       // buf reused by the next F inputs, the bins complete
   }
