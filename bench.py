@@ -83,7 +83,7 @@ def _traffic_table():
 KERNEL_SRC = {"k_upchan": "upchan.cu", "k_upchan_mr": "upchan_mr.cu", "k_xeng_tc": "xengine.cu",
               "k_grid_prep": "imaging.cu", "k_grid_tiles": "imaging.cu", "k_fft_rows": "imaging.cu", "k_fft_cols": "imaging.cu",
               "k_stats": "detect.cu", "k_ztrans": "detect.cu", "k_rank": "detect.cu", "k_walk": "detect.cu",
-              "k_median_sub": "detect.cu", "k_mf": "detect.cu", "k_nms_warp": "detect.cu",
+              "k_mf": "detect.cu", "k_nms_warp": "detect.cu",
               "k_gather_bins": "detect.cu", "k_drift": "drift.cu"}
 
 
@@ -197,7 +197,8 @@ def roofline_models(cfg, n_kept_vis, peaks):
         # z' = z - median as a pass of its own (read ranks and z, write z'): k_mf
         # does it while staging, so no launch carries this name
         "k_median_sub": ("hbm", vox * 12, "B", cube),
-        # boxcars: read z', write SNR and width
+        # boxcars: read z, write SNR and width (the median ranks and the band's
+        # values that the kernel stages as well are intermediates)
         "k_mf": ("hbm", vox * 9, "B", cube),
         # NMS: one pass reading the SNR cube (the detections are few)
         "k_nms_warp": ("hbm", vox * 4, "B", cube),
@@ -414,7 +415,7 @@ def _case_drift(repeats=2):
         ovro.drift_search(zsub, 2.0 / 128, [512], freqs, 12.0)
 
 
-_DET = ("k_stats", "k_ztrans", "k_rank", "k_walk", "k_median_sub", "k_mf", "k_nms_warp", "k_gather_bins")
+_DET = ("k_stats", "k_ztrans", "k_rank", "k_walk", "k_mf", "k_nms_warp", "k_gather_bins")
 # per case: calls made, the work of one call per kernel, and the unit of that work
 CASE_META = {
     "imaging": (3, {k: 256 for k in ("k_grid_prep", "k_grid_tiles", "k_fft_rows", "k_fft_cols")},
@@ -841,7 +842,7 @@ def run_ours(args):
     torch.cuda.synchronize()
     stages = {"upchan": ("k_upchan",), "correlate": ("k_xeng_tc", "k_xeng_simt"),
               "grid_image": ("k_grid_prep", "k_grid_tiles", "k_fft_rows", "k_fft_cols"),
-              "detect": ("k_stats", "k_ztrans", "k_rank", "k_walk", "k_median_sub", "k_mf", "k_nms_warp")}
+              "detect": ("k_stats", "k_ztrans", "k_rank", "k_walk", "k_mf", "k_nms_warp")}
     stage_ms = {st: sum(kern[k][0] for k in ks if k in kern) / n_trace for st, ks in stages.items()}
 
     # ---- end to end through host buffers: H2D of the voltages, D2H of the candidates
